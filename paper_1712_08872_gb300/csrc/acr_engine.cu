@@ -436,12 +436,12 @@ class Engine : public EngineBase {
     owned.clear();
     for (auto& kv : plans) {
       cudaFree(kv.second->d_groups); cudaFree(kv.second->d_items); cudaFree(kv.second->d_targets);
-      cudaFree(kv.second->d_stack);
+      cudaFree(kv.second->d_stack); cudaFree(kv.second->d_torder);
     }
     plans.clear();
     for (auto& kv : merged_plans) {
       cudaFree(kv.second->d_groups); cudaFree(kv.second->d_items); cudaFree(kv.second->d_targets);
-      cudaFree(kv.second->d_stack);
+      cudaFree(kv.second->d_stack); cudaFree(kv.second->d_torder);
     }
     merged_plans.clear();
     if (scratch) cudaFree(scratch);
@@ -505,6 +505,11 @@ class Engine : public EngineBase {
     pl.d_items = dmalloc(std::max<size_t>(pl.items.size(), 1) * sizeof(GItem));
     pl.d_targets = dmalloc(std::max<size_t>(pl.targets.size(), 1) * sizeof(TInfo));
     pl.d_stack = dmalloc(std::max<size_t>(pl.stack.size(), 1) * sizeof(StackDim));
+    if (pp.fused && !pl.torder.empty()) {
+      pl.d_torder = dmalloc(pl.torder.size() * sizeof(int32_t));
+      ACR_CUDA(cudaMemcpy(pl.d_torder, pl.torder.data(), pl.torder.size() * sizeof(int32_t),
+                          cudaMemcpyHostToDevice));
+    }
     if (!pl.stack.empty())
       ACR_CUDA(cudaMemcpy(pl.d_stack, pl.stack.data(), pl.stack.size() * sizeof(StackDim),
                           cudaMemcpyHostToDevice));
@@ -627,14 +632,23 @@ class Engine : public EngineBase {
       T* const* d_tab = (T* const*)ring.push(tab.data(), sizeof(void*) * (3 * nr + 1) * pc, st);
       int* const* d_rtab = (int* const*)ring.push(rtab.data(), sizeof(void*) * (nr + 1) * pc, st);
       for (const Stage& sg : pl.stages) {
-        if (sg.kind == ST_GEMM)
+        if (sg.kind == ST_GEMM) {
           timed(0, [&] { gemm_stage(pl, sg, d_tab, (const int* const*)d_rtab, pc, st); }, sg.tag);
-        else if (sg.kind == ST_PCHOL || sg.kind == ST_PCHOL + 16)
-          timed(1, [&] { launch_pchol<T>(pl, sg.beg, sg.end, sg.kind == ST_PCHOL, tau_orth(), d_tab,
-                                         d_rtab, pc, st, d_sketch_stat, fl(1)); });
-        else if (sg.kind == ST_EIG)
-          timed(2, [&] { launch_eig<T>(pl, sg.beg, sg.end, eps, kc, c_role, d_tab, d_rtab, pc,
-                                       d_err, st, fl(2)); });
+          continue;
+        }
+        if constexpr (std::is_same<T, float>::value) {
+          if (sg.kind == ST_ORTH)
+            timed(1, [&] { launch_orth(pl, tau_orth(), d_tab, d_rtab, pc, st, d_sketch_stat, fl(1)); });
+          else
+            timed(2, [&] { launch_core(pl, eps, kc, c_role, d_tab, d_rtab, pc, d_err, st, fl(2)); });
+        } else {
+          if (sg.kind == ST_PCHOL || sg.kind == ST_PCHOL + 16)
+            timed(1, [&] { launch_pchol<T>(pl, sg.beg, sg.end, sg.kind == ST_PCHOL, tau_orth(), d_tab,
+                                           d_rtab, pc, st, d_sketch_stat, fl(1)); });
+          else
+            timed(2, [&] { launch_eig<T>(pl, sg.beg, sg.end, eps, kc, c_role, d_tab, d_rtab, pc,
+                                         d_err, st, fl(2)); });
+        }
       }
     }
   }
@@ -745,7 +759,7 @@ void Engine<T>::prepare(const double* const* coefs, cudaStream_t st, bool count_
   pp.kc = kc;
   pp.oversample = 8;
   pp.cholqr2 = true;
-  pp.gram_scale = (int)(sizeof(double) / sizeof(T));
+  pp.fused = std::is_same<T, float>::value;
   mvp.build(S);
   {
     size_t fr = 0, tot = 0;

@@ -3,7 +3,6 @@
 //  * k_gwarp     -- one warp per group (row panels of up to 64 rows);
 //  * k_gdot, k_gdot_warp -- inner-product stages (both operands contiguous
 //                   along the contraction);
-//  * k_gram_ff   -- Grams of float columns with FP64-accurate results;
 //  * launch_ggemm -- the stage dispatcher (kernel shape per stage tag).
 #include <cuda_runtime.h>
 
@@ -786,120 +785,6 @@ __global__ void __launch_bounds__(NT, sizeof(Acc) == 4 ? (TM == 4 ? 4 : 2) : 1) 
   if (flops && lane == 0 && fl > 0) atomicAdd(flops, (double)fl);
 }
 
-// Gram matrices C = Y^T Y of float columns (the range finder's sketch and
-// basis Grams and the core Gram) with FP64 results.  The rank decisions that
-// follow resolve singular values only down to sqrt(relative Gram error)
-// times the largest one, so a float-accumulated Gram (error ~1e-7) stops at
-// ~3e-4; here every product is exact (a*b split into its rounded value and
-// FMA remainder) and the sums are compensated (TwoSum per lane, float-float
-// state, the lanes' results summed the same way, then rounded to double):
-// the relative error is ~1e-13 of sum |y_i||y_j|, so the Grams resolve
-// singular values down to the float data's own noise (~1e-7).
-//
-// One CTA per Gram: the columns of Y pass through shared memory in chunks of
-// 64 rows; thread (tile, slice) owns a 4 x 4 tile of the upper triangle and
-// the rows slice, slice + S, ... of every chunk; the slices' float-float
-// partials are summed in float-float in a fixed order, then rounded to double.
-constexpr int GRAM_KCH = 64;
-
-__global__ void __launch_bounds__(NT) k_gram_ff(const GGroup* __restrict__ groups,
-                                                const GItem* __restrict__ items,
-                                                float* const* __restrict__ tab,
-                                                const int* const* __restrict__ rtab, int P,
-                                                int gbase, double* __restrict__ flops) {
-  const int p = blockIdx.y;
-  const GGroup G = groups[gbase + blockIdx.x];
-  float* Cf = tab[G.cbuf * P + p];
-  if (!Cf) return;
-  const int m = dimv(G.m_st, G.m_rb, G.m_ri, rtab, P, p);
-  if (m <= 0 || m > 64 || G.ie <= G.ib) return;
-  double* C = reinterpret_cast<double*>(Cf + G.coff);
-  const GItem I = items[G.ib];
-  const float* Y = tab[I.abuf * P + p];
-  if (!Y) return;
-  Y += I.aoff;
-  const int k = dimv(I.k_st, I.k_rb, I.k_ri, rtab, P, p);
-  const int ld = I.lda;
-  // ys[column][row of the chunk] during the sweep; then the per-thread tile
-  // results (float-float pairs) in the same storage
-  __shared__ __align__(16) double raw[NT * 16];
-  const int TM = (m + 3) >> 2, ntile = TM * (TM + 1) / 2;
-  // rows per chunk: the staged columns (4 TM of them) fill the buffer
-  const int kch = TM <= 4 ? 4 * GRAM_KCH : (TM <= 8 ? 2 * GRAM_KCH : GRAM_KCH);
-  float* ysb = reinterpret_cast<float*>(raw);   // ys(col, row) = ysb[col * (kch + 1) + row]
-  static_assert(64 * (GRAM_KCH + 1) * sizeof(float) <= NT * 16 * sizeof(double), "staging fits");
-  static_assert(32 * (2 * GRAM_KCH + 1) * sizeof(float) <= NT * 16 * sizeof(double), "staging fits");
-  static_assert(16 * (4 * GRAM_KCH + 1) * sizeof(float) <= NT * 16 * sizeof(double), "staging fits");
-  const int S = NT / ntile >= 1 ? NT / ntile : 1;   // ntile <= 136 < NT
-  const int tid = threadIdx.x;
-  const int tile0 = tid / S, slice = tid - tile0 * S;
-  const bool active = tile0 < ntile;
-  int ti = 0, tile = active ? tile0 : 0;
-  while (tile >= TM - ti) { tile -= TM - ti; ++ti; }   // upper triangle: tj >= ti
-  const int i0 = 4 * ti, j0 = 4 * (ti + tile);
-  if (flops && tid == 0 && k > 0) atomicAdd(flops, 2.0 * m * m * k);
-  float s[4][4], c[4][4];
-#pragma unroll
-  for (int a = 0; a < 4; ++a)
-#pragma unroll
-    for (int b = 0; b < 4; ++b) { s[a][b] = 0.f; c[a][b] = 0.f; }
-  const int mt = 4 * TM;   // columns the tiles read (>= m: the rest read as 0)
-  const int ysld = kch + 1;
-  for (int e = m * kch + tid; e < mt * kch; e += NT) ysb[(e / kch) * ysld + e % kch] = 0.f;
-  for (int l0 = 0; l0 < k; l0 += kch) {
-    const int kk = min(kch, k - l0);
-    __syncthreads();
-    for (int e = tid; e < m * kch; e += NT) {
-      const int col = e / kch, l = e - col * kch;
-      ysb[col * ysld + l] = l < kk ? Y[(l0 + l) + (int64_t)col * ld] : 0.f;
-    }
-    __syncthreads();
-    if (active)
-      for (int l = slice; l < kk; l += S) {
-        float av[4], bv[4];
-#pragma unroll
-        for (int a = 0; a < 4; ++a) {
-          av[a] = ysb[(i0 + a) * ysld + l];
-          bv[a] = ysb[(j0 + a) * ysld + l];
-        }
-#pragma unroll
-        for (int a = 0; a < 4; ++a)
-#pragma unroll
-          for (int b = 0; b < 4; ++b) ff_fma(s[a][b], c[a][b], av[a], bv[b]);
-      }
-  }
-  __syncthreads();   // every thread is done with ys
-  // the slices' float-float partials, summed in float-float (TwoSum) in a
-  // fixed order; one conversion to double per output (the FP64 pipe is a
-  // small fraction of the FP32 one)
-  float (*red_s)[16] = reinterpret_cast<float (*)[16]>(raw);
-  float (*red_c)[16] = reinterpret_cast<float (*)[16]>(reinterpret_cast<float*>(raw) + NT * 16);
-#pragma unroll
-  for (int e = 0; e < 16; ++e) {
-    red_s[tid][e] = active ? s[e & 3][e >> 2] : 0.f;
-    red_c[tid][e] = active ? c[e & 3][e >> 2] : 0.f;
-  }
-  __syncthreads();
-  for (int e = tid; e < ntile * 16; e += NT) {
-    const int t = e >> 4, q = e & 15;
-    float hi = 0.f, lo = 0.f;
-    for (int sl = 0; sl < S; ++sl) {
-      const float x = red_s[t * S + sl][q];
-      const float u = hi + x, bp = u - hi;
-      lo += ((hi - (u - bp)) + (x - bp)) + red_c[t * S + sl][q];
-      hi = u;
-    }
-    const double v = (double)hi + (double)lo;
-    int tt = t, a = 0;
-    while (tt >= TM - a) { tt -= TM - a; ++a; }
-    const int i = 4 * a + (q & 3), j = 4 * (a + tt) + (q >> 2);
-    if (i < m && j < m) {
-      C[i + (int64_t)j * G.ldc] = v;
-      C[j + (int64_t)i * G.ldc] = v;
-    }
-  }
-}
-
 }  // namespace
 
 template <typename T>
@@ -941,9 +826,7 @@ void launch_ggemm(const Plan& pl, int gbeg, int gend, T* const* d_tab, const int
     // the wide groups on the tensor cores; variant 4 as 2 with 32 columns per
     // pass; variant 5 (float, inner-product stages) 8 x 8 warp tiles.
     const bool warp_dot = (tag == TAG_M || (sizeof(T) == 4 && (tag == TAG_S || tag == TAG_P)));
-    if (sizeof(T) == 4 && (tag == TAG_G || tag == TAG_G2 || tag == TAG_H)) {
-      k_gram_ff<<<grid, NT, 0, st>>>(gr, it, (float* const*)d_tab, d_rtab, P, gbeg + g0, d_fl);
-    } else if ((variant == 2 || variant == 4) && sizeof(T) == 4 && d_err && !tag_is_dot(tag)) {
+    if ((variant == 2 || variant == 4) && sizeof(T) == 4 && d_err && !tag_is_dot(tag)) {
       const int cnt = std::min(maxg, ng - g0);
       dim3 gw((cnt + NT / 32 - 1) / (NT / 32), P);
       if (variant == 4)

@@ -62,7 +62,7 @@ void launch_ggemm_tc(const Plan& pl, int gbeg, int gend, float* const* d_tab,
                      const int* const* d_rtab, int P, const double* d_coefs, cudaStream_t st,
                      double* d_fl, int* d_err);
 
-// Pivoted-Cholesky orthonormalisation cores (FP64) of plan targets.  The
+// Pivoted-Cholesky orthonormalisation cores of plan targets (FP64 factors).  The
 // truncating pass counts targets and stacked-rank overflows of the sketch
 // into d_sketch_stat[0..1] (may be null).
 template <typename T>
@@ -70,12 +70,21 @@ void launch_pchol(const Plan& pl, int tbeg, int tend, bool truncate, double tau,
                   T* const* d_tab, int* const* d_rtab, int P, cudaStream_t st,
                   unsigned long long* d_sketch_stat, double* d_flops = nullptr);
 
-// Jacobi eigen cores (FP64) of plan targets; writes the kept ranks into
+// Jacobi eigen cores of plan targets (FP64 factors); writes the kept ranks into
 // the rank buffer of role c_role and raises ERR_RANKCAP above kc.
 template <typename T>
 void launch_eig(const Plan& pl, int tbeg, int tend, double eps, int kc, int c_role,
                 T* const* d_tab, int* const* d_rtab, int P, int* d_err, cudaStream_t st,
                 double* d_flops = nullptr);
+
+// The fused stages ST_ORTH and ST_CORE of a plan's float targets: the sketches'
+// orthonormal bases, in place; core Grams, Jacobi cores and recomposition,
+// rank output and ERR_RANKCAP as launch_eig.
+void launch_orth(const Plan& pl, double tau, float* const* d_tab, int* const* d_rtab, int P,
+                 cudaStream_t st, unsigned long long* d_sketch_stat, double* d_flops = nullptr);
+void launch_core(const Plan& pl, double eps, int kc, int c_role, float* const* d_tab,
+                 int* const* d_rtab, int P, int* d_err, cudaStream_t st,
+                 double* d_flops = nullptr);
 
 // In-place Gauss-Jordan inverse (partial pivoting) of one dense lsz x lsz
 // leaf in each of P H-matrices (base pointers in d_dense[p]): FP64, or for

@@ -379,28 +379,31 @@ struct Builder {
     }
 
     // ---- scratch for low-rank targets
-    int64_t capsum_max = 0;
     for (LT& lt : lts) {
       const BNode& c = S.bn[lt.node];
       int m = S.cl[c.t].size, n = S.cl[c.s].size;
       int64_t capsum = 0;
       for (const LItem& li : lt.items) capsum += li.cap;
-      capsum_max = std::max(capsum_max, capsum);
       int p = (int)std::min<int64_t>(std::min(kc + pp.oversample, TILE), std::max<int64_t>(capsum, 1));
       lt.p = p;
       lt.y = alloc((int64_t)m * p);
-      lt.q = alloc((int64_t)m * p);
+      lt.q = pp.fused ? lt.y : alloc((int64_t)m * p);
       lt.bt = alloc((int64_t)n * p);
       for (LItem& li : lt.items) li.sp_off = alloc((int64_t)li.cap * p);
       TInfo& ti = lt.ti;
-      ti.g_off = alloc((int64_t)pp.gram_scale * p * p);
-      ti.t_off = alloc((int64_t)p * p);
-      ti.h_off = alloc((int64_t)pp.gram_scale * p * p);
-      ti.w_off = alloc((int64_t)p * p);
+      ti.g_off = ti.t_off = ti.h_off = ti.w_off = 0;
+      if (!pp.fused) {
+        ti.g_off = alloc((int64_t)p * p);
+        ti.t_off = alloc((int64_t)p * p);
+        ti.h_off = alloc((int64_t)p * p);
+        ti.w_off = alloc((int64_t)p * p);
+      }
       ti.p = p; ti.m = m; ti.n = n;
       ti.r_ri = alloc_rank();
       ti.c_leaf = c.leaf;
       ti.seed = 0;
+      ti.y_off = lt.y; ti.bt_off = lt.bt;
+      ti.u_off = S.lr_row0[c.leaf] * kc; ti.v_off = S.lr_col0[c.leaf] * kc;
       ti.sk_beg = (int)P.stack.size();
       for (const LItem& li : lt.items) {
         if (li.dense)
@@ -478,8 +481,12 @@ struct Builder {
       }
       stage(ST_GEMM, gg, (int)P.groups.size(), from_y ? TAG_Q : TAG_Q2);
     };
-    orth_pass(true);
-    if (pp.cholqr2) {
+    if (pp.fused) {
+      if (!lts.empty()) P.stages.push_back(Stage{ST_ORTH, 0, (int)lts.size()});
+    } else {
+      orth_pass(true);
+    }
+    if (pp.cholqr2 && !pp.fused) {
       orth_pass(false);
       for (LT& lt : lts) std::swap(lt.y, lt.q);   // the basis now lives in the former Y buffer
     }
@@ -520,6 +527,10 @@ struct Builder {
     }
     stage(ST_GEMM, g0, (int)P.groups.size(), TAG_BT);
 
+    if (pp.fused) {
+      if (!lts.empty()) P.stages.push_back(Stage{ST_CORE, 0, (int)lts.size()});
+      return;
+    }
     // H = (B^T)^T B^T   (r x r), core eigen-decomposition
     g0 = (int)P.groups.size();
     for (size_t i = 0; i < lts.size(); ++i) {
@@ -549,7 +560,6 @@ struct Builder {
       }
     }
     stage(ST_GEMM, g0, (int)P.groups.size(), TAG_UV);
-    (void)capsum_max;
   }
 };
 
@@ -559,10 +569,16 @@ namespace {
 // Order every GEMM stage's groups wide (static 64-column outputs) first and
 // record their count, so a launch can give the two kinds different kernels.
 // Groups of one stage write disjoint outputs: their order changes nothing.
-// Also records the widest sketch of the plan's targets.
+// Also records the widest sketch of the plan's targets and their order by size.
 void order_wide_first(Plan& plan) {
   plan.max_p = 0;
   for (const TInfo& ti : plan.targets) plan.max_p = std::max(plan.max_p, ti.p);
+  plan.torder.resize(plan.targets.size());
+  for (size_t i = 0; i < plan.targets.size(); ++i) plan.torder[i] = (int32_t)i;
+  std::stable_sort(plan.torder.begin(), plan.torder.end(), [&](int32_t a, int32_t b) {
+    const TInfo &x = plan.targets[a], &y = plan.targets[b];
+    return (int64_t)x.m * x.p < (int64_t)y.m * y.p;
+  });
   for (Stage& sg : plan.stages) {
     if (sg.kind != ST_GEMM) continue;
     auto wide = [](const GGroup& g) { return g.n_rb < 0 && g.n_st >= 64; };
@@ -599,6 +615,8 @@ int stage_slot(const Stage& sg) {
     static const int slot_of_tag[NTAGS] = {0, 1, 2, 3, 4, 5, 7, 8, 10, 11, 12, 13, 15};
     return slot_of_tag[sg.tag];
   }
+  if (sg.kind == ST_ORTH) return 5;
+  if (sg.kind == ST_CORE) return 13;
   if (sg.kind == ST_PCHOL) return 6;
   if (sg.kind == ST_PCHOL + 16) return 9;
   return 14;   // ST_EIG
@@ -622,6 +640,7 @@ void merge_plans(const std::vector<const Plan*>& ps, Plan& out) {
     out.stack.insert(out.stack.end(), ps[i]->stack.begin(), ps[i]->stack.end());
     for (TInfo ti : ps[i]->targets) {
       ti.g_off += soff[i]; ti.t_off += soff[i]; ti.h_off += soff[i]; ti.w_off += soff[i];
+      ti.y_off += soff[i]; ti.bt_off += soff[i];
       ti.r_ri += roff[i];
       ti.sk_beg += sk0; ti.sk_end += sk0;
       out.targets.push_back(ti);

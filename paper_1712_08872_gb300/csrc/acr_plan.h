@@ -73,6 +73,9 @@ struct TInfo {
   int32_t c_leaf;      // low-rank leaf index of C (rank output)
   int32_t seed;
   int32_t sk_beg, sk_end;  // the summed terms' inner dimensions: Plan::stack entries
+  int64_t y_off, bt_off;   // fused stages: scratch offsets of the sketch Y, replaced by the basis
+                           // Q (m x p, ld m), and of B^T (n x p, ld n)
+  int64_t u_off, v_off;    // the target leaf's factors in C's U and V buffers
 };
 
 // One summed term of a low-rank target, for the stacked-rank count: its
@@ -82,7 +85,10 @@ struct StackDim {
   int32_t st, rb, ri, g0, g1;
 };
 
-enum StageKind { ST_GEMM = 0, ST_PCHOL = 1, ST_EIG = 2 };
+// ST_ORTH and ST_CORE (PlanParams::fused) each stand for a run of the others:
+// the sketch's Gram, Cholesky and basis stages, and the core Gram, Jacobi and
+// recomposition stages.
+enum StageKind { ST_GEMM = 0, ST_PCHOL = 1, ST_EIG = 2, ST_ORTH = 3, ST_CORE = 4 };
 // what a GEMM stage computes (for profiling)
 enum StageTag {
   TAG_M = 0,       // phase 1: small inner products U^T V
@@ -134,18 +140,20 @@ struct Plan {
   int n_lr_targets = 0, n_dense_targets = 0, n_terms = 0;
   int64_t flops_static = 0;   // flops of the static-size GEMM parts (per plane)
   int32_t max_p = 0;          // widest sketch over the targets (bounds every core's size)
+  std::vector<int32_t> torder;   // target indices by increasing sketch size m * p
   // device copies (owned by the engine)
   void* d_groups = nullptr;
   void* d_items = nullptr;
   void* d_targets = nullptr;
   void* d_stack = nullptr;
+  void* d_torder = nullptr;
 };
 
 struct PlanParams {
   int kc;        // rank capacity of stored low-rank blocks
   int oversample;
   bool cholqr2;  // second orthonormalisation pass (single-precision forms)
-  int gram_scale = 1;   // storage elements per Gram entry: Grams are FP64 (2 for float)
+  bool fused = false;   // one basis and one core stage per plan (float factors)
 };
 
 // Build the plan of one formatted operation.

@@ -1,10 +1,9 @@
 // Setup kernels of the ACR engine (sm_103a), besides the grouped GEMMs of
-// acr_gemm_kernels.cu:
-//  * k_pchol   -- FP64 pivoted Cholesky of a sketch Gram: orthonormal basis
-//                 transform of the range finder;
-//  * k_eig     -- cyclic Jacobi of the small recompression core (FP64; for
-//                 float factors float-float), rank selection
-//                 sigma_i > eps * sigma_1 (Sec. 4.3 H_eps);
+// acr_gemm_kernels.cu and the float recompression cores of acr_core_kernels.cu:
+//  * k_pchol   -- pivoted Cholesky of a sketch Gram (FP64 factors): orthonormal
+//                 basis transform of the range finder;
+//  * k_eig     -- cyclic Jacobi of the small recompression core (FP64 factors),
+//                 rank selection sigma_i > eps * sigma_1 (Sec. 4.3 H_eps);
 //  * k_leaf_inv-- Gauss-Jordan inverse with partial pivoting of a dense
 //                 diagonal leaf (the leaves of the recursive H-inverse): FP64,
 //                 or for float storage float elimination refined to float
@@ -28,68 +27,7 @@ namespace {
 // ---------------------------------------------------------------- cores
 constexpr int CMAX = 64;   // largest sketch / core dimension
 
-// Float-float numbers (an unevaluated sum hi + lo of two floats, ~48
-// significant bits): the products and sums of the float form's small
-// Jacobi cores, on the FP32 pipe instead of this part's narrow FP64 pipe.
-struct FF {
-  float h, l;
-};
-__device__ __forceinline__ FF ff_of(double x) {
-  const float h = (float)x;
-  return FF{h, (float)(x - (double)h)};
-}
-__device__ __forceinline__ double ff_dbl(FF a) { return (double)a.h + (double)a.l; }
-// a * b: exact product of the high parts plus the cross terms, renormalised
-__device__ __forceinline__ FF ff_mul(FF a, FF b) {
-  const float p = a.h * b.h;
-  float e = fmaf(a.h, b.h, -p);
-  e = fmaf(a.h, b.l, e);
-  e = fmaf(a.l, b.h, e);
-  const float s = p + e;
-  return FF{s, e - (s - p)};
-}
-// a + b: TwoSum of the high parts, low parts added, renormalised
-__device__ __forceinline__ FF ff_add(FF a, FF b) {
-  const float s = a.h + b.h;
-  const float bp = s - a.h;
-  float e = (a.h - (s - bp)) + (b.h - bp);
-  e += a.l + b.l;
-  const float r = s + e;
-  return FF{r, e - (r - s)};
-}
-__device__ __forceinline__ FF ff_neg(FF a) { return FF{-a.h, -a.l}; }
-// (1 + t^2)^(-1/2) to float-float accuracy: one Newton step y + y (1 - x y^2) / 2
-// from the float estimate
-__device__ __forceinline__ FF ff_rsqrt1p(float t) {
-  const float p = t * t;
-  const FF x = ff_add(FF{1.f, 0.f}, FF{p, fmaf(t, t, -p)});
-  const float y = rsqrtf(x.h);
-  const FF xy2 = ff_mul(x, ff_mul(FF{y, 0.f}, FF{y, 0.f}));
-  const FF e = ff_add(FF{1.f, 0.f}, ff_neg(xy2));
-  return ff_add(FF{y, 0.f}, ff_mul(FF{y, 0.f}, FF{0.5f * e.h, 0.5f * e.l}));
-}
-
-// The Jacobi cores' element type: FP64 for FP64 factors; for float factors
-// float-float, whose products and sums run on the FP32 pipe instead of this
-// part's narrow FP64 pipe (~1e-14 relative, far below what float factors
-// keep).  jm, ja, jn: multiply, add, negate; jd: the value in double.
-template <typename T>
-using JacE = typename std::conditional<std::is_same<T, float>::value, FF, double>::type;
-__device__ __forceinline__ double jm(double a, double b) { return a * b; }
-__device__ __forceinline__ FF jm(FF a, FF b) { return ff_mul(a, b); }
-__device__ __forceinline__ double ja(double a, double b) { return a + b; }
-__device__ __forceinline__ FF ja(FF a, FF b) { return ff_add(a, b); }
-__device__ __forceinline__ double jn(double a) { return -a; }
-__device__ __forceinline__ FF jn(FF a) { return ff_neg(a); }
-__device__ __forceinline__ double jd(double a) { return a; }
-__device__ __forceinline__ double jd(FF a) { return ff_dbl(a); }
-__device__ __forceinline__ void jset(double& a, double x) { a = x; }
-__device__ __forceinline__ void jset(FF& a, double x) { a = ff_of(x); }
 // The rotation (c, s) that zeroes a_pq of the 2 x 2 block [a_pp a_pq; a_pq a_qq].
-// FP64: the textbook formulas.  Float-float: the angle in float (an angle off
-// by ~1e-7 leaves ~1e-7 of the entry, which later rotations remove), its
-// cosine and sine to float-float accuracy from that angle, so the rotation
-// itself is orthogonal to ~1e-14 and no FP64 operation remains in a sweep.
 __device__ __forceinline__ void jrot(double app, double aqq, double apq, double& c, double& s) {
   c = 1.0;
   s = 0.0;
@@ -100,17 +38,6 @@ __device__ __forceinline__ void jrot(double app, double aqq, double apq, double&
     s = t * c;
   }
 }
-__device__ __forceinline__ void jrot(FF app, FF aqq, FF apq, FF& c, FF& s) {
-  c = FF{1.f, 0.f};
-  s = FF{0.f, 0.f};
-  if (apq.h != 0.f) {
-    const float tau_ = (aqq.h - app.h) / (2.f * apq.h);
-    const float t = (tau_ >= 0.f ? 1.f : -1.f) / (fabsf(tau_) + sqrtf(1.f + tau_ * tau_));
-    c = ff_rsqrt1p(t);
-    s = ff_mul(FF{t, 0.f}, c);
-  }
-}
-
 
 // Pivoted Cholesky of G (pd x pd): G = P L L^T P^T, stop when the largest
 // remaining diagonal <= tau^2 * max diag(G) (truncating pass).  Writes
@@ -407,9 +334,8 @@ __global__ void __launch_bounds__(NT) k_eig_warp(const TInfo* __restrict__ tis, 
   const int p = blockIdx.y;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int t = tbase + blockIdx.x * (NT / 32) + warp;
-  using E = JacE<T>;
-  __shared__ E As[NT / 32][M][M + 1], Vs[NT / 32][M][M + 1];
-  __shared__ E css[NT / 32][M / 2], sns[NT / 32][M / 2];
+  __shared__ double As[NT / 32][M][M + 1], Vs[NT / 32][M][M + 1];
+  __shared__ double css[NT / 32][M / 2], sns[NT / 32][M / 2];
   __shared__ double lams[NT / 32][M];
   __shared__ int pps[NT / 32][M / 2], qqs[NT / 32][M / 2], ords[NT / 32][M];
   if (t >= tend) return;
@@ -425,29 +351,29 @@ __global__ void __launch_bounds__(NT) k_eig_warp(const TInfo* __restrict__ tis, 
   }
   if (r > M) return;   // k_eig's cores
   const int ld = ti.p;
-  E (*A)[M + 1] = As[warp];
-  E (*V)[M + 1] = Vs[warp];
-  E* cs = css[warp];
-  E* sn = sns[warp];
+  double (*A)[M + 1] = As[warp];
+  double (*V)[M + 1] = Vs[warp];
+  double* cs = css[warp];
+  double* sn = sns[warp];
   int* pp = pps[warp];
   int* qq = qqs[warp];
   const double* H = reinterpret_cast<const double*>(scr + ti.h_off);
   T* W = scr + ti.w_off;
   for (int e = lane; e < r * r; e += 32) {
     const int i = e % r, j = e / r;
-    jset(A[i][j], 0.5 * (H[i + (int64_t)j * ld] + H[j + (int64_t)i * ld]));
-    jset(V[i][j], (i == j) ? 1.0 : 0.0);
+    A[i][j] = 0.5 * (H[i + (int64_t)j * ld] + H[j + (int64_t)i * ld]);
+    V[i][j] = (i == j) ? 1.0 : 0.0;
   }
   __syncwarp();
   const int nn = (r + 1) & ~1;
   const int npair = nn / 2;
   int sweeps_done = 0;
-  const double conv = sizeof(T) == 8 ? 1e-30 : 1e-16;
+  const double conv = 1e-30;
   for (int sweep = 0; sweep < 40; ++sweep) {
     double off = 0, tot = 0;
     for (int e = lane; e < r * r; e += 32) {
       const int i = e % r, j = e / r;
-      const double a = jd(A[i][j]);
+      const double a = A[i][j];
       const double v = a * a;
       tot += v;
       if (i != j) off += v;
@@ -467,9 +393,7 @@ __global__ void __launch_bounds__(NT) k_eig_warp(const TInfo* __restrict__ tis, 
         const int b = 1 + ((pb - 1 + round) % (nn - 1));
         const int lo = a < b ? a : b, hi = a < b ? b : a;
         pp[k] = lo; qq[k] = hi;
-        E c, sv;
-        jset(c, 1.0);
-        jset(sv, 0.0);
+        double c = 1.0, sv = 0.0;
         if (hi < r) jrot(A[lo][lo], A[hi][hi], A[lo][hi], c, sv);
         cs[k] = c; sn[k] = sv;
       }
@@ -480,28 +404,27 @@ __global__ void __launch_bounds__(NT) k_eig_warp(const TInfo* __restrict__ tis, 
           const int k1 = e / npair, k2 = e - k1 * npair;
           const int a1 = pp[k1], b1 = qq[k1], a2 = pp[k2], b2 = qq[k2];
           const bool h1 = b1 < r, h2 = b2 < r;
-          const E c1 = cs[k1], s1 = sn[k1], c2 = cs[k2], s2 = sn[k2];
-          E z;
-          jset(z, 0.0);
-          const E x00 = A[a1][a2];
-          const E x01 = h2 ? A[a1][b2] : z;
-          const E x10 = h1 ? A[b1][a2] : z;
-          const E x11 = (h1 && h2) ? A[b1][b2] : z;
-          const E y00 = ja(jm(c2, x00), jn(jm(s2, x01))), y01 = ja(jm(s2, x00), jm(c2, x01));
-          const E y10 = ja(jm(c2, x10), jn(jm(s2, x11))), y11 = ja(jm(s2, x10), jm(c2, x11));
-          A[a1][a2] = ja(jm(c1, y00), jn(jm(s1, y10)));
-          if (h2) A[a1][b2] = ja(jm(c1, y01), jn(jm(s1, y11)));
-          if (h1) A[b1][a2] = ja(jm(s1, y00), jm(c1, y10));
-          if (h1 && h2) A[b1][b2] = ja(jm(s1, y01), jm(c1, y11));
+          const double c1 = cs[k1], s1 = sn[k1], c2 = cs[k2], s2 = sn[k2];
+          const double z = 0.0;
+          const double x00 = A[a1][a2];
+          const double x01 = h2 ? A[a1][b2] : z;
+          const double x10 = h1 ? A[b1][a2] : z;
+          const double x11 = (h1 && h2) ? A[b1][b2] : z;
+          const double y00 = c2 * x00 - s2 * x01, y01 = s2 * x00 + c2 * x01;
+          const double y10 = c2 * x10 - s2 * x11, y11 = s2 * x10 + c2 * x11;
+          A[a1][a2] = c1 * y00 - s1 * y10;
+          if (h2) A[a1][b2] = c1 * y01 - s1 * y11;
+          if (h1) A[b1][a2] = s1 * y00 + c1 * y10;
+          if (h1 && h2) A[b1][b2] = s1 * y01 + c1 * y11;
         } else {
           const int f = e - nblk;
           const int k = f / r, iv = f - k * r;
           const int a = pp[k], b = qq[k];
           if (b < r) {
-            const E c = cs[k], sv = sn[k];
-            const E vx = V[iv][a], vy = V[iv][b];
-            V[iv][a] = ja(jm(c, vx), jn(jm(sv, vy)));
-            V[iv][b] = ja(jm(sv, vx), jm(c, vy));
+            const double c = cs[k], sv = sn[k];
+            const double vx = V[iv][a], vy = V[iv][b];
+            V[iv][a] = c * vx - sv * vy;
+            V[iv][b] = sv * vx + c * vy;
           }
         }
       }
@@ -510,7 +433,7 @@ __global__ void __launch_bounds__(NT) k_eig_warp(const TInfo* __restrict__ tis, 
   }
   double* lam = lams[warp];
   int* order = ords[warp];
-  if (lane < r) lam[lane] = jd(A[lane][lane]);
+  if (lane < r) lam[lane] = A[lane][lane];
   __syncwarp();
   if (lane < r) {
     int pos = 0;
@@ -540,13 +463,12 @@ __global__ void __launch_bounds__(NT) k_eig_warp(const TInfo* __restrict__ tis, 
   k = __shfl_sync(0xffffffffu, k, 0);
   for (int e = lane; e < r * k; e += 32) {
     const int i = e % r, j = e / r;
-    W[i + (int64_t)j * ld] = (T)jd(V[i][order[j]]);
+    W[i + (int64_t)j * ld] = (T)V[i][order[j]];
   }
 }
 
 // Cyclic Jacobi (round-robin parallel order) on the r x r symmetric core H
-// (cores with r > 16; k_eig_warp takes the smaller ones), in the element
-// type JacE<T> (FP64, or float-float for float factors).
+// (cores with r > 16; k_eig_warp takes the smaller ones).
 template <typename T>
 __global__ void __launch_bounds__(NT) k_eig(const TInfo* __restrict__ tis, int tbase, double eps,
                                             int kc, int c_rbuf, T* const* __restrict__ tab,
@@ -561,12 +483,10 @@ __global__ void __launch_bounds__(NT) k_eig(const TInfo* __restrict__ tis, int t
   const int r = rs[ti.r_ri];
   const int ld = ti.p;
   if (r <= EIG_WARP_MAX) return;   // k_eig_warp's cores (and the empty bases)
-  using E = JacE<T>;
-  static_assert(sizeof(E) == sizeof(double), "the shared layout holds 8-byte elements");
   extern __shared__ double dsm[];
-  E (*A)[CMAX + 1] = reinterpret_cast<E (*)[CMAX + 1]>(dsm);
-  E (*V)[CMAX + 1] = reinterpret_cast<E (*)[CMAX + 1]>(dsm + CMAX * (CMAX + 1));
-  __shared__ E cs[CMAX / 2 + 1], sn[CMAX / 2 + 1];
+  double (*A)[CMAX + 1] = reinterpret_cast<double (*)[CMAX + 1]>(dsm);
+  double (*V)[CMAX + 1] = reinterpret_cast<double (*)[CMAX + 1]>(dsm + CMAX * (CMAX + 1));
+  __shared__ double cs[CMAX / 2 + 1], sn[CMAX / 2 + 1];
   __shared__ int pp[CMAX / 2 + 1], qq[CMAX / 2 + 1];
   __shared__ double red[NT];
   __shared__ int order[CMAX];
@@ -576,8 +496,8 @@ __global__ void __launch_bounds__(NT) k_eig(const TInfo* __restrict__ tis, int t
   T* W = scr + ti.w_off;
   for (int e = threadIdx.x; e < r * r; e += NT) {
     int i = e % r, j = e / r;
-    jset(A[i][j], 0.5 * ((double)H[i + (int64_t)j * ld] + (double)H[j + (int64_t)i * ld]));
-    jset(V[i][j], (i == j) ? 1.0 : 0.0);
+    A[i][j] = 0.5 * ((double)H[i + (int64_t)j * ld] + (double)H[j + (int64_t)i * ld]);
+    V[i][j] = (i == j) ? 1.0 : 0.0;
   }
   __syncthreads();
   const int nn = (r + 1) & ~1;   // even number of players (r may get a dummy)
@@ -590,7 +510,7 @@ __global__ void __launch_bounds__(NT) k_eig(const TInfo* __restrict__ tis, int t
       const int i = threadIdx.x & 63;
       if (i < r)
         for (int j = threadIdx.x >> 6; j < r; j += 4) {
-          const double a = jd(A[i][j]);
+          const double a = A[i][j];
           const double v = a * a;
           tot += v;
           if (i != j) off += v;
@@ -609,9 +529,8 @@ __global__ void __launch_bounds__(NT) k_eig(const TInfo* __restrict__ tis, int t
     double offs = 0, tots = 0;
     for (int w = 0; w < NT / 32; ++w) { offs += red[w]; tots += red[NT / 32 + w]; }
     __syncthreads();
-    // converged once the off-diagonal mass is below the storage precision's
-    // need: eigenvectors to ~1e-15 (FP64 factors) or ~1e-8 (float factors)
-    const double conv = sizeof(T) == 8 ? 1e-30 : 1e-16;
+    // converged: eigenvectors to ~1e-15
+    const double conv = 1e-30;
     if (offs <= conv * tots || r == 1) break;
     ++sweeps_done;
     for (int round = 0; round < nn - 1; ++round) {
@@ -622,9 +541,7 @@ __global__ void __launch_bounds__(NT) k_eig(const TInfo* __restrict__ tis, int t
         const int b = 1 + ((pb - 1 + round) % (nn - 1));
         int lo = a < b ? a : b, hi = a < b ? b : a;
         pp[k] = lo; qq[k] = hi;
-        E c, s;
-        jset(c, 1.0);
-        jset(s, 0.0);
+        double c = 1.0, s = 0.0;
         if (hi < r) jrot(A[lo][lo], A[hi][hi], A[lo][hi], c, s);
         cs[k] = c; sn[k] = s;
       }
@@ -641,28 +558,27 @@ __global__ void __launch_bounds__(NT) k_eig(const TInfo* __restrict__ tis, int t
           const int k1 = e / npair, k2 = e - k1 * npair;
           const int a1 = pp[k1], b1 = qq[k1], a2 = pp[k2], b2 = qq[k2];
           const bool h1 = b1 < r, h2 = b2 < r;
-          const E c1 = cs[k1], s1 = sn[k1], c2 = cs[k2], s2 = sn[k2];
-          E z;
-          jset(z, 0.0);
-          const E x00 = A[a1][a2];
-          const E x01 = h2 ? A[a1][b2] : z;
-          const E x10 = h1 ? A[b1][a2] : z;
-          const E x11 = (h1 && h2) ? A[b1][b2] : z;
-          const E y00 = ja(jm(c2, x00), jn(jm(s2, x01))), y01 = ja(jm(s2, x00), jm(c2, x01));
-          const E y10 = ja(jm(c2, x10), jn(jm(s2, x11))), y11 = ja(jm(s2, x10), jm(c2, x11));
-          A[a1][a2] = ja(jm(c1, y00), jn(jm(s1, y10)));
-          if (h2) A[a1][b2] = ja(jm(c1, y01), jn(jm(s1, y11)));
-          if (h1) A[b1][a2] = ja(jm(s1, y00), jm(c1, y10));
-          if (h1 && h2) A[b1][b2] = ja(jm(s1, y01), jm(c1, y11));
+          const double c1 = cs[k1], s1 = sn[k1], c2 = cs[k2], s2 = sn[k2];
+          const double z = 0.0;
+          const double x00 = A[a1][a2];
+          const double x01 = h2 ? A[a1][b2] : z;
+          const double x10 = h1 ? A[b1][a2] : z;
+          const double x11 = (h1 && h2) ? A[b1][b2] : z;
+          const double y00 = c2 * x00 - s2 * x01, y01 = s2 * x00 + c2 * x01;
+          const double y10 = c2 * x10 - s2 * x11, y11 = s2 * x10 + c2 * x11;
+          A[a1][a2] = c1 * y00 - s1 * y10;
+          if (h2) A[a1][b2] = c1 * y01 - s1 * y11;
+          if (h1) A[b1][a2] = s1 * y00 + c1 * y10;
+          if (h1 && h2) A[b1][b2] = s1 * y01 + c1 * y11;
         } else {
           const int f = e - nblk;
           const int k = f / r, iv = f - k * r;
           const int a = pp[k], b = qq[k];
           if (b < r) {
-            const E c = cs[k], s = sn[k];
-            const E vx = V[iv][a], vy = V[iv][b];
-            V[iv][a] = ja(jm(c, vx), jn(jm(s, vy)));
-            V[iv][b] = ja(jm(s, vx), jm(c, vy));
+            const double c = cs[k], s = sn[k];
+            const double vx = V[iv][a], vy = V[iv][b];
+            V[iv][a] = c * vx - s * vy;
+            V[iv][b] = s * vx + c * vy;
           }
         }
       }
@@ -670,7 +586,7 @@ __global__ void __launch_bounds__(NT) k_eig(const TInfo* __restrict__ tis, int t
     }
   }
   // sort eigenvalues descending (rank by counting; ties by index)
-  for (int i = threadIdx.x; i < r; i += NT) lam[i] = jd(A[i][i]);
+  for (int i = threadIdx.x; i < r; i += NT) lam[i] = A[i][i];
   __syncthreads();
   for (int i = threadIdx.x; i < r; i += NT) {
     int pos = 0;
@@ -702,7 +618,7 @@ __global__ void __launch_bounds__(NT) k_eig(const TInfo* __restrict__ tis, int t
   const int k = kkeep;
   for (int e = threadIdx.x; e < r * k; e += NT) {
     int i = e % r, j = e / r;
-    W[i + (int64_t)j * ld] = (T)jd(V[i][order[j]]);
+    W[i + (int64_t)j * ld] = (T)V[i][order[j]];
   }
 }
 
@@ -1267,11 +1183,11 @@ void launch_plane_to_h(const StructDev& sd, const double* coef, int n, const int
   ACR_LAUNCHED((sd.nd > 0) + (sd.nl > 0));
 }
 
+template void launch_pchol<double>(const Plan&, int, int, bool, double, double* const*,
+                                   int* const*, int, cudaStream_t, unsigned long long*, double*);
+template void launch_eig<double>(const Plan&, int, int, double, int, int, double* const*,
+                                 int* const*, int, int*, cudaStream_t, double*);
 #define ACR_INST(T)                                                                              \
-  template void launch_pchol<T>(const Plan&, int, int, bool, double, T* const*, int* const*, int, \
-                                cudaStream_t, unsigned long long*, double*);                     \
-  template void launch_eig<T>(const Plan&, int, int, double, int, int, T* const*, int* const*,   \
-                              int, int*, cudaStream_t, double*);                                 \
   template void launch_leaf_inv<T>(T* const*, int64_t, int, int, int*, cudaStream_t, double*,     \
                                    unsigned long long*);                                         \
   template void launch_hscale<T>(const StructDev&, T* const*, T* const*, T* const*, int* const*, \

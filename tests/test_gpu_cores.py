@@ -1,0 +1,54 @@
+"""The fused recompression stages of the float forms (basis and core kernels)
+at the edges of their range (GPU, through the C ABI): leaf sizes that are no
+multiple of a warp, sketches of every width up to the widest (rank cap 48), and
+weak admissibility, whose largest sketch (1152 x 56 floats) does not fit shared
+memory.
+
+The float factors differ from the FP64 form's by rounding, far below eps, so
+GMRES preconditioned with them takes the FP64 form's iterations, give or take
+one; the residual is confirmed by the oracle's SpMV.
+"""
+import numpy as np
+import pytest
+
+from inputs import codi_beta, gaussian_field_kappa, uniform_rhs
+from oracle.assembly import stencil_apply, stencil_codi, stencil_poisson
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("pde,n,eta,eps,cap", [
+    ("poisson", 20, 2.0, 1e-2, 19),     # 50-point leaves, 27-column sketches
+    ("codi", 24, 2.0, 1e-2, 24),        # 36-point leaves
+    ("poisson", 28, 2.0, 1e-5, 48),     # 49-point leaves, 56-column sketches
+    ("codi", 48, 96.0, 0.3, 48),        # one 1152 x 1152 admissible block per half
+])
+def test_float_cores(pde, n, eta, eps, cap):
+    from paper_1712_08872_gb300 import _build
+    _build.build()
+    import paper_1712_08872_gb300 as acr
+
+    def dev(x):
+        return torch.tensor(np.ascontiguousarray(x), dtype=torch.float64, device="cuda:0")
+
+    coef = torch.empty(7 * n ** 3, dtype=torch.float64, device="cuda:0")
+    if pde == "codi":
+        beta = codi_beta(n)
+        acr.acr_stencil_codi(n, dev(beta.ravel()), coef)
+        st = stencil_codi(beta, n)
+    else:
+        kappa = gaussian_field_kappa(n, 3)
+        acr.acr_stencil_poisson(n, dev(kappa), coef)
+        st = stencil_poisson(kappa, n)
+    f = uniform_rhs(n, 5)
+    its = {}
+    for prec in (acr.ACR_FP64, acr.ACR_FP32):
+        h = acr.Handle(n, coef, eps, eta, 64, prec, cap)
+        u = torch.zeros(n ** 3, dtype=torch.float64, device="cuda:0")
+        info, _ = acr.acr_krylov_solve(h.h, coef, acr.ACR_GMRES, 30, 1e-9, 200, dev(f), u)
+        h.close()
+        its[prec] = info.iterations
+        res = np.linalg.norm(f - stencil_apply(st, n, u.cpu().numpy())) / np.linalg.norm(f)
+        assert res <= 1.0001e-9, (prec, res)
+    assert abs(its[acr.ACR_FP32] - its[acr.ACR_FP64]) <= 1, its
