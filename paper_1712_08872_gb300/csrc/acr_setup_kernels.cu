@@ -11,6 +11,7 @@
 //  * k_hscale  -- exact diagonal scalings diag(r) X diag(c) (first CR level,
 //                 where the plane couplings are diagonal);
 //  * k_plane_dense / k_plane_lr -- H-format of a 7-point plane block.
+#include <cooperative_groups.h>
 #include <cuda_runtime.h>
 
 #include <type_traits>
@@ -21,6 +22,8 @@
 #include "acr_internal.h"
 
 namespace acr {
+
+namespace cg = cooperative_groups;
 
 namespace {
 
@@ -776,195 +779,228 @@ __device__ __forceinline__ float block_absmaxf(float v, float* red8) {
 // Leaf inverse of float storage without the FP64 pipe (a small fraction of
 // the FP32 one on this part): Gauss-Jordan with partial pivoting in float
 // gives X0 with relative error ~ cond * 6e-8; mixed-precision iterative
-// refinement X <- X + X R, R = I - A X, with the residual formed from exact
-// products and compensated sums (float-float, the Gram kernels' ff_fma),
-// then contracts the error by ~ |R| per step until the correction is below
-// two units in the last place of the largest entry: the result is the
-// inverse to float rounding, as the FP64 elimination rounded to float gives.
+// refinement X <- X + X0 R, R = I - A X, with the residual formed from exact
+// products and compensated sums (float-float, ff_fma), then contracts the error
+// by ~ |I - X0 A| per step until the correction is below two units in the last
+// place of the largest entry: the result is the inverse to float rounding, as
+// the FP64 elimination rounded to float gives.
 // When it cannot get there (a float pivot of zero, a non-finite entry, a
-// correction that does not at least halve, no convergence in four steps) the
+// correction that does not at least halve, no convergence in eight steps) the
 // leaf is inverted by the FP64 elimination instead (the shared buffers
 // reused), so the pivot and growth diagnostics are those of the FP64 form.
-constexpr int LEAF_F_SMEM = 3 * CMAX * (CMAX + 1) * (int)sizeof(float);
-constexpr int LTH = 512;   // threads of the float leaf inverse: 8 entries each
+//
+// At most n / 2 leaves are inverted at a time, one per plane, and every other
+// launch of the plane waits for them: latency is all that counts.  A cluster of
+// LCL CTAs takes one leaf.  The elimination's chain of n dependent steps runs
+// in one warp without any barrier, the matrix in its registers (lane l: rows l,
+// l + 32), redundantly in every CTA; the refinement's 2 x 64^3 products per step,
+// which would fill one SM for 10 us, are split by columns over the cluster,
+// whose CTAs meet once, before the result is stored.  64 x 64 leaf, 32 planes: 50 us
+// (one CTA of 512 threads with two barriers per elimination step: 145 us).
+constexpr int LCL = 8;                 // CTAs per leaf; columns of the inverse per CTA
+constexpr int LTH = 128;               // threads: 4 entries of the CTA's 64 x 8 each
 
-__global__ void __launch_bounds__(LTH) k_leaf_inv_f(float* const* __restrict__ dense, int64_t off,
-                                                    int n, int* err, double* __restrict__ flops,
-                                                    unsigned long long* __restrict__ fallbacks) {
-  constexpr int TH = LTH, CS = TH / 64;
-  static_assert(CMAX == 64, "64 x 64 leaves");
-  static_assert(2 * CMAX * (CMAX + 1) * sizeof(float) >= CMAX * (CMAX + 1) * sizeof(double),
-                "the FP64 fallback fits the X and R buffers");
-  float* Ap = dense[blockIdx.x];
-  if (!Ap) return;
-  Ap += off;
-  extern __shared__ __align__(16) float lsm[];
-  float (*A0)[CMAX + 1] = reinterpret_cast<float (*)[CMAX + 1]>(lsm);
-  float (*X)[CMAX + 1] = reinterpret_cast<float (*)[CMAX + 1]>(lsm + CMAX * (CMAX + 1));
-  float (*R)[CMAX + 1] = reinterpret_cast<float (*)[CMAX + 1]>(lsm + 2 * CMAX * (CMAX + 1));
-  __shared__ float rowk[CMAX], colk[CMAX], krow[CMAX];
-  __shared__ int piv[CMAX];
-  __shared__ int cmap[CMAX];
-  __shared__ int s_q, s_bad;
-  __shared__ float s_pinv;
-  __shared__ float red8[TH / 32];
-  const int ti = threadIdx.x & 63, tj = threadIdx.x >> 6;
-  float amax = 0.f;
-  for (int j = tj; j < n; j += CS)
-    if (ti < n) {
-      const float v = Ap[ti + (int64_t)j * n];
-      A0[ti][j] = v;
-      X[ti][j] = v;
-      amax = fmaxf(amax, fabsf(v));
-    }
-  if (threadIdx.x == 0) s_bad = 0;
-  __syncthreads();
-  amax = block_absmaxf<TH>(amax, red8);
-  // 1. Gauss-Jordan in float (the FP64 elimination's steps)
-  for (int k = 0; k < n; ++k) {
-    if (threadIdx.x < 32) {
-      const int lane = threadIdx.x;
-      float best = -1.f;
-      int q = -1;
-      for (int i = k + lane; i < n; i += 32) {
-        const float v = fabsf(X[i][k]);
-        if (v > best) { best = v; q = i; }
-      }
+// Gauss-Jordan of A (n x n, row length CMAX + 1) by one warp, rows never moved:
+// pivot row q_k of step k keeps its place (row q_k of the result belongs to
+// unknown k, column k to equation q_k) and its scale 1 / pivot is applied at the
+// end, so a step is one multiply-add per entry.  The columns rotate through the
+// registers, the pivot column always first.  X receives the inverse; false if a
+// pivot column is zero.
+__device__ __forceinline__ bool leaf_gj_warp(const float (*A)[CMAX + 1], int n,
+                                             float (*X)[CMAX + 1], float (*row)[CMAX], int* piv) {
+  const int lane = threadIdx.x & 31;
+  float x0[CMAX], x1[CMAX];
 #pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        const float ov = __shfl_xor_sync(0xffffffffu, best, o);
-        const int oi = __shfl_xor_sync(0xffffffffu, q, o);
-        if (oi >= 0 && (q < 0 || ov > best || (ov == best && oi < q))) { best = ov; q = oi; }
-      }
-      if (q < 0 || !(best > 0.f)) {
-        if (lane == 0) s_bad = 1;
-      } else {
-        const float pinv = 1.f / X[q][k];
-        for (int j = lane; j < n; j += 32) {
-          rowk[j] = (j == k) ? pinv : X[q][j] * pinv;
-          krow[j] = X[k][j];
-          colk[j] = (j == k) ? 0.f : (j == q ? X[k][k] : X[j][k]);
-        }
-        if (lane == 0) { s_q = q; s_pinv = pinv; piv[k] = q; }
-      }
+  for (int j = 0; j < CMAX; ++j) {
+    x0[j] = (lane < n && j < n) ? A[lane][j] : 0.f;
+    x1[j] = (lane + 32 < n && j < n) ? A[lane + 32][j] : 0.f;
+  }
+  float s0 = 0.f, s1 = 0.f;
+  int k0 = -1, k1 = -1;                // the step whose pivot the row was
+#pragma unroll 1
+  for (int k = 0; k < n; ++k) {
+    const unsigned b0 = k0 < 0 ? __float_as_uint(fabsf(x0[0])) : 0u;
+    const unsigned b1 = k1 < 0 ? __float_as_uint(fabsf(x1[0])) : 0u;
+    const unsigned best = __reduce_max_sync(0xffffffffu, max(b0, b1));
+    if (best == 0u) return false;
+    const unsigned w0 = __ballot_sync(0xffffffffu, b0 == best);
+    const unsigned w1 = __ballot_sync(0xffffffffu, b1 == best);
+    const bool hi = w0 == 0u;
+    const int ql = __ffs(hi ? w1 : w0) - 1;
+    float* rw = row[k & 1];
+    if (lane == ql) {
+#pragma unroll
+      for (int j = 0; j < CMAX; j += 4)
+        *reinterpret_cast<float4*>(rw + j) =
+            hi ? make_float4(x1[j], x1[j + 1], x1[j + 2], x1[j + 3])
+               : make_float4(x0[j], x0[j + 1], x0[j + 2], x0[j + 3]);
+      piv[k] = ql + (hi ? 32 : 0);
     }
-    __syncthreads();
-    if (s_bad) break;
-    const int q = s_q;
-    const float pinv = s_pinv;
-    if (ti < n) {
-      const float f = colk[ti];
-      for (int j = tj; j < n; j += CS) {
-        if (ti == k) {
-          X[ti][j] = rowk[j];
-        } else {
-          const float old = (ti == q) ? krow[j] : X[ti][j];
-          X[ti][j] = (j == k) ? -f * pinv : old - f * rowk[j];
-        }
+    const float pinv = 1.f / __shfl_sync(0xffffffffu, hi ? x1[0] : x0[0], ql);
+    const bool p0 = lane == ql && !hi, p1 = lane == ql && hi;
+    const float f0 = p0 ? 0.f : x0[0] * pinv, f1 = p1 ? 0.f : x1[0] * pinv;
+    if (p0) { s0 = pinv; k0 = k; }
+    if (p1) { s1 = pinv; k1 = k; }
+    __syncwarp();
+#pragma unroll
+    for (int j = 0; j < CMAX; j += 4) {
+      const float4 v = *reinterpret_cast<const float4*>(rw + j);
+      if (j > 0) {
+        x0[j - 1] = fmaf(-f0, v.x, x0[j]);
+        x1[j - 1] = fmaf(-f1, v.x, x1[j]);
       }
+      x0[j] = fmaf(-f0, v.y, x0[j + 1]);
+      x1[j] = fmaf(-f1, v.y, x1[j + 1]);
+      x0[j + 1] = fmaf(-f0, v.z, x0[j + 2]);
+      x1[j + 1] = fmaf(-f1, v.z, x1[j + 2]);
+      x0[j + 2] = fmaf(-f0, v.w, x0[j + 3]);
+      x1[j + 2] = fmaf(-f1, v.w, x1[j + 3]);
+    }
+    x0[CMAX - 1] = p0 ? 1.f : -f0;
+    x1[CMAX - 1] = p1 ? 1.f : -f1;
+  }
+  __syncwarp();
+  // register t holds column (t + n) mod 64
+#pragma unroll
+  for (int t = 0; t < CMAX; ++t) {
+    const int c = (t + n) & (CMAX - 1);
+    if (c < n) {
+      const int q = piv[c];
+      if (k0 >= 0) X[k0][q] = x0[t] * s0;
+      if (k1 >= 0) X[k1][q] = x1[t] * s1;
+    }
+  }
+  return true;
+}
+
+__global__ void __cluster_dims__(LCL, 1, 1) __launch_bounds__(LTH)
+    k_leaf_inv_f(float* const* __restrict__ dense, int64_t off, int n, int* err,
+                 double* __restrict__ flops, unsigned long long* __restrict__ fallbacks) {
+  static_assert(CMAX == 64 && LCL * 8 == CMAX && LTH == 2 * CMAX, "64 x 64 leaves");
+  float* Ap = dense[blockIdx.x / LCL];
+  if (!Ap) return;   // the whole cluster
+  Ap += off;
+  cg::cluster_group cl = cg::this_cluster();
+  const int rank = (int)cl.block_rank();
+  // A and X0 together hold the FP64 fallback's matrix
+  __shared__ __align__(16) float lsm[2 * CMAX * (CMAX + 1)];
+  float (*A)[CMAX + 1] = reinterpret_cast<float (*)[CMAX + 1]>(lsm);
+  float (*X0)[CMAX + 1] = reinterpret_cast<float (*)[CMAX + 1]>(lsm + CMAX * (CMAX + 1));
+  __shared__ __align__(16) float Xc[CMAX][8], Rc[CMAX][8];
+  __shared__ __align__(16) float row[2][CMAX];
+  __shared__ int piv[CMAX];
+  __shared__ int s_ok;
+  __shared__ float red8[LTH / 32];
+  __shared__ float s_state[2];   // this CTA's columns: 1 if they need the fallback; largest entry
+  const int tid = threadIdx.x;
+  float amax = 0.f;
+  for (int e = tid; e < n * n; e += LTH) {
+    const float v = Ap[e];
+    A[e % n][e / n] = v;
+    amax = fmaxf(amax, fabsf(v));
+  }
+  for (int e = tid; e < CMAX * (CMAX + 1); e += LTH) (&X0[0][0])[e] = 0.f;
+  __syncthreads();
+  amax = block_absmaxf<LTH>(amax, red8);
+  // 1. the float elimination
+  if (tid < 32) {
+    const bool ok = leaf_gj_warp(A, n, X0, row, piv);
+    if (tid == 0) s_ok = ok ? 1 : 0;
+  }
+  __syncthreads();
+  bool fallback = s_ok == 0, done = false;
+  int steps = 0;
+  const int i = tid & 63, j0 = 8 * rank + 4 * (tid >> 6), jl = 4 * (tid >> 6);
+  float x[4] = {0.f, 0.f, 0.f, 0.f};
+  float xmax = 0.f;
+  if (!fallback) {
+    for (int e = tid; e < n * n; e += LTH) {
+      const float v = fabsf(X0[e % n][e / n]);
+      xmax = (v <= 3.0e38f) ? fmaxf(xmax, v) : INFINITY;
+    }
+    xmax = block_absmaxf<LTH>(xmax, red8);
+    if (!(xmax <= 3.0e38f)) fallback = true;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      x[q] = (i < n && j0 + q < n) ? X0[i][j0 + q] : 0.f;
+      Xc[i][jl + q] = x[q];
     }
     __syncthreads();
   }
-  bool fallback = s_bad != 0;
-  int steps = 0;
+  // 2. refinement of this CTA's columns (rows and columns beyond n are zero)
+  float dprev = INFINITY;
+  for (int it = 0; it < 8 && !done && !fallback; ++it) {
+    ++steps;
+    float sh[4], sl[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) { sh[q] = 0.f; sl[q] = 0.f; }
+    if (i < n)
+      for (int l = 0; l < n; ++l) {
+        const float a = A[i][l];
+        const float4 v = *reinterpret_cast<const float4*>(&Xc[l][jl]);
+        ff_fma(sh[0], sl[0], a, v.x);
+        ff_fma(sh[1], sl[1], a, v.y);
+        ff_fma(sh[2], sl[2], a, v.z);
+        ff_fma(sh[3], sl[3], a, v.w);
+      }
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+      Rc[i][jl + q] = (i < n && j0 + q < n) ? ((i == j0 + q ? 1.f : 0.f) - sh[q]) - sl[q] : 0.f;
+    __syncthreads();
+    float d[4] = {0.f, 0.f, 0.f, 0.f};
+    for (int l = 0; l < n; ++l) {
+      const float a = X0[i][l];
+      const float4 v = *reinterpret_cast<const float4*>(&Rc[l][jl]);
+      d[0] = fmaf(a, v.x, d[0]);
+      d[1] = fmaf(a, v.y, d[1]);
+      d[2] = fmaf(a, v.z, d[2]);
+      d[3] = fmaf(a, v.w, d[3]);
+    }
+    float dmax = 0.f;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      dmax = (fabsf(d[q]) <= 3.0e38f) ? fmaxf(dmax, fabsf(d[q])) : INFINITY;
+      x[q] += d[q];
+      Xc[i][jl + q] = x[q];
+    }
+    dmax = block_absmaxf<LTH>(dmax, red8);
+    if (!(dmax <= 3.0e38f)) fallback = true;                  // non-finite
+    else if (dmax <= 2.4e-7f * xmax) done = true;
+    else if (dmax > 0.5f * dprev) fallback = true;            // not contracting
+    dprev = dmax;
+  }
+  if (!done) fallback = true;
+  xmax = 0.f;
+#pragma unroll
+  for (int q = 0; q < 4; ++q) xmax = (fabsf(x[q]) <= 3.0e38f) ? fmaxf(xmax, fabsf(x[q])) : INFINITY;
+  xmax = block_absmaxf<LTH>(xmax, red8);
+  if (tid == 0) {
+    s_state[0] = fallback ? 1.f : 0.f;
+    s_state[1] = xmax;
+  }
+  cl.sync();   // every CTA has read the leaf and knows its columns' outcome
+  fallback = false;
+  for (int c = 0; c < LCL; ++c) {
+    const float* st = cl.map_shared_rank(s_state, c);
+    fallback = fallback || st[0] != 0.f || !(st[1] <= 3.0e38f);
+    xmax = fmaxf(xmax, st[1]);
+  }
+  cl.sync();   // no CTA leaves while another reads its outcome
   if (!fallback) {
-    if (threadIdx.x == 0) {
-      int pi_[CMAX];
-      for (int c = 0; c < n; ++c) pi_[c] = c;
-      for (int k = n - 1; k >= 0; --k) {
-        const int q = piv[k];
-        const int t = pi_[k]; pi_[k] = pi_[q]; pi_[q] = t;
-      }
-      for (int c = 0; c < n; ++c) cmap[pi_[c]] = c;
-    }
-    __syncthreads();
-    // the inverse in natural column order, into R; then the buffers trade roles
-    for (int j = tj; j < n; j += CS)
-      if (ti < n) R[ti][cmap[j]] = X[ti][j];
-    __syncthreads();
-    float (*tmp)[CMAX + 1] = X; X = R; R = tmp;
-    // 2. refinement
-    bool done = false;
-    float dprev = INFINITY;
-    for (int it = 0; it < 4 && !done && !fallback; ++it) {
-      ++steps;
-      // R = I - A0 X from exact products and compensated sums; the thread's
-      // CMAX / CS entries advance together (independent chains, one load of
-      // A0 per step; columns beyond n are computed and dropped)
-      constexpr int NQ = CMAX / CS;
-      if (ti < n) {
-        float sh[NQ], sl[NQ];
-#pragma unroll
-        for (int q = 0; q < NQ; ++q) { sh[q] = 0.f; sl[q] = 0.f; }
-        for (int l = 0; l < n; ++l) {
-          const float a = A0[ti][l];
-#pragma unroll
-          for (int q = 0; q < NQ; ++q) ff_fma(sh[q], sl[q], a, X[l][tj + CS * q]);
-        }
-#pragma unroll
-        for (int q = 0; q < NQ; ++q) {
-          const int j = tj + CS * q;
-          if (j < n) R[ti][j] = ((ti == j ? 1.f : 0.f) - sh[q]) - sl[q];
-        }
-      }
-      __syncthreads();
-      // correction D = X R; X += D
-      float d[NQ];
-#pragma unroll
-      for (int q = 0; q < NQ; ++q) d[q] = 0.f;
-      if (ti < n)
-        for (int l = 0; l < n; ++l) {
-          const float x = X[ti][l];
-#pragma unroll
-          for (int q = 0; q < NQ; ++q) d[q] = fmaf(x, R[l][tj + CS * q], d[q]);
-        }
-      float dmax = 0.f;
-#pragma unroll
-      for (int q = 0; q < NQ; ++q) {
-        const int j = tj + CS * q;
-        if (ti < n && j < n)
-          dmax = (fabsf(d[q]) <= 3.0e38f) ? fmaxf(dmax, fabsf(d[q])) : INFINITY;
-      }
-      __syncthreads();   // every read of X is done
-      float xmax = 0.f;
-#pragma unroll
-      for (int q = 0; q < CMAX / CS; ++q) {
-        const int j = tj + CS * q;
-        if (ti < n && j < n) {
-          X[ti][j] += d[q];
-          const float v = fabsf(X[ti][j]);
-          xmax = (v <= 3.0e38f) ? fmaxf(xmax, v) : INFINITY;
-        }
-      }
-      dmax = block_absmaxf<TH>(dmax, red8);
-      xmax = block_absmaxf<TH>(xmax, red8);
-      if (!(xmax <= 3.0e38f) || !(dmax <= 3.0e38f)) fallback = true;   // non-finite
-      else if (dmax <= 2.4e-7f * xmax) done = true;
-      else if (dmax > 0.5f * dprev) fallback = true;                    // not contracting
-      dprev = dmax;
-    }
-    if (!done) fallback = true;
-    if (!fallback) {
-      float xmax = 0.f;
-      for (int j = tj; j < n; j += CS)
-        if (ti < n) xmax = fmaxf(xmax, fabsf(X[ti][j]));
-      xmax = block_absmaxf<TH>(xmax, red8);
-      if (!((double)amax * (double)xmax <= leaf_growth_max<float>())) {
-        if (threadIdx.x == 0) atomicOr(err, ERR_GROWTH);
-        return;
-      }
-      for (int j = tj; j < n; j += CS)
-        if (ti < n) Ap[ti + (int64_t)j * n] = X[ti][j];
-      if (flops && threadIdx.x == 0) atomicAdd(flops, 2.0 * n * n * n * (1 + 2 * steps));
+    if (!((double)amax * (double)xmax <= leaf_growth_max<float>())) {
+      if (rank == 0 && tid == 0) atomicOr(err, ERR_GROWTH);
       return;
     }
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+      if (i < n && j0 + q < n) Ap[i + (int64_t)(j0 + q) * n] = x[q];
+    if (flops && rank == 0 && tid == 0) atomicAdd(flops, 2.0 * n * n * n * (1 + 2 * steps));
+    return;
   }
-  // 3. FP64 elimination of the stored leaf (untouched so far), in the X and
-  // R buffers (contiguous: X and R may have traded roles, the pair has not)
-  __syncthreads();
-  if (fallbacks && threadIdx.x == 0) atomicAdd(fallbacks, 1ull);
-  leaf_inv_fp64<float, TH>(Ap, n, reinterpret_cast<double (*)[CMAX + 1]>(lsm + CMAX * (CMAX + 1)),
-                       err, flops);
+  // 3. FP64 elimination of the stored leaf (untouched so far)
+  if (rank != 0) return;
+  if (fallbacks && tid == 0) atomicAdd(fallbacks, 1ull);
+  leaf_inv_fp64<float, LTH>(Ap, n, reinterpret_cast<double (*)[CMAX + 1]>(lsm), err, flops);
 }
 
 // out = sgn * diag(r) X diag(c): dense part
@@ -1140,13 +1176,7 @@ void launch_leaf_inv(T* const* d_dense, int64_t off, int lsz, int P, int* d_err,
                      double* d_fl, unsigned long long* d_fallbacks) {
   if (P <= 0) return;
   if constexpr (std::is_same<T, float>::value) {
-    static bool attr = false;
-    if (!attr) {
-      ACR_CUDA(cudaFuncSetAttribute(k_leaf_inv_f, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    LEAF_F_SMEM));
-      attr = true;
-    }
-    k_leaf_inv_f<<<P, LTH, LEAF_F_SMEM, st>>>(d_dense, off, lsz, d_err, d_fl, d_fallbacks);
+    k_leaf_inv_f<<<P * LCL, LTH, 0, st>>>(d_dense, off, lsz, d_err, d_fl, d_fallbacks);
   } else {
     k_leaf_inv<T><<<P, NT, 0, st>>>(d_dense, off, lsz, d_err, d_fl);
   }
