@@ -791,84 +791,102 @@ __device__ __forceinline__ float block_absmaxf(float v, float* red8) {
 //
 // At most n / 2 leaves are inverted at a time, one per plane, and every other
 // launch of the plane waits for them: latency is all that counts.  A cluster of
-// LCL CTAs takes one leaf.  The elimination's chain of n dependent steps runs
-// in one warp without any barrier, the matrix in its registers (lane l: rows l,
-// l + 32), redundantly in every CTA; the refinement's 2 x 64^3 products per step,
-// which would fill one SM for 10 us, are split by columns over the cluster,
-// whose CTAs meet once, before the result is stored.  64 x 64 leaf, 32 planes: 50 us
-// (one CTA of 512 threads with two barriers per elimination step: 145 us).
+// LCL CTAs takes one leaf.  Every CTA eliminates the whole leaf (cheaper than
+// an exchange per step): panels of 8 columns in one warp's registers, whose
+// 8 dependent steps (pivot search by one warp-wide maximum, 8 shuffles, 16
+// multiply-adds per lane) need no barrier, then one rank-8 update of the other
+// columns by all warps.  The refinement's 2 x 64^3 products per step, which would
+// fill one SM for 10 us, are split by columns over the cluster; the outcomes are
+// pushed to every CTA before the one cluster barrier.  64 x 64 leaf, 1 to
+// 32 planes: 27 to 35 us (one CTA with two barriers per elimination step:
+// 141 to 145 us; the whole leaf in one warp's registers, 64 columns per step: 50 us).
 constexpr int LCL = 8;                 // CTAs per leaf; columns of the inverse per CTA
-constexpr int LTH = 128;               // threads: 4 entries of the CTA's 64 x 8 each
+constexpr int LTH = 256;               // threads: 2 entries of the CTA's 64 x 8 each
+constexpr int LPW = 8;                 // panel width
 
-// Gauss-Jordan of A (n x n, row length CMAX + 1) by one warp, rows never moved:
-// pivot row q_k of step k keeps its place (row q_k of the result belongs to
-// unknown k, column k to equation q_k) and its scale 1 / pivot is applied at the
-// end, so a step is one multiply-add per entry.  The columns rotate through the
-// registers, the pivot column always first.  X receives the inverse; false if a
-// pivot column is zero.
-__device__ __forceinline__ bool leaf_gj_warp(const float (*A)[CMAX + 1], int n,
-                                             float (*X)[CMAX + 1], float (*row)[CMAX], int* piv) {
-  const int lane = threadIdx.x & 31;
-  float x0[CMAX], x1[CMAX];
+// In-place Gauss-Jordan inverse of X (64 x 64, rows and columns from n on zero) by the CTA, rows
+// never moved: pivot row piv[k] of step k keeps its place, so that the result's
+// row piv[k] belongs to unknown k and its column k to equation piv[k].  False if
+// a pivot column is zero (to within 64 subnormal units).
+__device__ __forceinline__ bool leaf_gj(float (*X)[CMAX + 1], int n, float (*xq)[CMAX], int* piv,
+                                        int* step, int* s_ok) {
+  const int tid = threadIdx.x, lane = tid & 31;
+  constexpr int NC = CMAX / (LTH / 64);   // columns of a thread's row in the update
+  const int i = tid & 63, c0 = (tid >> 6) * NC;
+  unsigned used = 0;                   // warp 0: bit 0 row lane, bit 1 row lane + 32
+  if (tid == 0) *s_ok = 1;
+  if (tid < CMAX) step[tid] = -1;      // the step whose pivot a row was
+  __syncthreads();
+  for (int kb = 0; kb < n; kb += LPW) {
+    const int kw = min(LPW, n - kb);
+    if (tid < 32) {
+      float x0[LPW], x1[LPW], s0 = 1.f, s1 = 1.f;
 #pragma unroll
-  for (int j = 0; j < CMAX; ++j) {
-    x0[j] = (lane < n && j < n) ? A[lane][j] : 0.f;
-    x1[j] = (lane + 32 < n && j < n) ? A[lane + 32][j] : 0.f;
-  }
-  float s0 = 0.f, s1 = 0.f;
-  int k0 = -1, k1 = -1;                // the step whose pivot the row was
-#pragma unroll 1
-  for (int k = 0; k < n; ++k) {
-    const unsigned b0 = k0 < 0 ? __float_as_uint(fabsf(x0[0])) : 0u;
-    const unsigned b1 = k1 < 0 ? __float_as_uint(fabsf(x1[0])) : 0u;
-    const unsigned best = __reduce_max_sync(0xffffffffu, max(b0, b1));
-    if (best == 0u) return false;
-    const unsigned w0 = __ballot_sync(0xffffffffu, b0 == best);
-    const unsigned w1 = __ballot_sync(0xffffffffu, b1 == best);
-    const bool hi = w0 == 0u;
-    const int ql = __ffs(hi ? w1 : w0) - 1;
-    float* rw = row[k & 1];
-    if (lane == ql) {
+      for (int c = 0; c < LPW; ++c) { x0[c] = X[lane][kb + c]; x1[c] = X[lane + 32][kb + c]; }
 #pragma unroll
-      for (int j = 0; j < CMAX; j += 4)
-        *reinterpret_cast<float4*>(rw + j) =
-            hi ? make_float4(x1[j], x1[j + 1], x1[j + 2], x1[j + 3])
-               : make_float4(x0[j], x0[j + 1], x0[j + 2], x0[j + 3]);
-      piv[k] = ql + (hi ? 32 : 0);
-    }
-    const float pinv = 1.f / __shfl_sync(0xffffffffu, hi ? x1[0] : x0[0], ql);
-    const bool p0 = lane == ql && !hi, p1 = lane == ql && hi;
-    const float f0 = p0 ? 0.f : x0[0] * pinv, f1 = p1 ? 0.f : x1[0] * pinv;
-    if (p0) { s0 = pinv; k0 = k; }
-    if (p1) { s1 = pinv; k1 = k; }
-    __syncwarp();
+      for (int t = 0; t < LPW; ++t) {
+        if (t < kw) {
+          // the largest remaining |entry| of column kb + t, its row in the six low
+          // bits (entries that agree to 2^-17 count as equal: the lowest row)
+          const unsigned b0 = (used & 1u) ? 0u : ((__float_as_uint(fabsf(x0[t])) & ~63u) | (63u - lane));
+          const unsigned b1 = (used & 2u) ? 0u : ((__float_as_uint(fabsf(x1[t])) & ~63u) | (31u - lane));
+          const unsigned best = __reduce_max_sync(0xffffffffu, max(b0, b1));
+          const int q = 63 - (int)(best & 63u);
+          if ((best & ~63u) == 0u && lane == 0) *s_ok = 0;
+          const bool hi = q >= 32;
+          float v[LPW];
 #pragma unroll
-    for (int j = 0; j < CMAX; j += 4) {
-      const float4 v = *reinterpret_cast<const float4*>(rw + j);
-      if (j > 0) {
-        x0[j - 1] = fmaf(-f0, v.x, x0[j]);
-        x1[j - 1] = fmaf(-f1, v.x, x1[j]);
+          for (int c = 0; c < LPW; ++c) v[c] = __shfl_sync(0xffffffffu, hi ? x1[c] : x0[c], q & 31);
+          // (the pivot row is scaled when the panel is done: until then its entries,
+          // the multipliers it is updated with included, are 1 / s times their value)
+          const float pinv = 1.f / v[t];
+          const bool p0 = lane == q, p1 = lane + 32 == q;
+          used |= (p0 ? 1u : 0u) | (p1 ? 2u : 0u);
+          const float f0 = p0 ? 0.f : x0[t] * pinv, f1 = p1 ? 0.f : x1[t] * pinv;
+          s0 = p0 ? pinv : s0;
+          s1 = p1 ? pinv : s1;
+#pragma unroll
+          for (int c = 0; c < LPW; ++c)
+            if (c != t) {
+              x0[c] = fmaf(-f0, v[c], x0[c]);
+              x1[c] = fmaf(-f1, v[c], x1[c]);
+            }
+          x0[t] = p0 ? 1.f : -f0;
+          x1[t] = p1 ? 1.f : -f1;
+          if (lane == 0) { piv[kb + t] = q; step[q] = kb + t; }
+        }
       }
-      x0[j] = fmaf(-f0, v.y, x0[j + 1]);
-      x1[j] = fmaf(-f1, v.y, x1[j + 1]);
-      x0[j + 1] = fmaf(-f0, v.z, x0[j + 2]);
-      x1[j + 1] = fmaf(-f1, v.z, x1[j + 2]);
-      x0[j + 2] = fmaf(-f0, v.w, x0[j + 3]);
-      x1[j + 2] = fmaf(-f1, v.w, x1[j + 3]);
-    }
-    x0[CMAX - 1] = p0 ? 1.f : -f0;
-    x1[CMAX - 1] = p1 ? 1.f : -f1;
-  }
-  __syncwarp();
-  // register t holds column (t + n) mod 64
 #pragma unroll
-  for (int t = 0; t < CMAX; ++t) {
-    const int c = (t + n) & (CMAX - 1);
-    if (c < n) {
-      const int q = piv[c];
-      if (k0 >= 0) X[k0][q] = x0[t] * s0;
-      if (k1 >= 0) X[k1][q] = x1[t] * s1;
+      for (int c = 0; c < LPW; ++c)
+        if (c < kw) { X[lane][kb + c] = x0[c] * s0; X[lane + 32][kb + c] = x1[c] * s1; }
     }
+    __syncthreads();
+    if (!*s_ok) return false;
+    // the pivot rows' old entries, then X[i][j] <- (i not a pivot row) X[i][j] +
+    // sum_t X[i][kb + t] xq[t][j] for the columns outside the panel
+    float pr[LPW], y[NC];
+    const bool pivot = step[i] >= kb;
+#pragma unroll
+    for (int t = 0; t < LPW; ++t) pr[t] = t < kw ? X[i][kb + t] : 0.f;
+#pragma unroll
+    for (int u = 0; u < NC; ++u) y[u] = pivot ? 0.f : X[i][c0 + u];
+    for (int e = tid; e < LPW * CMAX; e += LTH)
+      xq[e >> 6][e & 63] = (e >> 6) < kw ? X[piv[kb + (e >> 6)]][e & 63] : 0.f;
+    __syncthreads();
+#pragma unroll
+    for (int t = 0; t < LPW; ++t)
+#pragma unroll
+      for (int u = 0; u < NC; u += 4) {
+        const float4 v = *reinterpret_cast<const float4*>(&xq[t][c0 + u]);
+        y[u] = fmaf(pr[t], v.x, y[u]);
+        y[u + 1] = fmaf(pr[t], v.y, y[u + 1]);
+        y[u + 2] = fmaf(pr[t], v.z, y[u + 2]);
+        y[u + 3] = fmaf(pr[t], v.w, y[u + 3]);
+      }
+#pragma unroll
+    for (int u = 0; u < NC; ++u)
+      if (c0 + u < kb || c0 + u >= kb + LPW) X[i][c0 + u] = y[u];
+    __syncthreads();
   }
   return true;
 }
@@ -876,7 +894,7 @@ __device__ __forceinline__ bool leaf_gj_warp(const float (*A)[CMAX + 1], int n,
 __global__ void __cluster_dims__(LCL, 1, 1) __launch_bounds__(LTH)
     k_leaf_inv_f(float* const* __restrict__ dense, int64_t off, int n, int* err,
                  double* __restrict__ flops, unsigned long long* __restrict__ fallbacks) {
-  static_assert(CMAX == 64 && LCL * 8 == CMAX && LTH == 2 * CMAX, "64 x 64 leaves");
+  static_assert(CMAX == 64 && LCL * 8 == CMAX && LTH == 4 * CMAX, "64 x 64 leaves");
   float* Ap = dense[blockIdx.x / LCL];
   if (!Ap) return;   // the whole cluster
   Ap += off;
@@ -887,41 +905,51 @@ __global__ void __cluster_dims__(LCL, 1, 1) __launch_bounds__(LTH)
   float (*A)[CMAX + 1] = reinterpret_cast<float (*)[CMAX + 1]>(lsm);
   float (*X0)[CMAX + 1] = reinterpret_cast<float (*)[CMAX + 1]>(lsm + CMAX * (CMAX + 1));
   __shared__ __align__(16) float Xc[CMAX][8], Rc[CMAX][8];
-  __shared__ __align__(16) float row[2][CMAX];
-  __shared__ int piv[CMAX];
+  float (*xq)[CMAX] = reinterpret_cast<float (*)[CMAX]>(&Rc[0][0]);   // elimination only
+  __shared__ int piv[CMAX], step[CMAX];
   __shared__ int s_ok;
   __shared__ float red8[LTH / 32];
-  __shared__ float s_state[2];   // this CTA's columns: 1 if they need the fallback; largest entry
+  __shared__ float s_state[LCL][2];   // per column group: 1 if it needs the fallback; largest entry
   const int tid = threadIdx.x;
+  const int i = tid & 63, jl = 2 * (tid >> 6), j0 = 8 * rank + jl;
   float amax = 0.f;
-  for (int e = tid; e < n * n; e += LTH) {
-    const float v = Ap[e];
-    A[e % n][e / n] = v;
-    amax = fmaxf(amax, fabsf(v));
+  {
+    float v[CMAX / 4];
+#pragma unroll
+    for (int q = 0; q < CMAX / 4; ++q) {
+      const int j = (tid >> 6) + 4 * q;
+      v[q] = (i < n && j < n) ? Ap[i + (int64_t)j * n] : 0.f;
+    }
+#pragma unroll
+    for (int q = 0; q < CMAX / 4; ++q) {
+      A[i][(tid >> 6) + 4 * q] = v[q];
+      X0[i][(tid >> 6) + 4 * q] = v[q];
+      amax = fmaxf(amax, fabsf(v[q]));
+    }
   }
-  for (int e = tid; e < CMAX * (CMAX + 1); e += LTH) (&X0[0][0])[e] = 0.f;
-  __syncthreads();
   amax = block_absmaxf<LTH>(amax, red8);
-  // 1. the float elimination
-  if (tid < 32) {
-    const bool ok = leaf_gj_warp(A, n, X0, row, piv);
-    if (tid == 0) s_ok = ok ? 1 : 0;
-  }
-  __syncthreads();
-  bool fallback = s_ok == 0, done = false;
+  // 1. the float elimination; its result in natural order
+  bool fallback = !leaf_gj(X0, n, xq, piv, step, &s_ok), done = false;
   int steps = 0;
-  const int i = tid & 63, j0 = 8 * rank + 4 * (tid >> 6), jl = 4 * (tid >> 6);
-  float x[4] = {0.f, 0.f, 0.f, 0.f};
+  float x[2] = {0.f, 0.f};
   float xmax = 0.f;
   if (!fallback) {
-    for (int e = tid; e < n * n; e += LTH) {
-      const float v = fabsf(X0[e % n][e / n]);
-      xmax = (v <= 3.0e38f) ? fmaxf(xmax, v) : INFINITY;
+    float v[CMAX / 4];
+    const int row = step[i];
+#pragma unroll
+    for (int q = 0; q < CMAX / 4; ++q) v[q] = X0[i][(tid >> 6) + 4 * q];
+    __syncthreads();
+#pragma unroll
+    for (int q = 0; q < CMAX / 4; ++q) {
+      const int j = (tid >> 6) + 4 * q;
+      if (i < n && j < n) X0[row][piv[j]] = v[q];
+      const float w = fabsf(v[q]);
+      if (i < n && j < n) xmax = (w <= 3.0e38f) ? fmaxf(xmax, w) : INFINITY;
     }
     xmax = block_absmaxf<LTH>(xmax, red8);
     if (!(xmax <= 3.0e38f)) fallback = true;
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
+    for (int q = 0; q < 2; ++q) {
       x[q] = (i < n && j0 + q < n) ? X0[i][j0 + q] : 0.f;
       Xc[i][jl + q] = x[q];
     }
@@ -931,34 +959,29 @@ __global__ void __cluster_dims__(LCL, 1, 1) __launch_bounds__(LTH)
   float dprev = INFINITY;
   for (int it = 0; it < 8 && !done && !fallback; ++it) {
     ++steps;
-    float sh[4], sl[4];
+    float sh[2] = {0.f, 0.f}, sl[2] = {0.f, 0.f};
+#pragma unroll 4
+    for (int l = 0; l < n; ++l) {
+      const float a = A[i][l];
+      const float2 v = *reinterpret_cast<const float2*>(&Xc[l][jl]);
+      ff_fma(sh[0], sl[0], a, v.x);
+      ff_fma(sh[1], sl[1], a, v.y);
+    }
 #pragma unroll
-    for (int q = 0; q < 4; ++q) { sh[q] = 0.f; sl[q] = 0.f; }
-    if (i < n)
-      for (int l = 0; l < n; ++l) {
-        const float a = A[i][l];
-        const float4 v = *reinterpret_cast<const float4*>(&Xc[l][jl]);
-        ff_fma(sh[0], sl[0], a, v.x);
-        ff_fma(sh[1], sl[1], a, v.y);
-        ff_fma(sh[2], sl[2], a, v.z);
-        ff_fma(sh[3], sl[3], a, v.w);
-      }
-#pragma unroll
-    for (int q = 0; q < 4; ++q)
+    for (int q = 0; q < 2; ++q)
       Rc[i][jl + q] = (i < n && j0 + q < n) ? ((i == j0 + q ? 1.f : 0.f) - sh[q]) - sl[q] : 0.f;
     __syncthreads();
-    float d[4] = {0.f, 0.f, 0.f, 0.f};
+    float d[2] = {0.f, 0.f};
+#pragma unroll 8
     for (int l = 0; l < n; ++l) {
       const float a = X0[i][l];
-      const float4 v = *reinterpret_cast<const float4*>(&Rc[l][jl]);
+      const float2 v = *reinterpret_cast<const float2*>(&Rc[l][jl]);
       d[0] = fmaf(a, v.x, d[0]);
       d[1] = fmaf(a, v.y, d[1]);
-      d[2] = fmaf(a, v.z, d[2]);
-      d[3] = fmaf(a, v.w, d[3]);
     }
     float dmax = 0.f;
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
+    for (int q = 0; q < 2; ++q) {
       dmax = (fabsf(d[q]) <= 3.0e38f) ? fmaxf(dmax, fabsf(d[q])) : INFINITY;
       x[q] += d[q];
       Xc[i][jl + q] = x[q];
@@ -972,27 +995,26 @@ __global__ void __cluster_dims__(LCL, 1, 1) __launch_bounds__(LTH)
   if (!done) fallback = true;
   xmax = 0.f;
 #pragma unroll
-  for (int q = 0; q < 4; ++q) xmax = (fabsf(x[q]) <= 3.0e38f) ? fmaxf(xmax, fabsf(x[q])) : INFINITY;
+  for (int q = 0; q < 2; ++q) xmax = (fabsf(x[q]) <= 3.0e38f) ? fmaxf(xmax, fabsf(x[q])) : INFINITY;
   xmax = block_absmaxf<LTH>(xmax, red8);
-  if (tid == 0) {
-    s_state[0] = fallback ? 1.f : 0.f;
-    s_state[1] = xmax;
+  if (tid < LCL) {   // to every CTA of the cluster
+    float* st = cl.map_shared_rank(&s_state[rank][0], tid);
+    st[0] = fallback ? 1.f : 0.f;
+    st[1] = xmax;
   }
-  cl.sync();   // every CTA has read the leaf and knows its columns' outcome
+  cl.sync();   // every CTA has read the leaf and knows all columns' outcome
   fallback = false;
   for (int c = 0; c < LCL; ++c) {
-    const float* st = cl.map_shared_rank(s_state, c);
-    fallback = fallback || st[0] != 0.f || !(st[1] <= 3.0e38f);
-    xmax = fmaxf(xmax, st[1]);
+    fallback = fallback || s_state[c][0] != 0.f || !(s_state[c][1] <= 3.0e38f);
+    xmax = fmaxf(xmax, s_state[c][1]);
   }
-  cl.sync();   // no CTA leaves while another reads its outcome
   if (!fallback) {
     if (!((double)amax * (double)xmax <= leaf_growth_max<float>())) {
       if (rank == 0 && tid == 0) atomicOr(err, ERR_GROWTH);
       return;
     }
 #pragma unroll
-    for (int q = 0; q < 4; ++q)
+    for (int q = 0; q < 2; ++q)
       if (i < n && j0 + q < n) Ap[i + (int64_t)(j0 + q) * n] = x[q];
     if (flops && rank == 0 && tid == 0) atomicAdd(flops, 2.0 * n * n * n * (1 + 2 * steps));
     return;
