@@ -58,12 +58,13 @@ typedef enum {
  * as in FP32; when it ends every stored factor (dense leaves, U, V) is
  * rounded to bfloat16 (round to nearest even), halving the factor memory and
  * the bytes an apply reads; the apply multiplies in float.  The Krylov
- * iteration is FP64 in every form, and so are the Grams that decide ranks
+ * iteration is FP64 in every form, and so are the core Grams that decide ranks
  * (FP64-accurate float-float sums in the float forms).  The dense leaf
  * inverses and the small recompression cores are FP64 in the FP64 form; in
  * the float forms the leaf inverses are float eliminations refined to float
- * accuracy (FP64 elimination when refinement cannot get there), the Jacobi
- * cores run in float-float and the pivoted Cholesky in FP64.
+ * accuracy (FP64 elimination when refinement cannot get there), the sketch bases come
+ * from a re-orthogonalised float Gram-Schmidt, and the core Grams and Jacobi
+ * cores run in float-float.
  * (Reduced-precision storage is not in the paper, whose H-arithmetic is
  * double precision throughout, Sec. 5.) */
 typedef enum { ACR_FP64 = 0, ACR_FP32 = 1, ACR_BF16 = 2 } acr_precision;
@@ -133,15 +134,17 @@ typedef struct {
 
 typedef struct {
   acr_kernel_stat gemm;      /* grouped small GEMMs (k_ggemm) */
-  acr_kernel_stat orth;      /* pivoted-Cholesky cores (k_pchol), FP64 */
-  acr_kernel_stat eig;       /* Jacobi recompression cores (k_eig; float-float for float factors) */
+  acr_kernel_stat orth;      /* FP64 pivoted-Cholesky cores (k_pchol); float factors: basis kernel (k_orth) */
+  acr_kernel_stat eig;       /* FP64 Jacobi cores (k_eig); float factors: Gram, float-float Jacobi and
+                                recomposition (k_core) */
   acr_kernel_stat leaf_inv;  /* dense leaf inverses (k_leaf_inv; refined float for float factors) */
   acr_kernel_stat other;     /* conversion, scaling */
   /* grouped-GEMM time and counted flops per plan stage: 0 inner products
    * U^T V of phase 1, 1 term factors (H-matrix x block products, dense
    * products), 2 dense-leaf sums, 3 sketches Z^T Omega, 4 sketch Y, 5 first
    * Gram, 6 first basis, 7 second Gram, 8 second basis, 9 X^T Q, 10 B^T,
-   * 11 core Gram, 12 recomposition U = Q W, V = B^T W; 13..15 unused */
+   * 11 core Gram, 12 recomposition U = Q W, V = B^T W (5 to 8 and 11, 12 for
+   * FP64 factors; the float forms' are inside orth and eig); 13..15 unused */
   double stage_ms[16];
   double stage_flops[16];
   /* wall time (CUDA events) of each CR level's H-inversion batch and of its
@@ -214,9 +217,10 @@ acr_status acr_autotune_leaf(const acr_grid* grid, const double* coef, const acr
 /* Autotuner of the setup's grouped-GEMM kernel shapes (the paper has no
  * counterpart): one profiled setup of coef with opt per shape (every stage in
  * shape 0, then every stage in shape 1, 2, 3), then per stage the fastest.
- * Shape 0: one CTA per group, 4 CTAs per SM; shape 1: for float factors 3
- * CTAs per SM with more registers (double: half the K-chunk), and the warp-
- * and CTA-per-group inner-product kernels swapped; shape 2 (float factors,
+ * Shape 0: one CTA per group with tabulated operand rows, and one per bundle of
+ * groups sharing their A operands in the factor stages; shape 1: one CTA per
+ * group staging item by item, and the warp- and CTA-per-group inner-product
+ * kernels swapped; shape 2 (float factors,
  * non-inner-product stages): one warp per group, groups with 64-column
  * outputs on the shape-0 kernel; shape 3: as 2 with those groups on the
  * tcgen05 tensor cores (split-TF32 operands); shape 4: as 2 with 32 output

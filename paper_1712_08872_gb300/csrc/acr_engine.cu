@@ -437,11 +437,13 @@ class Engine : public EngineBase {
     for (auto& kv : plans) {
       cudaFree(kv.second->d_groups); cudaFree(kv.second->d_items); cudaFree(kv.second->d_targets);
       cudaFree(kv.second->d_stack); cudaFree(kv.second->d_torder);
+      cudaFree(kv.second->d_bundles);
     }
     plans.clear();
     for (auto& kv : merged_plans) {
       cudaFree(kv.second->d_groups); cudaFree(kv.second->d_items); cudaFree(kv.second->d_targets);
       cudaFree(kv.second->d_stack); cudaFree(kv.second->d_torder);
+      cudaFree(kv.second->d_bundles);
     }
     merged_plans.clear();
     if (scratch) cudaFree(scratch);
@@ -505,6 +507,11 @@ class Engine : public EngineBase {
     pl.d_items = dmalloc(std::max<size_t>(pl.items.size(), 1) * sizeof(GItem));
     pl.d_targets = dmalloc(std::max<size_t>(pl.targets.size(), 1) * sizeof(TInfo));
     pl.d_stack = dmalloc(std::max<size_t>(pl.stack.size(), 1) * sizeof(StackDim));
+    if (!pl.bundles.empty()) {
+      pl.d_bundles = dmalloc(pl.bundles.size() * sizeof(int32_t));
+      ACR_CUDA(cudaMemcpy(pl.d_bundles, pl.bundles.data(), pl.bundles.size() * sizeof(int32_t),
+                          cudaMemcpyHostToDevice));
+    }
     if (pp.fused && !pl.torder.empty()) {
       pl.d_torder = dmalloc(pl.torder.size() * sizeof(int32_t));
       ACR_CUDA(cudaMemcpy(pl.d_torder, pl.torder.data(), pl.torder.size() * sizeof(int32_t),
@@ -658,8 +665,14 @@ class Engine : public EngineBase {
   void gemm_stage(const Plan& pl, const Stage& sg, T* const* d_tab, const int* const* d_rtab,
                   int pc, cudaStream_t st) {
     double* f = sg.tag >= 0 ? fl(5 + sg.tag) : fl(0);
-    launch_ggemm<T>(pl, sg.beg, sg.end, d_tab, d_rtab, pc, d_coefs, st, f, sg.tag,
-                    sg.tag >= 0 && sg.tag < 16 ? gemm_variant[sg.tag] : 0, d_err, sg.nwide);
+    const int variant = sg.tag >= 0 && sg.tag < 16 ? gemm_variant[sg.tag] : 0;
+    if (variant == 0 && sg.bend > sg.bbeg) {
+      launch_ggemm<T>(pl, sg.beg, sg.beg + sg.nwide, d_tab, d_rtab, pc, d_coefs, st, f, sg.tag);
+      launch_gbundle<T>(pl, sg.bbeg, sg.bend, d_tab, d_rtab, pc, d_coefs, st, f);
+      return;
+    }
+    launch_ggemm<T>(pl, sg.beg, sg.end, d_tab, d_rtab, pc, d_coefs, st, f, sg.tag, variant, d_err,
+                    sg.nwide);
   }
 
   double tau_orth() const {

@@ -1,5 +1,9 @@
 // Grouped small GEMMs of the setup plans (sm_103a, CUDA cores):
-//  * k_ggemm     -- one CTA per group, items K-concatenated in shared staging;
+//  * k_gcat      -- one CTA per group, items K-concatenated in shared staging
+//                   (the default of every stage that is no inner product);
+//  * k_gbundle   -- factor stages: one CTA per bundle of groups that share
+//                   their A operands;
+//  * k_ggemm     -- an earlier staged form, one of the autotuner's shapes;
 //  * k_gwarp     -- one warp per group (row panels of up to 64 rows);
 //  * k_gdot, k_gdot_warp -- inner-product stages (both operands contiguous
 //                   along the contraction);
@@ -351,6 +355,610 @@ __global__ void __launch_bounds__(NT, MINB) k_ggemm(const GGroup* __restrict__ g
     }
   }
   if (flops && threadIdx.x == 0 && fl > 0) atomicAdd(flops, (double)fl);
+}
+
+// Grouped products with outputs of up to 64 x 64 (every stage that is no inner
+// product), one CTA per group.  A group's items of dynamic rank (a few columns
+// each) are laid end to end along the inner dimension and cut into chunks of KC
+// rows whatever their own ranks are; a chunk's rows get their operand
+// addresses first (one thread per row), so that all of its loads are in flight
+// together -- a group of thirty rank-3 items costs two round trips to L2, not
+// thirty.  Its items with a dense leaf (inner dimension = leaf size) are chunks of
+// their own, addressed without a table.  Operands are staged without integer
+// divisions: those contiguous along the output with lanes along it, the
+// others (A transposed, B plain) as 8 x 4 patches per warp, whose loads fill
+// whole 32-byte sectors and whose stores meet no bank conflict.  4 x 4 register
+// tiles read both operands as 16-byte vectors (3 shared wavefronts per 16
+// multiply-adds); outputs with fewer than 256 tiles split the chunk's rows over
+// the spare threads, whose partial sums are added in a fixed order at the end.
+//
+// Bound by the latency of its chunks (three CTAs per SM, ~4 us per dense item at one
+// CTA), not by the FMA pipe: dense sums of the n = 64 convection-diffusion setup
+// 47 ms against 62 ms in k_ggemm, n = 80 (50-point leaves, which k_ggemm stages
+// with a division per entry) 110 against 172 ms, sketch products 91 against 140 ms.
+constexpr int CI = 64;         // items resolved at a time
+constexpr int CLD = TILE + 4;  // row length of the staged A: 16-byte rows, 8 x 4 patches conflict-free
+
+template <typename T>
+struct __align__(16) CatOp {   // one operand of a chunk row
+  const T* x;                  // A: first entry, contiguous; B: first entry
+  int info;                    // A: first output row | rows << 8; B: stride of the columns
+  float cf;                    // A: coefficient (+-1)
+};
+
+// 16-byte vectors of shared operands
+__device__ __forceinline__ void ld4(const float* p, float (&v)[4]) {
+  const float4 x = *reinterpret_cast<const float4*>(p);
+  v[0] = x.x; v[1] = x.y; v[2] = x.z; v[3] = x.w;
+}
+__device__ __forceinline__ void ld4(const double* p, double (&v)[4]) {
+  const double2 x = *reinterpret_cast<const double2*>(p), y = *reinterpret_cast<const double2*>(p + 2);
+  v[0] = x.x; v[1] = x.y; v[2] = y.x; v[3] = y.y;
+}
+
+template <typename T>
+__host__ __device__ constexpr int cat_bytes() { return 64 * 2 * CLD * (int)sizeof(T); }   // 64 rows of both operands
+
+template <typename T>
+__global__ void __launch_bounds__(NT, sizeof(T) == 4 ? 3 : 2)
+    k_gcat(const GGroup* __restrict__ groups, const GItem* __restrict__ items,
+           T* const* __restrict__ tab, const int* const* __restrict__ rtab, int P, int gbase,
+           const double* __restrict__ coefs, double* __restrict__ flops) {
+  const int p = blockIdx.y;
+  const GGroup G = groups[gbase + blockIdx.x];
+  T* C = tab[G.cbuf * P + p];
+  if (!C) return;
+  const int m = dimv(G.m_st, G.m_rb, G.m_ri, rtab, P, p);
+  const int nall = dimv(G.n_st, G.n_rb, G.n_ri, rtab, P, p);
+  // this CTA's columns j0 ... j0 + n - 1 of the group's output
+  const int nc = ((nall + 4 * (int)gridDim.z - 1) / (4 * (int)gridDim.z)) * 4;
+  const int j0 = blockIdx.z * nc, n = min(nc, nall - j0);
+  if (m <= 0 || n <= 0) return;
+  C += G.coff + (int64_t)j0 * G.ldc;
+  extern __shared__ __align__(16) unsigned char cat_raw[];
+  struct ItemR {
+    const T* A;
+    const T* B;
+    int rows, flags, lda, ldb, row_off, seed, omega_row0, k;
+    float cf;
+  };
+  __shared__ ItemR sit[CI];
+  __shared__ int koff[CI + 1];      // first row of each item in the batch
+  __shared__ int xlist[CI], s_cnt[4];   // dense items from the front, identity items from the back
+  __shared__ CatOp<T> ra[128], rb[128];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int MT = (m + 3) >> 2, N4 = (n + 3) >> 2, tiles = MT * N4;
+  const int ldb_s = 4 * N4 + 4;
+  const int KC = min(128, (cat_bytes<T>() / (int)sizeof(T) / (CLD + ldb_s)) & ~7);
+  T* As = reinterpret_cast<T*>(cat_raw);      // As[kk * CLD + i]
+  T* Bs = As + KC * CLD;                      // Bs[kk * ldb_s + j]
+  const int S = NT / tiles;                   // row slices (tiles <= 256)
+  const int slice = tid / tiles, tile = tid - slice * tiles;
+  const int ty = tile / N4, tx = tile - ty * N4;
+  const bool active = slice < S;
+  T acc[4][4];
+#pragma unroll
+  for (int a = 0; a < 4; ++a)
+#pragma unroll
+    for (int b = 0; b < 4; ++b) acc[a][b] = T(0);
+  auto compute = [&](int kf) {
+    __syncthreads();
+    if (active) {
+#pragma unroll 4
+      for (int kk = slice; kk < kf; kk += S) {
+        T a[4], b[4];
+        ld4(As + kk * CLD + 4 * ty, a);
+        ld4(Bs + kk * ldb_s + 4 * tx, b);
+#pragma unroll
+        for (int x = 0; x < 4; ++x)
+#pragma unroll
+          for (int y = 0; y < 4; ++y) acc[x][y] += a[x] * b[y];
+      }
+    }
+    __syncthreads();
+  };
+
+  for (int base = G.ib; base < G.ie; base += CI) {
+    const int cnt = min(CI, G.ie - base);
+    __syncthreads();   // the previous batch is done with the tables
+    if (tid < CI) {
+      ItemR R{};
+      bool dyn = false;
+      if (tid < cnt) {
+        const GItem J = items[base + tid];
+        bool ok = !(J.guard0 >= 0 && !tab[J.guard0 * P + p]) &&
+                  !(J.guard1 >= 0 && !tab[J.guard1 * P + p]);
+        if (ok && J.abuf >= 0) { R.A = tab[J.abuf * P + p]; ok = R.A != nullptr; if (ok) R.A += J.aoff; }
+        if (ok && J.bbuf >= 0) { R.B = tab[J.bbuf * P + p]; ok = R.B != nullptr; if (ok) R.B += J.boff; }
+        if (ok) {
+          R.k = dimv(J.k_st, J.k_rb, J.k_ri, rtab, P, p);
+          R.rows = dimv(J.r_st, J.r_rb, J.r_ri, rtab, P, p);
+          R.cf = (float)coefs[J.coef];
+          if (R.k <= 0 || R.rows <= 0) R.k = R.rows = 0;
+        }
+        // A transposed (1); B contiguous along the columns (2), sketch rows (8); identity A (16), B (32)
+        R.flags = ((J.aflags & FL_T) ? 1 : 0) | ((J.bflags & FL_T) ? 2 : 0) |
+                  ((J.bflags & FL_OMEGA) ? 8 : 0) | ((J.aflags & FL_IDENT) ? 16 : 0) |
+                  ((J.bflags & FL_IDENT) ? 32 : 0);
+        dyn = J.k_rb >= 0;
+        R.lda = J.lda; R.ldb = J.ldb;
+        R.row_off = J.row_off; R.seed = J.seed; R.omega_row0 = J.omega_row0;
+        if (flops && R.k > 0) {
+          const double w = (R.flags & 48) ? (double)R.rows * n : 2.0 * R.rows * n * R.k;
+          atomicAdd(flops, w);
+        }
+      }
+      sit[tid] = R;
+      const bool ident = R.k > 0 && (R.flags & 48), dense = R.k > 0 && !dyn && !ident;
+      int inc = (R.k > 0 && dyn) ? R.k : 0;   // inclusive scan over the warp's items
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int v = __shfl_up_sync(0xffffffffu, inc, o);
+        if (lane >= o) inc += v;
+      }
+      koff[tid + 1] = inc;
+      const unsigned md = __ballot_sync(0xffffffffu, dense), mi = __ballot_sync(0xffffffffu, ident);
+      if (lane == 0) { s_cnt[warp] = __popc(md); s_cnt[2 + warp] = __popc(mi); }
+      asm volatile("bar.sync 1, 64;" ::: "memory");   // the two resolving warps
+      if (tid >= 32) koff[tid + 1] = inc + koff[32];
+      if (tid == 0) koff[0] = 0;
+      const unsigned below = (1u << lane) - 1u;
+      if (dense) xlist[(warp ? s_cnt[0] : 0) + __popc(md & below)] = tid;
+      if (ident) xlist[CI - 1 - (warp ? s_cnt[2] : 0) - __popc(mi & below)] = tid;
+    }
+    __syncthreads();
+    const int ktot = koff[CI], ndense = s_cnt[0] + s_cnt[1], nident = s_cnt[2] + s_cnt[3];
+    if (active && slice == 0)
+      for (int q = 0; q < nident; ++q) {
+        // C(r0 + i, j) += cf * B(i, j)  or  cf * A(i, j)
+        const ItemR& I = sit[xlist[CI - 1 - q]];
+        const bool ai = I.flags & 16, bt = I.flags & 2;
+        const int64_t si = ai && bt ? I.ldb : 1, sj = ai ? (bt ? 1 : I.ldb) : I.lda;
+        const T* X = ai ? I.B : I.A;
+#pragma unroll
+        for (int a = 0; a < 4; ++a) {
+          const int i = 4 * ty + a - I.row_off;
+          if (i < 0 || i >= I.rows) continue;
+#pragma unroll
+          for (int b = 0; b < 4; ++b)
+            if (4 * tx + b < n) acc[a][b] += (T)I.cf * X[i * si + (j0 + 4 * tx + b) * sj];
+        }
+      }
+    // ---- the dynamic-rank items
+    for (int c0 = 0; c0 < ktot; c0 += KC) {
+      const int kf = min(KC, ktot - c0);
+      if (tid < kf) {   // each row's operands
+        const int r = c0 + tid;
+        int lo = 0, hi = CI;            // the item with koff[lo] <= r < koff[lo + 1]
+        while (hi - lo > 1) {
+          const int mid = (lo + hi) >> 1;
+          if (koff[mid] <= r) lo = mid;
+          else hi = mid;
+        }
+        const ItemR& I = sit[lo];
+        const int l = r - koff[lo];
+        ra[tid] = CatOp<T>{I.A + (int64_t)l * I.lda, I.row_off | I.rows << 8, I.cf};
+        rb[tid] = (I.flags & 2) ? CatOp<T>{I.B + (int64_t)l * I.ldb + j0, 1, 0.f}
+                                : CatOp<T>{I.B + l + (int64_t)j0 * I.ldb, I.ldb, 0.f};
+      }
+      __syncthreads();
+      {
+        const int i = tid & 63;
+        constexpr int U = 8;
+        for (int k0 = tid >> 6; k0 < kf; k0 += 4 * U) {
+          T v[U];
+#pragma unroll
+          for (int u = 0; u < U; ++u) {
+            v[u] = T(0);
+            if (k0 + 4 * u < kf) {
+              const CatOp<T> D = ra[k0 + 4 * u];
+              const int ii = i - (D.info & 255);
+              if (ii >= 0 && ii < (D.info >> 8)) v[u] = (T)D.cf * D.x[ii];
+            }
+          }
+#pragma unroll
+          for (int u = 0; u < U; ++u)
+            if (k0 + 4 * u < kf) As[(k0 + 4 * u) * CLD + i] = v[u];
+        }
+      }
+      {
+        const int jw = N4 <= 1 ? 4 : N4 <= 2 ? 8 : N4 <= 4 ? 16 : N4 <= 8 ? 32 : 64;
+        const int j = tid & (jw - 1), ks = NT / jw;
+        constexpr int U = 4;
+        for (int k0 = tid / jw; k0 < kf; k0 += ks * U) {
+          T v[U];
+#pragma unroll
+          for (int u = 0; u < U; ++u) {
+            v[u] = T(0);
+            if (k0 + ks * u < kf && j < n) {
+              const CatOp<T> D = rb[k0 + ks * u];
+              v[u] = D.x[(int64_t)j * D.info];
+            }
+          }
+#pragma unroll
+          for (int u = 0; u < U; ++u)
+            if (k0 + ks * u < kf && j < 4 * N4) Bs[(k0 + ks * u) * ldb_s + j] = v[u];
+        }
+      }
+      compute(kf);
+    }
+    // ---- the items with a dense leaf: all of a thread's loads in flight, the
+    // next item's (float) while the tiles of the one before are multiplied
+    const int lk = 8 * warp + (lane >> 2);   // row of the 8 x 4 patches
+    constexpr bool AHEAD = sizeof(T) == 4;
+    T va[16], vb[16];
+    auto load = [&](int q) {
+      const ItemR& I = sit[xlist[q]];
+      const int k = I.k, rows = I.rows, r0 = I.row_off, flags = I.flags;
+      if (flags & 1) {
+        const T* A = I.A + lk;
+        const int64_t ld = I.lda;
+#pragma unroll
+        for (int u = 0; u < 16; ++u) {
+          const int ii = 4 * u + (lane & 3) - r0;
+          va[u] = (lk < k && ii >= 0 && ii < rows) ? A[ii * ld] : T(0);
+        }
+      } else {
+        const int ii = (tid & 63) - r0;
+        const T* A = I.A + ii;
+        const int64_t ld = I.lda;
+        const bool in = ii >= 0 && ii < rows;
+#pragma unroll
+        for (int u = 0; u < 16; ++u) {
+          const int l = (tid >> 6) + 4 * u;
+          va[u] = (in && l < k) ? A[l * ld] : T(0);
+        }
+      }
+      if (!(flags & 10)) {
+        const T* B = I.B + lk;
+        const int64_t ld = I.ldb;
+#pragma unroll
+        for (int u = 0; u < 16; ++u) {
+          const int j = 4 * u + (lane & 3);
+          vb[u] = (u < N4 && lk < k && j < n) ? B[(j0 + j) * ld] : T(0);
+        }
+      }
+    };
+    if (AHEAD && ndense > 0) load(0);
+    for (int q = 0; q < ndense; ++q) {
+      if (!AHEAD) load(q);
+      const ItemR& I = sit[xlist[q]];
+      const int k = I.k, flags = I.flags;
+      const T cf = (T)I.cf;
+      if (flags & 1) {
+#pragma unroll
+        for (int u = 0; u < 16; ++u) As[lk * CLD + 4 * u + (lane & 3)] = cf * va[u];
+      } else {
+#pragma unroll
+        for (int u = 0; u < 16; ++u) As[((tid >> 6) + 4 * u) * CLD + (tid & 63)] = cf * va[u];
+      }
+      if (!(flags & 10)) {
+#pragma unroll
+        for (int u = 0; u < 16; ++u)
+          if (u < N4) Bs[lk * ldb_s + 4 * u + (lane & 3)] = vb[u];
+      } else {
+        for (int e = warp; e < k; e += NT / 32)
+          for (int j = lane; j < n; j += 32)
+            Bs[e * ldb_s + j] = (flags & 8) ? (T)omega((uint32_t)I.seed, (uint32_t)(I.omega_row0 + e),
+                                                       (uint32_t)(j0 + j))
+                                            : I.B[j0 + j + (int64_t)e * I.ldb];
+      }
+      if (AHEAD && q + 1 < ndense) load(q + 1);
+      compute(k);
+    }
+  }
+  // the slices' sums, laid out by columns: element (i, j) of slice s at
+  // red[s * R + j * 4 MT + i]; stored with lanes along the rows
+  T* red = reinterpret_cast<T*>(cat_raw);
+  const int R = 16 * tiles, m4 = 4 * MT;
+  const T beta = G.beta >= 0 ? (T)coefs[G.beta] : T(0);
+  __syncthreads();
+  if (active)
+#pragma unroll
+    for (int b = 0; b < 4; ++b)
+#pragma unroll
+      for (int a = 0; a < 4; ++a) red[slice * R + (4 * tx + b) * m4 + 4 * ty + a] = acc[a][b];
+  __syncthreads();
+  for (int jb = warp; jb < n; jb += 4 * (NT / 32)) {
+    T old[4][2];
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const int i = lane + 32 * h, j = jb + u * (NT / 32);
+        old[u][h] = (G.beta >= 0 && i < m && j < n) ? C[i + (int64_t)j * G.ldc] : T(0);
+      }
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const int i = lane + 32 * h, j = jb + u * (NT / 32);
+        if (i >= m || j >= n) continue;
+        T v = red[j * m4 + i];
+        for (int s = 1; s < S; ++s) v += red[s * R + j * m4 + i];
+        C[i + (int64_t)j * G.ldc] = G.beta >= 0 ? v + beta * old[u][h] : v;
+      }
+  }
+}
+
+// The factor products of a bundle: groups whose items read the same A operands
+// (the leaves of one block B(r, s), or A(t, r)) against the factors of different
+// low-rank blocks.  The groups' columns stand side by side, up to 64 at a time, so
+// that every dense leaf is staged once for all of them: alone, a group of rank
+// 3 does 6 flops per entry of the 64 x 64 leaf it loads and the stage is
+// bound by L2; a bundle of 16 does about 100 (n = 64 setup: 45 ms against 88 ms with
+// one CTA per group and 71 ms with one warp per group; n = 80: 127 against 342 and
+// 181 ms).  Tiles, chunks and staging as in
+// k_gcat (A plain or transposed, B plain, C overwritten).
+constexpr int BI = 32;         // items resolved at a time
+
+template <typename T>
+__global__ void __launch_bounds__(NT, sizeof(T) == 4 ? 3 : 2)
+    k_gbundle(const int* __restrict__ bundles, const GGroup* __restrict__ groups,
+              const GItem* __restrict__ items, T* const* __restrict__ tab,
+              const int* const* __restrict__ rtab, int P, const double* __restrict__ coefs,
+              double* __restrict__ flops) {
+  const int p = blockIdx.y;
+  const int gb = bundles[2 * blockIdx.x], ng = bundles[2 * blockIdx.x + 1] - gb;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  extern __shared__ __align__(16) unsigned char cat_raw[];
+  struct ItemA {
+    const T* A;
+    int k, rows, flags, lda, row_off;
+    float cf;
+  };
+  __shared__ ItemA sit[BI];
+  __shared__ const T* bp[BI][BUNDLE_MAX];   // B operand of (item, group)
+  __shared__ int bld[BI][BUNDLE_MAX];
+  __shared__ T* cp[BUNDLE_MAX];             // output of each group
+  __shared__ int cld[BUNDLE_MAX], noff[BUNDLE_MAX + 1], ib[BUNDLE_MAX];
+  __shared__ int koff[BI + 1], xlist[BI], s_nd;
+  __shared__ short colg[TILE], coll[TILE];  // group and own column of each output column
+  __shared__ CatOp<T> ra[128];
+  __shared__ int2 rb[128];                  // item and row of each chunk row
+  const GGroup G0 = groups[gb];
+  const int m = dimv(G0.m_st, G0.m_rb, G0.m_ri, rtab, P, p);
+  if (tid < 32) {
+    int n = 0;
+    if (lane < ng) {
+      const GGroup G = groups[gb + lane];
+      T* C = tab[G.cbuf * P + p];
+      n = C ? max(0, dimv(G.n_st, G.n_rb, G.n_ri, rtab, P, p)) : 0;
+      cp[lane] = C ? C + G.coff : nullptr;
+      cld[lane] = G.ldc;
+      ib[lane] = G.ib;
+    }
+    int inc = n;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int v = __shfl_up_sync(0xffffffffu, inc, o);
+      if (lane >= o) inc += v;
+    }
+    if (lane < ng) noff[lane + 1] = inc;
+    if (lane == 0) noff[0] = 0;
+  }
+  __syncthreads();
+  const int nall = noff[ng], nitems = G0.ie - G0.ib;
+  if (m <= 0 || nall <= 0) return;
+  const int MT = (m + 3) >> 2;
+  for (int j0 = 0; j0 < nall; j0 += TILE) {
+    const int n = min(TILE, nall - j0);
+    const int N4 = (n + 3) >> 2, tiles = MT * N4, ldb_s = 4 * N4 + 4;
+    const int KC = min(128, (cat_bytes<T>() / (int)sizeof(T) / (CLD + ldb_s)) & ~7);
+    T* As = reinterpret_cast<T*>(cat_raw);
+    T* Bs = As + KC * CLD;
+    const int S = NT / tiles;
+    const int slice = tid / tiles, tile = tid - slice * tiles;
+    const int ty = tile / N4, tx = tile - ty * N4;
+    const bool active = slice < S;
+    T acc[4][4];
+#pragma unroll
+    for (int a = 0; a < 4; ++a)
+#pragma unroll
+      for (int b = 0; b < 4; ++b) acc[a][b] = T(0);
+    auto compute = [&](int kf) {
+      __syncthreads();
+      if (active) {
+#pragma unroll 4
+        for (int kk = slice; kk < kf; kk += S) {
+          T a[4], b[4];
+          ld4(As + kk * CLD + 4 * ty, a);
+          ld4(Bs + kk * ldb_s + 4 * tx, b);
+#pragma unroll
+          for (int x = 0; x < 4; ++x)
+#pragma unroll
+            for (int y = 0; y < 4; ++y) acc[x][y] += a[x] * b[y];
+        }
+      }
+      __syncthreads();
+    };
+    if (tid < TILE) {
+      int g = 0;
+      if (tid < n)
+        while (noff[g + 1] <= j0 + tid) ++g;
+      colg[tid] = (short)g;
+      coll[tid] = (short)(j0 + tid - noff[g]);
+    }
+    for (int base = 0; base < nitems; base += BI) {
+      const int cnt = min(BI, nitems - base);
+      __syncthreads();
+      if (tid < 32) {
+        ItemA R{};
+        bool dyn = false;
+        if (lane < cnt) {
+          const GItem J = items[G0.ib + base + lane];
+          R.A = tab[J.abuf * P + p];
+          if (R.A) {
+            R.A += J.aoff;
+            R.k = dimv(J.k_st, J.k_rb, J.k_ri, rtab, P, p);
+            R.rows = dimv(J.r_st, J.r_rb, J.r_ri, rtab, P, p);
+            R.cf = (float)coefs[J.coef];
+            if (R.k <= 0 || R.rows <= 0) R.k = R.rows = 0;
+          }
+          R.flags = (J.aflags & FL_T) ? 1 : 0;
+          R.lda = J.lda; R.row_off = J.row_off;
+          dyn = J.k_rb >= 0;
+          if (flops && R.k > 0) atomicAdd(flops, 2.0 * R.rows * n * R.k);
+        }
+        sit[lane] = R;
+        const bool dense = R.k > 0 && !dyn;
+        int inc = (R.k > 0 && dyn) ? R.k : 0;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+          const int v = __shfl_up_sync(0xffffffffu, inc, o);
+          if (lane >= o) inc += v;
+        }
+        koff[lane + 1] = inc;
+        if (lane == 0) koff[0] = 0;
+        const unsigned md = __ballot_sync(0xffffffffu, dense);
+        if (dense) xlist[__popc(md & ((1u << lane) - 1u))] = lane;
+        if (lane == 0) s_nd = __popc(md);
+      } else {
+        for (int e = tid - 32; e < cnt * ng; e += NT - 32) {
+          const int q = e / ng, g = e - q * ng;
+          const GItem& J = items[ib[g] + base + q];
+          const T* B = tab[J.bbuf * P + p];
+          bp[q][g] = B ? B + J.boff : nullptr;
+          bld[q][g] = J.ldb;
+        }
+      }
+      __syncthreads();
+      const int ktot = koff[BI], ndense = s_nd;
+      // ---- the dynamic-rank items
+      for (int c0 = 0; c0 < ktot; c0 += KC) {
+        const int kf = min(KC, ktot - c0);
+        if (tid < kf) {
+          const int r = c0 + tid;
+          int lo = 0, hi = BI;
+          while (hi - lo > 1) {
+            const int mid = (lo + hi) >> 1;
+            if (koff[mid] <= r) lo = mid;
+            else hi = mid;
+          }
+          const ItemA& I = sit[lo];
+          const int l = r - koff[lo];
+          ra[tid] = CatOp<T>{I.A + (int64_t)l * I.lda, I.row_off | I.rows << 8, I.cf};
+          rb[tid] = make_int2(lo, l);
+        }
+        __syncthreads();
+        {
+          const int i = tid & 63;
+          constexpr int U = 8;
+          for (int k0 = tid >> 6; k0 < kf; k0 += 4 * U) {
+            T v[U];
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+              v[u] = T(0);
+              if (k0 + 4 * u < kf) {
+                const CatOp<T> D = ra[k0 + 4 * u];
+                const int ii = i - (D.info & 255);
+                if (ii >= 0 && ii < (D.info >> 8)) v[u] = (T)D.cf * D.x[ii];
+              }
+            }
+#pragma unroll
+            for (int u = 0; u < U; ++u)
+              if (k0 + 4 * u < kf) As[(k0 + 4 * u) * CLD + i] = v[u];
+          }
+        }
+        {   // lanes along the rows, which are contiguous within an item
+          constexpr int U = 4;
+          const int kk = tid & 127;
+          const int2 r = rb[kk < kf ? kk : 0];
+          for (int jb = tid >> 7; jb < 4 * N4; jb += 2 * U) {
+            T v[U];
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+              const int j = jb + 2 * u;
+              v[u] = T(0);
+              if (kk < kf && j < n) {
+                const int g = colg[j];
+                const T* B = bp[r.x][g];
+                if (B) v[u] = B[r.y + (int64_t)coll[j] * bld[r.x][g]];
+              }
+            }
+#pragma unroll
+            for (int u = 0; u < U; ++u)
+              if (kk < kf && jb + 2 * u < 4 * N4) Bs[kk * ldb_s + jb + 2 * u] = v[u];
+          }
+        }
+        compute(kf);
+      }
+      // ---- the dense leaves
+      const int lk = 8 * warp + (lane >> 2);   // row of the 8 x 4 patches
+      T va[16], vb[16];
+      auto load = [&](int x) {
+        const int q = xlist[x];
+        const ItemA& I = sit[q];
+        const int k = I.k, rows = I.rows, r0 = I.row_off;
+        if (I.flags & 1) {
+          const T* A = I.A + lk;
+          const int64_t ld = I.lda;
+#pragma unroll
+          for (int u = 0; u < 16; ++u) {
+            const int ii = 4 * u + (lane & 3) - r0;
+            va[u] = (lk < k && ii >= 0 && ii < rows) ? A[ii * ld] : T(0);
+          }
+        } else {
+          const int ii = (tid & 63) - r0;
+          const T* A = I.A + ii;
+          const int64_t ld = I.lda;
+          const bool in = ii >= 0 && ii < rows;
+#pragma unroll
+          for (int u = 0; u < 16; ++u) {
+            const int l = (tid >> 6) + 4 * u;
+            va[u] = (in && l < k) ? A[l * ld] : T(0);
+          }
+        }
+#pragma unroll
+        for (int u = 0; u < 16; ++u) {
+          const int j = 4 * u + (lane & 3);
+          vb[u] = T(0);
+          if (u < N4 && lk < k && j < n) {
+            const int g = colg[j];
+            const T* B = bp[q][g];
+            if (B) vb[u] = B[lk + (int64_t)coll[j] * bld[q][g]];
+          }
+        }
+      };
+      if (ndense > 0) load(0);
+      for (int x = 0; x < ndense; ++x) {
+        const ItemA& I = sit[xlist[x]];
+        const int k = I.k;
+        const T cf = (T)I.cf;
+        if (I.flags & 1) {
+#pragma unroll
+          for (int u = 0; u < 16; ++u) As[lk * CLD + 4 * u + (lane & 3)] = cf * va[u];
+        } else {
+#pragma unroll
+          for (int u = 0; u < 16; ++u) As[((tid >> 6) + 4 * u) * CLD + (tid & 63)] = cf * va[u];
+        }
+#pragma unroll
+        for (int u = 0; u < 16; ++u)
+          if (u < N4) Bs[lk * ldb_s + 4 * u + (lane & 3)] = vb[u];
+        if (x + 1 < ndense) load(x + 1);
+        compute(k);
+      }
+    }
+    T* red = reinterpret_cast<T*>(cat_raw);
+    const int R = 16 * tiles, m4 = 4 * MT;
+    __syncthreads();
+    if (active)
+#pragma unroll
+      for (int b = 0; b < 4; ++b)
+#pragma unroll
+        for (int a = 0; a < 4; ++a) red[slice * R + (4 * tx + b) * m4 + 4 * ty + a] = acc[a][b];
+    __syncthreads();
+    for (int j = warp; j < n; j += NT / 32) {
+      const int g = colg[j];
+      T* C = cp[g] + (int64_t)coll[j] * cld[g];
+      for (int i = lane; i < m; i += 32) {
+        T v = red[j * m4 + i];
+        for (int s = 1; s < S; ++s) v += red[s * R + j * m4 + i];
+        C[i] = v;
+      }
+    }
+    __syncthreads();
+  }
 }
 
 // Warp-per-group form of k_ggemm for float operands and row panels
@@ -788,6 +1396,22 @@ __global__ void __launch_bounds__(NT, sizeof(Acc) == 4 ? (TM == 4 ? 4 : 2) : 1) 
 }  // namespace
 
 template <typename T>
+void launch_gbundle(const Plan& pl, int bbeg, int bend, T* const* d_tab, const int* const* d_rtab,
+                    int P, const double* d_coefs, cudaStream_t st, double* d_fl) {
+  if (bend <= bbeg || P <= 0) return;
+  if (cat_bytes<T>() > 48 * 1024)
+    ACR_CUDA(cudaFuncSetAttribute(k_gbundle<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                  cat_bytes<T>()));
+  for (int b0 = bbeg; b0 < bend; b0 += 65535) {
+    const dim3 grid(std::min(65535, bend - b0), P);
+    k_gbundle<T><<<grid, NT, cat_bytes<T>(), st>>>(
+        (const int*)pl.d_bundles + 2 * b0, (const GGroup*)pl.d_groups, (const GItem*)pl.d_items,
+        d_tab, d_rtab, P, d_coefs, d_fl);
+    ACR_LAUNCHED(1);
+  }
+}
+
+template <typename T>
 void launch_ggemm(const Plan& pl, int gbeg, int gend, T* const* d_tab, const int* const* d_rtab,
                   int P, const double* d_coefs, cudaStream_t st, double* d_fl, int tag,
                   int variant, int* d_err, int nwide) {
@@ -810,6 +1434,13 @@ void launch_ggemm(const Plan& pl, int gbeg, int gend, T* const* d_tab, const int
   }
   if (variant == 3) variant = 2;   // no wide groups: shape 3 is shape 2
   using Acc = T;
+  if (cat_bytes<T>() > 48 * 1024)
+    ACR_CUDA(cudaFuncSetAttribute(k_gcat<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                  cat_bytes<T>()));
+  // A stage of few groups per plane leaves most of the SMs idle whenever few
+  // planes are left: its outputs' columns are then split over 2 or 4 CTAs.  (By the
+  // plan alone, not by P: a plane's result must not depend on the batch.)
+  const int zsplit = ng <= 38 ? 4 : ng <= 76 ? 2 : 1;
   const int maxg = 65535;
   for (int g0 = 0; g0 < ng; g0 += maxg) {
     dim3 grid(std::min(maxg, ng - g0), P);
@@ -854,12 +1485,16 @@ void launch_ggemm(const Plan& pl, int gbeg, int gend, T* const* d_tab, const int
       k_ggemm<T, Acc, STAGE_BYTES / 2, 2>
           <<<grid, NT, 0, st>>>(gr, it, d_tab, d_rtab, P, gbeg + g0, d_coefs, d_fl);
     else
-      k_ggemm<T, Acc, STAGE_BYTES, sizeof(Acc) == 4 ? 4 : 2>
-          <<<grid, NT, 0, st>>>(gr, it, d_tab, d_rtab, P, gbeg + g0, d_coefs, d_fl);
+      k_gcat<T><<<dim3(grid.x, grid.y, zsplit), NT, cat_bytes<T>(), st>>>(gr, it, d_tab, d_rtab, P,
+                                                                          gbeg + g0, d_coefs, d_fl);
     ACR_LAUNCHED(1);
   }
 }
 
+template void launch_gbundle<double>(const Plan&, int, int, double* const*, const int* const*, int,
+                                     const double*, cudaStream_t, double*);
+template void launch_gbundle<float>(const Plan&, int, int, float* const*, const int* const*, int,
+                                    const double*, cudaStream_t, double*);
 template void launch_ggemm<double>(const Plan&, int, int, double* const*, const int* const*, int,
                                    const double*, cudaStream_t, double*, int, int, int*, int);
 template void launch_ggemm<float>(const Plan&, int, int, float* const*, const int* const*, int,

@@ -56,6 +56,11 @@ void launch_ggemm(const Plan& pl, int gbeg, int gend, T* const* d_tab, const int
                   int P, const double* d_coefs, cudaStream_t st, double* d_flops = nullptr,
                   int tag = -1, int variant = 0, int* d_err = nullptr, int nwide = 0);
 
+// The bundles [bbeg, bend) of a factor stage, one CTA per (bundle, plane).
+template <typename T>
+void launch_gbundle(const Plan& pl, int bbeg, int bend, T* const* d_tab, const int* const* d_rtab,
+                    int P, const double* d_coefs, cudaStream_t st, double* d_flops = nullptr);
+
 // The wide (dense-output, up to 64 x 64) groups [gbeg, gend) of a float GEMM
 // stage on the tcgen05 tensor cores (split-TF32 operands, FP32 results).
 void launch_ggemm_tc(const Plan& pl, int gbeg, int gend, float* const* d_tab,

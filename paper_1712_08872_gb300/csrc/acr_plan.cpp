@@ -566,6 +566,63 @@ struct Builder {
 }  // namespace
 
 namespace {
+// Do two groups' items read the same A operands in the same order (same inner
+// dimensions, rows and coefficients)?
+bool same_a(const Plan& pl, const GGroup& x, const GGroup& y) {
+  if (x.ie - x.ib != y.ie - y.ib || x.m_st != y.m_st || x.m_rb != y.m_rb || x.m_ri != y.m_ri ||
+      x.beta != y.beta)
+    return false;
+  for (int i = 0; i < x.ie - x.ib; ++i) {
+    const GItem &a = pl.items[x.ib + i], &b = pl.items[y.ib + i];
+    if (a.abuf != b.abuf || a.aoff != b.aoff || a.lda != b.lda || a.aflags != b.aflags ||
+        a.bflags != b.bflags || a.k_st != b.k_st || a.k_rb != b.k_rb || a.k_ri != b.k_ri ||
+        a.r_st != b.r_st || a.r_rb != b.r_rb || a.r_ri != b.r_ri || a.row_off != b.row_off ||
+        a.coef != b.coef || a.guard0 != b.guard0 || a.guard1 != b.guard1)
+      return false;
+  }
+  return true;
+}
+
+// Bundles of a factor stage's narrow groups, in the order of their first group.
+// Small stages keep more, smaller bundles (at least ~150, one per SM, where
+// there are that many groups).
+void make_bundles(Plan& plan, Stage& sg) {
+  const int beg = sg.beg + sg.nwide, n = sg.end - beg;
+  const int most = std::max(1, std::min(BUNDLE_MAX, n / 152));
+  std::unordered_map<uint64_t, std::vector<int>> open;   // key -> bundles of that key
+  std::vector<std::vector<int>> bd;
+  for (int i = 0; i < n; ++i) {
+    const GGroup& g = plan.groups[beg + i];
+    uint64_t key = (uint64_t)(g.ie - g.ib);
+    for (int q = g.ib; q < g.ie; ++q) {
+      const GItem& it = plan.items[q];
+      key = (key ^ (uint64_t)it.aoff ^ ((uint64_t)it.abuf << 48)) * 0x9E3779B97F4A7C15ull;
+      key ^= key >> 29;
+    }
+    int at = -1;
+    std::vector<int>& cand = open[key];
+    if (!cand.empty() && (int)bd[cand.back()].size() < most &&
+        same_a(plan, plan.groups[beg + bd[cand.back()][0]], g))
+      at = cand.back();
+    if (at < 0) {
+      at = (int)bd.size();
+      bd.emplace_back();
+      cand.push_back(at);
+    }
+    bd[at].push_back(i);
+  }
+  std::vector<GGroup> re;
+  re.reserve(n);
+  sg.bbeg = (int)plan.bundles.size() / 2;
+  for (const auto& b : bd) {
+    plan.bundles.push_back(beg + (int)re.size());
+    for (int i : b) re.push_back(plan.groups[beg + i]);
+    plan.bundles.push_back(beg + (int)re.size());
+  }
+  sg.bend = (int)plan.bundles.size() / 2;
+  std::copy(re.begin(), re.end(), plan.groups.begin() + beg);
+}
+
 // Order every GEMM stage's groups wide (static 64-column outputs) first and
 // record their count, so a launch can give the two kinds different kernels.
 // Groups of one stage write disjoint outputs: their order changes nothing.
@@ -585,6 +642,7 @@ void order_wide_first(Plan& plan) {
     auto mid = std::stable_partition(plan.groups.begin() + sg.beg, plan.groups.begin() + sg.end,
                                      wide);
     sg.nwide = (int)(mid - (plan.groups.begin() + sg.beg));
+    if (sg.tag == TAG_FACT) make_bundles(plan, sg);
   }
 }
 }  // namespace

@@ -113,8 +113,13 @@ inline bool tag_is_dot(int t) {
 }
 
 // A GEMM stage's groups are ordered with those of a static 64-column output
-// (dense leaf products) first: nwide of them, then the narrow ones.
-struct Stage { int kind; int beg, end; int tag = -1; int nwide = 0; };
+// (dense leaf products) first: nwide of them, then the narrow ones.  The narrow
+// groups of a factor stage (TAG_FACT) are further ordered into the bundles
+// [bbeg, bend) of Plan::bundles: runs of groups whose items read the same A operands in
+// the same order (one H-matrix block times the factors of several low-rank
+// blocks), so that a kernel can stage those operands once per bundle.
+struct Stage { int kind; int beg, end; int tag = -1; int nwide = 0; int bbeg = 0, bend = 0; };
+constexpr int BUNDLE_MAX = 16;   // groups per bundle
 
 // Operand roles: role r owns buffers 3r (dense), 3r+1 (U), 3r+2 (V) and
 // rank buffer r.  The scratch real buffer is 3*nroles, the scratch rank
@@ -134,6 +139,7 @@ struct Plan {
   std::vector<TInfo> targets;
   std::vector<StackDim> stack;
   std::vector<Stage> stages;
+  std::vector<int32_t> bundles;   // first and past-the-last group of each bundle
   int64_t scratch = 0;        // real scratch elements per plane
   int32_t scratch_ranks = 0;  // int scratch entries per plane
   int nroles = 1;
@@ -147,6 +153,7 @@ struct Plan {
   void* d_targets = nullptr;
   void* d_stack = nullptr;
   void* d_torder = nullptr;
+  void* d_bundles = nullptr;
 };
 
 struct PlanParams {
