@@ -512,7 +512,7 @@ class Engine : public EngineBase {
       ACR_CUDA(cudaMemcpy(pl.d_bundles, pl.bundles.data(), pl.bundles.size() * sizeof(int32_t),
                           cudaMemcpyHostToDevice));
     }
-    if (pp.fused && !pl.torder.empty()) {
+    if (!pl.torder.empty()) {
       pl.d_torder = dmalloc(pl.torder.size() * sizeof(int32_t));
       ACR_CUDA(cudaMemcpy(pl.d_torder, pl.torder.data(), pl.torder.size() * sizeof(int32_t),
                           cudaMemcpyHostToDevice));
@@ -669,6 +669,10 @@ class Engine : public EngineBase {
     if (variant == 0 && sg.bend > sg.bbeg) {
       launch_ggemm<T>(pl, sg.beg, sg.beg + sg.nwide, d_tab, d_rtab, pc, d_coefs, st, f, sg.tag);
       launch_gbundle<T>(pl, sg.bbeg, sg.bend, d_tab, d_rtab, pc, d_coefs, st, f);
+      return;
+    }
+    if (variant == 0 && (sg.tag == TAG_S || sg.tag == TAG_P)) {
+      launch_tdot<T>(pl, sg.tag == TAG_S, d_tab, d_rtab, pc, st, f);
       return;
     }
     launch_ggemm<T>(pl, sg.beg, sg.end, d_tab, d_rtab, pc, d_coefs, st, f, sg.tag, variant, d_err,

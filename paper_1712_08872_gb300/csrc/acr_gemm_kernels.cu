@@ -1393,7 +1393,229 @@ __global__ void __launch_bounds__(NT, sizeof(Acc) == 4 ? (TM == 4 ? 4 : 2) : 1) 
   if (flops && lane == 0 && fl > 0) atomicAdd(flops, (double)fl);
 }
 
+// The inner products of a low-rank target with its common right factor: the
+// sketch rows S_i = Z_i^T Omega (SK) or the projections P_i = X_i^T Q of all
+// summed terms i.  One CTA per target holds the common factor (generated once,
+// instead of once per term, for Omega) in shared memory, row by row; a warp takes 8 columns of
+// one Z_i at a time: 32 rows of them pass through the warp's own shared
+// slice, and each lane accumulates 8 products of its own output column -- no
+// shuffles per output, 3 shared loads per 8 multiply-adds.  Narrow outputs (W < 32
+// columns) split the 32 rows over the lanes' spare groups.  Sums are per 32 rows, then
+// over the blocks.  Factors of more than 512 (FP64: 256) rows go through in blocks, added
+// in global memory.  n = 64 setup: sketches 33 -> 20 ms, projections 39 -> 22 ms (n = 80: 118 -> 59, 100 -> 60)
+// against one warp per term with lanes along the rows.
+// rows of the common factor held at a time
+template <typename T>
+__host__ __device__ constexpr int tdr() { return sizeof(T) == 4 ? 512 : 256; }
+constexpr int TDI = 64;        // terms resolved at a time
+
+template <typename T>
+constexpr size_t tdot_smem(int rows, int p) {
+  const int w = p <= 8 ? 8 : p <= 16 ? 16 : p <= 32 ? 32 : 64;
+  return ((size_t)(rows < tdr<T>() ? rows : tdr<T>()) * (w + 1) + (NT / 32) * 32 * 8) * sizeof(T) + 16;
+}
+
+template <typename T, bool SK>
+__global__ void __launch_bounds__(NT, sizeof(T) == 4 ? 4 : 2)
+    k_tdot(const TInfo* __restrict__ tis, const int* __restrict__ order,
+           const GGroup* __restrict__ groups, const GItem* __restrict__ items,
+           T* const* __restrict__ tab, const int* const* __restrict__ rtab, int P, int scr_buf,
+           int scr_rbuf, double* __restrict__ flops) {
+  const int p = blockIdx.y;
+  const TInfo ti = tis[order[blockIdx.x]];
+  T* scr = tab[scr_buf * P + p];
+  const int* rs = rtab[scr_rbuf * P + p];
+  const int gb = SK ? ti.s_beg : ti.x_beg, ge = SK ? ti.s_end : ti.x_end;
+  if (!scr || !rs || ge <= gb) return;
+  const int nc = SK ? ti.p : rs[ti.r_ri];       // output columns
+  if (nc <= 0) return;
+  const int rows = SK ? ti.n : ti.m;            // rows of the common factor
+  const int W = nc <= 8 ? 8 : nc <= 16 ? 16 : nc <= 32 ? 32 : 64, LD = W + 1;
+  extern __shared__ __align__(16) unsigned char td_raw[];
+  T* zsall = reinterpret_cast<T*>(td_raw);      // 32 x 8 per warp
+  T* F = zsall + (NT / 32) * 32 * 8;            // F(row, col) = F[row * LD + col]
+  struct Term {
+    const T* Z;
+    T* C;
+    int k, rows, lda, ldc, off;
+  };
+  __shared__ Term term[TDI];
+  __shared__ int uoff[TDI + 1];                 // first unit (8 columns of Z) of each term
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  T* zs = zsall + warp * 32 * 8;
+  const int w32 = min(W, 32), col = lane & (w32 - 1), sub = lane / w32, RS = 32 / w32;
+  for (int f0 = 0; f0 < rows; f0 += tdr<T>()) {
+    const int fr = min(tdr<T>(), rows - f0);
+    __syncthreads();
+    if (SK) {
+      for (int e = tid; e < fr * (W / 2); e += NT) {
+        const int r = e / (W / 2), c = e - r * (W / 2);     // (W a power of two)
+        if (2 * c < nc) {
+          const uint32_t b = omega_bits((uint32_t)ti.seed, (uint32_t)(f0 + r), (uint32_t)c);
+          F[r * LD + 2 * c] = (T)omega_half(b, 0u);
+          F[r * LD + 2 * c + 1] = (T)omega_half(b, 1u);
+        }
+      }
+    } else {
+      const T* Q = scr + ti.y_off + f0;
+      for (int c = warp; c < nc; c += NT / 32)
+        for (int r = lane; r < fr; r += 32) F[r * LD + c] = Q[r + (int64_t)c * rows];
+    }
+    for (int base = gb; base < ge; base += TDI) {
+      const int cnt = min(TDI, ge - base);
+      __syncthreads();
+      if (tid < TDI) {
+        Term R{};
+        if (tid < cnt) {
+          const GGroup G = groups[base + tid];
+          const GItem I = items[G.ib];
+          const T* Z = tab[I.abuf * P + p];
+          if (Z) {
+            R.Z = Z + I.aoff;
+            R.C = scr + G.coff;
+            R.k = dimv(G.m_st, G.m_rb, G.m_ri, rtab, P, p);
+            R.rows = I.k_st;
+            R.off = SK ? I.omega_row0 : (int)(I.boff - ti.y_off);
+            R.lda = I.lda; R.ldc = G.ldc;
+            if (flops && f0 == 0 && R.k > 0) atomicAdd(flops, 2.0 * R.rows * nc * R.k);
+          }
+          // (a term without rows in this block has no units here)
+          if (R.k <= 0 || R.off >= f0 + fr || R.off + R.rows <= f0) R.k = 0;
+        }
+        term[tid] = R;
+        int inc = (R.k + 7) >> 3;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+          const int v = __shfl_up_sync(0xffffffffu, inc, o);
+          if (lane >= o) inc += v;
+        }
+        uoff[tid + 1] = inc;
+        if (tid == 0) uoff[0] = 0;
+      }
+      __syncthreads();
+      const int half = uoff[32], units = half + uoff[TDI];
+      for (int u = warp; u < units; u += NT / 32) {
+        // the term of unit u (the second half's offsets are its own)
+        int lo, hi, add;
+        if (u < half) { lo = 0; hi = 32; add = 0; } else { lo = 32; hi = TDI; add = half; }
+        while (hi - lo > 1) {
+          const int mid = (lo + hi) >> 1;
+          if ((mid == 32 ? 0 : uoff[mid]) <= u - add) lo = mid;
+          else hi = mid;
+        }
+        const Term R = term[lo];
+        const int i0 = 8 * (u - add - (lo == 32 ? 0 : uoff[lo]));
+        const int kc = min(8, R.k - i0);
+        // rows [l0, l1) of the term lie in this block; F row of term row l: l + sh
+        const int l0 = max(0, f0 - R.off), l1 = min(R.rows, f0 + fr - R.off), sh = R.off - f0;
+        const T* Z = R.Z + (int64_t)i0 * R.lda;
+        for (int h = 0; h < W; h += 32) {
+          T acc[8], z[8];
+#pragma unroll
+          for (int c = 0; c < 8; ++c) acc[c] = T(0);
+#pragma unroll
+          for (int c = 0; c < 8; ++c)
+            z[c] = (c < kc && l0 + lane < l1) ? Z[l0 + lane + (int64_t)c * R.lda] : T(0);
+          for (int l = l0; l < l1; l += 32) {
+            __syncwarp();
+#pragma unroll
+            for (int c = 0; c < 8; c += 16 / (int)sizeof(T)) {
+              if (sizeof(T) == 4)
+                *reinterpret_cast<float4*>(zs + lane * 8 + c) =
+                    make_float4((float)z[c], (float)z[c + 1], (float)z[c + 2], (float)z[c + 3]);
+              else
+                *reinterpret_cast<double2*>(zs + lane * 8 + c) = make_double2((double)z[c], (double)z[c + 1]);
+            }
+            __syncwarp();
+#pragma unroll
+            for (int c = 0; c < 8; ++c)   // the next rows, while these are multiplied
+              z[c] = (c < kc && l + 32 + lane < l1) ? Z[l + 32 + lane + (int64_t)c * R.lda] : T(0);
+            const int nr = min(32, l1 - l), per = 32 / RS;
+            const T* f = F + (int64_t)(l + sh + sub * per) * LD + h + col;
+            const T* zr = zs + sub * per * 8;
+            const int my = min(per, nr - sub * per);
+            T s[8];
+#pragma unroll
+            for (int c = 0; c < 8; ++c) s[c] = T(0);
+            if (kc > 4) {
+#pragma unroll 4
+              for (int r = 0; r < my; ++r) {
+                T a[4], b[4];
+                ld4(zr + r * 8, a);
+                ld4(zr + r * 8 + 4, b);
+                const T t = f[r * LD];
+#pragma unroll
+                for (int c = 0; c < 4; ++c) { s[c] += a[c] * t; s[c + 4] += b[c] * t; }
+              }
+            } else {
+#pragma unroll 4
+              for (int r = 0; r < my; ++r) {
+                T a[4];
+                ld4(zr + r * 8, a);
+                const T t = f[r * LD];
+#pragma unroll
+                for (int c = 0; c < 4; ++c) s[c] += a[c] * t;
+              }
+            }
+#pragma unroll
+            for (int c = 0; c < 8; ++c) acc[c] += s[c];
+          }
+          for (int o = w32; o < 32; o <<= 1)
+#pragma unroll
+            for (int c = 0; c < 8; ++c) acc[c] += __shfl_xor_sync(0xffffffffu, acc[c], o);
+          // through the warp's slice: the 8 rows of a column are contiguous
+          __syncwarp();
+          if (sub == 0)
+#pragma unroll
+            for (int c = 0; c < 8; ++c) zs[col * 8 + c] = acc[c];
+          __syncwarp();
+          const int i = lane & 7;
+          for (int j = lane >> 3; j < w32; j += 4) {
+            if (i >= kc || h + j >= nc) continue;
+            T* c = R.C + i0 + i + (int64_t)(h + j) * R.ldc;
+            const T v = zs[j * 8 + i];
+            *c = l0 > 0 ? *c + v : v;
+          }
+        }
+      }
+    }
+  }
+}
+
 }  // namespace
+
+template <typename T>
+void launch_tdot(const Plan& pl, bool sketch, T* const* d_tab, const int* const* d_rtab, int P,
+                 cudaStream_t st, double* d_fl) {
+  const int nt = (int)pl.torder.size();
+  if (nt <= 0 || P <= 0) return;
+  auto kern = sketch ? k_tdot<T, true> : k_tdot<T, false>;
+  auto smem = [&](int q) {
+    const TInfo& ti = pl.targets[pl.torder[q]];
+    return tdot_smem<T>(std::max(ti.m, ti.n), ti.p);
+  };
+  // targets by increasing size: those that leave room for 4 (double: 2) CTAs per
+  // SM first, then the larger ones; few targets go in one launch
+  const size_t small = sizeof(T) == 4 ? 56320 : 112640;
+  const bool few = (int64_t)nt * P <= device_sm_count();
+  ACR_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                (int)tdot_smem<T>(tdr<T>(), 64)));
+  for (int beg = 0; beg < nt;) {
+    int end = nt;
+    if (!few && smem(beg) <= small)
+      for (end = beg + 1; end < nt && smem(end) <= small; ++end) {}
+    size_t need = 0;
+    for (int q = beg; q < end; ++q) need = std::max(need, smem(q));
+    for (int t0 = beg; t0 < end; t0 += 65535) {
+      const dim3 grid(std::min(65535, end - t0), P);
+      kern<<<grid, NT, need, st>>>((const TInfo*)pl.d_targets, (const int*)pl.d_torder + t0,
+                                   (const GGroup*)pl.d_groups, (const GItem*)pl.d_items, d_tab,
+                                   d_rtab, P, 3 * pl.nroles, pl.nroles, d_fl);
+      ACR_LAUNCHED(1);
+    }
+    beg = end;
+  }
+}
 
 template <typename T>
 void launch_gbundle(const Plan& pl, int bbeg, int bend, T* const* d_tab, const int* const* d_rtab,
@@ -1491,6 +1713,10 @@ void launch_ggemm(const Plan& pl, int gbeg, int gend, T* const* d_tab, const int
   }
 }
 
+template void launch_tdot<double>(const Plan&, bool, double* const*, const int* const*, int,
+                                  cudaStream_t, double*);
+template void launch_tdot<float>(const Plan&, bool, float* const*, const int* const*, int,
+                                 cudaStream_t, double*);
 template void launch_gbundle<double>(const Plan&, int, int, double* const*, const int* const*, int,
                                      const double*, cudaStream_t, double*);
 template void launch_gbundle<float>(const Plan&, int, int, float* const*, const int* const*, int,

@@ -61,6 +61,12 @@ template <typename T>
 void launch_gbundle(const Plan& pl, int bbeg, int bend, T* const* d_tab, const int* const* d_rtab,
                     int P, const double* d_coefs, cudaStream_t st, double* d_flops = nullptr);
 
+// The sketch products (sketch) or projections of a plan's low-rank targets, one
+// CTA per (target, plane).
+template <typename T>
+void launch_tdot(const Plan& pl, bool sketch, T* const* d_tab, const int* const* d_rtab, int P,
+                 cudaStream_t st, double* d_flops = nullptr);
+
 // The wide (dense-output, up to 64 x 64) groups [gbeg, gend) of a float GEMM
 // stage on the tcgen05 tensor cores (split-TF32 operands, FP32 results).
 void launch_ggemm_tc(const Plan& pl, int gbeg, int gend, float* const* d_tab,

@@ -402,6 +402,7 @@ struct Builder {
       ti.r_ri = alloc_rank();
       ti.c_leaf = c.leaf;
       ti.seed = 0;
+      ti.s_beg = ti.s_end = ti.x_beg = ti.x_end = 0;
       ti.y_off = lt.y; ti.bt_off = lt.bt;
       ti.u_off = S.lr_row0[c.leaf] * kc; ti.v_off = S.lr_col0[c.leaf] * kc;
       ti.sk_beg = (int)P.stack.size();
@@ -419,13 +420,16 @@ struct Builder {
     stage(ST_GEMM, gdense0, (int)P.groups.size(), TAG_DENSE);
     // S_i = Z_i^T Omega (k_i x p)
     const int gs0 = (int)P.groups.size();
-    for (LT& lt : lts) {
+    for (size_t i = 0; i < lts.size(); ++i) {
+      LT& lt = lts[i];
+      P.targets[i].s_beg = (int)P.groups.size();
       for (const LItem& li : lt.items) {
         if (li.dense) continue;
         begin_group(bscr(), li.sp_off, li.cap, li.k, dconst(lt.p), -1);
         add_item(li.zbuf, li.zoff, li.zld, FL_T, -1, 0, 0, FL_OMEGA, dconst(li.zrows), li.k, 0, 0,
                  (int)(1000003u * (uint32_t)(lt.node + 1)), li.col_off);
       }
+      P.targets[i].s_end = (int)P.groups.size();
     }
     stage(ST_GEMM, gs0, (int)P.groups.size(), TAG_S);
 
@@ -495,7 +499,9 @@ struct Builder {
     g0 = (int)P.groups.size();
     for (size_t i = 0; i < lts.size(); ++i) {
       LT& lt = lts[i];
-      const TInfo& ti = P.targets[i];
+      TInfo& ti = P.targets[i];
+      ti.x_beg = (int)P.groups.size();
+      ti.x_end = ti.x_beg + (int)lt.items.size();
       for (const LItem& li : lt.items) {
         Dim kd = li.dense ? dconst(lsz) : li.k;
         begin_group(bscr(), li.sp_off, li.cap, kd, drank(rscr(), ti.r_ri), -1);
@@ -716,6 +722,13 @@ void merge_plans(const std::vector<const Plan*>& ps, Plan& out) {
         kind = sg.kind;
         tag = sg.tag;
         if (sg.kind == ST_GEMM) {
+          const int shift = (int)out.groups.size() - sg.beg;
+          if (sg.tag == TAG_S || sg.tag == TAG_P)
+            for (size_t t = 0; t < ps[i]->targets.size(); ++t) {
+              TInfo& ti = out.targets[toff[i] + t];
+              (sg.tag == TAG_S ? ti.s_beg : ti.x_beg) += shift;
+              (sg.tag == TAG_S ? ti.s_end : ti.x_end) += shift;
+            }
           for (int g = sg.beg; g < sg.end; ++g) {
             GGroup G = ps[i]->groups[g];
             const int ib = (int)out.items.size();

@@ -73,9 +73,11 @@ struct TInfo {
   int32_t c_leaf;      // low-rank leaf index of C (rank output)
   int32_t seed;
   int32_t sk_beg, sk_end;  // the summed terms' inner dimensions: Plan::stack entries
-  int64_t y_off, bt_off;   // fused stages: scratch offsets of the sketch Y, replaced by the basis
-                           // Q (m x p, ld m), and of B^T (n x p, ld n)
+  int64_t y_off, bt_off;   // scratch offsets of the sketch Y, replaced by the final basis Q
+                           // (m x p, ld m), and of B^T (n x p, ld n)
   int64_t u_off, v_off;    // the target leaf's factors in C's U and V buffers
+  int32_t s_beg, s_end;    // groups of the target's sketch products Z_i^T Omega (TAG_S) ...
+  int32_t x_beg, x_end;    // ... and of its projections X_i^T Q (TAG_P)
 };
 
 // One summed term of a low-rank target, for the stacked-rank count: its
