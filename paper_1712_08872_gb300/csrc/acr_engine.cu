@@ -125,6 +125,79 @@ struct TableRing {
   }
 };
 
+// Device copies of plans: carved out of large chunks and filled through two
+// pinned halves on the setup's stream, so that the host can build the next plan
+// while the device runs the last one (a cudaMalloc and a synchronous copy per array
+// made the device idle through every plan's construction).
+struct PlanStore {
+  static constexpr size_t HALF = size_t(4) << 20, CHUNK = size_t(16) << 20;
+  std::vector<char*> chunks;
+  size_t left = 0;
+  char* at = nullptr;
+  char* pin = nullptr;
+  size_t off = 0;
+  int half = 0;
+  cudaEvent_t free_[2] = {nullptr, nullptr};
+  bool used[2] = {false, false};
+  void* alloc(size_t bytes) {
+    const size_t b = (std::max<size_t>(bytes, 16) + 255) & ~size_t(255);
+    if (b > left) {
+      const size_t c = std::max(b, CHUNK);
+      at = (char*)dmalloc(c);
+      chunks.push_back(at);
+      left = c;
+    }
+    void* p = at;
+    at += b;
+    left -= b;
+    return p;
+  }
+  void copy(void* dst, const void* src, size_t bytes, cudaStream_t st) {
+    if (!pin) {
+      count_allocs(1);
+      ACR_CUDA(cudaMallocHost(&pin, 2 * HALF));
+      for (cudaEvent_t& e : free_) ACR_CUDA(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
+    }
+    for (size_t done = 0; done < bytes;) {
+      if (off == HALF) {   // the other half, once its copies are done
+        ACR_CUDA(cudaEventRecord(free_[half], st));
+        used[half] = true;
+        half ^= 1;
+        off = 0;
+        if (used[half]) ACR_CUDA(cudaEventSynchronize(free_[half]));
+      }
+      const size_t n = std::min(bytes - done, HALF - off);
+      char* h = pin + half * HALF + off;
+      std::memcpy(h, (const char*)src + done, n);
+      ACR_CUDA(cudaMemcpyAsync((char*)dst + done, h, n, cudaMemcpyHostToDevice, st));
+      off = std::min(HALF, (off + n + 255) & ~size_t(255));
+      done += n;
+    }
+  }
+  template <typename V>
+  void* put(const std::vector<V>& v, cudaStream_t st) {
+    void* p = alloc(v.size() * sizeof(V));
+    if (!v.empty()) copy(p, v.data(), v.size() * sizeof(V), st);
+    return p;
+  }
+  // the staging is idle (its stream was synchronised)
+  void release_staging() {
+    if (pin) cudaFreeHost(pin);
+    for (cudaEvent_t& e : free_) {
+      if (e) cudaEventDestroy(e);
+      e = nullptr;
+    }
+    pin = nullptr;
+    off = 0;
+    used[0] = used[1] = false;
+  }
+  void release() {
+    for (char* c : chunks) cudaFree(c);
+    chunks.clear();
+    left = 0;
+  }
+};
+
 }  // namespace
 
 struct HM {
@@ -274,6 +347,10 @@ class Engine : public EngineBase {
   MatvecDev mvd{};
   PlanParams pp{};
   std::map<std::vector<int>, std::unique_ptr<Plan>> plans;
+  static constexpr size_t PLAN_LARGE = 65536;   // items
+  std::vector<GGroup> spare_groups;
+  std::vector<GItem> spare_items;
+  PlanStore store;
   std::vector<void*> owned;          // structure / plan / table arrays
   std::vector<HM> D;                 // plane blocks (X in place after inversion), count * n
   SlotPool pool, pool_b;             // T-typed H-matrices; bfloat16 copies (BF16 form)
@@ -434,18 +511,10 @@ class Engine : public EngineBase {
     pool_b.release();
     for (void* p : owned) cudaFree(p);
     owned.clear();
-    for (auto& kv : plans) {
-      cudaFree(kv.second->d_groups); cudaFree(kv.second->d_items); cudaFree(kv.second->d_targets);
-      cudaFree(kv.second->d_stack); cudaFree(kv.second->d_torder);
-      cudaFree(kv.second->d_bundles);
-    }
     plans.clear();
-    for (auto& kv : merged_plans) {
-      cudaFree(kv.second->d_groups); cudaFree(kv.second->d_items); cudaFree(kv.second->d_targets);
-      cudaFree(kv.second->d_stack); cudaFree(kv.second->d_torder);
-      cudaFree(kv.second->d_bundles);
-    }
     merged_plans.clear();
+    store.release_staging();
+    store.release();
     if (scratch) cudaFree(scratch);
     if (scratch_ranks) cudaFree(scratch_ranks);
     scratch = nullptr; scratch_ranks = nullptr;
@@ -469,8 +538,21 @@ class Engine : public EngineBase {
     for (auto& a : op.adds) { key.push_back(a.m_role); key.push_back(a.coef); }
     auto it = plans.find(key);
     if (it != plans.end()) return *it->second;
+    // Built in storage that goes from plan to plan (page faults of fresh memory
+    // cost as much as the construction); small plans are copied out of it,
+    // large ones give it back when they have been uploaded.
     auto pl = std::make_unique<Plan>();
+    pl->groups = std::move(spare_groups);
+    pl->items = std::move(spare_items);
     build_plan(S, op, pp, *pl);
+    if (pl->items.size() < PLAN_LARGE) {
+      std::vector<GGroup> g(pl->groups);
+      std::vector<GItem> i(pl->items);
+      g.swap(pl->groups);
+      i.swap(pl->items);
+      spare_groups = std::move(g);
+      spare_items = std::move(i);
+    }
     Plan& ref = *pl;
     plans[key] = std::move(pl);
     return ref;
@@ -501,34 +583,24 @@ class Engine : public EngineBase {
     }
   }
 
-  void upload_plan(Plan& pl) {
-    if (pl.d_groups) return;
-    pl.d_groups = dmalloc(std::max<size_t>(pl.groups.size(), 1) * sizeof(GGroup));
-    pl.d_items = dmalloc(std::max<size_t>(pl.items.size(), 1) * sizeof(GItem));
-    pl.d_targets = dmalloc(std::max<size_t>(pl.targets.size(), 1) * sizeof(TInfo));
-    pl.d_stack = dmalloc(std::max<size_t>(pl.stack.size(), 1) * sizeof(StackDim));
-    if (!pl.bundles.empty()) {
-      pl.d_bundles = dmalloc(pl.bundles.size() * sizeof(int32_t));
-      ACR_CUDA(cudaMemcpy(pl.d_bundles, pl.bundles.data(), pl.bundles.size() * sizeof(int32_t),
-                          cudaMemcpyHostToDevice));
+  void upload_plan(Plan& pl, cudaStream_t st) {
+    if (pl.uploaded) return;
+    pl.d_groups = store.put(pl.groups, st);
+    pl.d_items = store.put(pl.items, st);
+    pl.d_targets = store.put(pl.targets, st);
+    pl.d_stack = store.put(pl.stack, st);
+    pl.d_torder = store.put(pl.torder, st);
+    pl.d_bundles = store.put(pl.bundles, st);
+    pl.uploaded = true;
+    if (pl.items.size() >= PLAN_LARGE) {
+      pl.stripped = true;
+      if (spare_items.capacity() < pl.items.capacity()) {
+        spare_groups = std::move(pl.groups);
+        spare_items = std::move(pl.items);
+      }
+      pl.groups = std::vector<GGroup>();
+      pl.items = std::vector<GItem>();
     }
-    if (!pl.torder.empty()) {
-      pl.d_torder = dmalloc(pl.torder.size() * sizeof(int32_t));
-      ACR_CUDA(cudaMemcpy(pl.d_torder, pl.torder.data(), pl.torder.size() * sizeof(int32_t),
-                          cudaMemcpyHostToDevice));
-    }
-    if (!pl.stack.empty())
-      ACR_CUDA(cudaMemcpy(pl.d_stack, pl.stack.data(), pl.stack.size() * sizeof(StackDim),
-                          cudaMemcpyHostToDevice));
-    if (!pl.groups.empty())
-      ACR_CUDA(cudaMemcpy(pl.d_groups, pl.groups.data(), pl.groups.size() * sizeof(GGroup),
-                          cudaMemcpyHostToDevice));
-    if (!pl.items.empty())
-      ACR_CUDA(cudaMemcpy(pl.d_items, pl.items.data(), pl.items.size() * sizeof(GItem),
-                          cudaMemcpyHostToDevice));
-    if (!pl.targets.empty())
-      ACR_CUDA(cudaMemcpy(pl.d_targets, pl.targets.data(), pl.targets.size() * sizeof(TInfo),
-                          cudaMemcpyHostToDevice));
   }
 
   // Run a formatted operation, splitting it into the four child target
@@ -597,6 +669,13 @@ class Engine : public EngineBase {
     auto it = merged_plans.find(key);
     if (it == merged_plans.end()) {
       auto mp = std::make_unique<Plan>();
+      std::vector<std::unique_ptr<Plan>> again;   // plans whose host copies were given up
+      for (size_t i = 0; i < ps.size(); ++i)
+        if (ps[i]->stripped) {
+          again.push_back(std::make_unique<Plan>());
+          build_plan(S, ops[i], pp, *again.back());
+          ps[i] = again.back().get();
+        }
       merge_plans(ps, *mp);
       it = merged_plans.emplace(key, std::move(mp)).first;
     }
@@ -613,7 +692,7 @@ class Engine : public EngineBase {
 
   void run_plan(Plan& pl, int c_role, const std::vector<std::vector<HM>>& roles, int P,
                 cudaStream_t st) {
-    upload_plan(pl);
+    upload_plan(pl, st);
     const int nr = pl.nroles;
     size_t per_plane = std::max<size_t>((size_t)pl.scratch * sizeof(T), 256);
     int Pc = (int)std::max<size_t>(1, std::min<size_t>(P, scratch_budget / per_plane));
@@ -734,13 +813,16 @@ class Engine : public EngineBase {
     for (HM& h : roles[1]) free_hm(h);   // reusable by later launches (stream order)
   }
 
+  // A pointer table of an apply program: its place in the program's one upload
+  // (build_program), as an offset until then.
+  std::vector<char> blob;
   template <typename V>
   void** put_tables(const std::vector<V>& host) {
-    void* p = dmalloc(std::max<size_t>(host.size() * sizeof(V), 16));
-    if (!host.empty())
-      ACR_CUDA(cudaMemcpy(p, host.data(), host.size() * sizeof(V), cudaMemcpyHostToDevice));
-    owned.push_back(p);
-    return (void**)p;
+    const size_t at = blob.size();
+    const size_t bytes = host.size() * sizeof(V);
+    blob.resize(at + ((std::max<size_t>(bytes, 16) + 255) & ~size_t(255)));
+    if (bytes) std::memcpy(blob.data() + at, host.data(), bytes);
+    return reinterpret_cast<void**>(at);
   }
   // a pointer table of the setup, through the ring (capturable)
   template <typename V>
@@ -755,7 +837,7 @@ class Engine : public EngineBase {
   void run_steps(const std::vector<ApplyStep>& steps, int nr, cudaStream_t st, double* tv);
   static constexpr int RB = 8;       // right-hand sides per apply pass (multi-RHS apply)
   int64_t tvs = 0;                   // doubles of projection scratch per right-hand side
-  void collect_info();
+  void collect_info(cudaStream_t st);
 };
 
 template <typename T>
@@ -884,7 +966,7 @@ void Engine<T>::prepare(const double* const* coefs, cudaStream_t st, bool count_
   if (!count_pass) {
     // one-shot: plans are built as the real pass first needs them (host
     // work overlapping the device's), memory grows on demand
-    ring.init(size_t(64) << 20);
+    ring.init(size_t(32) << 20);
   } else {
     // counting pass: the same host sequence with no device work sizes the
     // H-matrix slots, the setup scratch and the table ring exactly
@@ -908,6 +990,8 @@ void Engine<T>::prepare(const double* const* coefs, cudaStream_t st, bool count_
     scratch_rank_cnt = std::max<size_t>(scratch_rank_need, 1);
     ring.init(ring_need);
     ring.fixed = true;
+    ACR_CUDA(cudaStreamSynchronize(st));   // the plans are on the device
+    store.release_staging();
   }
   info.structure_ms = std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - h0).count();
 }
@@ -1157,6 +1241,9 @@ void Engine<T>::finish(cudaStream_t st, bool one_shot) {
     info.sketch_overflows = (int64_t)ss[1];
     info.leaf_fp64_fallbacks = (int64_t)ss[2];
   }
+  store.release_staging();
+  spare_groups = std::vector<GGroup>();
+  spare_items = std::vector<GItem>();
   if (one_shot) {
     // the scratch arena is only needed by the setup; in the BF16 form the
     // FP32 arena holds no stored factor any more
@@ -1164,24 +1251,39 @@ void Engine<T>::finish(cudaStream_t st, bool one_shot) {
     if (scratch_ranks) { cudaFree(scratch_ranks); scratch_ranks = nullptr; scratch_rank_cnt = 0; }
     if (bf16) pool.release();
   }
-  collect_info();
+  collect_info(st);
   if (!Fv) build_apply_program();
 }
 
 template <typename T>
-void Engine<T>::collect_info() {
+void Engine<T>::collect_info(cudaStream_t st) {
   // ranks of every stored low-rank block
   std::vector<int> rk(S.lleaf.size());
   int64_t sumr = 0, cnt = 0;
   int mx = 0;
   int64_t bytes = 0;
-  std::vector<const void*> seen;
-  auto account = [&](const HM& h) {
-    if (!h.dense) return;
-    if (std::find(seen.begin(), seen.end(), h.dense) != seen.end()) return;
-    seen.push_back(h.dense);
-    if (!rk.empty())
-      ACR_CUDA(cudaMemcpy(rk.data(), h.rank, rk.size() * sizeof(int), cudaMemcpyDeviceToHost));
+  // every stored H-matrix once; their ranks through the (idle) pinned ring, as
+  // many at a time as it holds
+  std::vector<HM> seen;
+  {
+    std::vector<std::pair<const void*, HM>> all;
+    auto note = [&](const HM& h) {
+      if (h.dense) all.push_back({h.dense, h});
+    };
+    for (const Level& lev : levels) {
+      for (int i : lev.red) note(D[i]);
+      for (int in = 0; in < count; ++in)
+        for (int k = 0; k < n; k += lev.s) { note(lev.L[in * n + k]); note(lev.U[in * n + k]); }
+    }
+    for (int in = 0; in < count; ++in) note(D[in * n]);
+    std::sort(all.begin(), all.end(), [](const auto& a, const auto& b) { return a.first < b.first; });
+    for (size_t i = 0; i < all.size(); ++i)
+      if (i == 0 || all[i].first != all[i - 1].first) seen.push_back(all[i].second);
+  }
+  const size_t rkb = rk.size() * sizeof(int);
+  const size_t per = rkb == 0 ? seen.size() : ring.cap / rkb;
+  auto account = [&](const HM& h, const int* host) {
+    if (!rk.empty()) std::memcpy(rk.data(), host, rkb);
     int64_t used = (int64_t)S.dleaf.size() * S.lsz * S.lsz;
     for (size_t l = 0; l < rk.size(); ++l) {
       mx = std::max(mx, rk[l]);
@@ -1192,19 +1294,31 @@ void Engine<T>::collect_info() {
     hm_used[h.dense] = used;
     bytes += used * (int64_t)store_bytes();
   };
-  for (const Level& lev : levels) {
-    for (int i : lev.red) account(D[i]);
-    for (int in = 0; in < count; ++in)
-      for (int k = 0; k < n; k += lev.s) { account(lev.L[in * n + k]); account(lev.U[in * n + k]); }
+  std::vector<int> one(per == 0 ? rk.size() : 0);
+  for (size_t b = 0; b < seen.size();) {
+    if (per == 0) {   // a ring smaller than one rank list
+      ACR_CUDA(cudaMemcpy(one.data(), seen[b].rank, rkb, cudaMemcpyDeviceToHost));
+      account(seen[b], one.data());
+      ++b;
+      continue;
+    }
+    const size_t e = std::min(seen.size(), b + per);
+    if (rkb > 0) {
+      for (size_t q = b; q < e; ++q)
+        ACR_CUDA(cudaMemcpyAsync(ring.host + (q - b) * rkb, seen[q].rank, rkb,
+                                 cudaMemcpyDeviceToHost, st));
+      ACR_CUDA(cudaStreamSynchronize(st));
+    }
+    for (size_t q = b; q < e; ++q) account(seen[q], (const int*)(ring.host + (q - b) * rkb));
+    b = e;
   }
-  for (int in = 0; in < count; ++in) account(D[in * n]);
   info.max_rank = mx;
   info.avg_rank = cnt ? (double)sumr / cnt : 0.0;
   info.factor_bytes = bytes + 2 * N * count * (int64_t)sizeof(double);
-  int64_t per = ((int64_t)S.dleaf.size() * S.lsz * S.lsz + (S.sumM + S.sumN) * kc) *
-                (int64_t)store_bytes();
+  const int64_t hm_bytes = ((int64_t)S.dleaf.size() * S.lsz * S.lsz + (S.sumM + S.sumN) * kc) *
+                           (int64_t)store_bytes();
   info.factor_capacity_bytes =
-      per * (int64_t)seen.size() + 2 * N * count * (int64_t)sizeof(double);
+      hm_bytes * (int64_t)seen.size() + 2 * N * count * (int64_t)sizeof(double);
 }
 
 template <typename T>
@@ -1411,6 +1525,12 @@ void Engine<T>::build_program(Program& pg, int inst, bool count_bytes, double* F
       bw.push_back(copy_step(us, gs));      // u_i = g_i
       bw.push_back(mv_step(X, tmp, us, -1.0, 1.0, tr));  // u_i -= X_i tmp
     }
+  }
+  {   // the program's tables in one copy
+    char* base = (char*)upload(blob, owned);
+    for (auto* steps : {&pg.fwd, &pg.bwd, &pg.fwdT, &pg.bwdT})
+      for (ApplyStep& q : *steps) q.tabs = (void**)(base + reinterpret_cast<size_t>(q.tabs));
+    blob = std::vector<char>();
   }
   if (count_bytes) {
     // the two permutations between natural and cluster order

@@ -18,6 +18,8 @@ struct Term {
   int prod, t, r, s, type, anode, bnode, a_role, b_role, coef;
   int64_t off;   // scratch offset of the computed factor (W, Y or the dense product)
   int ld;        // its leading dimension
+  int next;      // the next term of the same block (t, s), -1: none
+  size_t m0;     // its small inner products: Builder::moff from here
 };
 
 struct Dim { int32_t st, rb, ri; };
@@ -32,10 +34,38 @@ struct Builder {
   int nroles;
   int kc;
   std::vector<Term> terms;
-  std::unordered_map<int64_t, std::vector<int>> terms_at;   // key t*ncl+s
+  // first and last term of each block (t, s): a table reset entry by entry where it is small
+  // enough, a map otherwise
+  struct Ends { int head = -1, tail = -1; };
+  std::vector<Ends>& tab;
+  std::unordered_map<int64_t, Ends> far;
+  std::vector<int64_t> moff;     // scratch offsets of the small inner products
+
+  static std::vector<Ends>& table() {
+    thread_local std::vector<Ends> t;
+    return t;
+  }
+  Ends* find_ends(int t, int s) {
+    const int64_t k = key(t, s);
+    if (!tab.empty()) return &tab[k];
+    auto it = far.find(k);
+    return it == far.end() ? nullptr : &it->second;
+  }
+  int first_term(int t, int s) {
+    Ends* e = find_ends(t, s);
+    return e ? e->head : -1;
+  }
+  ~Builder() {
+    if (!tab.empty())
+      for (const Term& q : terms) tab[key(q.t, q.s)] = Ends();
+  }
 
   Builder(const Structure& s_, const OpDesc& o, const PlanParams& p, Plan& pl)
-      : S(s_), op(o), pp(p), P(pl), nroles(o.nroles), kc(p.kc) {}
+      : S(s_), op(o), pp(p), P(pl), nroles(o.nroles), kc(p.kc), tab(table()) {
+    const size_t n2 = S.cl.size() * S.cl.size();
+    if (S.cl.size() > 2048) tab.clear();
+    else if (tab.size() < n2) tab.resize(n2);
+  }
 
   int bdense(int role) const { return 3 * role; }
   int bU(int role) const { return 3 * role + 1; }
@@ -52,25 +82,26 @@ struct Builder {
   int alloc_rank() { return P.scratch_ranks++; }
 
   int begin_group(int cbuf, int64_t coff, int ldc, Dim m, Dim n, int beta) {
-    GGroup g;
-    g.coff = coff; g.cbuf = cbuf; g.ldc = ldc;
-    g.m_st = m.st; g.m_rb = m.rb; g.m_ri = m.ri;
-    g.n_st = n.st; g.n_rb = n.rb; g.n_ri = n.ri;
+    GGroup g{};
+    g.coff = coff; g.cbuf = (int8_t)cbuf; g.ldc = ldc;
+    g.m_st = (int16_t)m.st; g.m_rb = (int8_t)m.rb; g.m_ri = m.ri;
+    g.n_st = (int16_t)n.st; g.n_rb = (int8_t)n.rb; g.n_ri = n.ri;
     g.ib = g.ie = (int)P.items.size();
-    g.beta = beta; g.pad = 0;
+    g.beta = (int8_t)beta;
     P.groups.push_back(g);
     return (int)P.groups.size() - 1;
   }
   void add_item(int abuf, int64_t aoff, int lda, int aflags, int bbuf, int64_t boff, int ldb,
                 int bflags, Dim k, Dim rows, int row_off, int coef, int seed = 0, int orow0 = 0,
                 int guard0 = -1, int guard1 = -1) {
-    GItem it;
-    it.aoff = aoff; it.boff = boff; it.abuf = abuf; it.bbuf = bbuf; it.lda = lda; it.ldb = ldb;
-    it.aflags = aflags; it.bflags = bflags;
-    it.k_st = k.st; it.k_rb = k.rb; it.k_ri = k.ri;
-    it.r_st = rows.st; it.r_rb = rows.rb; it.r_ri = rows.ri;
-    it.row_off = row_off; it.coef = coef; it.seed = seed; it.omega_row0 = orow0;
-    it.guard0 = guard0; it.guard1 = guard1;
+    GItem it{};
+    it.aoff = aoff; it.boff = boff; it.abuf = (int8_t)abuf; it.bbuf = (int8_t)bbuf;
+    it.lda = lda; it.ldb = ldb;
+    it.aflags = (int8_t)aflags; it.bflags = (int8_t)bflags;
+    it.k_st = k.st; it.k_rb = (int8_t)k.rb; it.k_ri = k.ri;
+    it.r_st = (int16_t)rows.st; it.r_rb = (int8_t)rows.rb; it.r_ri = rows.ri;
+    it.row_off = (int16_t)row_off; it.coef = (int8_t)coef; it.seed = seed; it.omega_row0 = orow0;
+    it.guard0 = (int8_t)guard0; it.guard1 = (int8_t)guard1;
     P.items.push_back(it);
     P.groups.back().ie = (int)P.items.size();
   }
@@ -98,35 +129,36 @@ struct Builder {
     else if (kb == BK_LOWRANK) q.type = TERM_B;
     else if (ka == BK_DENSE && kb == BK_DENSE) q.type = TERM_D;
     else throw std::runtime_error("unbalanced block trees (dense x inner) are not supported");
-    terms_at[key(t, s)].push_back((int)terms.size());
+    q.next = -1;
+    q.m0 = 0;
+    const int id = (int)terms.size();
     terms.push_back(q);
+    Ends& e = tab.empty() ? far[key(t, s)] : tab[key(t, s)];
+    if (e.head < 0) e.head = id;
+    else terms[e.tail].next = id;
+    e.tail = id;
   }
 
   // ---------------------------------------------------------------- phase 1
   void phase1() {
     const int lsz = S.lsz;
-    std::vector<int> leaves;
-    // stage 1a: small inner products M
+    // stage 1a: small inner products M, one per low-rank leaf of the other operand
     int g0 = (int)P.groups.size();
-    struct MRef { int term, leaf_node; int64_t off; };
-    std::vector<MRef> mrefs;
-    for (int qi = 0; qi < (int)terms.size(); ++qi) {
-      Term& q = terms[qi];
+    for (Term& q : terms) {
       if (q.type == TERM_A) {
         q.ld = S.cl[q.s].size;
         q.off = alloc((int64_t)q.ld * kc);
+        q.m0 = moff.size();
         int la = S.bn[q.anode].leaf;
-        leaves.clear();
-        S.subtree_leaves(q.bnode, leaves);
         const Cluster& cr = S.cl[q.r];
-        for (int bnode : leaves) {
-          if (S.bn[bnode].kind != BK_LOWRANK) continue;
-          int lb = S.bn[bnode].leaf;
-          const Cluster& crb = S.cl[S.bn[bnode].t];
-          int64_t moff = alloc((int64_t)kc * kc);
-          mrefs.push_back(MRef{qi, bnode, moff});
+        for (int pos = S.bn[q.bnode].lbeg; pos < S.bn[q.bnode].lend; ++pos) {
+          const BNode& b = S.bn[S.leafseq[pos]];
+          if (b.kind != BK_LOWRANK) continue;
+          int lb = b.leaf;
+          const Cluster& crb = S.cl[b.t];
+          moff.push_back(alloc((int64_t)kc * kc));
           // M = U_b^T V_a[r_b]   (k_b x k_a)
-          begin_group(bscr(), moff, kc, drank(q.b_role, lb), drank(q.a_role, la), -1);
+          begin_group(bscr(), moff.back(), kc, drank(q.b_role, lb), drank(q.a_role, la), -1);
           add_item(bU(q.b_role), S.lr_row0[lb] * kc, crb.size, FL_T,
                    bV(q.a_role), S.lr_col0[la] * kc + (crb.begin - cr.begin), cr.size, 0,
                    dconst(crb.size), drank(q.b_role, lb), 0, 0);
@@ -134,18 +166,17 @@ struct Builder {
       } else if (q.type == TERM_B) {
         q.ld = S.cl[q.t].size;
         q.off = alloc((int64_t)q.ld * kc);
+        q.m0 = moff.size();
         int lb = S.bn[q.bnode].leaf;
-        leaves.clear();
-        S.subtree_leaves(q.anode, leaves);
         const Cluster& cr = S.cl[q.r];
-        for (int anode : leaves) {
-          if (S.bn[anode].kind != BK_LOWRANK) continue;
-          int la = S.bn[anode].leaf;
-          const Cluster& cra = S.cl[S.bn[anode].s];
-          int64_t moff = alloc((int64_t)kc * kc);
-          mrefs.push_back(MRef{qi, anode, moff});
+        for (int pos = S.bn[q.anode].lbeg; pos < S.bn[q.anode].lend; ++pos) {
+          const BNode& a = S.bn[S.leafseq[pos]];
+          if (a.kind != BK_LOWRANK) continue;
+          int la = a.leaf;
+          const Cluster& cra = S.cl[a.s];
+          moff.push_back(alloc((int64_t)kc * kc));
           // M' = V_a^T U_b[r_a]   (k_a x k_b)
-          begin_group(bscr(), moff, kc, drank(q.a_role, la), drank(q.b_role, lb), -1);
+          begin_group(bscr(), moff.back(), kc, drank(q.a_role, la), drank(q.b_role, lb), -1);
           add_item(bV(q.a_role), S.lr_col0[la] * kc, cra.size, FL_T,
                    bU(q.b_role), S.lr_row0[lb] * kc + (cra.begin - cr.begin), cr.size, 0,
                    dconst(cra.size), drank(q.a_role, la), 0, 0);
@@ -153,27 +184,26 @@ struct Builder {
       }
     }
     stage(ST_GEMM, g0, (int)P.groups.size(), TAG_M);
-    // index M by (term, leaf node)
-    std::unordered_map<int64_t, int64_t> moff_of;
-    for (const MRef& m : mrefs) moff_of[(int64_t)m.term * (int64_t)S.bn.size() + m.leaf_node] = m.off;
+    // the inner product of term q with the leaf at position pos of node's subtree
+    auto moff_of = [&](const Term& q, int node, int pos) {
+      return moff[q.m0 + S.lr_before[pos] - S.lr_before[S.bn[node].lbeg]];
+    };
 
     // stage 1b: chunked factors W = B^T V_a, Y = A U_b, dense products
     g0 = (int)P.groups.size();
-    for (int qi = 0; qi < (int)terms.size(); ++qi) {
-      Term& q = terms[qi];
+    for (Term& q : terms) {
       if (q.type == TERM_A) {
         int la = S.bn[q.anode].leaf;
         const Cluster& cr = S.cl[q.r];
         const Cluster& cs = S.cl[q.s];
-        leaves.clear();
-        S.subtree_leaves(q.bnode, leaves);
-        for (int c0 = cs.begin; c0 < cs.begin + cs.size; c0 += lsz) {
+        const ChunkLeaves& cc = S.chunk_leaves(q.bnode, true);
+        for (int c = 0; c < cs.size / lsz; ++c) {
+          const int c0 = cs.begin + c * lsz;
           begin_group(bscr(), q.off + (c0 - cs.begin), q.ld, dconst(lsz), drank(q.a_role, la), -1);
-          for (int bnode : leaves) {
-            const BNode& b = S.bn[bnode];
+          for (int e = cc.ptr[c]; e < cc.ptr[c + 1]; ++e) {
+            const BNode& b = S.bn[S.leafseq[cc.at[e]]];
             const Cluster& crb = S.cl[b.t];
             const Cluster& csb = S.cl[b.s];
-            if (c0 < csb.begin || c0 >= csb.begin + csb.size) continue;
             if (b.kind == BK_DENSE) {
               // W[c] += B_b^T V_a[r_b]
               add_item(bdense(q.b_role), S.dense_off(b.leaf), lsz, FL_T,
@@ -182,9 +212,9 @@ struct Builder {
               P.flops_static += 2LL * lsz * lsz * kc;
             } else {
               // W[c] += V_b[c] M
-              int64_t moff = moff_of.at((int64_t)qi * (int64_t)S.bn.size() + bnode);
               add_item(bV(q.b_role), S.lr_col0[b.leaf] * kc + (c0 - csb.begin), csb.size, 0,
-                       bscr(), moff, kc, 0, drank(q.b_role, b.leaf), dconst(lsz), 0, 0);
+                       bscr(), moff_of(q, q.bnode, cc.at[e]), kc, 0, drank(q.b_role, b.leaf),
+                       dconst(lsz), 0, 0);
             }
           }
         }
@@ -192,15 +222,14 @@ struct Builder {
         int lb = S.bn[q.bnode].leaf;
         const Cluster& cr = S.cl[q.r];
         const Cluster& ct = S.cl[q.t];
-        leaves.clear();
-        S.subtree_leaves(q.anode, leaves);
-        for (int c0 = ct.begin; c0 < ct.begin + ct.size; c0 += lsz) {
+        const ChunkLeaves& cc = S.chunk_leaves(q.anode, false);
+        for (int c = 0; c < ct.size / lsz; ++c) {
+          const int c0 = ct.begin + c * lsz;
           begin_group(bscr(), q.off + (c0 - ct.begin), q.ld, dconst(lsz), drank(q.b_role, lb), -1);
-          for (int anode : leaves) {
-            const BNode& a = S.bn[anode];
+          for (int e = cc.ptr[c]; e < cc.ptr[c + 1]; ++e) {
+            const BNode& a = S.bn[S.leafseq[cc.at[e]]];
             const Cluster& cta = S.cl[a.t];
             const Cluster& csa = S.cl[a.s];
-            if (c0 < cta.begin || c0 >= cta.begin + cta.size) continue;
             if (a.kind == BK_DENSE) {
               // Y[c] += A_a U_b[r_a]
               add_item(bdense(q.a_role), S.dense_off(a.leaf), lsz, 0,
@@ -208,9 +237,9 @@ struct Builder {
                        dconst(lsz), dconst(lsz), 0, 0);
               P.flops_static += 2LL * lsz * lsz * kc;
             } else {
-              int64_t moff = moff_of.at((int64_t)qi * (int64_t)S.bn.size() + anode);
               add_item(bU(q.a_role), S.lr_row0[a.leaf] * kc + (c0 - cta.begin), cta.size, 0,
-                       bscr(), moff, kc, 0, drank(q.a_role, a.leaf), dconst(lsz), 0, 0);
+                       bscr(), moff_of(q, q.anode, cc.at[e]), kc, 0, drank(q.a_role, a.leaf),
+                       dconst(lsz), 0, 0);
             }
           }
         }
@@ -240,22 +269,22 @@ struct Builder {
     int64_t sp_off;        // scratch for S_i (k x p) then P_i (k x r)
   };
 
+  std::vector<std::pair<int, int>> pairs;   // collect_terms' stack
+
   // terms restricted / embedded into target leaf (tc, sc)
   void collect_terms(int tc, int sc, bool lowrank, std::vector<int>& anc_self,
                      std::vector<int>& desc) {
     const BNode& root = S.bn[op.c_node];
     int t = tc, s = sc;
     while (true) {
-      auto it = terms_at.find(key(t, s));
-      if (it != terms_at.end())
-        for (int q : it->second) anc_self.push_back(q);
+      for (int q = first_term(t, s); q >= 0; q = terms[q].next) anc_self.push_back(q);
       if (t == root.t && s == root.s) break;
       t = S.cl[t].parent;
       s = S.cl[s].parent;
       if (t < 0 || s < 0) break;
     }
     if (!lowrank) return;
-    std::vector<std::pair<int, int>> st;
+    std::vector<std::pair<int, int>>& st = pairs;
     const Cluster &ct = S.cl[tc], &cs = S.cl[sc];
     if (ct.child[0] >= 0 && cs.child[0] >= 0)
       for (int i = 0; i < 2; ++i)
@@ -263,9 +292,7 @@ struct Builder {
     while (!st.empty()) {
       auto [a, b] = st.back();
       st.pop_back();
-      auto it = terms_at.find(key(a, b));
-      if (it != terms_at.end())
-        for (int q : it->second) desc.push_back(q);
+      for (int q = first_term(a, b); q >= 0; q = terms[q].next) desc.push_back(q);
       const Cluster &ca = S.cl[a], &cb = S.cl[b];
       if (ca.child[0] >= 0 && cb.child[0] >= 0)
         for (int i = 0; i < 2; ++i)
@@ -348,6 +375,7 @@ struct Builder {
       ++P.n_lr_targets;
       LT lt;
       lt.node = node;
+      lt.items.reserve(anc.size() + desc.size() + op.adds.size() + 1);
       int lc = c.leaf;
       if (op.alpha >= 0) {
         LItem li{};
@@ -595,8 +623,9 @@ bool same_a(const Plan& pl, const GGroup& x, const GGroup& y) {
 void make_bundles(Plan& plan, Stage& sg) {
   const int beg = sg.beg + sg.nwide, n = sg.end - beg;
   const int most = std::max(1, std::min(BUNDLE_MAX, n / 152));
-  std::unordered_map<uint64_t, std::vector<int>> open;   // key -> bundles of that key
-  std::vector<std::vector<int>> bd;
+  std::unordered_map<uint64_t, int> open;   // key -> its last bundle
+  open.reserve(n);
+  std::vector<int> of(n), size, first;      // bundle of each group; size and first group of each
   for (int i = 0; i < n; ++i) {
     const GGroup& g = plan.groups[beg + i];
     uint64_t key = (uint64_t)(g.ie - g.ib);
@@ -605,27 +634,29 @@ void make_bundles(Plan& plan, Stage& sg) {
       key = (key ^ (uint64_t)it.aoff ^ ((uint64_t)it.abuf << 48)) * 0x9E3779B97F4A7C15ull;
       key ^= key >> 29;
     }
-    int at = -1;
-    std::vector<int>& cand = open[key];
-    if (!cand.empty() && (int)bd[cand.back()].size() < most &&
-        same_a(plan, plan.groups[beg + bd[cand.back()][0]], g))
-      at = cand.back();
-    if (at < 0) {
-      at = (int)bd.size();
-      bd.emplace_back();
-      cand.push_back(at);
+    auto [at, fresh] = open.try_emplace(key, (int)size.size());
+    if (!fresh && (size[at->second] >= most ||
+                   !same_a(plan, plan.groups[beg + first[at->second]], g))) {
+      at->second = (int)size.size();
+      fresh = true;
     }
-    bd[at].push_back(i);
+    if (fresh) {
+      size.push_back(0);
+      first.push_back(i);
+    }
+    of[i] = at->second;
+    ++size[at->second];
   }
-  std::vector<GGroup> re;
-  re.reserve(n);
+  std::vector<int> at(size.size() + 1, 0);
   sg.bbeg = (int)plan.bundles.size() / 2;
-  for (const auto& b : bd) {
-    plan.bundles.push_back(beg + (int)re.size());
-    for (int i : b) re.push_back(plan.groups[beg + i]);
-    plan.bundles.push_back(beg + (int)re.size());
+  for (size_t b = 0; b < size.size(); ++b) {
+    at[b + 1] = at[b] + size[b];
+    plan.bundles.push_back(beg + at[b]);
+    plan.bundles.push_back(beg + at[b + 1]);
   }
   sg.bend = (int)plan.bundles.size() / 2;
+  std::vector<GGroup> re(n);
+  for (int i = 0; i < n; ++i) re[at[of[i]]++] = plan.groups[beg + i];
   std::copy(re.begin(), re.end(), plan.groups.begin() + beg);
 }
 
@@ -645,16 +676,22 @@ void order_wide_first(Plan& plan) {
   for (Stage& sg : plan.stages) {
     if (sg.kind != ST_GEMM) continue;
     auto wide = [](const GGroup& g) { return g.n_rb < 0 && g.n_st >= 64; };
-    auto mid = std::stable_partition(plan.groups.begin() + sg.beg, plan.groups.begin() + sg.end,
-                                     wide);
-    sg.nwide = (int)(mid - (plan.groups.begin() + sg.beg));
+    const auto beg = plan.groups.begin() + sg.beg, end = plan.groups.begin() + sg.end;
+    sg.nwide = (int)std::count_if(beg, end, wide);
+    if (sg.nwide > 0 && sg.nwide < sg.end - sg.beg) std::stable_partition(beg, end, wide);
     if (sg.tag == TAG_FACT) make_bundles(plan, sg);
   }
 }
 }  // namespace
 
 void build_plan(const Structure& S, const OpDesc& op, const PlanParams& pp, Plan& plan) {
+  std::vector<GGroup> groups = std::move(plan.groups);
+  std::vector<GItem> items = std::move(plan.items);
+  groups.clear();
+  items.clear();
   plan = Plan();
+  plan.groups = std::move(groups);
+  plan.items = std::move(items);
   plan.nroles = op.nroles;
   Builder b(S, op, pp, plan);
   const BNode& c = S.bn[op.c_node];

@@ -42,26 +42,33 @@ namespace acr {
 enum : int32_t { FL_T = 1, FL_IDENT = 2, FL_OMEGA = 4 };
 
 // A dimension: the constant `st`, or rank[ri] of rank buffer rb of the plane.
-struct GItem {
+// (A plan of one plane-sized product holds hundreds of thousands of items: the
+// records are as small as their ranges allow -- buffers and rank buffers below
+// 128, output tiles of at most 64 -- 64 and 40 bytes.)
+struct alignas(16) GItem {
   int64_t aoff, boff;
-  int32_t abuf, bbuf, lda, ldb;
-  int32_t aflags, bflags;
-  int32_t k_st, k_rb, k_ri;     // inner dimension
-  int32_t r_st, r_rb, r_ri;     // rows this item contributes (<= group rows)
-  int32_t row_off;              // first output row of the contribution
-  int32_t coef;                 // index into the coefficient array
+  int32_t lda, ldb;
+  int32_t k_st, k_ri;           // inner dimension
+  int32_t r_ri;                 // rows this item contributes (<= group rows)
   int32_t seed, omega_row0;     // FL_OMEGA: B(l, j) = omega(seed, omega_row0 + l, j)
-  int32_t guard0, guard1;       // buffers that must be present for the plane (-1: none)
+  int16_t r_st;
+  int16_t row_off;              // first output row of the contribution
+  int8_t abuf, bbuf;
+  int8_t aflags, bflags;
+  int8_t k_rb, r_rb;
+  int8_t coef;                  // index into the coefficient array
+  int8_t guard0, guard1;        // buffers that must be present for the plane (-1: none)
 };
+static_assert(sizeof(GItem) == 64, "four 16-byte loads per item");
 
 struct GGroup {
   int64_t coff;
-  int32_t cbuf, ldc;
-  int32_t m_st, m_rb, m_ri;
-  int32_t n_st, n_rb, n_ri;
+  int32_t ldc;
+  int32_t m_ri, n_ri;
   int32_t ib, ie;
-  int32_t beta;                 // coefficient of the old C; -1: C is overwritten
-  int32_t pad;
+  int16_t m_st, n_st;
+  int8_t cbuf, m_rb, n_rb;
+  int8_t beta;                  // coefficient of the old C; -1: C is overwritten
 };
 
 // one low-rank target of phase 2 (core kernels)
@@ -150,6 +157,8 @@ struct Plan {
   int32_t max_p = 0;          // widest sketch over the targets (bounds every core's size)
   std::vector<int32_t> torder;   // target indices by increasing sketch size m * p
   // device copies (owned by the engine)
+  bool uploaded = false;
+  bool stripped = false;      // host copies of groups and items given up after the upload
   void* d_groups = nullptr;
   void* d_items = nullptr;
   void* d_targets = nullptr;
@@ -165,7 +174,8 @@ struct PlanParams {
   bool fused = false;   // one basis and one core stage per plan (float factors)
 };
 
-// Build the plan of one formatted operation.
+// Build the plan of one formatted operation (plan.groups and plan.items keep
+// the storage they come with).
 void build_plan(const Structure& S, const OpDesc& op, const PlanParams& pp, Plan& plan);
 
 // Merge plans of independent operations (same roles, same target role):

@@ -64,6 +64,7 @@ int Structure::block(int t, int s, int parent) {
   for (int k = 0; k < 4; ++k) b.child[k] = -1;
   bn.push_back(b);
   node_of[(int64_t)t * (int64_t)cl.size() + s] = id;
+  bn[id].lbeg = (int)leafseq.size();
   const Cluster& ct = cl[t];
   const Cluster& cs = cl[s];
   if (admissible(t, s)) {
@@ -79,6 +80,8 @@ int Structure::block(int t, int s, int parent) {
         bn[id].child[k++] = c;
       }
   }
+  if (bn[id].kind != BK_INNER) leafseq.push_back(id);
+  bn[id].lend = (int)leafseq.size();
   return id;
 }
 
@@ -92,7 +95,15 @@ void Structure::build(int n_, double eta_, int leaf_) {
     if (c.child[0] < 0)
       for (int iy = c.y0; iy < c.y1; ++iy)
         for (int ix = c.x0; ix < c.x1; ++ix) perm.push_back(ix + n * iy);
+  leafseq.clear(); node_tab.clear(); lr_before.clear();
+  chunks_[0].clear(); chunks_[1].clear();
   block(0, 0, -1);
+  if (cl.size() <= 2048) {
+    node_tab.assign(cl.size() * cl.size(), -1);
+    for (const auto& kv : node_of) node_tab[kv.first] = kv.second;
+  }
+  lr_before.push_back(0);
+  for (int id : leafseq) lr_before.push_back(lr_before.back() + (bn[id].kind == BK_LOWRANK));
   // leaf enumeration in depth-first order (storage order)
   for (int i = 0; i < (int)bn.size(); ++i) {
     if (bn[i].kind == BK_DENSE) { bn[i].leaf = (int)dleaf.size(); dleaf.push_back(i); }
@@ -130,16 +141,36 @@ void Structure::build(int n_, double eta_, int leaf_) {
 }
 
 void Structure::subtree_leaves(int node_id, std::vector<int>& out) const {
-  std::vector<int> stack{node_id};
-  while (!stack.empty()) {
-    int b = stack.back();
-    stack.pop_back();
-    if (bn[b].kind == BK_INNER) {
-      for (int k = 3; k >= 0; --k) stack.push_back(bn[b].child[k]);
-    } else {
-      out.push_back(b);
-    }
+  out.insert(out.end(), leafseq.begin() + bn[node_id].lbeg, leafseq.begin() + bn[node_id].lend);
+}
+
+const ChunkLeaves& Structure::chunk_leaves(int id, bool cols) const {
+  auto& cache = chunks_[cols ? 1 : 0];
+  auto it = cache.find(id);
+  if (it != cache.end()) return it->second;
+  const BNode& b = bn[id];
+  const Cluster& c = cl[cols ? b.s : b.t];
+  ChunkLeaves cc;
+  cc.ptr.assign(c.size / lsz + 1, 0);
+  auto span = [&](int pos, int& c0, int& c1) {
+    const BNode& l = bn[leafseq[pos]];
+    const Cluster& lc = cl[cols ? l.s : l.t];
+    c0 = (lc.begin - c.begin) / lsz;
+    c1 = c0 + lc.size / lsz;
+  };
+  int c0, c1;
+  for (int pos = b.lbeg; pos < b.lend; ++pos) {
+    span(pos, c0, c1);
+    for (int q = c0; q < c1; ++q) ++cc.ptr[q + 1];
   }
+  for (size_t q = 1; q < cc.ptr.size(); ++q) cc.ptr[q] += cc.ptr[q - 1];
+  cc.at.resize(cc.ptr.back());
+  std::vector<int> w(cc.ptr.begin(), cc.ptr.end() - 1);
+  for (int pos = b.lbeg; pos < b.lend; ++pos) {
+    span(pos, c0, c1);
+    for (int q = c0; q < c1; ++q) cc.at[w[q]++] = pos;
+  }
+  return cache.emplace(id, std::move(cc)).first->second;
 }
 
 }  // namespace acr

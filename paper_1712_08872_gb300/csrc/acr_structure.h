@@ -25,6 +25,13 @@ struct BNode {
   int child[4];         // inner nodes: (t0,s0),(t0,s1),(t1,s0),(t1,s1)
   int parent;
   int leaf;             // dense-leaf index or low-rank-leaf index, -1 for inner
+  int lbeg, lend;       // its subtree's leaves: positions in Structure::leafseq
+};
+
+// The leaves of a block subtree by the leaf-size chunks of its columns (or
+// rows): those of chunk c at at[ptr[c]] ... at[ptr[c + 1] - 1], positions in Structure::leafseq.
+struct ChunkLeaves {
+  std::vector<int> ptr, at;
 };
 
 struct Structure {
@@ -43,13 +50,21 @@ struct Structure {
   int nleafcl = 0;              // number of leaf clusters
   bool balanced = false;
   std::vector<int> leaf_cluster_at;  // leaf cluster id by position / lsz
+  std::vector<int> leafseq;     // block nodes of all leaves, in node order (= depth first)
+  std::vector<int> lr_before;   // low-rank leaves among the first i of leafseq
   std::unordered_map<int64_t, int> node_of;
+  std::vector<int> node_tab;    // the same as a table, where it is small enough
 
   void build(int n, double eta, int leaf);
   int node(int t, int s) const {
-    auto it = node_of.find((int64_t)t * (int64_t)cl.size() + s);
+    const int64_t key = (int64_t)t * (int64_t)cl.size() + s;
+    if (!node_tab.empty()) return node_tab[key];
+    auto it = node_of.find(key);
     return it == node_of.end() ? -1 : it->second;
   }
+  // leaves of node id's subtree by column (or row) chunk (balanced trees), built on
+  // first use: a structure is used from one host thread
+  const ChunkLeaves& chunk_leaves(int id, bool cols) const;
   bool admissible(int t, int s) const;
   double diam(int t) const;
   double dist(int t, int s) const;
@@ -60,6 +75,7 @@ struct Structure {
  private:
   int split(int x0, int x1, int y0, int y1, int begin, int level, int parent);
   int block(int t, int s, int parent);
+  mutable std::unordered_map<int, ChunkLeaves> chunks_[2];
 };
 
 }  // namespace acr
