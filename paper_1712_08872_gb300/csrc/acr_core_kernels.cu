@@ -49,19 +49,22 @@ __device__ __forceinline__ void count_stacked_warp(const TInfo& ti,
 
 // Orthonormal basis Q of range(Y) (m x p, in place): the column of largest
 // remaining norm is taken, projected once more against the basis so far (the
-// second pass that makes Gram-Schmidt orthonormal to rounding), normalised, and
-// removed from the remaining columns, whose norms are then recomputed; stops
-// when the largest remaining norm is at most tau times the largest of Y.
+// second pass that makes Gram-Schmidt orthonormal to rounding), and removed from
+// the remaining columns, whose norms are then recomputed; stops when the largest
+// remaining norm is at most tau times the largest of Y.  Basis columns are kept
+// unscaled with the square of their reciprocal norm, and scaled at the end.
 //
 // Bound by the latency of the r dependent steps, not by arithmetic or bytes
 // (64 x 32 floats per typical target): Y stays in shared memory, a warp owns
-// whole columns in the update (no barrier between its dot and its axpy), and a
-// step has four barriers.  It replaces six launches of the plan (two
-// compensated Grams, two FP64 pivoted Cholesky cores, two basis products).
+// whole columns (CPW of them, their sums and reductions side by side; no barrier
+// between a column's dot and its axpy), and a step has three barriers.  It
+// replaces six launches of the plan (two compensated Grams, two FP64 pivoted
+// Cholesky cores, two basis products: 95 ms of the n = 64 setup; here 25 ms, and
+// 30 ms with the columns of a warp one after another and a fourth barrier).
 constexpr int ONT = 256;
 
-template <bool SMEM>
-__global__ void __launch_bounds__(ONT) k_orth(const TInfo* __restrict__ tis,
+template <bool SMEM, int CPW>
+__global__ void __launch_bounds__(ONT, 6) k_orth(const TInfo* __restrict__ tis,
                                               const int* __restrict__ order, double tau_,
                                               float* const* __restrict__ tab,
                                               int* const* __restrict__ rtab, int P, int scr_buf,
@@ -70,7 +73,9 @@ __global__ void __launch_bounds__(ONT) k_orth(const TInfo* __restrict__ tis,
                                               double* __restrict__ flops) {
   constexpr int NW = ONT / 32;
   extern __shared__ float ysm[];
-  __shared__ float nrm[CMAX], dot[CMAX], part[NW];
+  __shared__ float nrm[CMAX], rn2[CMAX];
+  __shared__ __align__(16) float dot[CMAX];
+  __shared__ __align__(16) float part[NW];
   const int p = blockIdx.y;
   const TInfo ti = tis[order[blockIdx.x]];
   float* scr = tab[scr_buf * P + p];
@@ -80,54 +85,115 @@ __global__ void __launch_bounds__(ONT) k_orth(const TInfo* __restrict__ tis,
   float* Yg = scr + ti.y_off;
   float* Y = SMEM ? ysm : Yg;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  for (int c = warp; c < pc; c += NW) {
-    const float* g = Yg + (int64_t)c * m;
-    float* y = Y + (int64_t)c * m;
-    float s = 0.f;
-    for (int i = lane; i < m; i += 32) {
-      const float v = g[i];
-      if (SMEM) y[i] = v;
-      s = fmaf(v, v, s);
-    }
-    s = warp_sum(s);
-    if (lane == 0) nrm[c] = s;
+  {
+    float s[CPW];
+#pragma unroll
+    for (int u = 0; u < CPW; ++u) s[u] = 0.f;
+    for (int i = lane; i < m; i += 32)
+#pragma unroll
+      for (int u = 0; u < CPW; ++u) {
+        const int c = warp + NW * u;
+        if (c < pc) {
+          const float v = Yg[i + (int64_t)c * m];
+          if (SMEM) Y[i + c * m] = v;
+          s[u] = fmaf(v, v, s[u]);
+        }
+      }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+      for (int u = 0; u < CPW; ++u) s[u] += __shfl_xor_sync(FULL, s[u], o);
+#pragma unroll
+    for (int u = 0; u < CPW; ++u)
+      if (lane == 0 && warp + NW * u < pc) nrm[warp + NW * u] = s[u];
   }
   if (sketch_stat && warp == NW - 1)
     count_stacked_warp(ti, stack, tab, (const int* const*)rtab, P, p, sketch_stat);
   __syncthreads();
   const float tau2 = (float)(tau_ * tau_);
   float tol = 0.f;
+  bool scaled = false;
   int r = 0;
   for (int j = 0; j < pc; ++j) {
-    // every warp finds the largest remaining column (the lowest index on ties)
-    const float a = (j + lane < pc) ? nrm[j + lane] : -1.f;
-    const float b = (j + lane + 32 < pc) ? nrm[j + lane + 32] : -1.f;
-    float best = fmaxf(a, b);
-    int q = a >= b ? j + lane : j + lane + 32;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      const float ov = __shfl_xor_sync(FULL, best, o);
-      const int oq = __shfl_xor_sync(FULL, q, o);
-      if (ov > best || (ov == best && oq < q)) { best = ov; q = oq; }
+    // every warp finds the largest remaining column: bits of the squared norms
+    // order like the norms, the low six hold the column (norms that agree to
+    // 2^-17 count as equal: the lowest column); NaN norms are passed over
+    unsigned ka = 0u, kb = 0u;
+    if (j + lane < pc && nrm[j + lane] > 0.f)
+      ka = (__float_as_uint(nrm[j + lane]) & ~63u) | (63u - (j + lane));
+    if (CPW > 4 && j + lane + 32 < pc && nrm[j + lane + 32] > 0.f)
+      kb = (__float_as_uint(nrm[j + lane + 32]) & ~63u) | (63u - (j + lane + 32));
+    const unsigned kbest = __reduce_max_sync(FULL, max(ka, kb));
+    if (kbest == 0u) break;
+    const int q = 63 - (int)(kbest & 63u);
+    const float best = nrm[q];
+    if (j == 0) {
+      // a sketch so small that its squares would lose bits: scaled by a power of
+      // two (Q does not depend on it)
+      if (best < 0x1p-80f && !scaled) {
+        const float f = ldexpf(1.f, -(ilogbf(best) / 2));
+        for (int c = warp; c < pc; c += NW) {
+          float s = 0.f;
+          for (int i = lane; i < m; i += 32) {
+            const float v = f * Y[i + (int64_t)c * m];
+            Y[i + (int64_t)c * m] = v;
+            s = fmaf(v, v, s);
+          }
+          s = warp_sum(s);
+          __syncwarp();
+          if (lane == 0) rn2[c] = s;
+        }
+        __syncthreads();
+        if (tid < pc) nrm[tid] = rn2[tid];
+        __syncthreads();
+        scaled = true;
+        j = -1;
+        continue;
+      }
+      tol = tau2 * best;
     }
-    if (j == 0) tol = tau2 * best;
-    if (!(best > tol) || !(best > 0.f)) break;
+    if (!(best > tol)) break;
     float* yq = Y + (int64_t)q * m;
     float* yj = Y + (int64_t)j * m;
     // second projection against the basis so far
-    for (int c = warp; c < j; c += NW) {
-      const float* y = Y + (int64_t)c * m;
-      float s = 0.f;
-      for (int i = lane; i < m; i += 32) s = fmaf(y[i], yq[i], s);
-      s = warp_sum(s);
-      if (lane == 0) dot[c] = s;
+    if (warp < j) {
+      float s[CPW];
+#pragma unroll
+      for (int u = 0; u < CPW; ++u) s[u] = 0.f;
+      for (int i = lane; i < m; i += 32) {
+        const float v = yq[i];
+#pragma unroll
+        for (int u = 0; u < CPW; ++u) {
+          const int c = warp + NW * u;
+          if (c < j) s[u] = fmaf(Y[i + (int64_t)c * m], v, s[u]);
+        }
+      }
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+        for (int u = 0; u < CPW; ++u) s[u] += __shfl_xor_sync(FULL, s[u], o);
+#pragma unroll
+      for (int u = 0; u < CPW; ++u) {
+        const int c = warp + NW * u;
+        if (lane == 0 && c < j) dot[c] = s[u] * rn2[c];
+      }
     }
     __syncthreads();
     // (the interchange of columns j and q folded in: a thread owns its rows)
     float s2 = 0.f;
     for (int i = tid; i < m; i += ONT) {
       float v = yq[i];
-      for (int c = 0; c < j; ++c) v = fmaf(-dot[c], Y[i + (int64_t)c * m], v);
+      int c = 0;
+      for (; c + 4 <= j; c += 4) {
+        const float4 d = *reinterpret_cast<const float4*>(dot + c);
+        const float* y = Y + i + (int64_t)c * m;
+        const float y0 = y[0], y1 = y[m], y2 = y[2 * (int64_t)m], y3 = y[3 * (int64_t)m];
+        v = fmaf(-d.x, y0, v);
+        v = fmaf(-d.y, y1, v);
+        v = fmaf(-d.z, y2, v);
+        v = fmaf(-d.w, y3, v);
+      }
+      for (; c < j; ++c) v = fmaf(-dot[c], Y[i + (int64_t)c * m], v);
       if (q != j) yq[i] = yj[i];
       yj[i] = v;
       s2 = fmaf(v, v, s2);
@@ -135,32 +201,55 @@ __global__ void __launch_bounds__(ONT) k_orth(const TInfo* __restrict__ tis,
     s2 = warp_sum(s2);
     if (lane == 0) part[warp] = s2;
     __syncthreads();
-    float nv = 0.f;
+    const float4 p0 = *reinterpret_cast<const float4*>(part);
+    const float4 p1 = *reinterpret_cast<const float4*>(part + 4);
+    const float nv = ((p0.x + p0.y) + (p0.z + p0.w)) + ((p1.x + p1.y) + (p1.z + p1.w));
+    const float rr = nv >= 0x1p-126f ? 1.f / nv : 0.f;
+    if (tid == 0) rn2[j] = rr;
+    // remove it from the remaining columns (this warp's from c0 on); their norms afresh
+    const int c0 = warp + NW * ((j + 1 - warp + NW - 1) / NW);
+    if (c0 < pc) {
+      float s[CPW], t[CPW];
 #pragma unroll
-    for (int w = 0; w < NW; ++w) nv += part[w];
-    const float rn = nv > 0.f ? 1.f / sqrtf(nv) : 0.f;
-    for (int i = tid; i < m; i += ONT) yj[i] *= rn;
-    __syncthreads();
-    // remove it from the remaining columns; their norms afresh
-    for (int c = j + 1 + warp; c < pc; c += NW) {
-      float* y = Y + (int64_t)c * m;
-      float s = 0.f;
-      for (int i = lane; i < m; i += 32) s = fmaf(yj[i], y[i], s);
-      s = warp_sum(s);
-      float t = 0.f;
+      for (int u = 0; u < CPW; ++u) s[u] = t[u] = 0.f;
       for (int i = lane; i < m; i += 32) {
-        const float v = fmaf(-s, yj[i], y[i]);
-        y[i] = v;
-        t = fmaf(v, v, t);
+        const float v = yj[i];
+#pragma unroll
+        for (int u = 0; u < CPW; ++u)
+          if (c0 + NW * u < pc) s[u] = fmaf(v, Y[i + (int64_t)(c0 + NW * u) * m], s[u]);
       }
-      t = warp_sum(t);
-      if (lane == 0) nrm[c] = t;
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+        for (int u = 0; u < CPW; ++u) s[u] += __shfl_xor_sync(FULL, s[u], o);
+#pragma unroll
+      for (int u = 0; u < CPW; ++u) s[u] *= rr;
+      for (int i = lane; i < m; i += 32) {
+        const float v = yj[i];
+#pragma unroll
+        for (int u = 0; u < CPW; ++u)
+          if (c0 + NW * u < pc) {
+            float* y = Y + i + (int64_t)(c0 + NW * u) * m;
+            const float w = fmaf(-s[u], v, *y);
+            *y = w;
+            t[u] = fmaf(w, w, t[u]);
+          }
+      }
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+        for (int u = 0; u < CPW; ++u) t[u] += __shfl_xor_sync(FULL, t[u], o);
+#pragma unroll
+      for (int u = 0; u < CPW; ++u)
+        if (lane == 0 && c0 + NW * u < pc) nrm[c0 + NW * u] = t[u];
     }
     r = j + 1;
     __syncthreads();
   }
-  if (SMEM)
-    for (int e = tid; e < r * m; e += ONT) Yg[e] = Y[e];
+  for (int c = warp; c < r; c += NW) {
+    const float f = sqrtf(rn2[c]);
+    for (int i = lane; i < m; i += 32) Yg[i + (int64_t)c * m] = f * Y[i + (int64_t)c * m];
+  }
   if (tid == 0) {
     rs[ti.r_ri] = r;
     if (flops) atomicAdd(flops, (double)m * r * (4.0 * pc));
@@ -203,15 +292,17 @@ __device__ __forceinline__ FF ff_rsqrt1p(float t) {
   return ff_add(FF{y, 0.f}, ff_mul(FF{y, 0.f}, FF{0.5f * e.h, 0.5f * e.l}));
 }
 // The rotation (c, s) that zeroes a_pq of [a_pp a_pq; a_pq a_qq]: the angle in
-// float (an angle off by ~1e-7 leaves ~1e-7 of the entry, which later rotations
-// remove), its cosine and sine to float-float accuracy from that angle, so the
+// float with the fast divide (an angle off by ~1e-6 leaves ~1e-6 of the entry, which
+// later rotations remove), its cosine and sine to float-float accuracy from that angle, so the
 // rotation itself is orthogonal to ~1e-14.
 __device__ __forceinline__ void ff_rot(FF app, FF aqq, FF apq, FF& c, FF& s) {
   c = FF{1.f, 0.f};
   s = FF{0.f, 0.f};
   if (apq.h != 0.f) {
-    const float tau = (aqq.h - app.h) / (2.f * apq.h);
-    const float t = (tau >= 0.f ? 1.f : -1.f) / (fabsf(tau) + sqrtf(1.f + tau * tau));
+    const float tau =
+        fminf(fmaxf(__fdividef(aqq.h - app.h, 2.f * apq.h), -1e15f), 1e15f);
+    const float h = fmaf(tau, tau, 1.f);
+    const float t = copysignf(__fdividef(1.f, fabsf(tau) + h * rsqrtf(h)), tau);
     c = ff_rsqrt1p(t);
     s = ff_mul(FF{t, 0.f}, c);
   }
@@ -229,16 +320,20 @@ __device__ __forceinline__ void ff_rot(FF app, FF aqq, FF apq, FF& c, FF& s) {
 // the factors U = Q W, V = B^T W straight into the target's leaf.
 //
 // Bound by the latency of the ~6 (r - 1) dependent rounds of a core, each a
-// rotation angle (float divide, square root) and a handful of float-float
-// operations per thread; four warps so that a typical core's round (r = 12:
-// 21 blocks and 72 row pairs of V) is one pass over the threads.
+// rotation angle and a handful of float-float operations per thread.  Four warps,
+// so that a typical core's round (r = 12: 21 blocks and 72 row pairs of V) is one
+// pass over the threads; every warp computes all rotations in its lanes and
+// hands them round by shuffles, and a round writes the other copy of A, so
+// that it has one barrier.  n = 64 setup: the four stages 90 ms, here 31 ms (36 ms with
+// rotations through shared memory and A updated in place).
 constexpr int CNT = 128;
 constexpr int CRAW = CNT * 16;   // float-float partial sums of the Gram's tiles
 
 __host__ __device__ constexpr size_t core_smem(int p) {
-  // A; the Gram's staging, then V in its place (p x (p + 1) float-float each); W
+  // A; the Gram's staging, then the other A and V in its place (p x (p + 1)
+  // float-float each); W
   const size_t a = (size_t)p * (p + 1) * sizeof(FF), g = CRAW * sizeof(FF);
-  return a + (a > g ? a : g) + (size_t)p * ((p + 3) & ~3) * sizeof(float);
+  return a + (2 * a > g ? 2 * a : g) + (size_t)p * ((p + 3) & ~3) * sizeof(float);
 }
 
 __global__ void __launch_bounds__(CNT) k_core(const TInfo* __restrict__ tis, int tbase, double eps,
@@ -261,12 +356,10 @@ __global__ void __launch_bounds__(CNT) k_core(const TInfo* __restrict__ tis, int
   extern __shared__ __align__(16) unsigned char csm[];
   const int lda = r | 1;   // odd row length: no bank conflicts down a column
   FF* A = reinterpret_cast<FF*>(csm);
-  FF* V = A + (size_t)maxp * (maxp + 1);
-  FF* raw = V;   // the Gram is done before V begins
-  float* W = reinterpret_cast<float*>(
-      V + max((size_t)maxp * (maxp + 1), (size_t)CRAW));
-  __shared__ FF cs[CMAX / 2], sn[CMAX / 2];
-  __shared__ short pp[CMAX / 2], qq[CMAX / 2];
+  FF* A2 = A + (size_t)maxp * (maxp + 1);
+  FF* V = A2 + (size_t)maxp * (maxp + 1);
+  FF* raw = A2;   // the Gram is done before the second A and V begin
+  float* W = reinterpret_cast<float*>(A2 + max(2 * (size_t)maxp * (maxp + 1), (size_t)CRAW));
   __shared__ float red[2][CNT / 32];
   __shared__ float lam[CMAX];
   __shared__ int ord[CMAX];
@@ -361,16 +454,43 @@ __global__ void __launch_bounds__(CNT) k_core(const TInfo* __restrict__ tis, int
   // ---- cyclic Jacobi
   const int nn = (r + 1) & ~1;   // even number of players (an odd r gets a dummy)
   const int np = nn / 2, nblk = np * (np + 1) / 2;
+  // work items of a round: the blocks k1 <= k2 of A, then from a whole warp on
+  // the (pair, row) items of V; a thread's items stay its own, the first few's
+  // indices in registers (x | y << 8: k1, k2 or pair, row; -1: none)
+  const int vbase = (nblk + 31) & ~31, nitem = vbase + np * r;
+  constexpr int KEEP = 3;
+  auto item = [&](int e) {
+    if (e < vbase) {
+      if (e >= nblk) return -1;
+      int k1 = 0, k2 = e;
+      while (k2 >= np - k1) { k2 -= np - k1; ++k1; }
+      return k1 | (k1 + k2) << 8;
+    }
+    if (e >= nitem) return -1;
+    const int k = (e - vbase) / r;
+    return k | (e - vbase - k * r) << 8;
+  };
+  int kept[KEEP];
+#pragma unroll
+  for (int u = 0; u < KEEP; ++u) kept[u] = item(tid + CNT * u);
+  // circle method: player 0 fixed, the others rotate
+  auto pair_of = [&](int k, int round, int& lo, int& hi) {
+    int a = k == 0 ? 0 : k + round, b = nn - 1 - k + round;
+    if (a >= nn) a -= nn - 1;
+    if (b >= nn) b -= nn - 1;
+    lo = min(a, b);
+    hi = max(a, b);
+  };
   int sweeps = 0;
   for (int sweep = 0; sweep < 40 && r > 1; ++sweep) {
     // off-diagonal and total mass; converged at 1e-16 (eigenvectors to ~1e-8)
     float off = 0.f, tot = 0.f;
-    for (int e = tid; e < r * r; e += CNT) {
-      const int i = e / r, j = e - i * r;
-      const float v = A[i * lda + j].h;
-      if (i != j) off = fmaf(v, v, off);
-      else tot = fmaf(v, v, tot);
-    }
+    for (int i = tid >> 5; i < r; i += CNT / 32)
+      for (int j = lane; j < r; j += 32) {
+        const float v = A[i * lda + j].h;
+        if (i != j) off = fmaf(v, v, off);
+        else tot = fmaf(v, v, tot);
+      }
     off = warp_sum(off);
     tot = warp_sum(tot);
     if (lane == 0) { red[0][tid >> 5] = off; red[1][tid >> 5] = tot; }
@@ -380,59 +500,70 @@ __global__ void __launch_bounds__(CNT) k_core(const TInfo* __restrict__ tis, int
     if (off <= 1e-16f * (tot + off)) break;
     ++sweeps;
     for (int round = 0; round < nn - 1; ++round) {
-      if (tid < np) {   // circle method: player 0 fixed, the others rotate
-        int a = tid == 0 ? 0 : tid + round, b = nn - 1 - tid + round;
-        if (a >= nn) a -= nn - 1;
-        if (b >= nn) b -= nn - 1;
-        const int lo = min(a, b), hi = max(a, b);
-        FF c{1.f, 0.f}, s{0.f, 0.f};
-        if (hi < r) ff_rot(A[lo * lda + lo], A[hi * lda + hi], A[lo * lda + hi], c, s);
-        pp[tid] = (short)lo; qq[tid] = (short)hi;
-        cs[tid] = c; sn[tid] = s;
+      // lane k: the rotation of pair k
+      FF rc{1.f, 0.f}, rsn{0.f, 0.f};
+      if (lane < np) {
+        int lo, hi;
+        pair_of(lane, round, lo, hi);
+        if (hi < r) ff_rot(A[lo * lda + lo], A[hi * lda + hi], A[lo * lda + hi], rc, rsn);
       }
-      __syncthreads();
-      // A <- J^T A J: the 2 x 2 block (rows of pair k1, columns of pair k2) is
-      // rotated on its own, columns first, then rows, and mirrored; V <- V J
-      for (int e = tid; e < nblk + np * r; e += CNT) {
-        if (e < nblk) {
-          // block e of the pairs k1 <= k2, row by row
-          int k1 = 0, k2 = e;
-          while (k2 >= np - k1) { k2 -= np - k1; ++k1; }
-          k2 += k1;
-          const int a1 = pp[k1], b1 = qq[k1], a2 = pp[k2], b2 = qq[k2];
-          const bool h1 = b1 < r, h2 = b2 < r;
-          const FF c1 = cs[k1], s1 = sn[k1], c2 = cs[k2], s2 = sn[k2];
-          const FF z{0.f, 0.f};
-          const FF x00 = A[a1 * lda + a2];
-          const FF x01 = h2 ? A[a1 * lda + b2] : z;
-          const FF x10 = h1 ? A[b1 * lda + a2] : z;
-          const FF x11 = (h1 && h2) ? A[b1 * lda + b2] : z;
-          const FF y00 = ff_add(ff_mul(c2, x00), ff_neg(ff_mul(s2, x01)));
-          const FF y01 = ff_add(ff_mul(s2, x00), ff_mul(c2, x01));
-          const FF y10 = ff_add(ff_mul(c2, x10), ff_neg(ff_mul(s2, x11)));
-          const FF y11 = ff_add(ff_mul(s2, x10), ff_mul(c2, x11));
-          const FF z00 = ff_add(ff_mul(c1, y00), ff_neg(ff_mul(s1, y10)));
-          const FF z01 = ff_add(ff_mul(c1, y01), ff_neg(ff_mul(s1, y11)));
-          const FF z10 = ff_add(ff_mul(s1, y00), ff_mul(c1, y10));
-          const FF z11 = ff_add(ff_mul(s1, y01), ff_mul(c1, y11));
-          A[a1 * lda + a2] = z00;
-          if (h2) A[a1 * lda + b2] = z01;
-          if (h1 && (k1 != k2)) A[b1 * lda + a2] = z10;
-          if (h1 && h2) A[b1 * lda + b2] = z11;
-          if (k1 != k2) {
-            A[a2 * lda + a1] = z00;
-            if (h2) A[b2 * lda + a1] = z01;
-            if (h1) A[a2 * lda + b1] = z10;
-            if (h1 && h2) A[b2 * lda + b1] = z11;
-          } else if (h1) {
-            A[b1 * lda + a1] = z01;   // a diagonal block stays symmetric
-          }
+      auto rot = [&](int k, FF& c, FF& s) {
+        c.h = __shfl_sync(FULL, rc.h, k); c.l = __shfl_sync(FULL, rc.l, k);
+        s.h = __shfl_sync(FULL, rsn.h, k); s.l = __shfl_sync(FULL, rsn.l, k);
+      };
+      for (int u = 0, e0 = tid & ~31; e0 < nitem; ++u, e0 += CNT) {
+        int id = 0;
+        if (u < KEEP) {
+#pragma unroll
+          for (int x = 0; x < KEEP; ++x)
+            if (u == x) id = kept[x];
         } else {
-          const int f = e - nblk;
-          const int k = f / r, iv = f - k * r;
-          const int a = pp[k], b = qq[k];
-          if (b < r) {
-            const FF c = cs[k], s = sn[k];
+          id = item(e0 + lane);
+        }
+        const bool on = id >= 0;
+        if (e0 < vbase) {
+          // A <- J^T A J into the other copy: the 2 x 2 block (rows of pair k1,
+          // columns of pair k2) is rotated on its own, columns first, then
+          // rows, and mirrored
+          const int k1 = on ? id & 255 : 0, k2 = on ? id >> 8 : 0;
+          FF c1, s1, c2, s2;
+          rot(k1, c1, s1);
+          rot(k2, c2, s2);
+          if (on) {
+            int a1, b1, a2, b2;
+            pair_of(k1, round, a1, b1);
+            pair_of(k2, round, a2, b2);
+            const bool h1 = b1 < r, h2 = b2 < r;
+            const FF z{0.f, 0.f};
+            const FF x00 = A[a1 * lda + a2];
+            const FF x01 = h2 ? A[a1 * lda + b2] : z;
+            const FF x10 = h1 ? A[b1 * lda + a2] : z;
+            const FF x11 = (h1 && h2) ? A[b1 * lda + b2] : z;
+            const FF y00 = ff_add(ff_mul(c2, x00), ff_neg(ff_mul(s2, x01)));
+            const FF y01 = ff_add(ff_mul(s2, x00), ff_mul(c2, x01));
+            const FF y10 = ff_add(ff_mul(c2, x10), ff_neg(ff_mul(s2, x11)));
+            const FF y11 = ff_add(ff_mul(s2, x10), ff_mul(c2, x11));
+            const FF z00 = ff_add(ff_mul(c1, y00), ff_neg(ff_mul(s1, y10)));
+            const FF z01 = ff_add(ff_mul(c1, y01), ff_neg(ff_mul(s1, y11)));
+            const FF z10 = ff_add(ff_mul(s1, y00), ff_mul(c1, y10));
+            const FF z11 = ff_add(ff_mul(s1, y01), ff_mul(c1, y11));
+            const bool same = k1 == k2;   // a diagonal block stays symmetric
+            A2[a1 * lda + a2] = z00;
+            if (!same) A2[a2 * lda + a1] = z00;
+            if (h2) { A2[a1 * lda + b2] = z01; A2[b2 * lda + a1] = z01; }
+            if (h1 && !same) { A2[b1 * lda + a2] = z10; A2[a2 * lda + b1] = z10; }
+            if (h1 && h2) {
+              A2[b1 * lda + b2] = z11;
+              if (!same) A2[b2 * lda + b1] = z11;
+            }
+          }
+        } else {   // V <- V J
+          const int k = on ? id & 255 : 0, iv = on ? id >> 8 : 0;
+          FF c, s;
+          rot(k, c, s);
+          int a, b;
+          pair_of(k, round, a, b);
+          if (on && b < r) {
             const FF vx = V[iv * lda + a], vy = V[iv * lda + b];
             V[iv * lda + a] = ff_add(ff_mul(c, vx), ff_neg(ff_mul(s, vy)));
             V[iv * lda + b] = ff_add(ff_mul(s, vx), ff_mul(c, vy));
@@ -440,6 +571,9 @@ __global__ void __launch_bounds__(CNT) k_core(const TInfo* __restrict__ tis, int
         }
       }
       __syncthreads();
+      FF* t = A;
+      A = A2;
+      A2 = t;
     }
   }
   // ---- eigenvalues descending (rank by counting; ties by index), the kept rank
@@ -489,28 +623,32 @@ __global__ void __launch_bounds__(CNT) k_core(const TInfo* __restrict__ tis, int
     W[e] = w;
   }
   __syncthreads();
-  auto mul = [&](const float* X, float* Z, int rows) {   // Z = X W, rows x k
-    for (int j0 = 0; j0 < k; j0 += 4)
-      for (int i = tid; i < rows; i += CNT) {
-        float4 acc{0.f, 0.f, 0.f, 0.f};
-#pragma unroll 4
-        for (int l = 0; l < r; ++l) {
-          const float x = X[i + (int64_t)l * rows];
-          const float4 w = *reinterpret_cast<const float4*>(W + l * ldw + j0);
-          acc.x = fmaf(x, w.x, acc.x); acc.y = fmaf(x, w.y, acc.y);
-          acc.z = fmaf(x, w.z, acc.z); acc.w = fmaf(x, w.w, acc.w);
-        }
-        float* z = Z + i + (int64_t)j0 * rows;
-        z[0] = acc.x;
-        if (j0 + 1 < k) z[rows] = acc.y;
-        if (j0 + 2 < k) z[2 * (int64_t)rows] = acc.z;
-        if (j0 + 3 < k) z[3 * (int64_t)rows] = acc.w;
-      }
-  };
   float* Uo = tab[(3 * c_role + 1) * P + p];
   float* Vo = tab[(3 * c_role + 2) * P + p];
-  if (Uo) mul(scr + ti.y_off, Uo + ti.u_off, ti.m);
-  if (Vo) mul(B, Vo + ti.v_off, n);
+  const int m = ti.m;
+  for (int e = tid; e < m + n; e += CNT) {   // a row of U = Q W, then of V = B^T W
+    const bool u = e < m;
+    const int rows = u ? m : n, i = u ? e : e - m;
+    const float* X = (u ? scr + ti.y_off : B) + i;
+    float* Z = u ? Uo : Vo;
+    if (!Z) continue;
+    Z += (u ? ti.u_off : ti.v_off) + i;
+    for (int j0 = 0; j0 < k; j0 += 4) {
+      float4 acc{0.f, 0.f, 0.f, 0.f};
+#pragma unroll 8
+      for (int l = 0; l < r; ++l) {
+        const float x = X[(int64_t)l * rows];
+        const float4 w = *reinterpret_cast<const float4*>(W + l * ldw + j0);
+        acc.x = fmaf(x, w.x, acc.x); acc.y = fmaf(x, w.y, acc.y);
+        acc.z = fmaf(x, w.z, acc.z); acc.w = fmaf(x, w.w, acc.w);
+      }
+      float* z = Z + (int64_t)j0 * rows;
+      z[0] = acc.x;
+      if (j0 + 1 < k) z[rows] = acc.y;
+      if (j0 + 2 < k) z[2 * (int64_t)rows] = acc.z;
+      if (j0 + 3 < k) z[3 * (int64_t)rows] = acc.w;
+    }
+  }
 }
 
 }  // namespace
@@ -536,21 +674,19 @@ void launch_orth(const Plan& pl, double tau, float* const* d_tab, int* const* d_
     int end = nt;
     if (c < NCLS)
       for (end = beg; end < nt && bytes(end) <= cls[c]; ++end) {}
-    if (c < NCLS && end > beg && bytes(end - 1) > 48 * 1024)
-      ACR_CUDA(cudaFuncSetAttribute(k_orth<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    (int)cls[NCLS - 1]));
-    for (int t0 = beg; t0 < end; t0 += 65535) {
-      const dim3 grid(std::min(65535, end - t0), P);
-      const int* ord = (const int*)pl.d_torder + t0;
-      if (c < NCLS)
-        k_orth<true><<<grid, ONT, bytes(end - 1), st>>>(
-            (const TInfo*)pl.d_targets, ord, tau, d_tab, d_rtab, P, 3 * pl.nroles, pl.nroles,
-            (const StackDim*)pl.d_stack, d_sketch_stat, d_fl);
-      else
-        k_orth<false><<<grid, ONT, 0, st>>>(
-            (const TInfo*)pl.d_targets, ord, tau, d_tab, d_rtab, P, 3 * pl.nroles, pl.nroles,
-            (const StackDim*)pl.d_stack, d_sketch_stat, d_fl);
-      ACR_LAUNCHED(1);
+    if (end > beg) {
+      auto kern = c < NCLS ? (pl.max_p <= 32 ? k_orth<true, 4> : k_orth<true, 8>)
+                           : (pl.max_p <= 32 ? k_orth<false, 4> : k_orth<false, 8>);
+      const size_t smem = c < NCLS ? bytes(end - 1) : 0;
+      if (smem > 48 * 1024)
+        ACR_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                      (int)cls[NCLS - 1]));
+      for (int t0 = beg; t0 < end; t0 += 65535) {
+        kern<<<dim3(std::min(65535, end - t0), P), ONT, smem, st>>>(
+            (const TInfo*)pl.d_targets, (const int*)pl.d_torder + t0, tau, d_tab, d_rtab, P,
+            3 * pl.nroles, pl.nroles, (const StackDim*)pl.d_stack, d_sketch_stat, d_fl);
+        ACR_LAUNCHED(1);
+      }
     }
     beg = end;
   }
