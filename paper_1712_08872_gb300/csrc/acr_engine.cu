@@ -89,6 +89,7 @@ struct TableRing {
   char* host = nullptr;
   char* dev = nullptr;
   size_t cap = 0, off = 0;
+  int64_t epoch = 0;    // tables pushed in an earlier epoch may have been overwritten
   bool counting = false;
   bool fixed = false;   // sized by a counting pass: never wraps
   void init(size_t c) {
@@ -98,6 +99,10 @@ struct TableRing {
     ACR_CUDA(cudaMallocHost(&host, cap));
     dev = (char*)dmalloc(cap);
     off = 0;
+  }
+  void restart() {
+    off = 0;
+    ++epoch;
   }
   void release() {
     if (host) cudaFreeHost(host);
@@ -115,7 +120,7 @@ struct TableRing {
     if (off + b > cap) {
       if (fixed) throw AcrError{S_OOM, "setup pointer tables exceed their sized ring"};
       ACR_CUDA(cudaStreamSynchronize(st));   // earlier copies out of the ring are done
-      off = 0;
+      restart();
     }
     std::memcpy(host + off, data, bytes);
     ACR_CUDA(cudaMemcpyAsync(dev + off, host + off, bytes, cudaMemcpyHostToDevice, st));
@@ -365,6 +370,14 @@ class Engine : public EngineBase {
   };
   std::vector<Level> levels;
   TableRing ring;
+  struct {                           // the pointer tables of the last plan run
+    int64_t epoch = -1;
+    int nr = 0, pc = 0;
+    const void *scr = nullptr, *rscr = nullptr;
+    size_t stride = 0, rstride = 0;  // scratch bytes and rank slots per plane
+    std::vector<void*> host;
+    void** dev = nullptr;
+  } tabs;
   void* scratch = nullptr;
   size_t scratch_bytes = 0;
   int* scratch_ranks = nullptr;
@@ -694,29 +707,60 @@ class Engine : public EngineBase {
                 cudaStream_t st) {
     upload_plan(pl, st);
     const int nr = pl.nroles;
-    size_t per_plane = std::max<size_t>((size_t)pl.scratch * sizeof(T), 256);
+    const size_t per_plane =
+        (std::max<size_t>((size_t)pl.scratch * sizeof(T), 256) + 255) & ~size_t(255);
+    const size_t ranks = std::max(pl.scratch_ranks, 1);
     int Pc = (int)std::max<size_t>(1, std::min<size_t>(P, scratch_budget / per_plane));
-    ensure_scratch(per_plane * Pc, (size_t)std::max(pl.scratch_ranks, 1) * Pc, st);
+    ensure_scratch(per_plane * Pc, ranks * Pc, st);
     char* scr_base = dry ? fake_base() : (char*)scratch;
     int* scr_rank_base = dry ? (int*)fake_base() : scratch_ranks;
-    std::vector<void*> tab((3 * nr + 1) * (size_t)Pc);
-    std::vector<void*> rtab((nr + 1) * (size_t)Pc);
     for (int c0 = 0; c0 < P; c0 += Pc) {
       const int pc = std::min(Pc, P - c0);
-      for (int r = 0; r < nr; ++r)
+      // The tables of the last run serve again when the operands are the same and
+      // its planes' scratch is large enough (one H-inverse runs some 250 plans on the
+      // same two H-matrices per plane: a copy before each of them cost as much as
+      // a small plan's kernel).  New ones spread the planes over all of the scratch.
+      const bool same = tabs.epoch == ring.epoch && tabs.nr == nr && tabs.pc == pc &&
+                        tabs.scr == scr_base && tabs.rscr == scr_rank_base &&
+                        tabs.stride >= per_plane && tabs.rstride >= ranks && [&] {
+                          for (int r = 0; r < nr; ++r)
+                            for (int p = 0; p < pc; ++p) {
+                              const HM& h = roles[r][c0 + p];
+                              if (tabs.host[(3 * r) * pc + p] != h.dense ||
+                                  tabs.host[(3 * nr + 1 + r) * pc + p] != h.rank)
+                                return false;
+                            }
+                          return true;
+                        }();
+      if (!same) {
+        const size_t have = dry ? scratch_need : scratch_bytes;
+        const size_t have_r = dry ? scratch_rank_need : scratch_rank_cnt;
+        tabs.nr = nr;
+        tabs.pc = pc;
+        tabs.scr = scr_base;
+        tabs.rscr = scr_rank_base;
+        tabs.stride = std::max(per_plane, (have / pc) & ~size_t(255));
+        tabs.rstride = std::max(ranks, have_r / pc);
+        // pointers [buffer][plane], then rank pointers [buffer][plane]
+        std::vector<void*>& t = tabs.host;
+        t.resize((4 * nr + 2) * (size_t)pc);
+        for (int r = 0; r < nr; ++r)
+          for (int p = 0; p < pc; ++p) {
+            const HM& h = roles[r][c0 + p];
+            t[(3 * r + 0) * pc + p] = h.dense;
+            t[(3 * r + 1) * pc + p] = h.U;
+            t[(3 * r + 2) * pc + p] = h.V;
+            t[(3 * nr + 1 + r) * pc + p] = h.rank;
+          }
         for (int p = 0; p < pc; ++p) {
-          const HM& h = roles[r][c0 + p];
-          tab[(3 * r + 0) * pc + p] = h.dense;
-          tab[(3 * r + 1) * pc + p] = h.U;
-          tab[(3 * r + 2) * pc + p] = h.V;
-          rtab[r * pc + p] = h.rank;
+          t[(3 * nr) * pc + p] = scr_base + (size_t)p * tabs.stride;
+          t[(4 * nr + 1) * pc + p] = scr_rank_base + (size_t)p * tabs.rstride;
         }
-      for (int p = 0; p < pc; ++p) {
-        tab[(3 * nr) * pc + p] = scr_base + (size_t)p * per_plane;
-        rtab[nr * pc + p] = scr_rank_base + (size_t)p * std::max(pl.scratch_ranks, 1);
+        tabs.dev = (void**)ring.push(t.data(), sizeof(void*) * t.size(), st);
+        tabs.epoch = ring.epoch;
       }
-      T* const* d_tab = (T* const*)ring.push(tab.data(), sizeof(void*) * (3 * nr + 1) * pc, st);
-      int* const* d_rtab = (int* const*)ring.push(rtab.data(), sizeof(void*) * (nr + 1) * pc, st);
+      T* const* d_tab = (T* const*)tabs.dev;
+      int* const* d_rtab = (int* const*)(tabs.dev + (size_t)(3 * nr + 1) * pc);
       for (const Stage& sg : pl.stages) {
         if (sg.kind == ST_GEMM) {
           timed(0, [&] { gemm_stage(pl, sg, d_tab, (const int* const*)d_rtab, pc, st); }, sg.tag);
@@ -972,7 +1016,7 @@ void Engine<T>::prepare(const double* const* coefs, cudaStream_t st, bool count_
     // H-matrix slots, the setup scratch and the table ring exactly
     dry = true;
     ring.counting = true;
-    ring.off = 0;
+    ring.restart();
     scratch_need = scratch_rank_need = 0;
     execute(st);
     dry = false;
@@ -1000,7 +1044,7 @@ template <typename T>
 void Engine<T>::execute(cudaStream_t st) {
   cur_st = st;
   pool.restart();
-  ring.off = 0;
+  ring.restart();
   D.assign((size_t)count * n, HM());
   levels.clear();
   if (!dry) {
