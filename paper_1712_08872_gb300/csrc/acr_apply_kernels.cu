@@ -19,6 +19,7 @@
 
 #include <type_traits>
 
+#include "acr_device.h"
 #include "acr_internal.h"
 
 namespace acr {
@@ -70,6 +71,7 @@ __global__ void __launch_bounds__(256) k_lr_proj(MatvecDev mv, T* const* __restr
                                                  const int* const* __restrict__ rank,
                                                  const double* const* __restrict__ x, double* tv,
                                                  bool trans, int64_t vs) {
+  chain_begin();
   using Acc = AccT<T>;
   __shared__ Acc xs[R][64];
   __shared__ int64_t s_off[MAXQ];
@@ -170,6 +172,7 @@ __global__ void __launch_bounds__(256) k_hmv_rows(MatvecDev mv, T* const* __rest
                                                   double* const* __restrict__ y, double alpha,
                                                   double beta, const double* __restrict__ tv,
                                                   bool trans, int64_t vs) {
+  chain_begin();
   using Acc = AccT<T>;
   extern __shared__ __align__(16) unsigned char smraw[];
   Acc* xs = reinterpret_cast<Acc*>(smraw);
@@ -332,6 +335,7 @@ __global__ void __launch_bounds__(256) k_hmv_rows_v1(MatvecDev mv, T* const* __r
                                                      double* const* __restrict__ y, double alpha,
                                                      double beta, const double* __restrict__ tv,
                                                      bool trans, int64_t vs) {
+  chain_begin();
   extern __shared__ __align__(16) unsigned char smraw[];
   float* xs = reinterpret_cast<float*>(smraw);
   __shared__ double part[9][64];
@@ -470,6 +474,7 @@ __global__ void __launch_bounds__(256) k_hmv_rows_v1(MatvecDev mv, T* const* __r
 
 __global__ void k_permute(const double* __restrict__ in, double* __restrict__ out,
                           const int* __restrict__ perm, int n2, int64_t total, bool to_cluster) {
+  chain_begin();
   for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < total;
        e += (int64_t)gridDim.x * blockDim.x) {
     const int64_t k = e / n2;
@@ -484,6 +489,7 @@ __global__ void k_diag_update(double* const* __restrict__ y, const double* const
                               const double* const* __restrict__ b,
                               const double* const* __restrict__ z, int n2, double sgn,
                               int64_t vs) {
+  chain_begin();
   const int p = blockIdx.y;
   const int64_t o = blockIdx.z * vs;   // right-hand side blockIdx.z
   double* yp = y[p];
@@ -502,6 +508,7 @@ __global__ void k_diag_update(double* const* __restrict__ y, const double* const
 
 __global__ void k_copy_planes(double* const* __restrict__ dst, const double* const* __restrict__ src,
                               int n2, int64_t vs) {
+  chain_begin();
   const int p = blockIdx.y;
   const int64_t o = blockIdx.z * vs;   // right-hand side blockIdx.z
   double* d = dst[p];
@@ -531,6 +538,7 @@ __global__ void __launch_bounds__(256) k_lr_proj32(MatvecDev mv, T* const* __res
                                                    const int* const* __restrict__ rank,
                                                    const double* const* __restrict__ x,
                                                    double* tv, bool trans, int64_t vs) {
+  chain_begin();
   constexpr int R = 32;
   __shared__ float xs[64][R + 1];
   __shared__ int64_t s_off[MAXQ];
@@ -614,7 +622,7 @@ static void hmatvec_r(const MatvecDev& mv, T* const* dense, T* const* U, T* cons
   if (sm_rows > 180 * 1024)
     throw CudaError{cudaErrorInvalidConfiguration, "apply staging exceeds shared memory"};
   if (mv.nl > 0)
-    k_lr_proj<T, R><<<dim3(mv.nchunks, P), 256, 0, st>>>(mv, U, V, rank, x, tv, trans, vs);
+    launch_chain(k_lr_proj<T, R>, dim3(mv.nchunks, P), 256, 0, st, mv, U, V, rank, x, tv, trans, vs);
   bool done = false;
   if constexpr (R == 1 && !std::is_same<T, double>::value) {
     if (mv.lsz == 64 && mv.kc % 4 == 0) {
@@ -625,17 +633,17 @@ static void hmatvec_r(const MatvecDev& mv, T* const* dense, T* const* U, T* cons
         attr_v1 = true;
       }
       const size_t sm1 = ((size_t)mv.max_d * 64 + (size_t)mv.max_l * mv.kc) * sizeof(float);
-      k_hmv_rows_v1<T><<<dim3(mv.nchunks, P), 256, sm1, st>>>(mv, dense, U, V, rank, x, y, alpha,
+      launch_chain(k_hmv_rows_v1<T>, dim3(mv.nchunks, P), 256, sm1, st, mv, dense, U, V, rank, x, y, alpha,
                                                              beta, tv, trans, vs);
       done = true;
     }
   }
   if (done) {
   } else if (mv.lsz == 64)
-    k_hmv_rows<T, 64, R><<<dim3(mv.nchunks, P), 256, sm_rows, st>>>(
+    launch_chain(k_hmv_rows<T, 64, R>, dim3(mv.nchunks, P), 256, sm_rows, st, 
         mv, dense, U, V, rank, x, y, alpha, beta, tv, trans, vs);
   else
-    k_hmv_rows<T, 0, R><<<dim3(mv.nchunks, P), 256, sm_rows, st>>>(
+    launch_chain(k_hmv_rows<T, 0, R>, dim3(mv.nchunks, P), 256, sm_rows, st, 
         mv, dense, U, V, rank, x, y, alpha, beta, tv, trans, vs);
   ACR_LAUNCHED(mv.nl > 0 ? 2 : 1);
 }
@@ -661,7 +669,7 @@ void launch_lr_proj(const MatvecDev& mv, T* const* U, T* const* V, const int* co
                     cudaStream_t st) {
   if (P <= 0 || mv.nl <= 0) return;
   if (nr != 32) throw CudaError{cudaErrorInvalidValue, "projection group of 32 expected"};
-  k_lr_proj32<T><<<dim3(mv.nchunks, P), 256, 0, st>>>(mv, U, V, rank, x, tv, trans, vs);
+  launch_chain(k_lr_proj32<T>, dim3(mv.nchunks, P), 256, 0, st, mv, U, V, rank, x, tv, trans, vs);
   ACR_LAUNCHED(1);
 }
 
@@ -677,7 +685,7 @@ void launch_permute(const double* in, double* out, const int* perm, int n2, int 
                     bool to_cluster, cudaStream_t st) {
   int64_t total = (int64_t)n2 * nplanes;
   int blocks = (int)std::min<int64_t>((total + 255) / 256, (int64_t)device_sm_count() * 16);
-  k_permute<<<blocks, 256, 0, st>>>(in, out, perm, n2, total, to_cluster);
+  launch_chain(k_permute, blocks, 256, 0, st, in, out, perm, n2, total, to_cluster);
   ACR_LAUNCHED(1);
 }
 
@@ -686,7 +694,7 @@ void launch_diag_update(double* const* y, const double* const* a, const double* 
                         double sgn, int nr, int64_t vs, cudaStream_t st) {
   if (P <= 0) return;
   dim3 grid((n2 + 255) / 256 < 64 ? (n2 + 255) / 256 : 64, P, nr);
-  k_diag_update<<<grid, 256, 0, st>>>(y, a, x, b, z, n2, sgn, vs);
+  launch_chain(k_diag_update, grid, 256, 0, st, y, a, x, b, z, n2, sgn, vs);
   ACR_LAUNCHED(1);
 }
 
@@ -694,7 +702,7 @@ void launch_copy_planes(double* const* dst, const double* const* src, int n2, in
                         int64_t vs, cudaStream_t st) {
   if (P <= 0) return;
   dim3 grid((n2 + 255) / 256 < 64 ? (n2 + 255) / 256 : 64, P, nr);
-  k_copy_planes<<<grid, 256, 0, st>>>(dst, src, n2, vs);
+  launch_chain(k_copy_planes, grid, 256, 0, st, dst, src, n2, vs);
   ACR_LAUNCHED(1);
 }
 

@@ -13,6 +13,14 @@ namespace acr {
 
 constexpr int NT = 256;   // threads per CTA of the setup kernels
 
+// First statement of a kernel launched by launch_chain: every thread waits for the
+// kernels before it (whose results may be anything the kernel reads), then the next
+// launch of the chain may be set up.
+__device__ __forceinline__ void chain_begin() {
+  cudaGridDependencySynchronize();
+  cudaTriggerProgrammaticLaunchCompletion();
+}
+
 __device__ __forceinline__ int dimv(int st, int rb, int ri, const int* const* rtab, int P, int p) {
   if (rb < 0) return st;
   const int* r = rtab[rb * P + p];
