@@ -63,8 +63,8 @@ typedef enum {
  * inverses and the small recompression cores are FP64 in the FP64 form; in
  * the float forms the leaf inverses are float eliminations refined to float
  * accuracy (FP64 elimination when refinement cannot get there), the sketch bases come
- * from a re-orthogonalised float Gram-Schmidt, and the core Grams and Jacobi
- * cores run in float-float.
+ * from a re-orthogonalised float Gram-Schmidt, and the core Grams and the cores'
+ * eigenvectors are float-float.
  * (Reduced-precision storage is not in the paper, whose H-arithmetic is
  * double precision throughout, Sec. 5.) */
 typedef enum { ACR_FP64 = 0, ACR_FP32 = 1, ACR_BF16 = 2 } acr_precision;
@@ -135,16 +135,15 @@ typedef struct {
 typedef struct {
   acr_kernel_stat gemm;      /* grouped small GEMMs (k_ggemm) */
   acr_kernel_stat orth;      /* FP64 pivoted-Cholesky cores (k_pchol); float factors: basis kernel (k_orth) */
-  acr_kernel_stat eig;       /* FP64 Jacobi cores (k_eig); float factors: Gram, float-float Jacobi and
-                                recomposition (k_core) */
+  acr_kernel_stat eig;       /* core Grams, Jacobi cores and recomposition (k_core) */
   acr_kernel_stat leaf_inv;  /* dense leaf inverses (k_leaf_inv; refined float for float factors) */
   acr_kernel_stat other;     /* conversion, scaling */
   /* grouped-GEMM time and counted flops per plan stage: 0 inner products
    * U^T V of phase 1, 1 term factors (H-matrix x block products, dense
    * products), 2 dense-leaf sums, 3 sketches Z^T Omega, 4 sketch Y, 5 first
    * Gram, 6 first basis, 7 second Gram, 8 second basis, 9 X^T Q, 10 B^T,
-   * 11 core Gram, 12 recomposition U = Q W, V = B^T W (5 to 8 and 11, 12 for
-   * FP64 factors; the float forms' are inside orth and eig); 13..15 unused */
+   * 11 core Gram, 12 recomposition U = Q W, V = B^T W (5 to 8 for FP64
+   * factors, inside orth for float ones; 11 and 12 are inside eig); 13..15 unused */
   double stage_ms[16];
   double stage_flops[16];
   /* wall time (CUDA events) of each CR level's H-inversion batch and of its

@@ -1,14 +1,15 @@
-// Recompression cores of float targets (sm_103a), one CTA per low-rank target:
-//  * k_orth -- orthonormal basis of the sketch Y: pivoted Gram-Schmidt with
-//              re-orthogonalisation, truncated at tau;
-//  * k_core -- core Gram (B^T)^T B^T, its Jacobi eigen-decomposition, the rank
+// Recompression cores (sm_103a), one CTA per low-rank target:
+//  * k_orth -- float factors: orthonormal basis of the sketch Y by pivoted
+//              Gram-Schmidt with re-orthogonalisation, truncated at tau (FP64
+//              factors take the plan's Gram, k_pchol and basis stages);
+//  * k_core -- core Gram (B^T)^T B^T, its eigen-decomposition by Jacobi, the rank
 //              rule sigma_i > eps * sigma_1 (Sec. 4.3 H_eps), and the
 //              recomposed factors U = Q W_k, V = B^T W_k.
-// (FP64 factors go through the Gram, k_pchol and k_eig stages of the plan.)
 #include <cuda_runtime.h>
 
 #include <algorithm>
 #include <cstdint>
+#include <type_traits>
 
 #include "acr_device.h"
 #include "acr_internal.h"
@@ -256,9 +257,9 @@ __global__ void __launch_bounds__(ONT, 6) k_orth(const TInfo* __restrict__ tis,
   }
 }
 
-// ------------------------------------------------------------ float-float
+// ------------------------------------------------------------ Jacobi cores
 // Numbers held as an unevaluated sum hi + lo of two floats (~48 significant
-// bits): the core Gram and its Jacobi rotations run on the FP32 pipe instead of
+// bits): the float forms' core Gram and rotations run on the FP32 pipe instead of
 // this part's narrow FP64 pipe.
 struct FF {
   float h, l;
@@ -281,182 +282,88 @@ __device__ __forceinline__ FF ff_add(FF a, FF b) {
   return FF{r, e - (r - s)};
 }
 __device__ __forceinline__ FF ff_neg(FF a) { return FF{-a.h, -a.l}; }
-// (1 + t^2)^(-1/2) to float-float accuracy: one Newton step y + y (1 - x y^2) / 2
-// from the float estimate
-__device__ __forceinline__ FF ff_rsqrt1p(float t) {
+
+// The three element types of a core: float (first sweeps), FF and double.
+__device__ __forceinline__ float em(float a, float b) { return a * b; }
+__device__ __forceinline__ double em(double a, double b) { return a * b; }
+__device__ __forceinline__ FF em(FF a, FF b) { return ff_mul(a, b); }
+__device__ __forceinline__ float ea(float a, float b) { return a + b; }
+__device__ __forceinline__ double ea(double a, double b) { return a + b; }
+__device__ __forceinline__ FF ea(FF a, FF b) { return ff_add(a, b); }
+__device__ __forceinline__ float en(float a) { return -a; }
+__device__ __forceinline__ double en(double a) { return -a; }
+__device__ __forceinline__ FF en(FF a) { return ff_neg(a); }
+__device__ __forceinline__ float ef(float a) { return a; }              // to float
+__device__ __forceinline__ float ef(double a) { return (float)a; }
+__device__ __forceinline__ float ef(FF a) { return a.h; }
+__device__ __forceinline__ double ed(double a) { return a; }            // to double
+__device__ __forceinline__ double ed(FF a) { return (double)a.h + (double)a.l; }
+__device__ __forceinline__ void es(float& a, float x) { a = x; }        // from float
+__device__ __forceinline__ void es(double& a, float x) { a = x; }
+__device__ __forceinline__ void es(FF& a, float x) { a = FF{x, 0.f}; }
+__device__ __forceinline__ float eshfl(float a, int k) { return __shfl_sync(FULL, a, k); }
+__device__ __forceinline__ double eshfl(double a, int k) { return __shfl_sync(FULL, a, k); }
+__device__ __forceinline__ FF eshfl(FF a, int k) {
+  return FF{__shfl_sync(FULL, a.h, k), __shfl_sync(FULL, a.l, k)};
+}
+__device__ __forceinline__ double escale(double a, int e) { return ldexp(a, e); }
+__device__ __forceinline__ FF escale(FF a, int e) { return FF{ldexpf(a.h, e), ldexpf(a.l, e)}; }
+
+// (1 + t^2)^(-1/2): Newton steps y + y (1 - x y^2) / 2 from the float estimate
+__device__ __forceinline__ void cos_of(float t, float& c) { c = rsqrtf(fmaf(t, t, 1.f)); }
+__device__ __forceinline__ void cos_of(float t, FF& c) {
   const float p = t * t;
   const FF x = ff_add(FF{1.f, 0.f}, FF{p, fmaf(t, t, -p)});
   const float y = rsqrtf(x.h);
   const FF xy2 = ff_mul(x, ff_mul(FF{y, 0.f}, FF{y, 0.f}));
   const FF e = ff_add(FF{1.f, 0.f}, ff_neg(xy2));
-  return ff_add(FF{y, 0.f}, ff_mul(FF{y, 0.f}, FF{0.5f * e.h, 0.5f * e.l}));
+  c = ff_add(FF{y, 0.f}, ff_mul(FF{y, 0.f}, FF{0.5f * e.h, 0.5f * e.l}));
+}
+__device__ __forceinline__ void cos_of(float t, double& c) {
+  const double x = fma((double)t, (double)t, 1.0);
+  double y = (double)rsqrtf((float)x);
+  y = fma(0.5 * y, fma(-x * y, y, 1.0), y);
+  c = fma(0.5 * y, fma(-x * y, y, 1.0), y);
 }
 // The rotation (c, s) that zeroes a_pq of [a_pp a_pq; a_pq a_qq]: the angle in
 // float with the fast divide (an angle off by ~1e-6 leaves ~1e-6 of the entry, which
-// later rotations remove), its cosine and sine to float-float accuracy from that angle, so the
-// rotation itself is orthogonal to ~1e-14.
-__device__ __forceinline__ void ff_rot(FF app, FF aqq, FF apq, FF& c, FF& s) {
-  c = FF{1.f, 0.f};
-  s = FF{0.f, 0.f};
-  if (apq.h != 0.f) {
-    const float tau =
-        fminf(fmaxf(__fdividef(aqq.h - app.h, 2.f * apq.h), -1e15f), 1e15f);
-    const float h = fmaf(tau, tau, 1.f);
-    const float t = copysignf(__fdividef(1.f, fabsf(tau) + h * rsqrtf(h)), tau);
-    c = ff_rsqrt1p(t);
-    s = ff_mul(FF{t, 0.f}, c);
+// later rotations remove), its cosine and sine to the element type's accuracy from that angle, so the
+// rotation itself is orthogonal to rounding.
+template <typename EL>
+__device__ __forceinline__ void jrot(EL app, EL aqq, EL apq, EL& c, EL& s) {
+  es(c, 1.f);
+  es(s, 0.f);
+  const float q = ef(apq);
+  if (q != 0.f) {
+    const float d = ef(ea(aqq, en(app)));
+    const float tau = __fdividef(d, 2.f * q), at = fabsf(tau), h = fmaf(tau, tau, 1.f);
+    // (beyond 1e9 the square root is tau itself; an infinite tau gives the angle 0)
+    const float t = copysignf(__fdividef(1.f, at + (at > 1e9f ? at : h * rsqrtf(h))), tau);
+    cos_of(t, c);
+    EL te;
+    es(te, t);
+    s = em(te, c);
   }
 }
 
-// The core H = (B^T)^T B^T of a target (r x r, r the basis size): exact
-// products and compensated float-float sums, since the rank rule resolves
-// singular values only down to the square root of the Gram's relative error;
-// scaled by a power of two to a largest diagonal in [1/2, 1), so that blocks whose
-// squares would leave the float range keep the full float-float accuracy (an
-// exact scaling: the eigenvectors and the ratios sigma_i / sigma_1 are
-// unchanged); cyclic Jacobi in round-robin order, the symmetric half of each
-// round's 2 x 2 blocks rotated by one thread each (the mirror entry written
-// alongside) together with V; then the kept columns W of V, largest eigenvalue first, and
-// the factors U = Q W, V = B^T W straight into the target's leaf.
-//
-// Bound by the latency of the ~6 (r - 1) dependent rounds of a core, each a
-// rotation angle and a handful of float-float operations per thread.  Four warps,
-// so that a typical core's round (r = 12: 21 blocks and 72 row pairs of V) is one
-// pass over the threads; every warp computes all rotations in its lanes and
-// hands them round by shuffles, and a round writes the other copy of A, so
-// that it has one barrier.  n = 64 setup: the four stages 90 ms, here 31 ms (36 ms with
-// rotations through shared memory and A updated in place).
 constexpr int CNT = 128;
-constexpr int CRAW = CNT * 16;   // float-float partial sums of the Gram's tiles
 
-__host__ __device__ constexpr size_t core_smem(int p) {
-  // A; the Gram's staging, then the other A and V in its place (p x (p + 1)
-  // float-float each); W
-  const size_t a = (size_t)p * (p + 1) * sizeof(FF), g = CRAW * sizeof(FF);
-  return a + (2 * a > g ? 2 * a : g) + (size_t)p * ((p + 3) & ~3) * sizeof(float);
-}
-
-__global__ void __launch_bounds__(CNT) k_core(const TInfo* __restrict__ tis, int tbase, double eps,
-                                              int kc, int c_role, int maxp,
-                                              float* const* __restrict__ tab,
-                                              int* const* __restrict__ rtab, int P, int scr_buf,
-                                              int scr_rbuf, int* err, double* __restrict__ flops) {
-  const int p = blockIdx.y;
-  const TInfo ti = tis[tbase + blockIdx.x];
-  float* scr = tab[scr_buf * P + p];
-  int* rs = rtab[scr_rbuf * P + p];
-  int* crank = rtab[c_role * P + p];
-  if (!scr || !rs || !crank) return;
+// Cyclic Jacobi of the symmetric r x r matrix A in round-robin order, rotations
+// accumulated into V, until the off-diagonal mass is at most conv of the total.
+// Every warp computes all rotations of a round in its lanes and hands them
+// round by shuffles; a thread rotates 2 x 2 blocks (rows of pair k1, columns of
+// pair k2, k1 <= k2, the mirror entry written alongside) into the other copy A2 and
+// row pairs of V in place: one barrier per round.  A and A2 trade places with
+// every round.  Returns the sweeps done.
+template <typename EL>
+__device__ int jacobi(EL*& A, EL*& A2, EL* V, int r, int lda, float conv, int most,
+                      float (*red)[CNT / 32]) {
   const int tid = threadIdx.x, lane = tid & 31;
-  const int r = rs[ti.r_ri];
-  if (r <= 0) {   // an empty basis: rank 0
-    if (tid == 0) crank[ti.c_leaf] = 0;
-    return;
-  }
-  extern __shared__ __align__(16) unsigned char csm[];
-  const int lda = r | 1;   // odd row length: no bank conflicts down a column
-  FF* A = reinterpret_cast<FF*>(csm);
-  FF* A2 = A + (size_t)maxp * (maxp + 1);
-  FF* V = A2 + (size_t)maxp * (maxp + 1);
-  FF* raw = A2;   // the Gram is done before the second A and V begin
-  float* W = reinterpret_cast<float*>(A2 + max(2 * (size_t)maxp * (maxp + 1), (size_t)CRAW));
-  __shared__ float red[2][CNT / 32];
-  __shared__ float lam[CMAX];
-  __shared__ int ord[CMAX];
-  __shared__ int kkeep;
-
-  // ---- Gram of B^T (n x r): thread (tile, slice) owns a 4 x 4 tile of the
-  // upper triangle and every S-th row
-  const float* B = scr + ti.bt_off;
-  const int n = ti.n;
-  {
-    const int TM = (r + 3) >> 2, ntile = TM * (TM + 1) / 2, mt = 4 * TM;
-    // (CRAW float-float entries staged as 2 CRAW floats; at least 31 rows)
-    const int kch = min(256, ((2 * CRAW / mt) - 1) & ~1), ysld = kch + 1;
-    float* ys = reinterpret_cast<float*>(raw);
-    for (int tb = 0; tb < ntile; tb += CNT) {   // (one pass up to r = 60)
-      const int nt = min(CNT, ntile - tb);
-      const int S = CNT / nt;
-      const int tl = tid / S, slice = tid - tl * S;
-      const bool active = tl < nt;
-      int a0 = 0, t = tb + (active ? tl : 0);
-      while (t >= TM - a0) { t -= TM - a0; ++a0; }
-      const int i0 = 4 * a0, j0 = 4 * (a0 + t);
-      float s[4][4], c[4][4];
-#pragma unroll
-      for (int x = 0; x < 4; ++x)
-#pragma unroll
-        for (int y = 0; y < 4; ++y) { s[x][y] = 0.f; c[x][y] = 0.f; }
-      for (int l0 = 0; l0 < n; l0 += kch) {
-        const int kk = min(kch, n - l0);
-        __syncthreads();
-        for (int col = tid >> 5; col < mt; col += CNT / 32)
-          for (int l = lane; l < kk; l += 32)
-            ys[col * ysld + l] = col < r ? B[(l0 + l) + (int64_t)col * n] : 0.f;
-        __syncthreads();
-        if (active)
-          for (int l = slice; l < kk; l += S) {
-            float av[4], bv[4];
-#pragma unroll
-            for (int x = 0; x < 4; ++x) {
-              av[x] = ys[(i0 + x) * ysld + l];
-              bv[x] = ys[(j0 + x) * ysld + l];
-            }
-#pragma unroll
-            for (int x = 0; x < 4; ++x)
-#pragma unroll
-              for (int y = 0; y < 4; ++y) ff_fma(s[x][y], c[x][y], av[x], bv[y]);
-          }
-      }
-      __syncthreads();
-#pragma unroll
-      for (int e = 0; e < 16; ++e)
-        raw[e * CNT + tid] = active ? FF{s[e & 3][e >> 2], c[e & 3][e >> 2]} : FF{0.f, 0.f};
-      __syncthreads();
-      // the slices' partial sums in float-float, in a fixed order
-      for (int e = tid; e < nt * 16; e += CNT) {
-        const int tq = e >> 4, q = e & 15;
-        FF h{0.f, 0.f};
-        for (int sl = 0; sl < S; ++sl) {
-          const FF x = raw[q * CNT + tq * S + sl];
-          const float u = h.h + x.h, bp = u - h.h;
-          h.l += ((h.h - (u - bp)) + (x.h - bp)) + x.l;
-          h.h = u;
-        }
-        const float u = h.h + h.l;
-        h.l = h.l - (u - h.h);
-        h.h = u;
-        int tt = tb + tq, a = 0;
-        while (tt >= TM - a) { tt -= TM - a; ++a; }
-        const int i = 4 * a + (q & 3), j = 4 * (a + tt) + (q >> 2);
-        if (i < r && j < r) {
-          A[i * lda + j] = h;
-          A[j * lda + i] = h;
-        }
-      }
-    }
-  }
-  __syncthreads();
-  // ---- power-of-two scale: the largest diagonal to [1/2, 1)
-  float dmax = 0.f;
-  for (int i = 0; i < r; ++i) dmax = fmaxf(dmax, A[i * lda + i].h);
-  int ex = 0;
-  if (dmax > 0.f && dmax <= 3.0e38f) frexpf(dmax, &ex);
-  __syncthreads();
-  for (int e = tid; e < r * lda; e += CNT) {
-    const int i = e / lda, j = e - i * lda;
-    A[e].h = ldexpf(A[e].h, -ex);
-    A[e].l = ldexpf(A[e].l, -ex);
-    V[e] = FF{i == j ? 1.f : 0.f, 0.f};
-  }
-  __syncthreads();
-
-  // ---- cyclic Jacobi
   const int nn = (r + 1) & ~1;   // even number of players (an odd r gets a dummy)
   const int np = nn / 2, nblk = np * (np + 1) / 2;
-  // work items of a round: the blocks k1 <= k2 of A, then from a whole warp on
-  // the (pair, row) items of V; a thread's items stay its own, the first few's
-  // indices in registers (x | y << 8: k1, k2 or pair, row; -1: none)
+  // work items of a round: the blocks of A, then from a whole warp on the (pair,
+  // row) items of V; a thread's items stay its own, the first few's indices
+  // in registers (x | y << 8: k1, k2 or pair, row; -1: none)
   const int vbase = (nblk + 31) & ~31, nitem = vbase + np * r;
   constexpr int KEEP = 3;
   auto item = [&](int e) {
@@ -482,12 +389,12 @@ __global__ void __launch_bounds__(CNT) k_core(const TInfo* __restrict__ tis, int
     hi = max(a, b);
   };
   int sweeps = 0;
-  for (int sweep = 0; sweep < 40 && r > 1; ++sweep) {
-    // off-diagonal and total mass; converged at 1e-16 (eigenvectors to ~1e-8)
+  for (int sweep = 0; sweep < most && r > 1; ++sweep) {
+    // off-diagonal and total mass
     float off = 0.f, tot = 0.f;
     for (int i = tid >> 5; i < r; i += CNT / 32)
       for (int j = lane; j < r; j += 32) {
-        const float v = A[i * lda + j].h;
+        const float v = ef(A[i * lda + j]);
         if (i != j) off = fmaf(v, v, off);
         else tot = fmaf(v, v, tot);
       }
@@ -497,20 +404,18 @@ __global__ void __launch_bounds__(CNT) k_core(const TInfo* __restrict__ tis, int
     __syncthreads();
     off = (red[0][0] + red[0][1]) + (red[0][2] + red[0][3]);
     tot = (red[1][0] + red[1][1]) + (red[1][2] + red[1][3]);
-    if (off <= 1e-16f * (tot + off)) break;
+    if (off <= conv * (tot + off)) break;
     ++sweeps;
     for (int round = 0; round < nn - 1; ++round) {
       // lane k: the rotation of pair k
-      FF rc{1.f, 0.f}, rsn{0.f, 0.f};
+      EL rc, rsn;
+      es(rc, 1.f);
+      es(rsn, 0.f);
       if (lane < np) {
         int lo, hi;
         pair_of(lane, round, lo, hi);
-        if (hi < r) ff_rot(A[lo * lda + lo], A[hi * lda + hi], A[lo * lda + hi], rc, rsn);
+        if (hi < r) jrot(A[lo * lda + lo], A[hi * lda + hi], A[lo * lda + hi], rc, rsn);
       }
-      auto rot = [&](int k, FF& c, FF& s) {
-        c.h = __shfl_sync(FULL, rc.h, k); c.l = __shfl_sync(FULL, rc.l, k);
-        s.h = __shfl_sync(FULL, rsn.h, k); s.l = __shfl_sync(FULL, rsn.l, k);
-      };
       for (int u = 0, e0 = tid & ~31; e0 < nitem; ++u, e0 += CNT) {
         int id = 0;
         if (u < KEEP) {
@@ -521,32 +426,24 @@ __global__ void __launch_bounds__(CNT) k_core(const TInfo* __restrict__ tis, int
           id = item(e0 + lane);
         }
         const bool on = id >= 0;
-        if (e0 < vbase) {
-          // A <- J^T A J into the other copy: the 2 x 2 block (rows of pair k1,
-          // columns of pair k2) is rotated on its own, columns first, then
-          // rows, and mirrored
+        if (e0 < vbase) {   // a block: columns first, then rows
           const int k1 = on ? id & 255 : 0, k2 = on ? id >> 8 : 0;
-          FF c1, s1, c2, s2;
-          rot(k1, c1, s1);
-          rot(k2, c2, s2);
+          const EL c1 = eshfl(rc, k1), s1 = eshfl(rsn, k1), c2 = eshfl(rc, k2), s2 = eshfl(rsn, k2);
           if (on) {
             int a1, b1, a2, b2;
             pair_of(k1, round, a1, b1);
             pair_of(k2, round, a2, b2);
             const bool h1 = b1 < r, h2 = b2 < r;
-            const FF z{0.f, 0.f};
-            const FF x00 = A[a1 * lda + a2];
-            const FF x01 = h2 ? A[a1 * lda + b2] : z;
-            const FF x10 = h1 ? A[b1 * lda + a2] : z;
-            const FF x11 = (h1 && h2) ? A[b1 * lda + b2] : z;
-            const FF y00 = ff_add(ff_mul(c2, x00), ff_neg(ff_mul(s2, x01)));
-            const FF y01 = ff_add(ff_mul(s2, x00), ff_mul(c2, x01));
-            const FF y10 = ff_add(ff_mul(c2, x10), ff_neg(ff_mul(s2, x11)));
-            const FF y11 = ff_add(ff_mul(s2, x10), ff_mul(c2, x11));
-            const FF z00 = ff_add(ff_mul(c1, y00), ff_neg(ff_mul(s1, y10)));
-            const FF z01 = ff_add(ff_mul(c1, y01), ff_neg(ff_mul(s1, y11)));
-            const FF z10 = ff_add(ff_mul(s1, y00), ff_mul(c1, y10));
-            const FF z11 = ff_add(ff_mul(s1, y01), ff_mul(c1, y11));
+            EL z;
+            es(z, 0.f);
+            const EL x00 = A[a1 * lda + a2];
+            const EL x01 = h2 ? A[a1 * lda + b2] : z;
+            const EL x10 = h1 ? A[b1 * lda + a2] : z;
+            const EL x11 = (h1 && h2) ? A[b1 * lda + b2] : z;
+            const EL y00 = ea(em(c2, x00), en(em(s2, x01))), y01 = ea(em(s2, x00), em(c2, x01));
+            const EL y10 = ea(em(c2, x10), en(em(s2, x11))), y11 = ea(em(s2, x10), em(c2, x11));
+            const EL z00 = ea(em(c1, y00), en(em(s1, y10))), z01 = ea(em(c1, y01), en(em(s1, y11)));
+            const EL z10 = ea(em(s1, y00), em(c1, y10)), z11 = ea(em(s1, y01), em(c1, y11));
             const bool same = k1 == k2;   // a diagonal block stays symmetric
             A2[a1 * lda + a2] = z00;
             if (!same) A2[a2 * lda + a1] = z00;
@@ -559,45 +456,289 @@ __global__ void __launch_bounds__(CNT) k_core(const TInfo* __restrict__ tis, int
           }
         } else {   // V <- V J
           const int k = on ? id & 255 : 0, iv = on ? id >> 8 : 0;
-          FF c, s;
-          rot(k, c, s);
+          const EL c = eshfl(rc, k), s = eshfl(rsn, k);
           int a, b;
           pair_of(k, round, a, b);
           if (on && b < r) {
-            const FF vx = V[iv * lda + a], vy = V[iv * lda + b];
-            V[iv * lda + a] = ff_add(ff_mul(c, vx), ff_neg(ff_mul(s, vy)));
-            V[iv * lda + b] = ff_add(ff_mul(s, vx), ff_mul(c, vy));
+            const EL vx = V[iv * lda + a], vy = V[iv * lda + b];
+            V[iv * lda + a] = ea(em(c, vx), en(em(s, vy)));
+            V[iv * lda + b] = ea(em(s, vx), em(c, vy));
           }
         }
       }
       __syncthreads();
-      FF* t = A;
+      EL* t = A;
       A = A2;
       A2 = t;
     }
   }
+  return sweeps;
+}
+
+// The core of a target (r x r, r the basis size): H = (B^T)^T B^T with
+// FP64-accurate sums (float factors: exact products, compensated float-float sums; the
+// rank rule resolves singular values only down to the square root of the
+// Gram's relative error), scaled by a power of two to a largest diagonal in
+// [1/2, 1), so that blocks whose squares would leave the float range keep the
+// full accuracy (an exact scaling: eigenvectors and ratios sigma_i / sigma_1 are
+// unchanged); its eigenvectors; the kept ones W, largest eigenvalue first, and the
+// factors U = Q W, V = B^T W straight into the target's leaf.
+//
+// The eigenvectors: Jacobi sweeps in plain float to an off-diagonal 1e-5 of
+// the norm; the float rotations' product made orthonormal (Newton-Schulz, V =
+// W + W (I - W^T W) / 2: exact W^T W, the correction small enough for float; twice
+// for FP64); H transformed by it in the core's full arithmetic; then sweeps in
+// that arithmetic -- float-float to an off-diagonal mass of 1e-16, FP64 to 1e-30 --
+// which find a nearly diagonal matrix and need one (FP64: two) instead of six
+// to eight.  The result has the accuracy of sweeps in full arithmetic
+// throughout, at a twelfth of the operations per float sweep (FP64: a 64th).
+//
+// Bound by the latency of the ~6 (r - 1) dependent rounds of a core.  Four warps, so that a
+// typical core's round (r = 12: 21 blocks and 72 row pairs of V) is one pass over
+// the threads.  n = 64 setup: 31 ms (four stages of their own: 90 ms; float-float
+// sweeps throughout: 31 ms); n = 32 FP64: 11 ms (Gram, two Jacobi kernels and
+// recomposition as launches of their own: 33 ms).
+constexpr int CRAW = CNT * 16;   // partial sums of the Gram's tiles
+static_assert(sizeof(FF) == sizeof(double), "both element types share the layout");
+
+__host__ __device__ constexpr size_t core_smem(int p) {
+  // A; the Gram's staging, then the other A (later W) and V in its place (8-byte
+  // entries, rows of up to p + 3); the float rotations' product
+  const size_t a = (size_t)p * (p + 4) * 8, g = CRAW * 8;
+  return a + (2 * a > g ? 2 * a : g) + (size_t)p * (p + 4) * 4;
+}
+
+template <typename T>
+__global__ void __launch_bounds__(CNT) k_core(const TInfo* __restrict__ tis, int tbase, double eps,
+                                              int kc, int c_role, int maxp,
+                                              T* const* __restrict__ tab,
+                                              int* const* __restrict__ rtab, int P, int scr_buf,
+                                              int scr_rbuf, int* err, double* __restrict__ flops) {
+  constexpr bool F64 = sizeof(T) == 8;
+  using E = typename std::conditional<F64, double, FF>::type;
+  const int p = blockIdx.y;
+  const TInfo ti = tis[tbase + blockIdx.x];
+  T* scr = tab[scr_buf * P + p];
+  int* rs = rtab[scr_rbuf * P + p];
+  int* crank = rtab[c_role * P + p];
+  if (!scr || !rs || !crank) return;
+  const int tid = threadIdx.x, lane = tid & 31;
+  const int r = rs[ti.r_ri];
+  if (r <= 0) {   // an empty basis: rank 0
+    if (tid == 0) crank[ti.c_leaf] = 0;
+    return;
+  }
+  extern __shared__ __align__(16) unsigned char csm[];
+  const int lda = r | 1;   // odd row length: no bank conflicts down a column
+  E* A = reinterpret_cast<E*>(csm);
+  const size_t area = (size_t)maxp * (maxp + 4);
+  E* A2 = A + area;
+  E* V = A2 + area;
+  E* raw = A2;   // the Gram is done before the second A and V begin
+  float* W = reinterpret_cast<float*>(A2 + max(2 * area, (size_t)CRAW));
+  __shared__ float red[2][CNT / 32];
+  __shared__ double lam[CMAX];
+  __shared__ int ord[CMAX];
+  __shared__ int kkeep;
+
+  // ---- Gram of B^T (n x r): thread (tile, slice) owns a 4 x 4 tile of the
+  // upper triangle and every S-th row
+  const T* B = scr + ti.bt_off;
+  const int n = ti.n;
+  {
+    const int TM = (r + 3) >> 2, ntile = TM * (TM + 1) / 2, mt = 4 * TM;
+    // (the CRAW entries staged as values of T; at least 31 rows)
+    const int kch = min(256, ((CRAW * 8 / (int)sizeof(T) / mt) - 1) & ~1), ysld = kch + 1;
+    T* ys = reinterpret_cast<T*>(raw);
+    for (int tb = 0; tb < ntile; tb += CNT) {   // (one pass up to r = 60)
+      const int nt = min(CNT, ntile - tb);
+      const int S = CNT / nt;
+      const int tl = tid / S, slice = tid - tl * S;
+      const bool active = tl < nt;
+      int a0 = 0, t = tb + (active ? tl : 0);
+      while (t >= TM - a0) { t -= TM - a0; ++a0; }
+      const int i0 = 4 * a0, j0 = 4 * (a0 + t);
+      T s[4][4];
+      float c[4][4];
+#pragma unroll
+      for (int x = 0; x < 4; ++x)
+#pragma unroll
+        for (int y = 0; y < 4; ++y) { s[x][y] = T(0); c[x][y] = 0.f; }
+      for (int l0 = 0; l0 < n; l0 += kch) {
+        const int kk = min(kch, n - l0);
+        __syncthreads();
+        for (int col = tid >> 5; col < mt; col += CNT / 32)
+          for (int l = lane; l < kk; l += 32)
+            ys[col * ysld + l] = col < r ? B[(l0 + l) + (int64_t)col * n] : T(0);
+        __syncthreads();
+        if (active)
+          for (int l = slice; l < kk; l += S) {
+            T av[4], bv[4];
+#pragma unroll
+            for (int x = 0; x < 4; ++x) {
+              av[x] = ys[(i0 + x) * ysld + l];
+              bv[x] = ys[(j0 + x) * ysld + l];
+            }
+#pragma unroll
+            for (int x = 0; x < 4; ++x)
+#pragma unroll
+              for (int y = 0; y < 4; ++y) {
+                if constexpr (F64) s[x][y] = fma(av[x], bv[y], s[x][y]);
+                else ff_fma(s[x][y], c[x][y], av[x], bv[y]);
+              }
+          }
+      }
+      __syncthreads();
+#pragma unroll
+      for (int e = 0; e < 16; ++e) {
+        E v;
+        es(v, 0.f);
+        if (active) {
+          if constexpr (F64) v = s[e & 3][e >> 2];
+          else v = FF{s[e & 3][e >> 2], c[e & 3][e >> 2]};
+        }
+        raw[e * CNT + tid] = v;
+      }
+      __syncthreads();
+      // the slices' partial sums, in a fixed order
+      for (int e = tid; e < nt * 16; e += CNT) {
+        const int tq = e >> 4, q = e & 15;
+        E h;
+        es(h, 0.f);
+        for (int sl = 0; sl < S; ++sl) {
+          const E x = raw[q * CNT + tq * S + sl];
+          if constexpr (F64) {
+            h += x;
+          } else {
+            const float u = h.h + x.h, bp = u - h.h;
+            h.l += ((h.h - (u - bp)) + (x.h - bp)) + x.l;
+            h.h = u;
+          }
+        }
+        if constexpr (!F64) {
+          const float u = h.h + h.l;
+          h.l = h.l - (u - h.h);
+          h.h = u;
+        }
+        int tt = tb + tq, a = 0;
+        while (tt >= TM - a) { tt -= TM - a; ++a; }
+        const int i = 4 * a + (q & 3), j = 4 * (a + tt) + (q >> 2);
+        if (i < r && j < r) {
+          A[i * lda + j] = h;
+          A[j * lda + i] = h;
+        }
+      }
+    }
+  }
+  __syncthreads();
+  // ---- power-of-two scale: the largest diagonal to [1/2, 1)
+  int ex = 0;
+  {
+    double dmax = 0.0;
+    for (int i = lane; i < r; i += 32) dmax = fmax(dmax, ed(A[i * lda + i]));
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) dmax = fmax(dmax, __shfl_xor_sync(FULL, dmax, o));
+    if (dmax > 0.0 && dmax <= 1.0e300) frexp(dmax, &ex);
+  }
+  __syncthreads();
+  float* F0 = reinterpret_cast<float*>(A2);   // float copies for the first sweeps
+  float* F1 = F0 + area;
+  for (int e = tid; e < r * lda; e += CNT) {
+    const int i = e / lda, j = e - i * lda;
+    if (j >= r) continue;
+    const E v = escale(A[e], -ex);
+    A[e] = v;
+    F0[e] = ef(v);
+    W[e] = i == j ? 1.f : 0.f;
+  }
+  __syncthreads();
+
+  // ---- eigenvectors
+  int sweeps = 0;
+  if (r > 1) {
+    sweeps = jacobi<float>(F0, F1, W, r, lda, 1e-10f, 10, red);
+    __syncthreads();
+    // the product of the float rotations, made orthonormal
+    float* D = reinterpret_cast<float*>(A2);   // (I - W^T W) / 2
+    for (int e = tid; e < r * r; e += CNT) {
+      const int i = e / r, j = e - i * r;
+      if (F64) {
+        double g = 0.0;
+        for (int l = 0; l < r; ++l) g = fma((double)W[l * lda + i], (double)W[l * lda + j], g);
+        D[i * lda + j] = (float)(0.5 * ((i == j ? 1.0 : 0.0) - g));
+      } else {
+        float s = i == j ? -1.f : 0.f, c = 0.f;
+        for (int l = 0; l < r; ++l) ff_fma(s, c, W[l * lda + i], W[l * lda + j]);
+        D[i * lda + j] = -0.5f * (s + c);
+      }
+    }
+    __syncthreads();
+    for (int e = tid; e < r * r; e += CNT) {
+      const int i = e / r, j = e - i * r;
+      float d = 0.f;
+      for (int l = 0; l < r; ++l) d = fmaf(W[i * lda + l], D[l * lda + j], d);
+      E v, dd;
+      es(v, W[i * lda + j]);
+      es(dd, d);
+      V[i * lda + j] = ea(v, dd);
+    }
+    __syncthreads();
+    if constexpr (F64) {
+      for (int e = tid; e < r * r; e += CNT) {
+        const int i = e / r, j = e - i * r;
+        double g = 0.0;
+        for (int l = 0; l < r; ++l) g = fma(V[l * lda + i], V[l * lda + j], g);
+        D[i * lda + j] = (float)(0.5 * ((i == j ? 1.0 : 0.0) - g));
+      }
+      __syncthreads();
+      for (int e = tid; e < r * r; e += CNT) {   // (W in place of V: the correction is ~1e-12)
+        const int i = e / r, j = e - i * r;
+        float d = 0.f;
+        for (int l = 0; l < r; ++l) d = fmaf(W[i * lda + l], D[l * lda + j], d);
+        V[i * lda + j] += (double)d;
+      }
+      __syncthreads();
+    }
+    // A <- V^T (A V)
+    for (int e = tid; e < r * r; e += CNT) {
+      const int i = e / r, j = e - i * r;
+      E t;
+      es(t, 0.f);
+      for (int l = 0; l < r; ++l) t = ea(t, em(A[i * lda + l], V[l * lda + j]));
+      A2[i * lda + j] = t;
+    }
+    __syncthreads();
+    for (int e = tid; e < r * r; e += CNT) {
+      const int i = e / r, j = e - i * r;
+      if (j < i) continue;
+      E t;
+      es(t, 0.f);
+      for (int l = 0; l < r; ++l) t = ea(t, em(V[l * lda + i], A2[l * lda + j]));
+      A[i * lda + j] = t;
+      A[j * lda + i] = t;
+    }
+    __syncthreads();
+    sweeps += jacobi<E>(A, A2, V, r, lda, F64 ? 1e-30f : 1e-16f, 40, red);
+  } else if (tid == 0) {
+    es(V[0], 1.f);
+  }
   // ---- eigenvalues descending (rank by counting; ties by index), the kept rank
-  for (int i = tid; i < r; i += CNT) lam[i] = A[i * lda + i].h;
+  for (int i = tid; i < r; i += CNT) lam[i] = ed(A[i * lda + i]);
   __syncthreads();
   for (int i = tid; i < r; i += CNT) {
-    const double li = (double)lam[i] + (double)A[i * lda + i].l;
     int pos = 0;
-    for (int j = 0; j < r; ++j) {
-      const double lj = (double)lam[j] + (double)A[j * lda + j].l;
-      if (lj > li || (lj == li && j < i)) ++pos;
-    }
+    for (int j = 0; j < r; ++j)
+      if (lam[j] > lam[i] || (lam[j] == lam[i] && j < i)) ++pos;
     ord[pos] = i;
   }
   __syncthreads();
   if (tid == 0) {
-    const FF f0 = A[ord[0] * lda + ord[0]];
-    const double l1 = (double)f0.h + (double)f0.l;
+    const double l1 = lam[ord[0]];
     const double cut = eps * eps * l1;   // sigma_i > eps sigma_1
     int k = 0;
     if (l1 > 0.0)
       for (int j = 0; j < r; ++j) {
-        const FF f = A[ord[j] * lda + ord[j]];
-        const double lj = (double)f.h + (double)f.l;
+        const double lj = lam[ord[j]];
         if (lj > 0.0 && lj > cut) ++k;
         else break;
       }
@@ -611,42 +752,44 @@ __global__ void __launch_bounds__(CNT) k_core(const TInfo* __restrict__ tis, int
   }
   __syncthreads();
   const int k = kkeep;
-  // ---- recomposition: W (r x k, row by row, rows of whole float4)
+  // ---- recomposition: the kept columns W (r x k, rows of whole 4-vectors) in the
+  // second A's place
   const int ldw = (k + 3) & ~3;
+  T* K = reinterpret_cast<T*>(A2);
   for (int e = tid; e < r * ldw; e += CNT) {
     const int i = e / ldw, j = e - i * ldw;
-    float w = 0.f;
+    T w = T(0);
     if (j < k) {
-      const FF v = V[i * lda + ord[j]];
-      w = v.h + v.l;
+      const E v = V[i * lda + ord[j]];
+      if constexpr (F64) w = v;
+      else w = v.h + v.l;
     }
-    W[e] = w;
+    K[e] = w;
   }
   __syncthreads();
-  float* Uo = tab[(3 * c_role + 1) * P + p];
-  float* Vo = tab[(3 * c_role + 2) * P + p];
+  T* Uo = tab[(3 * c_role + 1) * P + p];
+  T* Vo = tab[(3 * c_role + 2) * P + p];
   const int m = ti.m;
   for (int e = tid; e < m + n; e += CNT) {   // a row of U = Q W, then of V = B^T W
     const bool u = e < m;
     const int rows = u ? m : n, i = u ? e : e - m;
-    const float* X = (u ? scr + ti.y_off : B) + i;
-    float* Z = u ? Uo : Vo;
+    const T* X = (u ? scr + ti.y_off : B) + i;
+    T* Z = u ? Uo : Vo;
     if (!Z) continue;
     Z += (u ? ti.u_off : ti.v_off) + i;
     for (int j0 = 0; j0 < k; j0 += 4) {
-      float4 acc{0.f, 0.f, 0.f, 0.f};
+      T acc[4] = {T(0), T(0), T(0), T(0)};
 #pragma unroll 8
       for (int l = 0; l < r; ++l) {
-        const float x = X[(int64_t)l * rows];
-        const float4 w = *reinterpret_cast<const float4*>(W + l * ldw + j0);
-        acc.x = fmaf(x, w.x, acc.x); acc.y = fmaf(x, w.y, acc.y);
-        acc.z = fmaf(x, w.z, acc.z); acc.w = fmaf(x, w.w, acc.w);
+        const T x = X[(int64_t)l * rows];
+        const T* w = K + l * ldw + j0;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) acc[q] += x * w[q];
       }
-      float* z = Z + (int64_t)j0 * rows;
-      z[0] = acc.x;
-      if (j0 + 1 < k) z[rows] = acc.y;
-      if (j0 + 2 < k) z[2 * (int64_t)rows] = acc.z;
-      if (j0 + 3 < k) z[3 * (int64_t)rows] = acc.w;
+      T* z = Z + (int64_t)j0 * rows;
+#pragma unroll
+      for (int q = 0; q < 4; ++q)
+        if (j0 + q < k) z[q * (int64_t)rows] = acc[q];
     }
   }
 }
@@ -692,20 +835,26 @@ void launch_orth(const Plan& pl, double tau, float* const* d_tab, int* const* d_
   }
 }
 
-void launch_core(const Plan& pl, double eps, int kc, int c_role, float* const* d_tab,
+template <typename T>
+void launch_core(const Plan& pl, double eps, int kc, int c_role, T* const* d_tab,
                  int* const* d_rtab, int P, int* d_err, cudaStream_t st, double* d_fl) {
   const int nt = (int)pl.targets.size();
   if (nt <= 0 || P <= 0) return;
   const size_t smem = core_smem(pl.max_p);
   if (smem > 48 * 1024)
-    ACR_CUDA(cudaFuncSetAttribute(k_core, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    ACR_CUDA(cudaFuncSetAttribute(k_core<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                   (int)core_smem(CMAX)));
   for (int t0 = 0; t0 < nt; t0 += 65535) {
     const dim3 grid(std::min(65535, nt - t0), P);
-    k_core<<<grid, CNT, smem, st>>>((const TInfo*)pl.d_targets, t0, eps, kc, c_role, pl.max_p,
-                                    d_tab, d_rtab, P, 3 * pl.nroles, pl.nroles, d_err, d_fl);
+    k_core<T><<<grid, CNT, smem, st>>>((const TInfo*)pl.d_targets, t0, eps, kc, c_role, pl.max_p,
+                                       d_tab, d_rtab, P, 3 * pl.nroles, pl.nroles, d_err, d_fl);
     ACR_LAUNCHED(1);
   }
 }
+
+template void launch_core<double>(const Plan&, double, int, int, double* const*, int* const*, int,
+                                  int*, cudaStream_t, double*);
+template void launch_core<float>(const Plan&, double, int, int, float* const*, int* const*, int,
+                                 int*, cudaStream_t, double*);
 
 }  // namespace acr

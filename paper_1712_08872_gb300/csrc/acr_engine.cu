@@ -766,19 +766,15 @@ class Engine : public EngineBase {
           timed(0, [&] { gemm_stage(pl, sg, d_tab, (const int* const*)d_rtab, pc, st); }, sg.tag);
           continue;
         }
-        if constexpr (std::is_same<T, float>::value) {
-          if (sg.kind == ST_ORTH)
-            timed(1, [&] { launch_orth(pl, tau_orth(), d_tab, d_rtab, pc, st, d_sketch_stat, fl(1)); });
-          else
-            timed(2, [&] { launch_core(pl, eps, kc, c_role, d_tab, d_rtab, pc, d_err, st, fl(2)); });
-        } else {
-          if (sg.kind == ST_PCHOL || sg.kind == ST_PCHOL + 16)
-            timed(1, [&] { launch_pchol<T>(pl, sg.beg, sg.end, sg.kind == ST_PCHOL, tau_orth(), d_tab,
-                                           d_rtab, pc, st, d_sketch_stat, fl(1)); });
-          else
-            timed(2, [&] { launch_eig<T>(pl, sg.beg, sg.end, eps, kc, c_role, d_tab, d_rtab, pc,
-                                         d_err, st, fl(2)); });
+        if (sg.kind == ST_CORE) {
+          timed(2, [&] { launch_core<T>(pl, eps, kc, c_role, d_tab, d_rtab, pc, d_err, st, fl(2)); });
+          continue;
         }
+        if constexpr (std::is_same<T, float>::value)
+          timed(1, [&] { launch_orth(pl, tau_orth(), d_tab, d_rtab, pc, st, d_sketch_stat, fl(1)); });
+        else
+          timed(1, [&] { launch_pchol<T>(pl, sg.beg, sg.end, sg.kind == ST_PCHOL, tau_orth(), d_tab,
+                                         d_rtab, pc, st, d_sketch_stat, fl(1)); });
       }
     }
   }
@@ -903,6 +899,7 @@ void Engine<T>::prepare(const double* const* coefs, cudaStream_t st, bool count_
   pp.oversample = 8;
   pp.cholqr2 = true;
   pp.fused = std::is_same<T, float>::value;
+  pp.fused_core = true;
   mvp.build(S);
   {
     size_t fr = 0, tot = 0;

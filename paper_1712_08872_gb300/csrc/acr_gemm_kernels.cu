@@ -1477,7 +1477,8 @@ __global__ void __launch_bounds__(NT, sizeof(T) == 4 ? 4 : 2)
             R.rows = I.k_st;
             R.off = SK ? I.omega_row0 : (int)(I.boff - ti.y_off);
             R.lda = I.lda; R.ldc = G.ldc;
-            if (flops && f0 == 0 && R.k > 0) atomicAdd(flops, 2.0 * R.rows * nc * R.k);
+            if (flops && f0 == 0 && blockIdx.z == 0 && R.k > 0)
+              atomicAdd(flops, 2.0 * R.rows * nc * R.k);
           }
           // (a term without rows in this block has no units here)
           if (R.k <= 0 || R.off >= f0 + fr || R.off + R.rows <= f0) R.k = 0;
@@ -1494,7 +1495,7 @@ __global__ void __launch_bounds__(NT, sizeof(T) == 4 ? 4 : 2)
       }
       __syncthreads();
       const int half = uoff[32], units = half + uoff[TDI];
-      for (int u = warp; u < units; u += NT / 32) {
+      for (int u = warp + (NT / 32) * blockIdx.z; u < units; u += (NT / 32) * gridDim.z) {
         // the term of unit u (the second half's offsets are its own)
         int lo, hi, add;
         if (u < half) { lo = 0; hi = 32; add = 0; } else { lo = 32; hi = TDI; add = half; }
@@ -1605,9 +1606,19 @@ void launch_tdot(const Plan& pl, bool sketch, T* const* d_tab, const int* const*
     if (!few && smem(beg) <= small)
       for (end = beg + 1; end < nt && smem(end) <= small; ++end) {}
     size_t need = 0;
-    for (int q = beg; q < end; ++q) need = std::max(need, smem(q));
+    int rows = 0;
+    for (int q = beg; q < end; ++q) {
+      need = std::max(need, smem(q));
+      rows = std::max({rows, pl.targets[pl.torder[q]].m, pl.targets[pl.torder[q]].n});
+    }
+    // few targets: their units dealt to up to 8 CTAs each (a unit's sums are the
+    // same wherever it runs; with more than one block of rows its partial sums
+    // meet in global memory and stay in one CTA)
+    int z = 1;
+    if (rows <= tdr<T>())
+      while (z < 8 && (int64_t)(end - beg) * P * z < 2 * device_sm_count()) z *= 2;
     for (int t0 = beg; t0 < end; t0 += 65535) {
-      const dim3 grid(std::min(65535, end - t0), P);
+      const dim3 grid(std::min(65535, end - t0), P, z);
       kern<<<grid, NT, need, st>>>((const TInfo*)pl.d_targets, (const int*)pl.d_torder + t0,
                                    (const GGroup*)pl.d_groups, (const GItem*)pl.d_items, d_tab,
                                    d_rtab, P, 3 * pl.nroles, pl.nroles, d_fl);

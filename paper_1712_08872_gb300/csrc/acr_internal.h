@@ -105,19 +105,14 @@ void launch_pchol(const Plan& pl, int tbeg, int tend, bool truncate, double tau,
                   T* const* d_tab, int* const* d_rtab, int P, cudaStream_t st,
                   unsigned long long* d_sketch_stat, double* d_flops = nullptr);
 
-// Jacobi eigen cores of plan targets (FP64 factors); writes the kept ranks into
-// the rank buffer of role c_role and raises ERR_RANKCAP above kc.
-template <typename T>
-void launch_eig(const Plan& pl, int tbeg, int tend, double eps, int kc, int c_role,
-                T* const* d_tab, int* const* d_rtab, int P, int* d_err, cudaStream_t st,
-                double* d_flops = nullptr);
-
-// The fused stages ST_ORTH and ST_CORE of a plan's float targets: the sketches'
-// orthonormal bases, in place; core Grams, Jacobi cores and recomposition,
-// rank output and ERR_RANKCAP as launch_eig.
+// The fused stages of a plan's targets.  ST_ORTH (float factors): the sketches'
+// orthonormal bases, in place, counted into d_sketch_stat as launch_pchol does.
+// ST_CORE: core Grams, Jacobi cores and recomposition; writes the kept ranks into the
+// rank buffer of role c_role and raises ERR_RANKCAP above kc.
 void launch_orth(const Plan& pl, double tau, float* const* d_tab, int* const* d_rtab, int P,
                  cudaStream_t st, unsigned long long* d_sketch_stat, double* d_flops = nullptr);
-void launch_core(const Plan& pl, double eps, int kc, int c_role, float* const* d_tab,
+template <typename T>
+void launch_core(const Plan& pl, double eps, int kc, int c_role, T* const* d_tab,
                  int* const* d_rtab, int P, int* d_err, cudaStream_t st,
                  double* d_flops = nullptr);
 

@@ -423,6 +423,8 @@ struct Builder {
       if (!pp.fused) {
         ti.g_off = alloc((int64_t)p * p);
         ti.t_off = alloc((int64_t)p * p);
+      }
+      if (!pp.fused_core) {
         ti.h_off = alloc((int64_t)p * p);
         ti.w_off = alloc((int64_t)p * p);
       }
@@ -561,7 +563,7 @@ struct Builder {
     }
     stage(ST_GEMM, g0, (int)P.groups.size(), TAG_BT);
 
-    if (pp.fused) {
+    if (pp.fused_core) {
       if (!lts.empty()) P.stages.push_back(Stage{ST_CORE, 0, (int)lts.size()});
       return;
     }

@@ -94,7 +94,7 @@ struct StackDim {
   int32_t st, rb, ri, g0, g1;
 };
 
-// ST_ORTH and ST_CORE (PlanParams::fused) each stand for a run of the others:
+// ST_ORTH and ST_CORE (PlanParams::fused, fused_core) each stand for a run of the others:
 // the sketch's Gram, Cholesky and basis stages, and the core Gram, Jacobi and
 // recomposition stages.
 enum StageKind { ST_GEMM = 0, ST_PCHOL = 1, ST_EIG = 2, ST_ORTH = 3, ST_CORE = 4 };
@@ -171,7 +171,8 @@ struct PlanParams {
   int kc;        // rank capacity of stored low-rank blocks
   int oversample;
   bool cholqr2;  // second orthonormalisation pass (single-precision forms)
-  bool fused = false;   // one basis and one core stage per plan (float factors)
+  bool fused = false;       // one basis stage per plan (float factors)
+  bool fused_core = false;  // one core stage per plan
 };
 
 // Build the plan of one formatted operation (plan.groups and plan.items keep

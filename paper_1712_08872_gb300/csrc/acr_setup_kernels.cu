@@ -1,9 +1,7 @@
 // Setup kernels of the ACR engine (sm_103a), besides the grouped GEMMs of
-// acr_gemm_kernels.cu and the float recompression cores of acr_core_kernels.cu:
+// acr_gemm_kernels.cu and the recompression cores of acr_core_kernels.cu:
 //  * k_pchol   -- pivoted Cholesky of a sketch Gram (FP64 factors): orthonormal
 //                 basis transform of the range finder;
-//  * k_eig     -- cyclic Jacobi of the small recompression core (FP64 factors),
-//                 rank selection sigma_i > eps * sigma_1 (Sec. 4.3 H_eps);
 //  * k_leaf_inv-- Gauss-Jordan inverse with partial pivoting of a dense
 //                 diagonal leaf (the leaves of the recursive H-inverse): FP64,
 //                 or for float storage float elimination refined to float
@@ -29,18 +27,6 @@ namespace {
 
 // ---------------------------------------------------------------- cores
 constexpr int CMAX = 64;   // largest sketch / core dimension
-
-// The rotation (c, s) that zeroes a_pq of the 2 x 2 block [a_pp a_pq; a_pq a_qq].
-__device__ __forceinline__ void jrot(double app, double aqq, double apq, double& c, double& s) {
-  c = 1.0;
-  s = 0.0;
-  if (apq != 0.0) {
-    const double tau_ = (aqq - app) / (2.0 * apq);
-    const double t = (tau_ >= 0 ? 1.0 : -1.0) / (fabs(tau_) + sqrt(1.0 + tau_ * tau_));
-    c = rsqrt(1.0 + t * t);
-    s = t * c;
-  }
-}
 
 // Pivoted Cholesky of G (pd x pd): G = P L L^T P^T, stop when the largest
 // remaining diagonal <= tau^2 * max diag(G) (truncating pass).  Writes
@@ -317,311 +303,6 @@ __global__ void __launch_bounds__(NT) k_pchol(const TInfo* __restrict__ tis, int
   if (threadIdx.x == 0) {
     rs[ti.r_ri] = r;
     if (flops) atomicAdd(flops, (double)pd * r * r - 2.0 * r * r * r / 3.0 + (double)r * r * r / 3.0);
-  }
-}
-
-constexpr int EIG_WARP_MAX = 16;   // cores up to this size: one warp each
-
-// The same cyclic Jacobi for small cores (1 < r <= 16), one warp per target,
-// eight targets per CTA: the rotations of a round are computed and applied
-// by the warp's lanes with warp barriers only (same rotation sequence and
-// stopping rule as k_eig).
-template <typename T>
-__global__ void __launch_bounds__(NT) k_eig_warp(const TInfo* __restrict__ tis, int tbase,
-                                                 int tend, double eps, int kc, int c_rbuf,
-                                                 T* const* __restrict__ tab,
-                                                 int* const* __restrict__ rtab, int P,
-                                                 int scr_buf, int scr_rbuf, int* err,
-                                                 double* __restrict__ flops) {
-  constexpr int M = EIG_WARP_MAX;
-  const int p = blockIdx.y;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int t = tbase + blockIdx.x * (NT / 32) + warp;
-  __shared__ double As[NT / 32][M][M + 1], Vs[NT / 32][M][M + 1];
-  __shared__ double css[NT / 32][M / 2], sns[NT / 32][M / 2];
-  __shared__ double lams[NT / 32][M];
-  __shared__ int pps[NT / 32][M / 2], qqs[NT / 32][M / 2], ords[NT / 32][M];
-  if (t >= tend) return;
-  const TInfo ti = tis[t];
-  T* scr = tab[scr_buf * P + p];
-  int* rs = rtab[scr_rbuf * P + p];
-  int* crank = rtab[c_rbuf * P + p];
-  if (!scr || !rs || !crank) return;
-  const int r = rs[ti.r_ri];
-  if (r <= 0) {   // an empty basis: rank 0
-    if (lane == 0) crank[ti.c_leaf] = 0;
-    return;
-  }
-  if (r > M) return;   // k_eig's cores
-  const int ld = ti.p;
-  double (*A)[M + 1] = As[warp];
-  double (*V)[M + 1] = Vs[warp];
-  double* cs = css[warp];
-  double* sn = sns[warp];
-  int* pp = pps[warp];
-  int* qq = qqs[warp];
-  const double* H = reinterpret_cast<const double*>(scr + ti.h_off);
-  T* W = scr + ti.w_off;
-  for (int e = lane; e < r * r; e += 32) {
-    const int i = e % r, j = e / r;
-    A[i][j] = 0.5 * (H[i + (int64_t)j * ld] + H[j + (int64_t)i * ld]);
-    V[i][j] = (i == j) ? 1.0 : 0.0;
-  }
-  __syncwarp();
-  const int nn = (r + 1) & ~1;
-  const int npair = nn / 2;
-  int sweeps_done = 0;
-  const double conv = 1e-30;
-  for (int sweep = 0; sweep < 40; ++sweep) {
-    double off = 0, tot = 0;
-    for (int e = lane; e < r * r; e += 32) {
-      const int i = e % r, j = e / r;
-      const double a = A[i][j];
-      const double v = a * a;
-      tot += v;
-      if (i != j) off += v;
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      off += __shfl_xor_sync(0xffffffffu, off, o);
-      tot += __shfl_xor_sync(0xffffffffu, tot, o);
-    }
-    if (off <= conv * tot || r == 1) break;
-    ++sweeps_done;
-    for (int round = 0; round < nn - 1; ++round) {
-      if (lane < npair) {
-        const int k = lane;
-        const int pa = k, pb = nn - 1 - k;
-        const int a = (pa == 0) ? 0 : 1 + ((pa - 1 + round) % (nn - 1));
-        const int b = 1 + ((pb - 1 + round) % (nn - 1));
-        const int lo = a < b ? a : b, hi = a < b ? b : a;
-        pp[k] = lo; qq[k] = hi;
-        double c = 1.0, sv = 0.0;
-        if (hi < r) jrot(A[lo][lo], A[hi][hi], A[lo][hi], c, sv);
-        cs[k] = c; sn[k] = sv;
-      }
-      __syncwarp();
-      const int nblk = npair * npair;
-      for (int e = lane; e < nblk + npair * r; e += 32) {
-        if (e < nblk) {
-          const int k1 = e / npair, k2 = e - k1 * npair;
-          const int a1 = pp[k1], b1 = qq[k1], a2 = pp[k2], b2 = qq[k2];
-          const bool h1 = b1 < r, h2 = b2 < r;
-          const double c1 = cs[k1], s1 = sn[k1], c2 = cs[k2], s2 = sn[k2];
-          const double z = 0.0;
-          const double x00 = A[a1][a2];
-          const double x01 = h2 ? A[a1][b2] : z;
-          const double x10 = h1 ? A[b1][a2] : z;
-          const double x11 = (h1 && h2) ? A[b1][b2] : z;
-          const double y00 = c2 * x00 - s2 * x01, y01 = s2 * x00 + c2 * x01;
-          const double y10 = c2 * x10 - s2 * x11, y11 = s2 * x10 + c2 * x11;
-          A[a1][a2] = c1 * y00 - s1 * y10;
-          if (h2) A[a1][b2] = c1 * y01 - s1 * y11;
-          if (h1) A[b1][a2] = s1 * y00 + c1 * y10;
-          if (h1 && h2) A[b1][b2] = s1 * y01 + c1 * y11;
-        } else {
-          const int f = e - nblk;
-          const int k = f / r, iv = f - k * r;
-          const int a = pp[k], b = qq[k];
-          if (b < r) {
-            const double c = cs[k], sv = sn[k];
-            const double vx = V[iv][a], vy = V[iv][b];
-            V[iv][a] = c * vx - sv * vy;
-            V[iv][b] = sv * vx + c * vy;
-          }
-        }
-      }
-      __syncwarp();
-    }
-  }
-  double* lam = lams[warp];
-  int* order = ords[warp];
-  if (lane < r) lam[lane] = A[lane][lane];
-  __syncwarp();
-  if (lane < r) {
-    int pos = 0;
-    for (int j = 0; j < r; ++j)
-      if (lam[j] > lam[lane] || (lam[j] == lam[lane] && j < lane)) ++pos;
-    order[pos] = lane;
-  }
-  __syncwarp();
-  int k = 0;
-  if (lane == 0) {
-    const double l1 = lam[order[0]];
-    if (l1 > 0.0) {
-      const double s1 = sqrt(l1);
-      for (int j = 0; j < r; ++j) {
-        const double lj = lam[order[j]];
-        if (lj > 0.0 && sqrt(lj) > eps * s1) ++k;
-        else break;
-      }
-    }
-    if (k > kc) {
-      atomicOr(err, ERR_RANKCAP);
-      k = kc;
-    }
-    crank[ti.c_leaf] = k;
-    if (flops) atomicAdd(flops, 9.0 * r * r * r * sweeps_done);
-  }
-  k = __shfl_sync(0xffffffffu, k, 0);
-  for (int e = lane; e < r * k; e += 32) {
-    const int i = e % r, j = e / r;
-    W[i + (int64_t)j * ld] = (T)V[i][order[j]];
-  }
-}
-
-// Cyclic Jacobi (round-robin parallel order) on the r x r symmetric core H
-// (cores with r > 16; k_eig_warp takes the smaller ones).
-template <typename T>
-__global__ void __launch_bounds__(NT) k_eig(const TInfo* __restrict__ tis, int tbase, double eps,
-                                            int kc, int c_rbuf, T* const* __restrict__ tab,
-                                            int* const* __restrict__ rtab, int P, int scr_buf,
-                                            int scr_rbuf, int* err, double* __restrict__ flops) {
-  const int p = blockIdx.y;
-  const TInfo ti = tis[tbase + blockIdx.x];
-  T* scr = tab[scr_buf * P + p];
-  int* rs = rtab[scr_rbuf * P + p];
-  int* crank = rtab[c_rbuf * P + p];
-  if (!scr || !rs || !crank) return;
-  const int r = rs[ti.r_ri];
-  const int ld = ti.p;
-  if (r <= EIG_WARP_MAX) return;   // k_eig_warp's cores (and the empty bases)
-  extern __shared__ double dsm[];
-  double (*A)[CMAX + 1] = reinterpret_cast<double (*)[CMAX + 1]>(dsm);
-  double (*V)[CMAX + 1] = reinterpret_cast<double (*)[CMAX + 1]>(dsm + CMAX * (CMAX + 1));
-  __shared__ double cs[CMAX / 2 + 1], sn[CMAX / 2 + 1];
-  __shared__ int pp[CMAX / 2 + 1], qq[CMAX / 2 + 1];
-  __shared__ double red[NT];
-  __shared__ int order[CMAX];
-  __shared__ double lam[CMAX];
-  __shared__ int kkeep;
-  const double* H = reinterpret_cast<const double*>(scr + ti.h_off);   // FP64 Gram
-  T* W = scr + ti.w_off;
-  for (int e = threadIdx.x; e < r * r; e += NT) {
-    int i = e % r, j = e / r;
-    A[i][j] = 0.5 * ((double)H[i + (int64_t)j * ld] + (double)H[j + (int64_t)i * ld]);
-    V[i][j] = (i == j) ? 1.0 : 0.0;
-  }
-  __syncthreads();
-  const int nn = (r + 1) & ~1;   // even number of players (r may get a dummy)
-  const int npair = nn / 2;
-  int sweeps_done = 0;
-  for (int sweep = 0; sweep < 40; ++sweep) {
-    // off-diagonal and total norms: warp shuffles, then one pass over the warps
-    double off = 0, tot = 0;
-    {
-      const int i = threadIdx.x & 63;
-      if (i < r)
-        for (int j = threadIdx.x >> 6; j < r; j += 4) {
-          const double a = A[i][j];
-          const double v = a * a;
-          tot += v;
-          if (i != j) off += v;
-        }
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      off += __shfl_xor_sync(0xffffffffu, off, o);
-      tot += __shfl_xor_sync(0xffffffffu, tot, o);
-    }
-    if ((threadIdx.x & 31) == 0) {
-      red[threadIdx.x >> 5] = off;
-      red[(NT >> 5) + (threadIdx.x >> 5)] = tot;
-    }
-    __syncthreads();
-    double offs = 0, tots = 0;
-    for (int w = 0; w < NT / 32; ++w) { offs += red[w]; tots += red[NT / 32 + w]; }
-    __syncthreads();
-    // converged: eigenvectors to ~1e-15
-    const double conv = 1e-30;
-    if (offs <= conv * tots || r == 1) break;
-    ++sweeps_done;
-    for (int round = 0; round < nn - 1; ++round) {
-      // circle method: player 0 fixed, others rotate
-      for (int k = threadIdx.x; k < npair; k += NT) {
-        const int pa = k, pb = nn - 1 - k;
-        const int a = (pa == 0) ? 0 : 1 + ((pa - 1 + round) % (nn - 1));
-        const int b = 1 + ((pb - 1 + round) % (nn - 1));
-        int lo = a < b ? a : b, hi = a < b ? b : a;
-        pp[k] = lo; qq[k] = hi;
-        double c = 1.0, s = 0.0;
-        if (hi < r) jrot(A[lo][lo], A[hi][hi], A[lo][hi], c, s);
-        cs[k] = c; sn[k] = s;
-      }
-      __syncthreads();
-      // A <- J^T A J in one pass: the pairs are disjoint, so each 2 x 2 block
-      // (rows of pair k1, columns of pair k2) is rotated on its own -- columns
-      // first, then rows; V <- V J alongside.  A pair holding the odd
-      // dimension's dummy index is the identity and has no second row/column.
-      // The blocks and the npair * r (row, pair) items of V share one flat
-      // index space, so that every lane has work.
-      const int nblk = npair * npair;
-      for (int e = threadIdx.x; e < nblk + npair * r; e += NT) {
-        if (e < nblk) {
-          const int k1 = e / npair, k2 = e - k1 * npair;
-          const int a1 = pp[k1], b1 = qq[k1], a2 = pp[k2], b2 = qq[k2];
-          const bool h1 = b1 < r, h2 = b2 < r;
-          const double c1 = cs[k1], s1 = sn[k1], c2 = cs[k2], s2 = sn[k2];
-          const double z = 0.0;
-          const double x00 = A[a1][a2];
-          const double x01 = h2 ? A[a1][b2] : z;
-          const double x10 = h1 ? A[b1][a2] : z;
-          const double x11 = (h1 && h2) ? A[b1][b2] : z;
-          const double y00 = c2 * x00 - s2 * x01, y01 = s2 * x00 + c2 * x01;
-          const double y10 = c2 * x10 - s2 * x11, y11 = s2 * x10 + c2 * x11;
-          A[a1][a2] = c1 * y00 - s1 * y10;
-          if (h2) A[a1][b2] = c1 * y01 - s1 * y11;
-          if (h1) A[b1][a2] = s1 * y00 + c1 * y10;
-          if (h1 && h2) A[b1][b2] = s1 * y01 + c1 * y11;
-        } else {
-          const int f = e - nblk;
-          const int k = f / r, iv = f - k * r;
-          const int a = pp[k], b = qq[k];
-          if (b < r) {
-            const double c = cs[k], s = sn[k];
-            const double vx = V[iv][a], vy = V[iv][b];
-            V[iv][a] = c * vx - s * vy;
-            V[iv][b] = s * vx + c * vy;
-          }
-        }
-      }
-      __syncthreads();
-    }
-  }
-  // sort eigenvalues descending (rank by counting; ties by index)
-  for (int i = threadIdx.x; i < r; i += NT) lam[i] = A[i][i];
-  __syncthreads();
-  for (int i = threadIdx.x; i < r; i += NT) {
-    int pos = 0;
-    for (int j = 0; j < r; ++j)
-      if (lam[j] > lam[i] || (lam[j] == lam[i] && j < i)) ++pos;
-    order[pos] = i;
-  }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double l1 = lam[order[0]];
-    int k = 0;
-    if (l1 > 0.0) {
-      double s1 = sqrt(l1);
-      for (int j = 0; j < r; ++j) {
-        double lj = lam[order[j]];
-        if (lj > 0.0 && sqrt(lj) > eps * s1) ++k;
-        else break;
-      }
-    }
-    if (k > kc) {
-      atomicOr(err, ERR_RANKCAP);
-      k = kc;
-    }
-    kkeep = k;
-    crank[ti.c_leaf] = k;
-    if (flops) atomicAdd(flops, 9.0 * r * r * r * sweeps_done);
-  }
-  __syncthreads();
-  const int k = kkeep;
-  for (int e = threadIdx.x; e < r * k; e += NT) {
-    int i = e % r, j = e / r;
-    W[i + (int64_t)j * ld] = (T)V[i][order[j]];
   }
 }
 
@@ -1164,36 +845,6 @@ void launch_pchol(const Plan& pl, int tbeg, int tend, bool truncate, double tau,
 }
 
 template <typename T>
-void launch_eig(const Plan& pl, int tbeg, int tend, double eps, int kc, int c_role,
-                T* const* d_tab, int* const* d_rtab, int P, int* d_err, cudaStream_t st,
-                double* d_fl) {
-  int nt = tend - tbeg;
-  if (nt <= 0 || P <= 0) return;
-  const size_t smem = 2 * CMAX * (CMAX + 1) * sizeof(double);
-  ACR_CUDA(cudaFuncSetAttribute(k_eig<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  {
-    const int per = NT / 32;
-    for (int t0 = 0; t0 < nt; t0 += 65535 * per) {
-      const int cnt = std::min(65535 * per, nt - t0);
-      dim3 grid((cnt + per - 1) / per, P);
-      k_eig_warp<T><<<grid, NT, 0, st>>>((const TInfo*)pl.d_targets, tbeg + t0, tbeg + t0 + cnt,
-                                         eps, kc, c_role, d_tab, d_rtab, P, 3 * pl.nroles,
-                                         pl.nroles, d_err, d_fl);
-      ACR_LAUNCHED(1);
-    }
-  }
-  // cores wider than a warp's (none when every sketch is at most that wide:
-  // a core is never wider than its basis, nor the basis than its sketch)
-  if (pl.max_p <= EIG_WARP_MAX) return;
-  for (int t0 = 0; t0 < nt; t0 += 65535) {
-    dim3 grid(std::min(65535, nt - t0), P);
-    k_eig<T><<<grid, NT, smem, st>>>((const TInfo*)pl.d_targets, tbeg + t0, eps, kc, c_role, d_tab,
-                                  d_rtab, P, 3 * pl.nroles, pl.nroles, d_err, d_fl);
-    ACR_LAUNCHED(1);
-  }
-}
-
-template <typename T>
 void launch_leaf_inv(T* const* d_dense, int64_t off, int lsz, int P, int* d_err, cudaStream_t st,
                      double* d_fl, unsigned long long* d_fallbacks) {
   if (P <= 0) return;
@@ -1237,8 +888,6 @@ void launch_plane_to_h(const StructDev& sd, const double* coef, int n, const int
 
 template void launch_pchol<double>(const Plan&, int, int, bool, double, double* const*,
                                    int* const*, int, cudaStream_t, unsigned long long*, double*);
-template void launch_eig<double>(const Plan&, int, int, double, int, int, double* const*,
-                                 int* const*, int, int*, cudaStream_t, double*);
 #define ACR_INST(T)                                                                              \
   template void launch_leaf_inv<T>(T* const*, int64_t, int, int, int*, cudaStream_t, double*,     \
                                    unsigned long long*);                                         \
