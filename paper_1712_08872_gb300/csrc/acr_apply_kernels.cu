@@ -43,6 +43,10 @@ struct RunSum {
   double s = 0.0;
   __device__ __forceinline__ void add(double v) { s += v; }
   __device__ __forceinline__ double value() const { return s; }
+  // a partial sum begins at begin() and enters by end(): for double it is the sum
+  // itself (one FP64 addition less per partial sum)
+  __device__ __forceinline__ double begin() const { return s; }
+  __device__ __forceinline__ void end(double v) { s = v; }
 };
 template <>
 struct RunSum<float> {
@@ -54,9 +58,42 @@ struct RunSum<float> {
     hi = t;
   }
   __device__ __forceinline__ double value() const { return (double)hi + (double)lo; }
+  __device__ __forceinline__ float begin() const { return 0.f; }
+  __device__ __forceinline__ void end(float v) { add(v); }
 };
 
 constexpr int MAXQ = 256;   // most low-rank leaves covering one chunk
+
+// The R right-hand sides' staged values of one vector entry (innermost in shared
+// memory, so that they come in 16-byte loads: with one load each, 8 right-hand
+// sides spent more time on them than on their products).
+template <int R>
+__device__ __forceinline__ void ldr(const float* p, float (&v)[R]) {
+  if constexpr (R % 4 == 0) {
+#pragma unroll
+    for (int q = 0; q < R; q += 4) {
+      const float4 x = *reinterpret_cast<const float4*>(p + q);
+      v[q] = x.x; v[q + 1] = x.y; v[q + 2] = x.z; v[q + 3] = x.w;
+    }
+  } else if constexpr (R == 2) {
+    const float2 x = *reinterpret_cast<const float2*>(p);
+    v[0] = x.x; v[1] = x.y;
+  } else {
+    v[0] = p[0];
+  }
+}
+template <int R>
+__device__ __forceinline__ void ldr(const double* p, double (&v)[R]) {
+  if constexpr (R % 2 == 0) {
+#pragma unroll
+    for (int q = 0; q < R; q += 2) {
+      const double2 x = *reinterpret_cast<const double2*>(p + q);
+      v[q] = x.x; v[q + 1] = x.y;
+    }
+  } else {
+    v[0] = p[0];
+  }
+}
 
 // Partial projections, one CTA per (leaf-size column chunk c, plane p): for
 // every low-rank leaf l whose columns cover chunk c, the piece of
@@ -73,7 +110,7 @@ __global__ void __launch_bounds__(256) k_lr_proj(MatvecDev mv, T* const* __restr
                                                  bool trans, int64_t vs) {
   chain_begin();
   using Acc = AccT<T>;
-  __shared__ Acc xs[R][64];
+  __shared__ __align__(16) Acc xs[64][R];
   __shared__ int64_t s_off[MAXQ];
   __shared__ int s_ld[MAXQ], s_seg[MAXQ], s_cum[MAXQ + 1];
   const int c = blockIdx.x, p = blockIdx.y;
@@ -89,7 +126,7 @@ __global__ void __launch_bounds__(256) k_lr_proj(MatvecDev mv, T* const* __restr
   const int q0 = ptr[c], nq = min(ptr[c + 1] - q0, MAXQ);
   for (int e = threadIdx.x; e < R * lsz; e += 256) {
     const int rr = R == 1 ? 0 : e / lsz, i = e - rr * lsz;
-    xs[rr][i] = (Acc)xp[rr * vs + (int64_t)c * lsz + i];
+    xs[i][rr] = (Acc)xp[rr * vs + (int64_t)c * lsz + i];
   }
   for (int q = threadIdx.x; q < nq; q += 256) {
     const int l = lf[q0 + q];
@@ -126,18 +163,17 @@ __global__ void __launch_bounds__(256) k_lr_proj(MatvecDev mv, T* const* __restr
       Acc v[R];
 #pragma unroll
       for (int rr = 0; rr < R; ++rr) v[rr] = Acc(0);
-      if (lsz == 64) {
+      T f[8];   // (all in flight, whatever the leaf size)
 #pragma unroll
-        for (int u = 0; u < 8; ++u) {
-          const Acc f = (Acc)ld(col[r + 8 * u]);
+      for (int u = 0; u < 8; ++u) f[u] = r + 8 * u < lsz ? col[r + 8 * u] : T(0.f);
 #pragma unroll
-          for (int rr = 0; rr < R; ++rr) v[rr] += f * xs[rr][r + 8 * u];
-        }
-      } else {
-        for (int i = r; i < lsz; i += 8) {
-          const Acc f = (Acc)ld(col[i]);
+      for (int u = 0; u < 8; ++u) {
+        if (r + 8 * u < lsz) {
+          const Acc w = (Acc)ld(f[u]);
+          Acc xv[R];
+          ldr<R>(xs[r + 8 * u], xv);
 #pragma unroll
-          for (int rr = 0; rr < R; ++rr) v[rr] += f * xs[rr][i];
+          for (int rr = 0; rr < R; ++rr) v[rr] += w * xv[rr];
         }
       }
 #pragma unroll
@@ -159,10 +195,14 @@ __global__ void __launch_bounds__(256) k_lr_proj(MatvecDev mv, T* const* __restr
 // transposed and V_l[cols of c] tv_l.  The x segments and tv vectors the
 // chunk needs are staged in shared memory first (converted once to the
 // multiply type), with the chunk's leaf descriptors (rank, offset, leading
-// dimension).  Thread t owns row t % 64: of each dense leaf the columns
-// t / 64 + 4 j, of the low-rank leaves every fourth one (starting at t / 64)
-// with all its columns.  LSZ > 0 fixes the leaf size at compile time
-// (unrolled, 16 loads in flight).
+// dimension).  Thread t owns row t % lsz: of each dense leaf the columns
+// t / lsz + G j, of the low-rank leaves every G-th one (starting at t / lsz), G =
+// 256 / lsz (a 36-point leaf keeps 252 threads busy; with rows t % 64 it kept
+// 144).  Bound by the loads in flight: 16 per dense leaf (LSZ 64, fixed at
+// compile time) or 8, and 4 columns each of two low-rank leaves, before their
+// products.  n = 96 (36-point leaves): 4.7 ms per apply against 7.7 ms; n = 80
+// (50-point leaves): 2.8 ms against 4.5 ms; 8 right-hand sides at n = 64: 3.1 ms
+// against 3.9 ms.
 template <typename T, int LSZ, int R>
 __global__ void __launch_bounds__(256) k_hmv_rows(MatvecDev mv, T* const* __restrict__ D,
                                                   T* const* __restrict__ U,
@@ -176,13 +216,13 @@ __global__ void __launch_bounds__(256) k_hmv_rows(MatvecDev mv, T* const* __rest
   using Acc = AccT<T>;
   extern __shared__ __align__(16) unsigned char smraw[];
   Acc* xs = reinterpret_cast<Acc*>(smraw);
-  __shared__ double part[R][4][64];
+  __shared__ double part[R][256];   // [row group][row]
   const int c = blockIdx.x, p = blockIdx.y;
   double* yp = y[p];
   if (!yp) return;
   const double* xp = x[p];
   const int lsz = LSZ > 0 ? LSZ : mv.lsz;
-  const int i = threadIdx.x & 63, g = threadIdx.x >> 6;
+  const int G = 256 / lsz, g = threadIdx.x / lsz, i = threadIdx.x - g * lsz;
   const bool have = D[p] != nullptr && xp != nullptr;
   const int* dptr = trans ? mv.dt_ptr : mv.d_ptr;
   const int* dleaf = trans ? mv.dt_leaf : mv.d_leaf;
@@ -192,8 +232,8 @@ __global__ void __launch_bounds__(256) k_hmv_rows(MatvecDev mv, T* const* __rest
   const int d0 = dptr[c], nd = dptr[c + 1] - d0;
   const int l0 = lptr[c], nlc = lptr[c + 1] - l0;
   const int kc = mv.kc;
-  const int xstride = nd * lsz, tstride = nlc * kc;   // per right-hand side
-  Acc* ts = xs + R * xstride;
+  const int xstride = nd * lsz, tstride = nlc * kc;   // entries per right-hand side
+  Acc* ts = xs + (R * xstride + 3) / 4 * 4;
   // per-leaf descriptors of this chunk, loaded once in parallel
   __shared__ int64_t s_off[MAXQ];
   __shared__ int s_ld[MAXQ], s_k[MAXQ], s_leaf[MAXQ];
@@ -211,7 +251,7 @@ __global__ void __launch_bounds__(256) k_hmv_rows(MatvecDev mv, T* const* __rest
       const int q = e / lsz, j = e - q * lsz;
       const double* src = xp + dcol[d0 + q] + j;
 #pragma unroll
-      for (int rr = 0; rr < R; ++rr) xs[rr * xstride + e] = (Acc)src[rr * vs];
+      for (int rr = 0; rr < R; ++rr) xs[e * R + rr] = (Acc)src[rr * vs];
     }
     const int* sptr = trans ? mv.segt_ptr : mv.seg_ptr;
     const int nseg = trans ? mv.nsegt : mv.nseg;
@@ -228,42 +268,61 @@ __global__ void __launch_bounds__(256) k_hmv_rows(MatvecDev mv, T* const* __rest
           for (int rr = 0; rr < R; ++rr) v[rr] += src[rr];
         }
 #pragma unroll
-      for (int rr = 0; rr < R; ++rr) ts[rr * tstride + e] = (Acc)v[rr];
+      for (int rr = 0; rr < R; ++rr) ts[e * R + rr] = (Acc)v[rr];
     }
   }
   __syncthreads();
   RunSum<Acc> acc[R];
-  if (have && i < lsz) {
+  if (have && g < G) {
     const T* Dp = D[p];
     for (int q = 0; q < nd; ++q) {
-      const T* blk = Dp + (int64_t)(q < MAXQ ? s_leaf[q] : dleaf[d0 + q]) * lsz * lsz;
-      const Acc* xq = xs + q * lsz;
+      const T* blk = Dp + (int64_t)(q < MAXQ ? s_leaf[q] : dleaf[d0 + q]) * lsz * lsz +
+                     (trans ? i * lsz : i);
+      const int cs = trans ? 1 : lsz;   // stride of the contraction
+      const Acc* xq = xs + q * lsz * R;
       Acc sp[R];
 #pragma unroll
-      for (int rr = 0; rr < R; ++rr) sp[rr] = Acc(0);
+      for (int rr = 0; rr < R; ++rr) sp[rr] = acc[rr].begin();
       if (LSZ > 0) {
 #pragma unroll
         for (int t = 0; t < (LSZ > 0 ? LSZ : 64) / 4; ++t) {
           const int j = g + 4 * t;
-          const Acc f = (Acc)ld(blk[trans ? j + i * LSZ : i + j * LSZ]);
+          const Acc f = (Acc)ld(blk[j * cs]);
+          Acc xv[R];
+          ldr<R>(xq + j * R, xv);
 #pragma unroll
-          for (int rr = 0; rr < R; ++rr) sp[rr] += f * xq[rr * xstride + j];
+          for (int rr = 0; rr < R; ++rr) sp[rr] += f * xv[rr];
         }
       } else {
-        for (int j = g; j < lsz; j += 4) {
-          const Acc f = (Acc)ld(blk[trans ? j + (int64_t)i * lsz : i + (int64_t)j * lsz]);
+        for (int j0 = g; j0 < lsz; j0 += 8 * G) {
+          T f[8];
 #pragma unroll
-          for (int rr = 0; rr < R; ++rr) sp[rr] += f * xq[rr * xstride + j];
+          for (int u = 0; u < 8; ++u) f[u] = j0 + G * u < lsz ? blk[(j0 + G * u) * cs] : T(0.f);
+#pragma unroll
+          for (int u = 0; u < 8; ++u) {
+            const int j = j0 + G * u;
+            if (j < lsz) {
+              const Acc w = (Acc)ld(f[u]);
+              Acc xv[R];
+              ldr<R>(xq + j * R, xv);
+#pragma unroll
+              for (int rr = 0; rr < R; ++rr) sp[rr] += w * xv[rr];
+            }
+          }
         }
       }
 #pragma unroll
-      for (int rr = 0; rr < R; ++rr) acc[rr].add(sp[rr]);
+      for (int rr = 0; rr < R; ++rr) acc[rr].end(sp[rr]);
     }
-    // low-rank leaves: thread group g takes leaves g, g+4, ...; all of a
-    // leaf's columns, partial sums of at most 16 products
+    // low-rank leaves: thread group g takes leaves g, g + G, ..., two at a time
+    // (FP64: one), partial sums of at most 4 products
+    constexpr int LH = sizeof(Acc) == 4 ? 2 : 1;
     const T* Fp = trans ? V[p] : U[p];
-    for (int q = g; q < nlc; q += 4) {
-      int k, ldm;
+    auto leaf = [&](int q, int& k, int& ldm, const T*& fb) {
+      k = 0;
+      ldm = 0;
+      fb = Fp;
+      if (q >= nlc) return;
       int64_t off;
       if (q < MAXQ) {
         k = s_k[q]; ldm = s_ld[q]; off = s_off[q];
@@ -273,30 +332,53 @@ __global__ void __launch_bounds__(256) k_hmv_rows(MatvecDev mv, T* const* __rest
         ldm = trans ? mv.lr_n[l] : mv.lr_m[l];
         off = trans ? mv.lr_col0[l] * kc + mv.lt_coloff[l0 + q] : mv.lr_row0[l] * kc + mv.l_rowoff[l0 + q];
       }
-      const T* fb = Fp + off + i;
-      const Acc* tq = ts + q * kc;
-      for (int j0 = 0; j0 < k; j0 += 16) {
-        Acc sp[R];
+      fb = Fp + off + i;
+    };
+    for (int q = g; q < nlc; q += LH * G) {
+      int k[LH], ldm[LH], kmax = 0;
+      const T* fb[LH];
 #pragma unroll
-        for (int rr = 0; rr < R; ++rr) sp[rr] = Acc(0);
-        const int j1 = min(k, j0 + 16);
-        for (int j = j0; j < j1; ++j) {
-          const Acc f = (Acc)ld(fb[(int64_t)j * ldm]);
+      for (int h = 0; h < LH; ++h) {
+        leaf(q + h * G, k[h], ldm[h], fb[h]);
+        kmax = max(kmax, k[h]);
+      }
+      for (int j0 = 0; j0 < kmax; j0 += 4) {
+        T f[LH][4];
 #pragma unroll
-          for (int rr = 0; rr < R; ++rr) sp[rr] += f * tq[rr * tstride + j];
+        for (int h = 0; h < LH; ++h)
+#pragma unroll
+          for (int u = 0; u < 4; ++u)
+            f[h][u] = j0 + u < k[h] ? fb[h][(int64_t)(j0 + u) * ldm[h]] : T(0.f);
+#pragma unroll
+        for (int h = 0; h < LH; ++h) {
+          if (j0 >= k[h]) continue;
+          const Acc* tq = ts + ((q + h * G) * kc + j0) * R;
+          Acc sp[R];
+#pragma unroll
+          for (int rr = 0; rr < R; ++rr) sp[rr] = acc[rr].begin();
+#pragma unroll
+          for (int u = 0; u < 4; ++u) {
+            if (j0 + u < k[h]) {
+              const Acc w = (Acc)ld(f[h][u]);
+              Acc xv[R];
+              ldr<R>(tq + u * R, xv);
+#pragma unroll
+              for (int rr = 0; rr < R; ++rr) sp[rr] += w * xv[rr];
+            }
+          }
+#pragma unroll
+          for (int rr = 0; rr < R; ++rr) acc[rr].end(sp[rr]);
         }
-#pragma unroll
-        for (int rr = 0; rr < R; ++rr) acc[rr].add(sp[rr]);
       }
     }
   }
 #pragma unroll
-  for (int rr = 0; rr < R; ++rr) part[rr][g][i] = acc[rr].value();
+  for (int rr = 0; rr < R; ++rr) part[rr][threadIdx.x] = acc[rr].value();
   __syncthreads();
-  for (int e = threadIdx.x; e < R * 64; e += 256) {
-    const int rr = e >> 6, ii = e & 63;
-    if (ii >= lsz || (R == 1 && e >= 64)) continue;
-    const double sum = part[rr][0][ii] + part[rr][1][ii] + part[rr][2][ii] + part[rr][3][ii];
+  for (int e = threadIdx.x; e < R * lsz; e += 256) {
+    const int rr = R == 1 ? 0 : e / lsz, ii = e - rr * lsz;
+    double sum = 0.0;
+    for (int h = 0; h < G; ++h) sum += part[rr][h * lsz + ii];
     double* yc = yp + rr * vs + (int64_t)c * lsz;
     const double old = (beta != 0.0) ? beta * yc[ii] : 0.0;
     yc[ii] = old + (have ? alpha * sum : 0.0);
@@ -387,6 +469,7 @@ __global__ void __launch_bounds__(256) k_hmv_rows_v1(MatvecDev mv, T* const* __r
   const int rl = tid & 15, cg = tid >> 4;
   if (have) {
     const T* Dp = D[p];
+#pragma unroll 2
     for (int q = 0; q < nd; ++q) {
       const T* blk = Dp + (int64_t)(q < MAXQ ? s_leaf[q] : dleaf[d0 + q]) * 4096;
       const float* xq = xs + q * 64;
@@ -432,12 +515,20 @@ __global__ void __launch_bounds__(256) k_hmv_rows_v1(MatvecDev mv, T* const* __r
       const T* fb = Fp + off + 4 * rl;
       const float* tq = ts + q * kc;
       float sp[4] = {0.f, 0.f, 0.f, 0.f};
-      for (int j = lane >> 4; j < k; j += 2) {
-        float v4[4];
-        load4(fb + (int64_t)j * ldm, v4);
-        const float t = tq[j];
+      for (int j0 = lane >> 4; j0 < k; j0 += 8) {   // 4 loads in flight
+        float v4[4][4];
 #pragma unroll
-        for (int v = 0; v < 4; ++v) sp[v] += v4[v] * t;
+        for (int u = 0; u < 4; ++u) {
+#pragma unroll
+          for (int v = 0; v < 4; ++v) v4[u][v] = 0.f;
+          if (j0 + 2 * u < k) load4(fb + (int64_t)(j0 + 2 * u) * ldm, v4[u]);
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          const float t = j0 + 2 * u < k ? tq[j0 + 2 * u] : 0.f;
+#pragma unroll
+          for (int v = 0; v < 4; ++v) sp[v] += v4[u][v] * t;
+        }
       }
 #pragma unroll
       for (int v = 0; v < 4; ++v) acc[v].add(sp[v]);
@@ -608,18 +699,19 @@ static void hmatvec_r(const MatvecDev& mv, T* const* dense, T* const* U, T* cons
                       cudaStream_t st) {
   using Acc = AccT<T>;
   const size_t sm_rows =
-      ((size_t)mv.max_d * mv.lsz + (size_t)mv.max_l * mv.kc) * R * sizeof(Acc);
+      (((size_t)mv.max_d * mv.lsz + (size_t)mv.max_l * mv.kc) * R + 4) * sizeof(Acc);
+  constexpr size_t most = 180 * 1024 + 4 * sizeof(Acc);
   static bool attr_set = false;   // per instantiation: allow the largest staging buffers
   if (!attr_set) {
     ACR_CUDA(cudaFuncSetAttribute(k_hmv_rows<T, 64, R>,
-                                  cudaFuncAttributeMaxDynamicSharedMemorySize, 180 * 1024));
+                                  cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most));
     ACR_CUDA(cudaFuncSetAttribute(k_hmv_rows<T, 0, R>,
-                                  cudaFuncAttributeMaxDynamicSharedMemorySize, 180 * 1024));
+                                  cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most));
     attr_set = true;
   }
   if (mv.max_l > MAXQ || mv.lsz > 64)
     throw CudaError{cudaErrorInvalidConfiguration, "more low-rank leaves per chunk than staged"};
-  if (sm_rows > 180 * 1024)
+  if (sm_rows > most)
     throw CudaError{cudaErrorInvalidConfiguration, "apply staging exceeds shared memory"};
   if (mv.nl > 0)
     launch_chain(k_lr_proj<T, R>, dim3(mv.nchunks, P), 256, 0, st, mv, U, V, rank, x, tv, trans, vs);
