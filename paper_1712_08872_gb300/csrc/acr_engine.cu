@@ -2214,8 +2214,7 @@ acr_status acr_spmv(const acr_grid* grid, const double* coef, const double* x, d
                     int32_t nrhs, cudaStream_t stream) {
   if (!grid_ok(grid) || !coef || !x || !y || nrhs < 1) return ACR_ERR_INVALID_ARG;
   return guarded([&] {
-    const int64_t N = (int64_t)grid->nx * grid->nx * grid->nx;
-    for (int k = 0; k < nrhs; ++k) acr::launch_spmv(coef, x + k * N, y + k * N, grid->nx, stream);
+    acr::launch_spmv(coef, x, y, grid->nx, stream, nrhs);
     return 0;
   });
 }

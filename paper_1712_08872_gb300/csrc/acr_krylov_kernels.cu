@@ -14,109 +14,139 @@ namespace {
 constexpr int RB = 256;      // threads per reduction block
 constexpr int RBLK = 592;    // partial sums per vector (4 per SM)
 
-// coefficient layout: [c | w | e | s | n | b | t], N each
-__global__ void k_stencil_poisson(const double* __restrict__ kap, double* __restrict__ coef, int n) {
-  const int64_t N = (int64_t)n * n * n;
-  const double h = 1.0 / (n + 1), ih2 = 1.0 / (h * h);
-  for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < N;
-       p += (int64_t)gridDim.x * blockDim.x) {
-    const int ix = (int)(p % n), iy = (int)((p / n) % n), iz = (int)(p / ((int64_t)n * n));
-    const double kp = kap[p];
-    const int64_t nb[6] = {p - 1, p + 1, p - n, p + n, p - (int64_t)n * n, p + (int64_t)n * n};
-    const bool in[6] = {ix > 0, ix < n - 1, iy > 0, iy < n - 1, iz > 0, iz < n - 1};
-    double c = 0.0;
-#pragma unroll
-    for (int d = 0; d < 6; ++d) {
-      double kf;
-      if (in[d]) {
-        const double kq = kap[nb[d]];
-        kf = 2.0 * kp * kq / (kp + kq);
-      } else {
-        kf = kp;
-      }
-      c += kf * ih2;
-      coef[(d + 1) * N + p] = in[d] ? -kf * ih2 : 0.0;
-    }
-    coef[p] = c;
-  }
+// The point kernels: CTA (x, y) takes 256 points of plane y % n, so that a point's
+// place needs one 32-bit division (with a flat 64-bit index, three 64-bit ones cost
+// more than the point's arithmetic).
+struct Point {
+  int ix, iy, iz;
+  int64_t p;
+  bool in;
+};
+__device__ __forceinline__ Point point_of(int n) {
+  Point q;
+  const unsigned e = blockIdx.x * 256u + threadIdx.x;
+  q.in = e < (unsigned)n * n;
+  q.iy = (int)(e / (unsigned)n);
+  q.ix = (int)(e - (unsigned)q.iy * n);
+  q.iz = (int)(blockIdx.y % (unsigned)n);
+  q.p = (int64_t)q.iz * n * n + e;
+  return q;
+}
+inline dim3 point_grid(int n, int groups = 1) {
+  return dim3((unsigned)(((int64_t)n * n + 255) / 256), (unsigned)n * groups);
 }
 
-__global__ void k_stencil_codi(const double* __restrict__ beta, double* __restrict__ coef, int n) {
-  const int64_t N = (int64_t)n * n * n;
-  const double h = 1.0 / (n + 1), ih2 = 1.0 / (h * h), ih = 1.0 / h;
-  for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < N;
-       p += (int64_t)gridDim.x * blockDim.x) {
-    const int ix = (int)(p % n), iy = (int)((p / n) % n), iz = (int)(p / ((int64_t)n * n));
-    const bool in[6] = {ix > 0, ix < n - 1, iy > 0, iy < n - 1, iz > 0, iz < n - 1};
-    double c = 6.0 * ih2;
+// coefficient layout: [c | w | e | s | n | b | t], N each
+__global__ void __launch_bounds__(256) k_stencil_poisson(const double* __restrict__ kap,
+                                                         double* __restrict__ coef, int n,
+                                                         double ih2) {
+  const Point q = point_of(n);
+  if (!q.in) return;
+  const int64_t N = (int64_t)n * n * n, p = q.p;
+  const double kp = kap[p];
+  const int64_t nb[6] = {p - 1, p + 1, p - n, p + n, p - (int64_t)n * n, p + (int64_t)n * n};
+  const bool in[6] = {q.ix > 0, q.ix < n - 1, q.iy > 0, q.iy < n - 1, q.iz > 0, q.iz < n - 1};
+  double c = 0.0;
 #pragma unroll
-    for (int a = 0; a < 3; ++a) {
-      const double b = beta[a * N + p];
-      c += fabs(b) * ih;
-      const double lo = -ih2 - fmax(b, 0.0) * ih;   // upstream for b > 0
-      const double hi = -ih2 + fmin(b, 0.0) * ih;   // upstream for b < 0
-      coef[(2 * a + 1) * N + p] = in[2 * a] ? lo : 0.0;
-      coef[(2 * a + 2) * N + p] = in[2 * a + 1] ? hi : 0.0;
+  for (int d = 0; d < 6; ++d) {
+    double kf;
+    if (in[d]) {
+      const double kq = kap[nb[d]];
+      kf = 2.0 * kp * kq / (kp + kq);
+    } else {
+      kf = kp;
     }
-    coef[p] = c;
+    c += kf * ih2;
+    coef[(d + 1) * N + p] = in[d] ? -kf * ih2 : 0.0;
   }
+  coef[p] = c;
+}
+
+// (the FP64 pipe bounds it before memory does: three multiply-adds per axis, the
+// upwind choice by the sign bit instead of FP64 comparisons)
+__global__ void __launch_bounds__(256) k_stencil_codi(const double* __restrict__ beta,
+                                                      double* __restrict__ coef, int n,
+                                                      double ih2, double ih) {
+  const Point q = point_of(n);
+  if (!q.in) return;
+  const int64_t N = (int64_t)n * n * n, p = q.p;
+  const bool in[6] = {q.ix > 0, q.ix < n - 1, q.iy > 0, q.iy < n - 1, q.iz > 0, q.iz < n - 1};
+  double c = 6.0 * ih2;
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    const double b = beta[a * N + p];
+    const bool neg = __double2hiint(b) < 0;
+    c += fabs(b) * ih;
+    const double lo = -ih2 - (neg ? 0.0 : b) * ih;   // upstream for b > 0
+    const double hi = -ih2 + (neg ? b : 0.0) * ih;   // upstream for b < 0
+    coef[(2 * a + 1) * N + p] = in[2 * a] ? lo : 0.0;
+    coef[(2 * a + 2) * N + p] = in[2 * a + 1] ? hi : 0.0;
+  }
+  coef[p] = c;
 }
 
 // Sec. 8 Eq. (HelmVarVel) with the 7-point Laplacian: -Lap u - sigma u,
 // sigma = (omega / c)^2 per node
-__global__ void k_stencil_helmholtz(const double* __restrict__ sigma, double* __restrict__ coef,
-                                    int n) {
-  const int64_t N = (int64_t)n * n * n;
-  const double h = 1.0 / (n + 1), ih2 = 1.0 / (h * h);
-  for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < N;
-       p += (int64_t)gridDim.x * blockDim.x) {
-    const int ix = (int)(p % n), iy = (int)((p / n) % n), iz = (int)(p / ((int64_t)n * n));
-    const bool in[6] = {ix > 0, ix < n - 1, iy > 0, iy < n - 1, iz > 0, iz < n - 1};
+__global__ void __launch_bounds__(256) k_stencil_helmholtz(const double* __restrict__ sigma,
+                                                           double* __restrict__ coef, int n,
+                                                           double ih2) {
+  const Point q = point_of(n);
+  if (!q.in) return;
+  const int64_t N = (int64_t)n * n * n, p = q.p;
+  const bool in[6] = {q.ix > 0, q.ix < n - 1, q.iy > 0, q.iy < n - 1, q.iz > 0, q.iz < n - 1};
 #pragma unroll
-    for (int d = 0; d < 6; ++d) coef[(d + 1) * N + p] = in[d] ? -ih2 : 0.0;
-    coef[p] = 6.0 * ih2 - sigma[p];
-  }
+  for (int d = 0; d < 6; ++d) coef[(d + 1) * N + p] = in[d] ? -ih2 : 0.0;
+  coef[p] = 6.0 * ih2 - sigma[p];
 }
 
-// y = A x; vector blockIdx.y of a batch sits blockIdx.y * N doubles further
-__global__ void k_spmv(const double* __restrict__ coef, const double* __restrict__ x,
-                       double* __restrict__ y, int n) {
-  const int64_t N = (int64_t)n * n * n;
-  const int64_t n2 = (int64_t)n * n;
-  x += blockIdx.y * N;
-  y += blockIdx.y * N;
-  for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < N;
-       p += (int64_t)gridDim.x * blockDim.x) {
-    const int ix = (int)(p % n), iy = (int)((p / n) % n), iz = (int)(p / n2);
-    double s = coef[p] * x[p];
-    if (ix > 0) s += coef[N + p] * x[p - 1];
-    if (ix < n - 1) s += coef[2 * N + p] * x[p + 1];
-    if (iy > 0) s += coef[3 * N + p] * x[p - n];
-    if (iy < n - 1) s += coef[4 * N + p] * x[p + n];
-    if (iz > 0) s += coef[5 * N + p] * x[p - n2];
-    if (iz < n - 1) s += coef[6 * N + p] * x[p + n2];
-    y[p] = s;
-  }
+// y = A x for R vectors at a time, N doubles apart (group blockIdx.y / n of
+// them): the seven coefficients are read once per group.  Seven FP64 multiply-adds
+// per point and vector bound it for R > 1 (23 us per vector at n = 127 on this
+// part's narrow FP64 pipe, 21 us of memory time for one vector alone).
+template <int R>
+__global__ void __launch_bounds__(256) k_spmv(const double* __restrict__ coef,
+                                              const double* __restrict__ x,
+                                              double* __restrict__ y, int n) {
+  const Point q = point_of(n);
+  if (!q.in) return;
+  const int64_t N = (int64_t)n * n * n, n2 = (int64_t)n * n, p = q.p;
+  const int64_t o = (int64_t)(blockIdx.y / (unsigned)n) * R * N;
+  double s[R];
+  auto add = [&](int d, int64_t off, bool in) {
+    if (!in) return;
+    const double a = coef[d * N + p];
+#pragma unroll
+    for (int r = 0; r < R; ++r) s[r] += a * x[o + r * N + p + off];
+  };
+  const double c = coef[p];
+#pragma unroll
+  for (int r = 0; r < R; ++r) s[r] = c * x[o + r * N + p];
+  add(1, -1, q.ix > 0);
+  add(2, 1, q.ix < n - 1);
+  add(3, -n, q.iy > 0);
+  add(4, n, q.iy < n - 1);
+  add(5, -n2, q.iz > 0);
+  add(6, n2, q.iz < n - 1);
+#pragma unroll
+  for (int r = 0; r < R; ++r) y[o + r * N + p] = s[r];
 }
 
 // y = A^T x: row p of A^T holds the coefficients that point at p from its
 // neighbours (the east coefficient of p-1, the west one of p+1, ...)
-__global__ void k_spmv_transpose(const double* __restrict__ coef, const double* __restrict__ x,
-                                 double* __restrict__ y, int n) {
-  const int64_t N = (int64_t)n * n * n;
-  const int64_t n2 = (int64_t)n * n;
-  for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < N;
-       p += (int64_t)gridDim.x * blockDim.x) {
-    const int ix = (int)(p % n), iy = (int)((p / n) % n), iz = (int)(p / n2);
-    double s = coef[p] * x[p];
-    if (ix > 0) s += coef[2 * N + p - 1] * x[p - 1];
-    if (ix < n - 1) s += coef[N + p + 1] * x[p + 1];
-    if (iy > 0) s += coef[4 * N + p - n] * x[p - n];
-    if (iy < n - 1) s += coef[3 * N + p + n] * x[p + n];
-    if (iz > 0) s += coef[6 * N + p - n2] * x[p - n2];
-    if (iz < n - 1) s += coef[5 * N + p + n2] * x[p + n2];
-    y[p] = s;
-  }
+__global__ void __launch_bounds__(256) k_spmv_transpose(const double* __restrict__ coef,
+                                                        const double* __restrict__ x,
+                                                        double* __restrict__ y, int n) {
+  const Point q = point_of(n);
+  if (!q.in) return;
+  const int64_t N = (int64_t)n * n * n, n2 = (int64_t)n * n, p = q.p;
+  double s = coef[p] * x[p];
+  if (q.ix > 0) s += coef[2 * N + p - 1] * x[p - 1];
+  if (q.ix < n - 1) s += coef[N + p + 1] * x[p + 1];
+  if (q.iy > 0) s += coef[4 * N + p - n] * x[p - n];
+  if (q.iy < n - 1) s += coef[3 * N + p + n] * x[p + n];
+  if (q.iz > 0) s += coef[6 * N + p - n2] * x[p - n2];
+  if (q.iz < n - 1) s += coef[5 * N + p + n2] * x[p + n2];
+  y[p] = s;
 }
 
 // grad_p = -lambda^T (dA/dkappa_p) u for the harmonic-mean Poisson stencil:
@@ -263,25 +293,48 @@ inline int grid_for(int64_t N) {
 
 }  // namespace
 
+// 1/h and 1/h^2 of the grid (here, not in every thread: FP64 divisions)
+static double inv_h(int n) { return 1.0 / (1.0 / (n + 1)); }
+static double inv_h2(int n) {
+  const double h = 1.0 / (n + 1);
+  return 1.0 / (h * h);
+}
+
 void launch_stencil_poisson(const double* kappa, double* coef, int n, cudaStream_t st) {
-  k_stencil_poisson<<<grid_for((int64_t)n * n * n), 256, 0, st>>>(kappa, coef, n);
+  k_stencil_poisson<<<point_grid(n), 256, 0, st>>>(kappa, coef, n, inv_h2(n));
   ACR_LAUNCHED(1);
 }
 
 void launch_stencil_codi(const double* beta, double* coef, int n, cudaStream_t st) {
-  k_stencil_codi<<<grid_for((int64_t)n * n * n), 256, 0, st>>>(beta, coef, n);
+  k_stencil_codi<<<point_grid(n), 256, 0, st>>>(beta, coef, n, inv_h2(n), inv_h(n));
   ACR_LAUNCHED(1);
 }
 
 void launch_stencil_helmholtz(const double* sigma, double* coef, int n, cudaStream_t st) {
-  k_stencil_helmholtz<<<grid_for((int64_t)n * n * n), 256, 0, st>>>(sigma, coef, n);
+  k_stencil_helmholtz<<<point_grid(n), 256, 0, st>>>(sigma, coef, n, inv_h2(n));
   ACR_LAUNCHED(1);
 }
 
 void launch_spmv(const double* coef, const double* x, double* y, int n, cudaStream_t st,
                  int nr) {
-  if (nr < 1) return;
-  k_spmv<<<dim3(grid_for((int64_t)n * n * n), nr), 256, 0, st>>>(coef, x, y, n);
+  const int64_t N = (int64_t)n * n * n;
+  // groups of 4 vectors (at most 16 groups in a launch: its rows of CTAs), then 2, then 1
+  while (nr > 0) {
+    const int g = std::min(nr / 4, 16);
+    const int r = g > 0 ? 4 * g : nr >= 2 ? 2 : 1;
+    if (g > 0) k_spmv<4><<<point_grid(n, g), 256, 0, st>>>(coef, x, y, n);
+    else if (r == 2) k_spmv<2><<<point_grid(n), 256, 0, st>>>(coef, x, y, n);
+    else k_spmv<1><<<point_grid(n), 256, 0, st>>>(coef, x, y, n);
+    ACR_LAUNCHED(1);
+    x += r * N;
+    y += r * N;
+    nr -= r;
+  }
+}
+
+void launch_spmv_transpose(const double* coef, const double* x, double* y, int n,
+                           cudaStream_t st) {
+  k_spmv_transpose<<<point_grid(n), 256, 0, st>>>(coef, x, y, n);
   ACR_LAUNCHED(1);
 }
 
@@ -308,12 +361,6 @@ void launch_baxpby(double* Y, const double* X, const double* a, double b, int64_
   if (nr <= 0) return;
   k_baxpby<<<dim3(std::max(1, grid_for(N) / std::max(1, nr / 4)), nr), 256, 0, st>>>(
       Y, X, a, b, ldr, N);
-  ACR_LAUNCHED(1);
-}
-
-void launch_spmv_transpose(const double* coef, const double* x, double* y, int n,
-                           cudaStream_t st) {
-  k_spmv_transpose<<<grid_for((int64_t)n * n * n), 256, 0, st>>>(coef, x, y, n);
   ACR_LAUNCHED(1);
 }
 
