@@ -1916,6 +1916,147 @@ int run_gmres(Krylov& K, int m, double rtol, int maxit, const double* f, double*
   return status;
 }
 
+// The iteration of run_pcg for nr right-hand sides of the same operator in
+// lockstep: each system has its own scalars; the SpMVs, dots, updates and
+// preconditioner applies of all run in single launches, and the applies share
+// passes over the factors (one system after another, 8 systems read them 8
+// times).  A system that has converged or broken down is frozen (its step is 0).
+int run_pcg_batch(Krylov& K, double rtol, int maxit, const double* f, double* u, int nr,
+                  acr_solve_info* info) {
+  const int64_t N = K.N, RN = (int64_t)nr * N;
+  double* R = K.dbuf(2 * RN);        // residuals, then the step before's
+  double* Z = K.dbuf(RN);
+  double* Pv = K.dbuf(RN);
+  double* Q = K.dbuf(RN);
+  double* part = K.dbuf((size_t)600 * 2 * nr);
+  double* dout = K.dbuf((size_t)3 * nr);
+  double* dco = K.dbuf(nr);
+  std::vector<double> h((size_t)3 * nr), co(nr);
+  auto fetch = [&](int cnt) {
+    ACR_CUDA(cudaMemcpyAsync(h.data(), dout, cnt * sizeof(double), cudaMemcpyDeviceToHost, K.st));
+    ACR_CUDA(cudaStreamSynchronize(K.st));
+  };
+  auto put = [&](const std::vector<double>& v) {
+    ACR_CUDA(cudaMemcpyAsync(dco, v.data(), nr * sizeof(double), cudaMemcpyHostToDevice, K.st));
+  };
+  // <X_r, Y_r> to dout[off + r]
+  auto dot = [&](const double* X, const double* Y, int off) {
+    launch_bmultidot(X, 0, N, 1, Y, N, nr, part, dout + off, K.st);
+  };
+  auto residual = [&]() {   // R = f - A u
+    launch_spmv(K.coef, u, Q, K.n, K.st, nr);
+    ACR_CUDA(cudaMemcpyAsync(R, f, RN * sizeof(double), cudaMemcpyDeviceToDevice, K.st));
+    std::fill(co.begin(), co.end(), 1.0);
+    put(co);
+    launch_bmultiaxpy(R, Q, 0, N, 1, dco, -1.0, N, nr, K.st);
+  };
+  // a system that broke down may hold NaN directions: none of its own from here on
+  auto still = [&](int r) {
+    ACR_CUDA(cudaMemsetAsync(Pv + r * N, 0, N * sizeof(double), K.st));
+    ACR_CUDA(cudaMemsetAsync(Q + r * N, 0, N * sizeof(double), K.st));
+  };
+  std::vector<double> nf(nr), res(nr, 0.0), rz(nr, 0.0), alpha(nr), beta(nr);
+  std::vector<int> its(nr, 0), status(nr, S_OK);
+  std::vector<char> done(nr, 0);
+  dot(f, f, 0);
+  fetch(nr);
+  for (int r = 0; r < nr; ++r) {
+    nf[r] = std::sqrt(std::max(h[r], 0.0));
+    if (nf[r] == 0.0) {
+      ACR_CUDA(cudaMemsetAsync(u + r * N, 0, N * sizeof(double), K.st));
+      done[r] = 1;
+    }
+  }
+  residual();
+  dot(R, R, 0);
+  fetch(nr);
+  bool any = false;
+  for (int r = 0; r < nr; ++r) {
+    if (done[r]) continue;
+    res[r] = std::sqrt(std::max(h[r], 0.0)) / nf[r];
+    if (res[r] <= rtol) done[r] = 1;
+    else any = true;
+  }
+  if (any) {
+    K.E->apply(R, Z, false, K.st, nr);
+    ACR_CUDA(cudaMemcpyAsync(Pv, Z, RN * sizeof(double), cudaMemcpyDeviceToDevice, K.st));
+    dot(R, Z, 0);
+    fetch(nr);
+    for (int r = 0; r < nr; ++r) {
+      rz[r] = h[r];
+      if (!done[r]) status[r] = S_NOT_CONVERGED;
+    }
+    for (int it = 1; it <= maxit && any; ++it) {
+      launch_spmv(K.coef, Pv, Q, K.n, K.st, nr);
+      dot(Pv, Q, 0);
+      fetch(nr);
+      for (int r = 0; r < nr; ++r) {
+        alpha[r] = 0.0;
+        if (done[r]) continue;
+        its[r] = it;
+        if (!std::isfinite(h[r]) || h[r] == 0.0) {
+          status[r] = S_BREAKDOWN;
+          done[r] = 1;
+          still(r);
+        } else {
+          alpha[r] = rz[r] / h[r];
+        }
+      }
+      put(alpha);
+      launch_bmultiaxpy(u, Pv, 0, N, 1, dco, 1.0, N, nr, K.st);
+      ACR_CUDA(cudaMemcpyAsync(R + RN, R, RN * sizeof(double), cudaMemcpyDeviceToDevice, K.st));
+      launch_bmultiaxpy(R, Q, 0, N, 1, dco, -1.0, N, nr, K.st);
+      K.E->apply(R, Z, false, K.st, nr);
+      launch_bmultidot(R, RN, N, 2, Z, N, nr, part, dout, K.st);   // <r, z>, <rold, z>
+      dot(R, R, 2 * nr);
+      fetch(3 * nr);
+      any = false;
+      for (int r = 0; r < nr; ++r) {
+        beta[r] = 0.0;
+        if (done[r]) continue;
+        res[r] = std::sqrt(std::max(h[2 * nr + r], 0.0)) / nf[r];
+        const double zr = h[2 * r], zro = h[2 * r + 1];
+        if (res[r] <= rtol) {
+          status[r] = S_OK;
+          done[r] = 1;
+        } else if (!std::isfinite(zr) || rz[r] == 0.0) {
+          status[r] = S_BREAKDOWN;
+          done[r] = 1;
+          still(r);
+        } else {
+          beta[r] = (zr - zro) / rz[r];
+          rz[r] = zr;
+          any = true;
+        }
+      }
+      if (!any) break;
+      put(beta);
+      launch_bmultiaxpy(Z, Pv, 0, N, 1, dco, 1.0, N, nr, K.st);   // z + beta p
+      std::swap(Z, Pv);
+      for (int r = 0; r < nr; ++r)
+        if (status[r] == S_BREAKDOWN) still(r);
+    }
+  }
+  // true residuals
+  residual();
+  dot(R, R, 0);
+  fetch(nr);
+  int s = S_OK;
+  acr_solve_info agg{};
+  agg.converged = 1;
+  for (int r = 0; r < nr; ++r) {
+    if (nf[r] != 0.0) res[r] = std::sqrt(std::max(h[r], 0.0)) / nf[r];
+    if (status[r] == S_OK && !(res[r] <= rtol * 1.0000001)) status[r] = S_NOT_CONVERGED;
+    if (status[r] == S_BREAKDOWN) s = S_BREAKDOWN;
+    else if (status[r] != S_OK && s == S_OK) s = status[r];
+    agg.iterations = std::max(agg.iterations, its[r]);
+    agg.rel_residual = std::max(agg.rel_residual, res[r]);
+    agg.converged &= status[r] == S_OK;
+  }
+  if (info) *info = agg;
+  return s;
+}
+
 // GMRES(m) for nr right-hand sides of the same operator in lockstep: every
 // system keeps its own Arnoldi basis, Hessenberg matrix and Givens rotations
 // (the iteration of run_gmres), while each step's preconditioner applies
@@ -2293,17 +2434,8 @@ static acr_status krylov_common(acr::EngineBase* E, const acr_grid* grid, const 
     if (nrhs > 1 && method == ACR_GMRES) {
       s = acr::run_gmres_batch(K, restart, rtol, maxit, f, u, nrhs, info);
     } else if (nrhs > 1) {
-      // PCG: one system after another; info reports the largest count and residual
-      acr_solve_info one{}, agg{};
-      agg.converged = 1;
-      for (int r = 0; r < nrhs && s != acr::S_BREAKDOWN; ++r) {
-        const int sr = acr::run_pcg(K, rtol, maxit, f + r * K.N, u + r * K.N, &one);
-        if (sr != acr::S_OK && s == acr::S_OK) s = sr;
-        agg.iterations = std::max(agg.iterations, one.iterations);
-        agg.rel_residual = std::max(agg.rel_residual, one.rel_residual);
-        agg.converged &= one.converged;
-      }
-      if (info) *info = agg;
+      // PCG: info reports the largest count and residual
+      s = acr::run_pcg_batch(K, rtol, maxit, f, u, nrhs, info);
     } else {
       s = method == ACR_PCG ? acr::run_pcg(K, rtol, maxit, f, u, info)
                             : acr::run_gmres(K, restart, rtol, maxit, f, u, info);
