@@ -2,7 +2,7 @@
 // acr_gemm_kernels.cu and the recompression cores of acr_core_kernels.cu:
 //  * k_pchol   -- pivoted Cholesky of a sketch Gram (FP64 factors): orthonormal
 //                 basis transform of the range finder;
-//  * k_leaf_inv-- Gauss-Jordan inverse with partial pivoting of a dense
+//  * k_leaf_inv_d, k_leaf_inv_f -- Gauss-Jordan inverse with partial pivoting of a dense
 //                 diagonal leaf (the leaves of the recursive H-inverse): FP64,
 //                 or for float storage float elimination refined to float
 //                 accuracy (FP64 when refinement cannot get there);
@@ -436,15 +436,6 @@ __device__ void leaf_inv_fp64(T* __restrict__ Ap, int n, double (*A)[CMAX + 1], 
   if (flops && threadIdx.x == 0) atomicAdd(flops, 2.0 * n * n * n);
 }
 
-template <typename T>
-__global__ void __launch_bounds__(NT) k_leaf_inv(T* const* __restrict__ dense, int64_t off, int n,
-                                                 int* err, double* __restrict__ flops) {
-  T* Ap = dense[blockIdx.x];
-  if (!Ap) return;
-  __shared__ double A[CMAX][CMAX + 1];
-  leaf_inv_fp64<T, NT>(Ap + off, n, A, err, flops);
-}
-
 template <int TH>
 __device__ __forceinline__ float block_absmaxf(float v, float* red8) {
 #pragma unroll
@@ -706,6 +697,166 @@ __global__ void __cluster_dims__(LCL, 1, 1) __launch_bounds__(LTH)
   leaf_inv_fp64<float, LTH>(Ap, n, reinterpret_cast<double (*)[CMAX + 1]>(lsm), err, flops);
 }
 
+// Leaf inverse of FP64 storage: the same elimination (rows never moved, panels of 8
+// columns) in FP64.  The 64^3 multiply-adds alone take one SM's FP64 pipe 63 us
+// (two lanes per clock), so a cluster of LCL CTAs shares a leaf by columns: the
+// owner of a panel eliminates it in one warp's registers and pushes it to every CTA, and
+// after one cluster barrier each updates its own 8 columns.  64 x 64 leaf: 123 us
+// against 219 us in one CTA.
+__global__ void __cluster_dims__(LCL, 1, 1) __launch_bounds__(128)
+    k_leaf_inv_d(double* const* __restrict__ dense, int64_t off, int n, int* err,
+                 double* __restrict__ flops) {
+  constexpr int TH = 128;
+  double* Ap = dense[blockIdx.x / LCL];
+  if (!Ap) return;   // the whole cluster
+  Ap += off;
+  cg::cluster_group cl = cg::this_cluster();
+  const int rank = (int)cl.block_rank();
+  __shared__ double X[CMAX][LPW + 1];            // this CTA's columns
+  __shared__ double Pn[2][CMAX][LPW + 1];        // the panel, by parity
+  __shared__ double xq[LPW][LPW];                // the pivot rows' old entries of X
+  __shared__ int piv[CMAX], step[CMAX];          // row of each step's pivot; step of each row
+  __shared__ int s_ok[2];
+  __shared__ double s_max[LCL][2];               // per CTA: largest entry of A, of the inverse
+  __shared__ double red8[TH / 32];
+  const int tid = threadIdx.x, lane = tid & 31;
+  const int i = tid & 63, jh = 4 * (tid >> 6), c0 = LPW * rank;
+  double amax = 0.0;
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    const int j = c0 + jh + q;
+    const double v = (i < n && j < n) ? Ap[i + (int64_t)j * n] : 0.0;
+    X[i][jh + q] = v;
+    amax = fmax(amax, fabs(v));
+  }
+  if (tid < CMAX) step[tid] = -1;
+  amax = block_absmax<TH>(amax, red8);
+  unsigned used = 0;   // warp 0: rows lane, lane + 32 that have been pivots
+  int buf = 0;
+  for (int kb = 0; kb < n; kb += LPW, buf ^= 1) {
+    const int kw = min(LPW, n - kb);
+    if (rank == kb / LPW) {
+      if (tid < 32) {
+        // (rows that were pivots of earlier panels)
+        used = (step[lane] >= 0 ? 1u : 0u) | (step[lane + 32] >= 0 ? 2u : 0u);
+        double x0[LPW], x1[LPW];
+        int pv[LPW], ok = 1;
+#pragma unroll
+        for (int c = 0; c < LPW; ++c) { x0[c] = X[lane][c]; x1[c] = X[lane + 32][c]; }
+#pragma unroll
+        for (int t = 0; t < LPW; ++t) {
+          pv[t] = -1;
+          if (t < kw) {
+            // the largest remaining |entry| by its upper bits (entries that agree to
+            // 2^-14 count as equal: the lowest row)
+            const unsigned h0 = (unsigned)__double2hiint(fabs(x0[t]));
+            const unsigned h1 = (unsigned)__double2hiint(fabs(x1[t]));
+            const unsigned b0 = (used & 1u) ? 0u : ((h0 & ~63u) | (63u - lane));
+            const unsigned b1 = (used & 2u) ? 0u : ((h1 & ~63u) | (31u - lane));
+            const unsigned best = __reduce_max_sync(0xffffffffu, max(b0, b1));
+            const int q = 63 - (int)(best & 63u);
+            if ((best & ~63u) == 0u) ok = 0;
+            const bool hi = q >= 32;
+            double v[LPW];
+#pragma unroll
+            for (int c = 0; c < LPW; ++c) v[c] = __shfl_sync(0xffffffffu, hi ? x1[c] : x0[c], q & 31);
+            const double pinv = 1.0 / v[t];
+            const bool p0 = lane == q, p1 = lane + 32 == q;
+            used |= (p0 ? 1u : 0u) | (p1 ? 2u : 0u);
+            pv[t] = q;
+            const double f0 = x0[t], f1 = x1[t];
+#pragma unroll
+            for (int c = 0; c < LPW; ++c) {
+              const double w = c == t ? pinv : v[c] * pinv;
+              x0[c] = p0 ? w : (c == t ? -f0 * pinv : fma(-f0, w, x0[c]));
+              x1[c] = p1 ? w : (c == t ? -f1 * pinv : fma(-f1, w, x1[c]));
+            }
+          }
+        }
+#pragma unroll
+        for (int c = 0; c < LPW; ++c) {
+          X[lane][c] = x0[c];
+          X[lane + 32][c] = x1[c];
+          Pn[buf][lane][c] = x0[c];
+          Pn[buf][lane + 32][c] = x1[c];
+        }
+        if (lane < LCL) {   // pivots and outcome to every CTA
+          int* dp = cl.map_shared_rank(piv, lane);
+          int* ds = cl.map_shared_rank(step, lane);
+          int* dk = cl.map_shared_rank(s_ok, lane);
+#pragma unroll
+          for (int t = 0; t < LPW; ++t)
+            if (pv[t] >= 0) {
+              dp[kb + t] = pv[t];
+              ds[pv[t]] = kb + t;
+            }
+          dk[buf] = ok;
+        }
+      }
+      __syncthreads();
+      for (int c = 0; c < LCL; ++c) {
+        if (c == rank) continue;
+        double* d = cl.map_shared_rank(&Pn[buf][0][0], c);
+        for (int e = tid; e < CMAX * (LPW + 1); e += TH) d[e] = (&Pn[buf][0][0])[e];
+      }
+    }
+    cl.sync();   // the panel is everywhere; everyone is done with the one before
+    if (!s_ok[buf]) {
+      if (rank == 0 && tid == 0) atomicOr(err, ERR_PIVOT);
+      cl.sync();
+      return;
+    }
+    if (rank != kb / LPW) {
+      if (tid < LPW * LPW)
+        xq[tid >> 3][tid & 7] = (tid >> 3) < kw ? X[piv[kb + (tid >> 3)]][tid & 7] : 0.0;
+      __syncthreads();
+      const int st = step[i];
+      const bool pivot = st >= kb && st < kb + LPW;
+      double y[4];
+#pragma unroll
+      for (int q = 0; q < 4; ++q) y[q] = pivot ? 0.0 : X[i][jh + q];
+#pragma unroll
+      for (int t = 0; t < LPW; ++t) {
+        const double pr = t < kw ? Pn[buf][i][t] : 0.0;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) y[q] = fma(pr, xq[t][jh + q], y[q]);
+      }
+#pragma unroll
+      for (int q = 0; q < 4; ++q) X[i][jh + q] = y[q];
+    }
+    __syncthreads();
+  }
+  // pivot growth of the computed inverse (a NaN or Inf entry fails too)
+  double xmax = 0.0;
+#pragma unroll
+  for (int q = 0; q < 4; ++q)
+    if (i < n && c0 + jh + q < n) {
+      const double v = fabs(X[i][jh + q]);
+      xmax = (v <= 1.7976931348623157e308) ? fmax(xmax, v) : INFINITY;
+    }
+  xmax = block_absmax<TH>(xmax, red8);
+  if (tid < LCL) {
+    double* d = cl.map_shared_rank(&s_max[rank][0], tid);
+    d[0] = amax;
+    d[1] = xmax;
+  }
+  cl.sync();
+  for (int c = 0; c < LCL; ++c) {
+    amax = fmax(amax, s_max[c][0]);
+    xmax = fmax(xmax, s_max[c][1]);
+  }
+  if (!(amax * xmax <= leaf_growth_max<double>())) {
+    if (rank == 0 && tid == 0) atomicOr(err, ERR_GROWTH);
+    return;
+  }
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    const int c = c0 + jh + q;
+    if (i < n && c < n) Ap[step[i] + (int64_t)piv[c] * n] = X[i][jh + q];
+  }
+  if (flops && rank == 0 && tid == 0) atomicAdd(flops, 2.0 * n * n * n);
+}
+
 // out = sgn * diag(r) X diag(c): dense part
 template <typename T>
 __global__ void k_hscale_dense(T* const* __restrict__ od, T* const* __restrict__ xd,
@@ -851,7 +1002,7 @@ void launch_leaf_inv(T* const* d_dense, int64_t off, int lsz, int P, int* d_err,
   if constexpr (std::is_same<T, float>::value) {
     k_leaf_inv_f<<<P * LCL, LTH, 0, st>>>(d_dense, off, lsz, d_err, d_fl, d_fallbacks);
   } else {
-    k_leaf_inv<T><<<P, NT, 0, st>>>(d_dense, off, lsz, d_err, d_fl);
+    k_leaf_inv_d<<<P * LCL, 128, 0, st>>>(d_dense, off, lsz, d_err, d_fl);
   }
   ACR_LAUNCHED(1);
 }
