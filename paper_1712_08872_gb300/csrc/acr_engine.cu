@@ -393,13 +393,15 @@ class Engine : public EngineBase {
   cudaEvent_t ev0 = nullptr, ev1 = nullptr;
   // apply work
   double *Fv = nullptr, *Gv = nullptr, *Uv = nullptr, *Tv = nullptr, *tvscr = nullptr;
-  // 32 right-hand sides per pass on the tensor cores (allocated on first use)
+  // 32 right-hand sides per pass (allocated on first use)
   double *Fw = nullptr, *Gw = nullptr, *Uw = nullptr, *Tw = nullptr, *tvw = nullptr;
+  float* xtw = nullptr;              // the vectors and projections of one product as floats
+  bool wide_failed = false;          // no memory for them: groups of 8 instead
   static constexpr int RW = 32;
   bool wide_ok() const {
-    return !std::is_same<T, double>::value && S.lsz == 64 && mvd.max_l <= 256 && count == 1;
+    return !std::is_same<T, double>::value && S.lsz <= 64 && mvd.max_l <= 256 && count == 1;
   }
-  void ensure_wide();
+  bool ensure_wide(cudaStream_t st);
   struct ApplyStep {
     int kind;                        // 0 hmatvec, 1 diag update, 2 copy
     int P;
@@ -410,7 +412,7 @@ class Engine : public EngineBase {
   struct Program { std::vector<ApplyStep> fwd, bwd, fwdT, bwdT; };
   Program prog_all;                  // every instance at once
   std::vector<Program> prog_inst;    // one instance (count > 1)
-  Program prog_wide;                 // 32 right-hand sides, tensor cores
+  Program prog_wide;                 // 32 right-hand sides
   int maxP = 1;
   std::map<const void*, int64_t> hm_used;   // stored entries an apply reads per H-matrix
 
@@ -1386,14 +1388,33 @@ void Engine<T>::build_apply_program() {
 }
 
 template <typename T>
-void Engine<T>::ensure_wide() {
-  if (Fw) return;
-  Fw = (double*)dmalloc(sizeof(double) * N * RW); owned.push_back(Fw);
-  Gw = (double*)dmalloc(sizeof(double) * N * RW); owned.push_back(Gw);
-  Uw = (double*)dmalloc(sizeof(double) * N * RW); owned.push_back(Uw);
-  Tw = (double*)dmalloc(sizeof(double) * N * RW); owned.push_back(Tw);
-  tvw = (double*)dmalloc(sizeof(double) * (size_t)tvs * RW); owned.push_back(tvw);
-  build_program(prog_wide, -1, false, Fw, Gw, Uw, Tw);
+bool Engine<T>::ensure_wide(cudaStream_t st) {
+  if (xtw) return true;
+  if (wide_failed) return false;
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  ACR_CUDA(cudaStreamIsCapturing(st, &cap));
+  if (cap != cudaStreamCaptureStatusNone) return false;   // nothing is allocated in a capture
+  std::vector<void*> got;
+  auto take = [&](size_t bytes) {
+    got.push_back(dmalloc(bytes));
+    return got.back();
+  };
+  try {
+    Fw = (double*)take(sizeof(double) * N * RW);
+    Gw = (double*)take(sizeof(double) * N * RW);
+    Uw = (double*)take(sizeof(double) * N * RW);
+    Tw = (double*)take(sizeof(double) * N * RW);
+    tvw = (double*)take(sizeof(double) * (size_t)tvs * RW);
+    xtw = (float*)take(sizeof(float) * wide_scratch_floats(mvd, maxP));
+    build_program(prog_wide, -1, false, Fw, Gw, Uw, Tw);
+  } catch (const AcrError&) {
+    for (void* q : got) cudaFree(q);
+    xtw = nullptr;
+    wide_failed = true;
+    return false;
+  }
+  owned.insert(owned.end(), got.begin(), got.end());
+  return true;
 }
 
 // The substitution as a list of batched steps over the plane slots of
@@ -1589,18 +1610,18 @@ void Engine<T>::run_steps(const std::vector<ApplyStep>& steps, int nr, cudaStrea
     void** t = s.tabs;
     if constexpr (!std::is_same<T, double>::value) {
       if (s.kind == 0 && nr == RW) {
-        // 32 right-hand sides: the H-matrix x matrix product on the tensor cores
+        // 32 right-hand sides: the H-matrix x matrix product
         if (bf16) {
           using B = __nv_bfloat16;
-          launch_hmatvec_tc<B>(mvd, (B* const*)t, (B* const*)(t + P), (B* const*)(t + 2 * P),
-                               (const int* const*)(t + 3 * P), (const double* const*)(t + 4 * P),
-                               (double* const*)(t + 5 * P), s.alpha, s.beta, s.trans, tvscr, P,
-                               vs, d_err, st);
+          launch_hmatvec_wide<B>(mvd, (B* const*)t, (B* const*)(t + P), (B* const*)(t + 2 * P),
+                                 (const int* const*)(t + 3 * P), (const double* const*)(t + 4 * P),
+                                 (double* const*)(t + 5 * P), s.alpha, s.beta, s.trans, tvscr, xtw,
+                                 P, vs, st);
         } else {
-          launch_hmatvec_tc<T>(mvd, (T* const*)t, (T* const*)(t + P), (T* const*)(t + 2 * P),
-                               (const int* const*)(t + 3 * P), (const double* const*)(t + 4 * P),
-                               (double* const*)(t + 5 * P), s.alpha, s.beta, s.trans, tvscr, P,
-                               vs, d_err, st);
+          launch_hmatvec_wide<T>(mvd, (T* const*)t, (T* const*)(t + P), (T* const*)(t + 2 * P),
+                                 (const int* const*)(t + 3 * P), (const double* const*)(t + 4 * P),
+                                 (double* const*)(t + 5 * P), s.alpha, s.beta, s.trans, tvscr, xtw,
+                                 P, vs, st);
         }
         continue;
       }
@@ -1642,12 +1663,10 @@ void Engine<T>::apply(const double* r, double* z, bool trans, cudaStream_t st, i
     launch_permute(Uv, z, sd.perm, n2, n * count, false, st);
     return;
   }
-  // groups of 32 right-hand sides on the tensor cores (float and bfloat16
-  // factors, 64-point leaves), then groups of 8, 4, 2, 1 on the CUDA cores;
-  // each group streams the factors once
+  // groups of 32 right-hand sides (float and bfloat16 factors), then of 8, 4, 2,
+  // 1; each group streams the factors once
   for (int k = 0; k < nrhs;) {
-    if (nrhs - k >= RW && wide_ok()) {
-      ensure_wide();
+    if (nrhs - k >= RW && wide_ok() && ensure_wide(st)) {
       launch_permute(r + (int64_t)k * N, Fw, sd.perm, n2, n * RW, true, st);
       run_program(prog_wide, trans, RW, st, tvw);
       launch_permute(Uw, z + (int64_t)k * N, sd.perm, n2, n * RW, false, st);
