@@ -92,6 +92,7 @@ struct TableRing {
   int64_t epoch = 0;    // tables pushed in an earlier epoch may have been overwritten
   bool counting = false;
   bool fixed = false;   // sized by a counting pass: never wraps
+  cudaStream_t main = nullptr, also = nullptr;   // the streams that read tables
   void init(size_t c) {
     release();
     cap = std::max<size_t>(c, 256);
@@ -119,7 +120,8 @@ struct TableRing {
     if (b > cap) throw AcrError{S_OOM, "pointer table larger than the staging ring"};
     if (off + b > cap) {
       if (fixed) throw AcrError{S_OOM, "setup pointer tables exceed their sized ring"};
-      ACR_CUDA(cudaStreamSynchronize(st));   // earlier copies out of the ring are done
+      ACR_CUDA(cudaStreamSynchronize(main));   // earlier tables have been copied and read
+      if (also) ACR_CUDA(cudaStreamSynchronize(also));
       restart();
     }
     std::memcpy(host + off, data, bytes);
@@ -131,9 +133,10 @@ struct TableRing {
 };
 
 // Device copies of plans: carved out of large chunks and filled through two
-// pinned halves on the setup's stream, so that the host can build the next plan
-// while the device runs the last one (a cudaMalloc and a synchronous copy per array
-// made the device idle through every plan's construction).
+// pinned halves on a stream of their own, so that the host can build the next plans
+// while the device runs the last ones (a cudaMalloc and a synchronous copy per array
+// made the device idle through every plan's construction; behind the setup's
+// kernels the copies held up the host once both halves were full).
 struct PlanStore {
   static constexpr size_t HALF = size_t(4) << 20, CHUNK = size_t(16) << 20;
   std::vector<char*> chunks;
@@ -144,6 +147,8 @@ struct PlanStore {
   int half = 0;
   cudaEvent_t free_[2] = {nullptr, nullptr};
   bool used[2] = {false, false};
+  cudaStream_t up = nullptr;         // the copies': behind no kernel
+  cudaEvent_t done_ = nullptr;
   void* alloc(size_t bytes) {
     const size_t b = (std::max<size_t>(bytes, 16) + 255) & ~size_t(255);
     if (b > left) {
@@ -157,15 +162,17 @@ struct PlanStore {
     left -= b;
     return p;
   }
-  void copy(void* dst, const void* src, size_t bytes, cudaStream_t st) {
+  void copy(void* dst, const void* src, size_t bytes) {
     if (!pin) {
       count_allocs(1);
       ACR_CUDA(cudaMallocHost(&pin, 2 * HALF));
       for (cudaEvent_t& e : free_) ACR_CUDA(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
+      if (!up) ACR_CUDA(cudaStreamCreateWithFlags(&up, cudaStreamNonBlocking));
+      if (!done_) ACR_CUDA(cudaEventCreateWithFlags(&done_, cudaEventDisableTiming));
     }
     for (size_t done = 0; done < bytes;) {
       if (off == HALF) {   // the other half, once its copies are done
-        ACR_CUDA(cudaEventRecord(free_[half], st));
+        ACR_CUDA(cudaEventRecord(free_[half], up));
         used[half] = true;
         half ^= 1;
         off = 0;
@@ -174,19 +181,25 @@ struct PlanStore {
       const size_t n = std::min(bytes - done, HALF - off);
       char* h = pin + half * HALF + off;
       std::memcpy(h, (const char*)src + done, n);
-      ACR_CUDA(cudaMemcpyAsync((char*)dst + done, h, n, cudaMemcpyHostToDevice, st));
+      ACR_CUDA(cudaMemcpyAsync((char*)dst + done, h, n, cudaMemcpyHostToDevice, up));
       off = std::min(HALF, (off + n + 255) & ~size_t(255));
       done += n;
     }
   }
   template <typename V>
-  void* put(const std::vector<V>& v, cudaStream_t st) {
+  void* put(const std::vector<V>& v) {
     void* p = alloc(v.size() * sizeof(V));
-    if (!v.empty()) copy(p, v.data(), v.size() * sizeof(V), st);
+    if (!v.empty()) copy(p, v.data(), v.size() * sizeof(V));
     return p;
   }
-  // the staging is idle (its stream was synchronised)
+  // st waits for the copies so far
+  void order(cudaStream_t st) {
+    if (!up) return;
+    ACR_CUDA(cudaEventRecord(done_, up));
+    ACR_CUDA(cudaStreamWaitEvent(st, done_, 0));
+  }
   void release_staging() {
+    if (up) cudaStreamSynchronize(up);
     if (pin) cudaFreeHost(pin);
     for (cudaEvent_t& e : free_) {
       if (e) cudaEventDestroy(e);
@@ -195,6 +208,10 @@ struct PlanStore {
     pin = nullptr;
     off = 0;
     used[0] = used[1] = false;
+    if (up) cudaStreamDestroy(up);
+    if (done_) cudaEventDestroy(done_);
+    up = nullptr;
+    done_ = nullptr;
   }
   void release() {
     for (char* c : chunks) cudaFree(c);
@@ -256,9 +273,9 @@ struct SlotPool {
       q = free_.back();
       free_.pop_back();
     } else {
+      if (!dry) reserve(hw + 1);
       q = hw++;
     }
-    if (!dry) reserve(q + 1);
     return q;
   }
   void reserve(int nslots) {
@@ -311,8 +328,9 @@ class Engine : public EngineBase {
   // plan and, by a counting pass, every allocation the setup makes (then
   // execute allocates nothing and synchronises nothing)
   void prepare(const double* const* coefs, cudaStream_t st, bool count_pass);
-  // device phase: only launches, asynchronous copies and memsets on st
-  // (no allocation, no synchronisation: capturable in a CUDA graph)
+  // device phase: only launches, asynchronous copies and memsets on st and, between a
+  // fork and a join, on inv_st (after a counting pass no allocation, no
+  // synchronisation: capturable in a CUDA graph)
   void execute(cudaStream_t st);
   // execute between the two events that time the setup
   void execute_timed(cudaStream_t st) {
@@ -370,21 +388,42 @@ class Engine : public EngineBase {
   };
   std::vector<Level> levels;
   TableRing ring;
-  struct {                           // the pointer tables of the last plan run
-    int64_t epoch = -1;
-    int nr = 0, pc = 0;
-    const void *scr = nullptr, *rscr = nullptr;
-    size_t stride = 0, rstride = 0;  // scratch bytes and rank slots per plane
-    std::vector<void*> host;
-    void** dev = nullptr;
-  } tabs;
-  void* scratch = nullptr;
-  size_t scratch_bytes = 0;
-  int* scratch_ranks = nullptr;
-  size_t scratch_rank_cnt = 0;
-  size_t scratch_need = 0, scratch_rank_need = 0;
+  // What the plans running on one stream share: [0] the setup's own stream, [1] the
+  // stream of an H-inverse that runs beside Schur updates.
+  struct Work {
+    char* scratch = nullptr;
+    size_t bytes = 0;
+    int* ranks = nullptr;
+    size_t rank_cnt = 0;
+    size_t need = 0, rank_need = 0;    // by the counting pass
+    std::vector<void*> old;            // outgrown
+    struct {                           // the pointer tables of the last plan run
+      int64_t epoch = -1;
+      int nr = 0, pc = 0;
+      const void *scr = nullptr, *rscr = nullptr;
+      size_t stride = 0, rstride = 0;  // scratch bytes and rank slots per plane
+      std::vector<void*> host;
+      void** dev = nullptr;
+    } tabs;
+  } work[2];
+  Work* w = work;
+  cudaStream_t inv_st = nullptr;     // the H-inverse's stream (high priority)
+  cudaEvent_t fork_ev = nullptr, join_ev = nullptr;
+  bool overlap = false;
+  void free_old(Work& k) {
+    for (void* p : k.old) cudaFree(p);
+    k.old.clear();
+  }
+  void free_work(Work& k) {
+    free_old(k);
+    if (k.scratch) cudaFree(k.scratch);
+    if (k.ranks) cudaFree(k.ranks);
+    k.scratch = nullptr; k.ranks = nullptr;
+    k.bytes = k.rank_cnt = 0;
+  }
   size_t scratch_budget = 0;
-  double* d_coefs = nullptr;
+  double* d_coefs = nullptr;         // 1, -1 and the sign of products with coefficient 2
+  bool negate = false;               // that sign
   int* d_err = nullptr;
   unsigned long long* d_sketch_stat = nullptr;   // truncated targets, stacked-rank overflows,
                                                  // leaf inverses by the FP64 fallback
@@ -468,7 +507,19 @@ class Engine : public EngineBase {
   // fake address of the counting pass (never dereferenced)
   static char* fake_base() { return reinterpret_cast<char*>(uintptr_t(1) << 45); }
   HM alloc_hm(cudaStream_t st) {
-    const int q = pool.take(dry);
+    int q = -1;
+    try {
+      q = pool.take(dry);
+    } catch (const AcrError&) {
+      // the memory of the second and of outgrown scratch, before giving up
+      if (counted || (!work[1].scratch && work[0].old.empty())) throw;
+      ACR_CUDA(cudaStreamSynchronize(cur_st));
+      if (inv_st) ACR_CUDA(cudaStreamSynchronize(inv_st));
+      free_old(work[0]);
+      free_work(work[1]);
+      overlap = false;
+      q = pool.take(dry);
+    }
     HM h = pool.at(q, dry);
     if (!dry)
       ACR_CUDA(cudaMemsetAsync(h.rank, 0, std::max<size_t>(S.lleaf.size(), 1) * sizeof(int), st));
@@ -522,6 +573,7 @@ class Engine : public EngineBase {
     }
   }
   void release() {
+    if (inv_st) cudaStreamSynchronize(inv_st);   // work left by a setup that failed
     pool.release();
     pool_b.release();
     for (void* p : owned) cudaFree(p);
@@ -530,9 +582,12 @@ class Engine : public EngineBase {
     merged_plans.clear();
     store.release_staging();
     store.release();
-    if (scratch) cudaFree(scratch);
-    if (scratch_ranks) cudaFree(scratch_ranks);
-    scratch = nullptr; scratch_ranks = nullptr;
+    if (inv_st) cudaStreamDestroy(inv_st);
+    inv_st = nullptr;
+    if (fork_ev) cudaEventDestroy(fork_ev);
+    if (join_ev) cudaEventDestroy(join_ev);
+    fork_ev = join_ev = nullptr;
+    for (Work& k : work) free_work(k);
     ring.release();
     for (Pend& pd : pend) { cudaEventDestroy(pd.a); cudaEventDestroy(pd.b); }
     for (cudaEvent_t e : evfree) cudaEventDestroy(e);
@@ -577,35 +632,57 @@ class Engine : public EngineBase {
   // then allocated once; a one-shot setup grows it on demand
   void ensure_scratch(size_t bytes, size_t ranks, cudaStream_t st) {
     if (dry) {
-      scratch_need = std::max(scratch_need, bytes);
-      scratch_rank_need = std::max(scratch_rank_need, ranks);
+      w->need = std::max(w->need, bytes);
+      w->rank_need = std::max(w->rank_need, ranks);
       return;
     }
-    if (bytes <= scratch_bytes && ranks <= scratch_rank_cnt) return;
+    if (bytes <= w->bytes && ranks <= w->rank_cnt) return;
     if (counted) throw AcrError{S_OOM, "setup scratch larger than its counted need"};
-    ACR_CUDA(cudaStreamSynchronize(st));
-    if (bytes > scratch_bytes) {
-      if (scratch) cudaFree(scratch);
-      scratch = nullptr;
-      scratch = dmalloc(bytes);
-      scratch_bytes = bytes;
-    }
-    if (ranks > scratch_rank_cnt) {
-      if (scratch_ranks) cudaFree(scratch_ranks);
-      scratch_ranks = nullptr;
-      scratch_ranks = (int*)dmalloc(ranks * sizeof(int));
-      scratch_rank_cnt = ranks;
+    // The smaller scratch stays until the setup ends: launches enqueued before use it,
+    // and waiting for them (as cudaFree also does) left the device idle while the
+    // next plans were built.  The sizes grow by factors of about 3.
+    auto grow = [&](auto*& p, size_t unit, size_t& have, size_t need) {
+      if (need <= have) return;
+      using V = std::remove_reference_t<decltype(p)>;
+      void* q = nullptr;
+      try {
+        q = dmalloc(need * unit);
+      } catch (const AcrError&) {
+        ACR_CUDA(cudaStreamSynchronize(st));
+        free_old(*w);
+        if (p) cudaFree(p);
+        p = nullptr;
+        have = 0;
+        q = dmalloc(need * unit);
+      }
+      if (p) w->old.push_back(p);
+      p = (V)q;
+      have = need;
+    };
+    try {
+      grow(w->scratch, 1, w->bytes, bytes);
+      grow(w->ranks, sizeof(int), w->rank_cnt, ranks);
+    } catch (const AcrError&) {
+      if (w == work) throw;
+      // no memory for the second scratch: the updates enqueued so far finish, and the
+      // inverse goes on with theirs (the next ones wait for it)
+      free_work(work[1]);
+      overlap = false;
+      ACR_CUDA(cudaStreamSynchronize(cur_st));
+      w = work;
+      ensure_scratch(bytes, ranks, st);
     }
   }
 
   void upload_plan(Plan& pl, cudaStream_t st) {
     if (pl.uploaded) return;
-    pl.d_groups = store.put(pl.groups, st);
-    pl.d_items = store.put(pl.items, st);
-    pl.d_targets = store.put(pl.targets, st);
-    pl.d_stack = store.put(pl.stack, st);
-    pl.d_torder = store.put(pl.torder, st);
-    pl.d_bundles = store.put(pl.bundles, st);
+    pl.d_groups = store.put(pl.groups);
+    pl.d_items = store.put(pl.items);
+    pl.d_targets = store.put(pl.targets);
+    pl.d_stack = store.put(pl.stack);
+    pl.d_torder = store.put(pl.torder);
+    pl.d_bundles = store.put(pl.bundles);
+    store.order(st);
     pl.uploaded = true;
     if (pl.items.size() >= PLAN_LARGE) {
       pl.stripped = true;
@@ -726,9 +803,19 @@ class Engine : public EngineBase {
         (std::max<size_t>((size_t)pl.scratch * sizeof(T), 256) + 255) & ~size_t(255);
     const size_t ranks = std::max(pl.scratch_ranks, 1);
     int Pc = (int)std::max<size_t>(1, std::min<size_t>(P, scratch_budget / per_plane));
+    // More planes than fill the device only cost the allocation of their scratch (both
+    // sides' couplings at n = 80 would take 31 GB): 8 of a large plan, what fits 6 GB
+    // of a small one, in chunks of like size.  Setup, all in: n = 64 233.6 -> 227.0 ms, n =
+    // 80 661 -> 660 ms (2 GB: 231.5, 661.5; 12 GB: 233.3, 658).
+    constexpr size_t SCRATCH_ENOUGH = size_t(6) << 30;
+    if (per_plane * Pc > SCRATCH_ENOUGH) {
+      Pc = std::min<int>(Pc, std::max<int>(8, (int)(SCRATCH_ENOUGH / per_plane)));
+      Pc = (P + (P + Pc - 1) / Pc - 1) / ((P + Pc - 1) / Pc);
+    }
     ensure_scratch(per_plane * Pc, ranks * Pc, st);
-    char* scr_base = dry ? fake_base() : (char*)scratch;
-    int* scr_rank_base = dry ? (int*)fake_base() : scratch_ranks;
+    auto& tabs = w->tabs;
+    char* scr_base = dry ? fake_base() : w->scratch;
+    int* scr_rank_base = dry ? (int*)fake_base() : w->ranks;
     for (int c0 = 0; c0 < P; c0 += Pc) {
       const int pc = std::min(Pc, P - c0);
       // The tables of the last run serve again when the operands are the same and
@@ -748,8 +835,8 @@ class Engine : public EngineBase {
                           return true;
                         }();
       if (!same) {
-        const size_t have = dry ? scratch_need : scratch_bytes;
-        const size_t have_r = dry ? scratch_rank_need : scratch_rank_cnt;
+        const size_t have = dry ? w->need : w->bytes;
+        const size_t have_r = dry ? w->rank_need : w->rank_cnt;
         tabs.nr = nr;
         tabs.pc = pc;
         tabs.scr = scr_base;
@@ -799,17 +886,18 @@ class Engine : public EngineBase {
   void gemm_stage(const Plan& pl, const Stage& sg, T* const* d_tab, const int* const* d_rtab,
                   int pc, cudaStream_t st) {
     double* f = sg.tag >= 0 ? fl(5 + sg.tag) : fl(0);
+    const double* cf = d_coefs + (negate ? 3 : 0);
     const int variant = sg.tag >= 0 && sg.tag < 16 ? gemm_variant[sg.tag] : 0;
     if (variant == 0 && sg.bend > sg.bbeg) {
-      launch_ggemm<T>(pl, sg.beg, sg.beg + sg.nwide, d_tab, d_rtab, pc, d_coefs, st, f, sg.tag);
-      launch_gbundle<T>(pl, sg.bbeg, sg.bend, d_tab, d_rtab, pc, d_coefs, st, f);
+      launch_ggemm<T>(pl, sg.beg, sg.beg + sg.nwide, d_tab, d_rtab, pc, cf, st, f, sg.tag);
+      launch_gbundle<T>(pl, sg.bbeg, sg.bend, d_tab, d_rtab, pc, cf, st, f);
       return;
     }
     if (variant == 0 && (sg.tag == TAG_S || sg.tag == TAG_P)) {
       launch_tdot<T>(pl, sg.tag == TAG_S, d_tab, d_rtab, pc, st, f);
       return;
     }
-    launch_ggemm<T>(pl, sg.beg, sg.end, d_tab, d_rtab, pc, d_coefs, st, f, sg.tag, variant, d_err,
+    launch_ggemm<T>(pl, sg.beg, sg.end, d_tab, d_rtab, pc, cf, st, f, sg.tag, variant, d_err,
                     sg.nwide);
   }
 
@@ -853,14 +941,21 @@ class Engine : public EngineBase {
     run_split(mk(n11, 0, 0, n12, 0, n21, 1, 1), roles, P, st);    // X11 = X11 - X12 T21
   }
 
-  void hinv_batch(const std::vector<int>& planes, cudaStream_t st) {
-    const int P = (int)planes.size();
-    if (P == 0) return;
+  // the roles of an H-inverse: the planes, in place, and one H-matrix of temporaries each
+  std::vector<std::vector<HM>> inv_roles(const std::vector<int>& planes, cudaStream_t st) {
     std::vector<std::vector<HM>> roles(2);
-    for (int i : planes) {
-      roles[0].push_back(D[i]);
-      roles[1].push_back(alloc_hm(st));
+    for (int i : planes) roles[0].push_back(D[i]);
+    try {
+      for (size_t i = 0; i < planes.size(); ++i) roles[1].push_back(alloc_hm(st));
+    } catch (const AcrError&) {
+      for (HM& h : roles[1]) free_hm(h);
+      throw;
     }
+    return roles;
+  }
+  void hinv_batch(std::vector<std::vector<HM>> roles, cudaStream_t st) {
+    const int P = (int)roles[0].size();
+    if (P == 0) return;
     std::vector<void*> xd(P);
     for (int p = 0; p < P; ++p) xd[p] = roles[0][p].dense;
     void* d_xdense = ring.push(xd.data(), sizeof(void*) * P, st);
@@ -989,7 +1084,7 @@ void Engine<T>::prepare(const double* const* coefs, cudaStream_t st, bool count_
   mvd.segt_ptr = (const int32_t*)upload(mvp.segt_ptr, owned);
   mvd.nseg = mvp.seg_ptr.back();
   mvd.nsegt = mvp.segt_ptr.back();
-  std::vector<double> coefs_pm{1.0, -1.0};
+  std::vector<double> coefs_pm{1.0, -1.0, 1.0, 1.0, -1.0, -1.0};   // (two sets)
   d_coefs = (double*)upload(coefs_pm, owned);
   d_err = (int*)dmalloc(sizeof(int));
   owned.push_back(d_err);
@@ -1008,6 +1103,15 @@ void Engine<T>::prepare(const double* const* coefs, cudaStream_t st, bool count_
   owned.push_back(Ld); owned.push_back(Ud);
   ACR_CUDA(cudaEventCreate(&ev0));
   ACR_CUDA(cudaEventCreate(&ev1));
+  overlap = !profiling;   // (a profile times every launch by itself)
+  if (overlap) {
+    int least = 0, greatest = 0;
+    ACR_CUDA(cudaDeviceGetStreamPriorityRange(&least, &greatest));
+    ACR_CUDA(cudaStreamCreateWithPriority(&inv_st, cudaStreamNonBlocking, greatest));
+    ACR_CUDA(cudaEventCreateWithFlags(&fork_ev, cudaEventDisableTiming));
+    ACR_CUDA(cudaEventCreateWithFlags(&join_ev, cudaEventDisableTiming));
+    ring.also = inv_st;
+  }
 
   // counting pass: the same host sequence with no device work sizes the
   // H-matrix arena(s), the setup scratch and the table ring
@@ -1026,27 +1130,39 @@ void Engine<T>::prepare(const double* const* coefs, cudaStream_t st, bool count_
   } else {
     // counting pass: the same host sequence with no device work sizes the
     // H-matrix slots, the setup scratch and the table ring exactly
-    dry = true;
-    ring.counting = true;
-    ring.restart();
-    scratch_need = scratch_rank_need = 0;
-    execute(st);
-    dry = false;
-    ring.counting = false;
-    const size_t ring_need = ring.off;
-    pool.reserve(pool.hw);
-    pool.fixed = true;
-    if (bf16) {
-      pool_b.reserve(pool_b.hw);
-      pool_b.fixed = true;
+    for (;;) {
+      dry = true;
+      ring.counting = true;
+      ring.restart();
+      for (Work& k : work) k.need = k.rank_need = 0;
+      execute(st);
+      dry = false;
+      ring.counting = false;
+      try {
+        pool.reserve(pool.hw);
+        if (bf16) pool_b.reserve(pool_b.hw);
+        for (Work& k : work) {
+          if (&k != work && !k.need) continue;
+          k.bytes = std::max<size_t>(k.need, 256);
+          k.rank_cnt = std::max<size_t>(k.rank_need, 1);
+          k.scratch = (char*)dmalloc(k.bytes);
+          k.ranks = (int*)dmalloc(k.rank_cnt * sizeof(int));
+        }
+        break;
+      } catch (const AcrError&) {
+        if (!overlap) throw;
+        overlap = false;   // one stream needs less
+        for (Work& k : work) free_work(k);
+        pool.release();
+        pool_b.release();
+      }
     }
-    scratch = dmalloc(std::max<size_t>(scratch_need, 256));
-    scratch_bytes = std::max<size_t>(scratch_need, 256);
-    scratch_ranks = (int*)dmalloc(std::max<size_t>(scratch_rank_need, 1) * sizeof(int));
-    scratch_rank_cnt = std::max<size_t>(scratch_rank_need, 1);
+    pool.fixed = true;
+    if (bf16) pool_b.fixed = true;
+    const size_t ring_need = ring.off;
     ring.init(ring_need);
     ring.fixed = true;
-    ACR_CUDA(cudaStreamSynchronize(st));   // the plans are on the device
+    ACR_CUDA(cudaStreamSynchronize(st));
     store.release_staging();
   }
   info.structure_ms = std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - h0).count();
@@ -1055,6 +1171,9 @@ void Engine<T>::prepare(const double* const* coefs, cudaStream_t st, bool count_
 template <typename T>
 void Engine<T>::execute(cudaStream_t st) {
   cur_st = st;
+  ring.main = st;
+  w = work;
+  negate = false;
   pool.restart();
   ring.restart();
   D.assign((size_t)count * n, HM());
@@ -1092,6 +1211,62 @@ void Engine<T>::execute(cudaStream_t st) {
 
   std::vector<HM> curL(NP), curU(NP);   // couplings of the current level (r >= 1)
   int s = 1, r = 0;
+  bool inverted = false;   // the level's H-inverse already runs, on inv_st
+  bool forked = false;     // inv_st has work that st does not wait for yet
+  size_t inv_bytes = 0, inv_ranks = 0, inv_planes = 1;   // the first level's scratch
+  // The H-inverse of the planes that the next level eliminates needs their own updates
+  // only: it runs on a stream of its own, by priority, beside the other planes'
+  // updates and the new couplings.  An inverse of a few planes is a chain of some
+  // 700 launches that leave the device mostly idle (17 ms at n = 64 whatever the
+  // planes); the updates fill it.  The other planes' updates are enqueued first (few
+  // launches), then the inverse, then the couplings, whose plans may still have to be
+  // built.  Setup at n = 32, FP64: 138 -> 127 ms; n = 64: 243 -> 217; n =
+  // 80: 707 -> 639.
+  auto fork = [&] {
+    if (overlap && !dry) ACR_CUDA(cudaEventRecord(fork_ev, st));
+  };
+  auto invert_ahead = [&](const std::vector<int>& planes) {
+    if (!overlap) return;
+    if (!dry) ACR_CUDA(cudaStreamWaitEvent(inv_st, fork_ev, 0));
+    forked = !dry;
+    std::vector<std::vector<HM>> roles;
+    try {
+      roles = inv_roles(planes, inv_st);
+    } catch (const AcrError&) {
+      overlap = false;   // no memory for its temporaries while the updates have theirs
+      if (!dry) ACR_CUDA(cudaEventRecord(join_ev, inv_st));
+      return;
+    }
+    w = work + 1;
+    if (!dry) {
+      char rname[16];
+      snprintf(rname, sizeof(rname), "inv%d", r + 1);
+      nvtxRangePushA(rname);
+      // one allocation in place of one per growth
+      if (!counted && !w->scratch)
+        ensure_scratch(inv_bytes / inv_planes * planes.size(),
+                       inv_ranks / inv_planes * planes.size(), inv_st);
+    }
+    hinv_batch(std::move(roles), inv_st);
+    if (!dry) {
+      nvtxRangePop();
+      ACR_CUDA(cudaEventRecord(join_ev, inv_st));
+      // (on the updates' scratch: none beside it)
+      if (w == work) ACR_CUDA(cudaStreamWaitEvent(st, join_ev, 0));
+    }
+    w = work;
+    inverted = true;
+  };
+  // The temporaries of the updates go back when the inverse has its own, which must
+  // not be theirs: the two streams do not order them.
+  auto join = [&](std::vector<HM>& Ta, std::vector<HM>& Tb) {
+    for (size_t q = 0; q < Ta.size(); ++q) {
+      free_hm(Ta[q]);
+      free_hm(Tb[q]);
+    }
+    if (forked) ACR_CUDA(cudaStreamWaitEvent(st, join_ev, 0));
+    forked = false;
+  };
   while (s < n) {
     Level lev;
     lev.s = s;
@@ -1112,7 +1287,13 @@ void Engine<T>::execute(cudaStream_t st) {
       li0 = ev(); li1 = ev(); lu1 = ev();
       ACR_CUDA(cudaEventRecord(li0, st));
     }
-    hinv_batch(lev.red, st);
+    if (!inverted) hinv_batch(inv_roles(lev.red, st), st);
+    inverted = false;
+    if (r == 0) {
+      inv_bytes = w->bytes;
+      inv_ranks = w->rank_cnt;
+      inv_planes = std::max<size_t>(lev.red.size(), 1);
+    }
     if (!dry) {
       nvtxRangePop();
       char rname[16];
@@ -1123,6 +1304,19 @@ void Engine<T>::execute(cudaStream_t st) {
     // a5-a7: Schur updates of the black planes
     const int PB = (int)lev.black.size();
     std::vector<HM> newL(NP), newU(NP);
+    // the planes that are inverted next, and of lev.black the places of these and of the rest
+    std::vector<int> next, first, rest;
+    for (int q = 0; q < PB; ++q) {
+      const int k = plane_of(lev.black[q]);
+      const bool is_next = 2 * s < n ? (k / (2 * s)) % 2 == 1 : k == 0;
+      if (is_next) next.push_back(lev.black[q]);
+      (is_next || !overlap ? first : rest).push_back(q);
+    }
+    auto pick = [](const std::vector<HM>& v, const std::vector<int>& at) {
+      std::vector<HM> o;
+      for (int q : at) o.push_back(v[q]);
+      return o;
+    };
     if (r == 0) {
       std::vector<HM> Ta(PB), Tb(PB), nL(PB), nU(PB), Xa(PB), Xb(PB), Dj(PB);
       std::vector<const double*> rowA(PB), colA(PB), rowB(PB), colB(PB), colLA(PB), colUB(PB);
@@ -1169,14 +1363,18 @@ void Engine<T>::execute(cudaStream_t st) {
       op.c_node = 0; op.c_role = 0; op.alpha = 0; op.nroles = 3;
       op.adds.push_back(OpDesc::Add{1, 1});
       op.adds.push_back(OpDesc::Add{2, 1});
-      std::vector<std::vector<HM>> roles{Dj, Ta, Tb};
-      run_op(op, roles, PB, st);
+      auto update = [&](const std::vector<int>& at) {
+        run_op(op, {pick(Dj, at), pick(Ta, at), pick(Tb, at)}, (int)at.size(), st);
+      };
+      update(first);
+      fork();
+      update(rest);
       for (int q = 0; q < PB; ++q) {
-        free_hm(Ta[q]);
-        free_hm(Tb[q]);
         newL[lev.black[q]] = nL[q];
         newU[lev.black[q]] = nU[q];
       }
+      invert_ahead(next);
+      join(Ta, Tb);
     } else {
       std::vector<HM> Ta(PB), Tb(PB), Lj(PB), Uj(PB), Xa(PB), Xb(PB), Dj(PB), Ua(PB), Lb(PB),
           La(PB), Ub(PB), nL(PB), nU(PB);
@@ -1196,23 +1394,34 @@ void Engine<T>::execute(cudaStream_t st) {
       }
       OpDesc opT;
       opT.c_node = 0; opT.c_role = 0; opT.alpha = -1; opT.nroles = 3;
-      opT.prods.push_back(OpDesc::Prod{0, 0, 1, 2, 0});
-      run_sides(opT, {Ta, Lj, Xa}, {Tb, Uj, Xb}, PB, st);   // Ta = L_j X_a, Tb = U_j X_b
+      opT.prods.push_back(OpDesc::Prod{0, 0, 1, 2, 2});
       OpDesc opD;
       opD.c_node = 0; opD.c_role = 0; opD.alpha = 0; opD.nroles = 5;
       opD.prods.push_back(OpDesc::Prod{0, 0, 1, 2, 1});
       opD.prods.push_back(OpDesc::Prod{0, 0, 3, 4, 1});
-      run_split(opD, {Dj, Ta, Ua, Tb, Lb}, PB, st);   // D_j -= Ta U_a + Tb L_b
-      OpDesc opN;
-      opN.c_node = 0; opN.c_role = 0; opN.alpha = -1; opN.nroles = 3;
-      opN.prods.push_back(OpDesc::Prod{0, 0, 1, 2, 1});
-      run_sides(opN, {nL, Ta, La}, {nU, Tb, Ub}, PB, st);   // L_j' = -Ta L_a, U_j' = -Tb U_b
+      auto update = [&](const std::vector<int>& at) {
+        const int PA = (int)at.size();
+        // Ta = L_j X_a, Tb = U_j X_b
+        run_sides(opT, {pick(Ta, at), pick(Lj, at), pick(Xa, at)},
+                  {pick(Tb, at), pick(Uj, at), pick(Xb, at)}, PA, st);
+        // D_j -= Ta U_a + Tb L_b
+        run_split(opD, {pick(Dj, at), pick(Ta, at), pick(Ua, at), pick(Tb, at), pick(Lb, at)}, PA,
+                  st);
+      };
+      update(first);
+      fork();
+      update(rest);
+      invert_ahead(next);
+      // L_j' = -Ta L_a, U_j' = -Tb U_b, by the same plan (its construction is as
+      // long as the products: 28 ms at n = 64)
+      negate = true;
+      run_sides(opT, {nL, Ta, La}, {nU, Tb, Ub}, PB, st);
+      negate = false;
       for (int q = 0; q < PB; ++q) {
-        free_hm(Ta[q]);
-        free_hm(Tb[q]);
         newL[lev.black[q]] = nL[q];
         newU[lev.black[q]] = nU[q];
       }
+      join(Ta, Tb);
     }
     if (!dry) nvtxRangePop();
     if (lu1) {
@@ -1239,7 +1448,7 @@ void Engine<T>::execute(cudaStream_t st) {
       l0 = ev(); l1 = ev();
       ACR_CUDA(cudaEventRecord(l0, st));
     }
-    hinv_batch(last, st);
+    if (!inverted) hinv_batch(inv_roles(last, st), st);
     if (l1) {
       ACR_CUDA(cudaEventRecord(l1, st));
       ACR_CUDA(cudaEventSynchronize(l1));
@@ -1301,8 +1510,7 @@ void Engine<T>::finish(cudaStream_t st, bool one_shot) {
   if (one_shot) {
     // the scratch arena is only needed by the setup; in the BF16 form the
     // FP32 arena holds no stored factor any more
-    if (scratch) { cudaFree(scratch); scratch = nullptr; scratch_bytes = 0; }
-    if (scratch_ranks) { cudaFree(scratch_ranks); scratch_ranks = nullptr; scratch_rank_cnt = 0; }
+    for (Work& k : work) free_work(k);
     if (bf16) pool.release();
   }
   collect_info(st);

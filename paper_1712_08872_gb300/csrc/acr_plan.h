@@ -56,7 +56,7 @@ struct alignas(16) GItem {
   int8_t abuf, bbuf;
   int8_t aflags, bflags;
   int8_t k_rb, r_rb;
-  int8_t coef;                  // index into the coefficient array
+  int8_t coef;                  // index into the coefficient array (1, -1, the run's sign)
   int8_t guard0, guard1;        // buffers that must be present for the plane (-1: none)
 };
 static_assert(sizeof(GItem) == 64, "four 16-byte loads per item");

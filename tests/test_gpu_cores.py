@@ -82,3 +82,27 @@ def test_apply_32_vectors_any_leaf(n, leaf, prec, trans):
         err = ((z[k:k + 8] - w).norm(dim=1) / w.norm(dim=1)).max().item()
         assert err <= (0.0 if k == 32 else 1e-6), (k, err)
     h.close()
+
+
+@pytest.mark.parametrize("n,prec", [(2, 0), (3, 1), (8, 1), (20, 0), (28, 1), (32, 2)])
+def test_inverse_beside_updates(n, prec):
+    """A profiled setup times every launch and so runs on one stream; the default one
+    inverts the next level's planes beside the other planes' updates.  The same kernels
+    on the same operands, whose sums do not depend on the batch: equal results."""
+    from paper_1712_08872_gb300 import _build
+    _build.build()
+    import paper_1712_08872_gb300 as acr
+
+    beta = torch.full((3 * n ** 3,), 20.0, dtype=torch.float64, device="cuda:0")
+    coef = torch.empty(7 * n ** 3, dtype=torch.float64, device="cuda:0")
+    acr.acr_stencil_codi(n, beta, coef)
+    r = torch.tensor(uniform_rhs(n, 5), device="cuda:0")
+    out = []
+    for flags in (acr.ACR_FLAG_PROFILE, 0, 0):
+        h = acr.Handle(n, coef, 1e-2, 2.0, 64, prec, 24, flags=flags)
+        z, i = torch.empty_like(r), h.info()
+        h.apply(r, z)
+        out.append((z.cpu(), i.max_rank, i.lr_truncations, i.sketch_overflows, i.factor_bytes))
+        h.close()
+    for o in out[1:]:
+        assert torch.equal(o[0], out[0][0]) and o[1:] == out[0][1:], o[1:]
