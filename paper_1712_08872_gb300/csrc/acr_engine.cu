@@ -2162,13 +2162,14 @@ int run_gmres(Krylov& K, int m, double rtol, int maxit, const double* f, double*
 int run_pcg_batch(Krylov& K, double rtol, int maxit, const double* f, double* u, int nr,
                   acr_solve_info* info) {
   const int64_t N = K.N, RN = (int64_t)nr * N;
-  double* R = K.dbuf(2 * RN);        // residuals, then the step before's
-  double* Z = K.dbuf(RN);
-  double* Pv = K.dbuf(RN);
-  double* Q = K.dbuf(RN);
-  double* part = K.dbuf((size_t)600 * 2 * nr);
-  double* dout = K.dbuf((size_t)3 * nr);
-  double* dco = K.dbuf(nr);
+  const int64_t RP = (RN + 31) / 32 * 32;
+  double* R = K.dbuf(5 * RP + (size_t)1204 * nr);
+  double* Z = R + (2 * RN + 31) / 32 * 32;   // (after the residuals and the step before's)
+  double* Pv = Z + RP;
+  double* Q = Pv + RP;
+  double* part = Q + RP;
+  double* dout = part + (size_t)1200 * nr;
+  double* dco = dout + (size_t)3 * nr;
   std::vector<double> h((size_t)3 * nr), co(nr);
   auto fetch = [&](int cnt) {
     ACR_CUDA(cudaMemcpyAsync(h.data(), dout, cnt * sizeof(double), cudaMemcpyDeviceToHost, K.st));
@@ -2672,8 +2673,23 @@ static acr_status krylov_common(acr::EngineBase* E, const acr_grid* grid, const 
     if (nrhs > 1 && method == ACR_GMRES) {
       s = acr::run_gmres_batch(K, restart, rtol, maxit, f, u, nrhs, info);
     } else if (nrhs > 1) {
-      // PCG: info reports the largest count and residual
-      s = acr::run_pcg_batch(K, rtol, maxit, f, u, nrhs, info);
+      // PCG: info reports the largest count and residual; one system after another
+      // where the vectors of all do not fit (their one allocation comes first)
+      try {
+        s = acr::run_pcg_batch(K, rtol, maxit, f, u, nrhs, info);
+      } catch (const acr::AcrError& e) {
+        if (e.status != acr::S_OOM) throw;
+        acr_solve_info one{}, agg{};
+        agg.converged = 1;
+        for (int r = 0; r < nrhs && s != acr::S_BREAKDOWN; ++r) {
+          const int sr = acr::run_pcg(K, rtol, maxit, f + r * K.N, u + r * K.N, &one);
+          if (sr != acr::S_OK && s == acr::S_OK) s = sr;
+          agg.iterations = std::max(agg.iterations, one.iterations);
+          agg.rel_residual = std::max(agg.rel_residual, one.rel_residual);
+          agg.converged &= one.converged;
+        }
+        if (info) *info = agg;
+      }
     } else {
       s = method == ACR_PCG ? acr::run_pcg(K, rtol, maxit, f, u, info)
                             : acr::run_gmres(K, restart, rtol, maxit, f, u, info);

@@ -106,3 +106,66 @@ def test_inverse_beside_updates(n, prec):
         h.close()
     for o in out[1:]:
         assert torch.equal(o[0], out[0][0]) and o[1:] == out[0][1:], o[1:]
+
+
+@pytest.mark.parametrize("n,prec,nr", [(12, 0, 3), (16, 1, 9), (20, 1, 33)])
+def test_pcg_in_lockstep(n, prec, nr):
+    """Several right-hand sides by PCG, one of them zero: every residual by the
+    oracle's SpMV meets the tolerance (slack for the final residual's own rounding), the
+    zero one's solution is zero, and the count is the largest single one, give or take
+    the one step that rounding can move at the tolerance."""
+    from paper_1712_08872_gb300 import _build
+    _build.build()
+    import paper_1712_08872_gb300 as acr
+
+    def dev(x):
+        return torch.tensor(np.ascontiguousarray(x), dtype=torch.float64, device="cuda:0")
+
+    kappa = gaussian_field_kappa(n, 4)
+    st = stencil_poisson(kappa, n)
+    coef = torch.empty(7 * n ** 3, dtype=torch.float64, device="cuda:0")
+    acr.acr_stencil_poisson(n, dev(kappa), coef)
+    F = np.stack([uniform_rhs(n, 60 + k) for k in range(nr)])
+    F[1] = 0.0
+    h = acr.Handle(n, coef, 1e-2, 2.0, 64, prec, 24)
+    u = torch.ones(nr * n ** 3, dtype=torch.float64, device="cuda:0")
+    info, _ = acr.acr_krylov_solve(h.h, coef, acr.ACR_PCG, 30, 1e-9, 200, dev(F.ravel()), u, nrhs=nr)
+    single = 0
+    for k in range(nr):
+        v = torch.ones(n ** 3, dtype=torch.float64, device="cuda:0")
+        one, _ = acr.acr_krylov_solve(h.h, coef, acr.ACR_PCG, 30, 1e-9, 200, dev(F[k]), v)
+        single = max(single, one.iterations)
+    h.close()
+    U = u.cpu().numpy().reshape(nr, -1)
+    assert not U[1].any()
+    for k in range(nr):
+        if k != 1:
+            res = np.linalg.norm(F[k] - stencil_apply(st, n, U[k])) / np.linalg.norm(F[k])
+            assert res <= 1.001e-9, (k, res)
+    assert abs(info.iterations - single) <= 1, (info.iterations, single)
+
+
+@pytest.mark.parametrize("n", [1, 7, 33])
+@pytest.mark.parametrize("nr", [1, 2, 3, 4, 5, 7])
+def test_spmv_vector_groups(n, nr):
+    """The SpMV reads the coefficients once per up to four vectors: every count of
+    vectors against the oracle's (seven products and their sum, so 8 units of
+    rounding of the terms' magnitudes)."""
+    from paper_1712_08872_gb300 import _build
+    _build.build()
+    import paper_1712_08872_gb300 as acr
+
+    kappa = gaussian_field_kappa(n, 4)
+    st = stencil_poisson(kappa, n)
+    coef = torch.empty(7 * n ** 3, dtype=torch.float64, device="cuda:0")
+    acr.acr_stencil_poisson(n, torch.tensor(np.ascontiguousarray(kappa), dtype=torch.float64,
+                                            device="cuda:0"), coef)
+    X = np.stack([uniform_rhs(n, k) for k in range(nr)])
+    x = torch.tensor(X, device="cuda:0").reshape(-1)
+    y = torch.empty_like(x)
+    acr.acr_spmv(n, coef, x, y, nr)
+    Y = y.cpu().numpy().reshape(nr, -1)
+    for k in range(nr):
+        ref = stencil_apply(st, n, X[k]).ravel()
+        mag = np.abs(st["c"]).max() * 2 * np.abs(X[k]).max()
+        assert np.abs(Y[k] - ref).max() <= 8 * 2.3e-16 * mag, k
