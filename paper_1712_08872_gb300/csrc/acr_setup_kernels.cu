@@ -721,6 +721,10 @@ __global__ void __cluster_dims__(LCL, 1, 1) __launch_bounds__(128)
   __shared__ double red8[TH / 32];
   const int tid = threadIdx.x, lane = tid & 31;
   const int i = tid & 63, jh = 4 * (tid >> 6), c0 = LPW * rank;
+  // No CTA writes into another's shared memory before that one has started and has set
+  // its own step[]: the arrival follows that, and the wait hides behind the loads.
+  if (tid < CMAX) step[tid] = -1;
+  cl.barrier_arrive();
   double amax = 0.0;
 #pragma unroll
   for (int q = 0; q < 4; ++q) {
@@ -729,8 +733,8 @@ __global__ void __cluster_dims__(LCL, 1, 1) __launch_bounds__(128)
     X[i][jh + q] = v;
     amax = fmax(amax, fabs(v));
   }
-  if (tid < CMAX) step[tid] = -1;
   amax = block_absmax<TH>(amax, red8);
+  cl.barrier_wait();
   unsigned used = 0;   // warp 0: rows lane, lane + 32 that have been pivots
   int buf = 0;
   for (int kb = 0; kb < n; kb += LPW, buf ^= 1) {
