@@ -571,6 +571,7 @@ __global__ void __cluster_dims__(LCL, 1, 1) __launch_bounds__(LTH)
   if (!Ap) return;   // the whole cluster
   Ap += off;
   cg::cluster_group cl = cg::this_cluster();
+  cl.barrier_arrive();   // (this CTA has started: the others may write its s_state)
   const int rank = (int)cl.block_rank();
   // A and X0 together hold the FP64 fallback's matrix
   __shared__ __align__(16) float lsm[2 * CMAX * (CMAX + 1)];
@@ -669,6 +670,7 @@ __global__ void __cluster_dims__(LCL, 1, 1) __launch_bounds__(LTH)
 #pragma unroll
   for (int q = 0; q < 2; ++q) xmax = (fabsf(x[q]) <= 3.0e38f) ? fmaxf(xmax, fabsf(x[q])) : INFINITY;
   xmax = block_absmaxf<LTH>(xmax, red8);
+  cl.barrier_wait();
   if (tid < LCL) {   // to every CTA of the cluster
     float* st = cl.map_shared_rank(&s_state[rank][0], tid);
     st[0] = fallback ? 1.f : 0.f;

@@ -26,7 +26,8 @@ def kernel_body(name):
 
 
 # (kernel, what a CTA sets in its own shared memory that others write into)
-@pytest.mark.parametrize("name,setup", [("k_leaf_inv_d", "step[tid] = -1;")])
+@pytest.mark.parametrize("name,setup", [("k_leaf_inv_d", "step[tid] = -1;"),
+                                        ("k_leaf_inv_f", None)])
 def test_cluster_has_started_before_the_first_remote_write(name, setup):
     body = kernel_body(name)
     remote = body.index("map_shared_rank")
