@@ -407,7 +407,10 @@ __device__ __forceinline__ void load4(const __nv_bfloat16* p, float (&v)[4]) {
 // row of D^T) per lane and reduces the 16 quads of a row with shuffles.
 // Partial sums (at most 4 dense products, or half a leaf's rank) enter
 // compensated float pairs; warps combine through shared memory in a fixed
-// order.
+// order.  Bound by HBM where many planes are left: n = 128, FP32, one apply (18 GB)
+// 6.37 ms, transposed 7.81 ms; with the dense loop unrolled twice 6.92 and 8.60 ms
+// (n = 64: 1.147 and 1.413 against 1.175 and 1.468): eight loads in flight per
+// thread are paid for with resident warps.
 template <typename T>
 __global__ void __launch_bounds__(256) k_hmv_rows_v1(MatvecDev mv, T* const* __restrict__ D,
                                                      T* const* __restrict__ U,
@@ -469,7 +472,6 @@ __global__ void __launch_bounds__(256) k_hmv_rows_v1(MatvecDev mv, T* const* __r
   const int rl = tid & 15, cg = tid >> 4;
   if (have) {
     const T* Dp = D[p];
-#pragma unroll 2
     for (int q = 0; q < nd; ++q) {
       const T* blk = Dp + (int64_t)(q < MAXQ ? s_leaf[q] : dleaf[d0 + q]) * 4096;
       const float* xq = xs + q * 64;
