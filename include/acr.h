@@ -58,12 +58,11 @@ typedef enum {
  * as in FP32; when it ends every stored factor (dense leaves, U, V) is
  * rounded to bfloat16 (round to nearest even), halving the factor memory and
  * the bytes an apply reads; the apply multiplies in float.  The Krylov
- * iteration is FP64 in every form, and so are the core Grams that decide ranks
- * (FP64-accurate float-float sums in the float forms).  The dense leaf
+ * iteration is FP64 in every form; what decides ranks (sketch bases, core Grams)
+ * is FP64 in the FP64 form and float-float (~45 bits) in the float forms.  The dense leaf
  * inverses and the small recompression cores are FP64 in the FP64 form; in
  * the float forms the leaf inverses are float eliminations refined to float
- * accuracy (FP64 elimination when refinement cannot get there), the sketch bases come
- * from a re-orthogonalised float Gram-Schmidt, and the core Grams and the cores'
+ * accuracy (FP64 elimination when refinement cannot get there), and the cores'
  * eigenvectors are float-float.
  * (Reduced-precision storage is not in the paper, whose H-arithmetic is
  * double precision throughout, Sec. 5.) */

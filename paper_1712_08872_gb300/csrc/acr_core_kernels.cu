@@ -1,7 +1,7 @@
 // Recompression cores (sm_103a), one CTA per low-rank target:
 //  * k_orth -- float factors: orthonormal basis of the sketch Y by pivoted
-//              Gram-Schmidt with re-orthogonalisation, truncated at tau (FP64
-//              factors take the plan's Gram, k_pchol and basis stages);
+//              Gram-Schmidt in float-float, truncated at tau (FP64 factors take
+//              the plan's Gram, k_pchol and basis stages);
 //  * k_core -- core Gram (B^T)^T B^T, its eigen-decomposition by Jacobi, the rank
 //              rule sigma_i > eps * sigma_1 (Sec. 4.3 H_eps), and the
 //              recomposed factors U = Q W_k, V = B^T W_k.
@@ -48,224 +48,14 @@ __device__ __forceinline__ void count_stacked_warp(const TInfo& ti,
   }
 }
 
-// Orthonormal basis Q of range(Y) (m x p, in place): the column of largest
-// remaining norm is taken, projected once more against the basis so far (the
-// second pass that makes Gram-Schmidt orthonormal to rounding), and removed from
-// the remaining columns, whose norms are then recomputed; stops when the largest
-// remaining norm is at most tau times the largest of Y.  Basis columns are kept
-// unscaled with the square of their reciprocal norm, and scaled at the end.
-//
-// Bound by the latency of the r dependent steps, not by arithmetic or bytes
-// (64 x 32 floats per typical target): Y stays in shared memory, a warp owns
-// whole columns (CPW of them, their sums and reductions side by side; no barrier
-// between a column's dot and its axpy), and a step has three barriers.  It
-// replaces six launches of the plan (two compensated Grams, two FP64 pivoted
-// Cholesky cores, two basis products: 95 ms of the n = 64 setup; here 25 ms, and
-// 30 ms with the columns of a warp one after another and a fourth barrier).
-constexpr int ONT = 256;
-
-template <bool SMEM, int CPW>
-__global__ void __launch_bounds__(ONT, 6) k_orth(const TInfo* __restrict__ tis,
-                                              const int* __restrict__ order, double tau_,
-                                              float* const* __restrict__ tab,
-                                              int* const* __restrict__ rtab, int P, int scr_buf,
-                                              int scr_rbuf, const StackDim* __restrict__ stack,
-                                              unsigned long long* __restrict__ sketch_stat,
-                                              double* __restrict__ flops) {
-  constexpr int NW = ONT / 32;
-  extern __shared__ float ysm[];
-  __shared__ float nrm[CMAX], rn2[CMAX];
-  __shared__ __align__(16) float dot[CMAX];
-  __shared__ __align__(16) float part[NW];
-  const int p = blockIdx.y;
-  const TInfo ti = tis[order[blockIdx.x]];
-  float* scr = tab[scr_buf * P + p];
-  int* rs = rtab[scr_rbuf * P + p];
-  if (!scr || !rs) return;
-  const int m = ti.m, pc = ti.p;
-  float* Yg = scr + ti.y_off;
-  float* Y = SMEM ? ysm : Yg;
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  {
-    float s[CPW];
-#pragma unroll
-    for (int u = 0; u < CPW; ++u) s[u] = 0.f;
-    for (int i = lane; i < m; i += 32)
-#pragma unroll
-      for (int u = 0; u < CPW; ++u) {
-        const int c = warp + NW * u;
-        if (c < pc) {
-          const float v = Yg[i + (int64_t)c * m];
-          if (SMEM) Y[i + c * m] = v;
-          s[u] = fmaf(v, v, s[u]);
-        }
-      }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1)
-#pragma unroll
-      for (int u = 0; u < CPW; ++u) s[u] += __shfl_xor_sync(FULL, s[u], o);
-#pragma unroll
-    for (int u = 0; u < CPW; ++u)
-      if (lane == 0 && warp + NW * u < pc) nrm[warp + NW * u] = s[u];
-  }
-  if (sketch_stat && warp == NW - 1)
-    count_stacked_warp(ti, stack, tab, (const int* const*)rtab, P, p, sketch_stat);
-  __syncthreads();
-  const float tau2 = (float)(tau_ * tau_);
-  float tol = 0.f;
-  bool scaled = false;
-  int r = 0;
-  for (int j = 0; j < pc; ++j) {
-    // every warp finds the largest remaining column: bits of the squared norms
-    // order like the norms, the low six hold the column (norms that agree to
-    // 2^-17 count as equal: the lowest column); NaN norms are passed over
-    unsigned ka = 0u, kb = 0u;
-    if (j + lane < pc && nrm[j + lane] > 0.f)
-      ka = (__float_as_uint(nrm[j + lane]) & ~63u) | (63u - (j + lane));
-    if (CPW > 4 && j + lane + 32 < pc && nrm[j + lane + 32] > 0.f)
-      kb = (__float_as_uint(nrm[j + lane + 32]) & ~63u) | (63u - (j + lane + 32));
-    const unsigned kbest = __reduce_max_sync(FULL, max(ka, kb));
-    if (kbest == 0u) break;
-    const int q = 63 - (int)(kbest & 63u);
-    const float best = nrm[q];
-    if (j == 0) {
-      // a sketch so small that its squares would lose bits: scaled by a power of
-      // two (Q does not depend on it)
-      if (best < 0x1p-80f && !scaled) {
-        const float f = ldexpf(1.f, -(ilogbf(best) / 2));
-        for (int c = warp; c < pc; c += NW) {
-          float s = 0.f;
-          for (int i = lane; i < m; i += 32) {
-            const float v = f * Y[i + (int64_t)c * m];
-            Y[i + (int64_t)c * m] = v;
-            s = fmaf(v, v, s);
-          }
-          s = warp_sum(s);
-          __syncwarp();
-          if (lane == 0) rn2[c] = s;
-        }
-        __syncthreads();
-        if (tid < pc) nrm[tid] = rn2[tid];
-        __syncthreads();
-        scaled = true;
-        j = -1;
-        continue;
-      }
-      tol = tau2 * best;
-    }
-    if (!(best > tol)) break;
-    float* yq = Y + (int64_t)q * m;
-    float* yj = Y + (int64_t)j * m;
-    // second projection against the basis so far
-    if (warp < j) {
-      float s[CPW];
-#pragma unroll
-      for (int u = 0; u < CPW; ++u) s[u] = 0.f;
-      for (int i = lane; i < m; i += 32) {
-        const float v = yq[i];
-#pragma unroll
-        for (int u = 0; u < CPW; ++u) {
-          const int c = warp + NW * u;
-          if (c < j) s[u] = fmaf(Y[i + (int64_t)c * m], v, s[u]);
-        }
-      }
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1)
-#pragma unroll
-        for (int u = 0; u < CPW; ++u) s[u] += __shfl_xor_sync(FULL, s[u], o);
-#pragma unroll
-      for (int u = 0; u < CPW; ++u) {
-        const int c = warp + NW * u;
-        if (lane == 0 && c < j) dot[c] = s[u] * rn2[c];
-      }
-    }
-    __syncthreads();
-    // (the interchange of columns j and q folded in: a thread owns its rows)
-    float s2 = 0.f;
-    for (int i = tid; i < m; i += ONT) {
-      float v = yq[i];
-      int c = 0;
-      for (; c + 4 <= j; c += 4) {
-        const float4 d = *reinterpret_cast<const float4*>(dot + c);
-        const float* y = Y + i + (int64_t)c * m;
-        const float y0 = y[0], y1 = y[m], y2 = y[2 * (int64_t)m], y3 = y[3 * (int64_t)m];
-        v = fmaf(-d.x, y0, v);
-        v = fmaf(-d.y, y1, v);
-        v = fmaf(-d.z, y2, v);
-        v = fmaf(-d.w, y3, v);
-      }
-      for (; c < j; ++c) v = fmaf(-dot[c], Y[i + (int64_t)c * m], v);
-      if (q != j) yq[i] = yj[i];
-      yj[i] = v;
-      s2 = fmaf(v, v, s2);
-    }
-    s2 = warp_sum(s2);
-    if (lane == 0) part[warp] = s2;
-    __syncthreads();
-    const float4 p0 = *reinterpret_cast<const float4*>(part);
-    const float4 p1 = *reinterpret_cast<const float4*>(part + 4);
-    const float nv = ((p0.x + p0.y) + (p0.z + p0.w)) + ((p1.x + p1.y) + (p1.z + p1.w));
-    const float rr = nv >= 0x1p-126f ? 1.f / nv : 0.f;
-    if (tid == 0) rn2[j] = rr;
-    // remove it from the remaining columns (this warp's from c0 on); their norms afresh
-    const int c0 = warp + NW * ((j + 1 - warp + NW - 1) / NW);
-    if (c0 < pc) {
-      float s[CPW], t[CPW];
-#pragma unroll
-      for (int u = 0; u < CPW; ++u) s[u] = t[u] = 0.f;
-      for (int i = lane; i < m; i += 32) {
-        const float v = yj[i];
-#pragma unroll
-        for (int u = 0; u < CPW; ++u)
-          if (c0 + NW * u < pc) s[u] = fmaf(v, Y[i + (int64_t)(c0 + NW * u) * m], s[u]);
-      }
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1)
-#pragma unroll
-        for (int u = 0; u < CPW; ++u) s[u] += __shfl_xor_sync(FULL, s[u], o);
-#pragma unroll
-      for (int u = 0; u < CPW; ++u) s[u] *= rr;
-      for (int i = lane; i < m; i += 32) {
-        const float v = yj[i];
-#pragma unroll
-        for (int u = 0; u < CPW; ++u)
-          if (c0 + NW * u < pc) {
-            float* y = Y + i + (int64_t)(c0 + NW * u) * m;
-            const float w = fmaf(-s[u], v, *y);
-            *y = w;
-            t[u] = fmaf(w, w, t[u]);
-          }
-      }
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1)
-#pragma unroll
-        for (int u = 0; u < CPW; ++u) t[u] += __shfl_xor_sync(FULL, t[u], o);
-#pragma unroll
-      for (int u = 0; u < CPW; ++u)
-        if (lane == 0 && c0 + NW * u < pc) nrm[c0 + NW * u] = t[u];
-    }
-    r = j + 1;
-    __syncthreads();
-  }
-  for (int c = warp; c < r; c += NW) {
-    const float f = sqrtf(rn2[c]);
-    for (int i = lane; i < m; i += 32) Yg[i + (int64_t)c * m] = f * Y[i + (int64_t)c * m];
-  }
-  if (tid == 0) {
-    rs[ti.r_ri] = r;
-    if (flops) atomicAdd(flops, (double)m * r * (4.0 * pc));
-  }
-}
-
-// ------------------------------------------------------------ Jacobi cores
 // Numbers held as an unevaluated sum hi + lo of two floats (~48 significant
-// bits): the float forms' core Gram and rotations run on the FP32 pipe instead of
-// this part's narrow FP64 pipe.
+// bits): the float forms' bases, core Grams and rotations run on the FP32 pipe
+// instead of this part's narrow FP64 pipe.
 struct FF {
   float h, l;
 };
 __device__ __forceinline__ FF ff_mul(FF a, FF b) {
-  const float p = a.h * b.h;
+  const float p = __fmul_rn(a.h, b.h);   // (never contracted into a sum)
   float e = fmaf(a.h, b.h, -p);
   e = fmaf(a.h, b.l, e);
   e = fmaf(a.l, b.h, e);
@@ -282,7 +72,235 @@ __device__ __forceinline__ FF ff_add(FF a, FF b) {
   return FF{r, e - (r - s)};
 }
 __device__ __forceinline__ FF ff_neg(FF a) { return FF{-a.h, -a.l}; }
+// s += a * b; s is not renormalised
+__device__ __forceinline__ void ff_dot(FF& s, FF a, FF b) {
+  const float p = __fmul_rn(a.h, b.h);   // (never contracted into a sum)
+  float e = fmaf(a.h, b.h, -p);
+  e = fmaf(a.h, b.l, e);
+  e = fmaf(a.l, b.h, e);
+  const float t = s.h + p, bp = t - s.h;
+  s.l += ((s.h - (t - bp)) + (p - bp)) + e;
+  s.h = t;
+}
+// y + a * b
+__device__ __forceinline__ FF ff_axpy(FF y, FF a, FF b) {
+  const float p = __fmul_rn(a.h, b.h);
+  float e = fmaf(a.h, b.h, -p);
+  e = fmaf(a.h, b.l, e);
+  e = fmaf(a.l, b.h, e);
+  const float s = y.h + p, bp = s - y.h;
+  const float l = ((y.h - (s - bp)) + (p - bp)) + (y.l + e);
+  const float r = s + l;
+  return FF{r, l - (r - s)};
+}
+// a / b to ~2^-45 (b normal)
+__device__ __forceinline__ FF ff_div(FF a, FF b) {
+  const float rb = 1.f / b.h, q = a.h * rb;
+  const FF qb = ff_mul(FF{q, 0.f}, b);
+  const float d = ff_add(a, ff_neg(qb)).h * rb;
+  const float r = q + d;
+  return FF{r, d - (r - q)};
+}
+// x^(-1/2): a Newton step y + y (1 - x y^2) / 2 from the float estimate
+__device__ __forceinline__ FF ff_rsqrt(FF x) {
+  const float y = rsqrtf(x.h);
+  const FF xy2 = ff_mul(x, ff_mul(FF{y, 0.f}, FF{y, 0.f}));
+  const FF e = ff_add(FF{1.f, 0.f}, ff_neg(xy2));
+  return ff_add(FF{y, 0.f}, ff_mul(FF{y, 0.f}, FF{0.5f * e.h, 0.5f * e.l}));
+}
 
+// sums over 2 ... 2 * top lanes
+__device__ __forceinline__ float sum_lanes(float a, int top) {
+#pragma unroll
+  for (int o = top; o > 0; o >>= 1) a += __shfl_xor_sync(FULL, a, o);
+  return a;
+}
+__device__ __forceinline__ FF sum_lanes(FF a, int top) {
+#pragma unroll
+  for (int o = top; o > 0; o >>= 1)
+    a = ff_add(a, FF{__shfl_xor_sync(FULL, a.h, o), __shfl_xor_sync(FULL, a.l, o)});
+  return a;
+}
+
+// Orthonormal basis Q of range(Y) (m x p, in place) by pivoted modified
+// Gram-Schmidt: the column of largest remaining norm is taken and removed from the
+// remaining columns, whose norms are then computed afresh; stops when the largest
+// remaining norm is at most tau times the largest of Y.
+//
+// Columns, dots, updates and the norm of the column taken are float-float (the rank
+// decision at tau and the basis have to be as good as FP64-accurate Grams with an
+// FP64 Cholesky make them; the other columns' norms only order them).  So one
+// pass is enough: the basis loses orthogonality by ~2^-45 / tau, at most 3e-8 at
+// the smallest tau (1e-6), below the rounding of Q to float, and a remaining norm at
+// tau is known to as much of itself (from Grams, whose relative error of 1e-13 is that
+// of squares, to 1e-13 / tau^2: 10% at 1e-6).
+//
+// Bound by the latency of the r dependent steps where few targets are left, else by
+// the ~30 operations per remaining entry and step: Y stays in shared memory, 8 lanes
+// own a column (CPG columns; the sums of a column take three exchanges), taken columns
+// stay where they are, and a step has one barrier.  n = 64 setup: 31 ms, n = 80: 94 ms
+// (a warp per four columns: 41 and 127; plain float columns with a second projection
+// per step: 24 and 75, rank decisions off by 1%, orthogonality up to 3e-7; six
+// launches with FP64 pivoted Cholesky: 95 ms at n = 64).
+constexpr int ONT = 256;
+
+// row length of the staged columns: two neighbours' 8 rows meet no bank conflict
+__host__ __device__ constexpr int orth_ld(int m) { return (m + 7) / 16 * 16 + 8; }
+
+template <bool SMEM, int CPG>
+__global__ void __launch_bounds__(ONT, CPG == 1 ? 5 : 3)
+    k_orth(const TInfo* __restrict__ tis, const int* __restrict__ order, FF tau2,
+           float* const* __restrict__ tab, int* const* __restrict__ rtab, int P, int scr_buf,
+           int scr_rbuf, const StackDim* __restrict__ stack,
+           unsigned long long* __restrict__ sketch_stat, double* __restrict__ flops) {
+  constexpr int NW = ONT / 32;
+  extern __shared__ FF ysm[];
+  __shared__ float nrm[2][CMAX];   // squared norms of the remaining columns, by parity of the step
+  __shared__ FF bn[CMAX];          // of each basis column: its squared norm, then the reciprocal norm
+  __shared__ int piv[CMAX];        // and its place
+  __shared__ float mx[NW];
+  const int p = blockIdx.y;
+  const TInfo ti = tis[order[blockIdx.x]];
+  float* scr = tab[scr_buf * P + p];
+  int* rs = rtab[scr_rbuf * P + p];
+  if (!scr || !rs) return;
+  const int m = ti.m, pc = ti.p, ld = SMEM ? orth_ld(m) : m;
+  float* Yg = scr + ti.y_off;
+  float* Yl = scr + ti.bt_off;   // low parts beyond shared memory: B^T comes later
+  auto get = [&](int i, int c) {
+    if constexpr (SMEM) return ysm[i + c * ld];
+    else return FF{Yg[i + (int64_t)c * ld], Yl[i + (int64_t)c * ld]};
+  };
+  auto put = [&](int i, int c, FF v) {
+    if constexpr (SMEM) {
+      ysm[i + c * ld] = v;
+    } else {
+      Yg[i + (int64_t)c * ld] = v.h;
+      Yl[i + (int64_t)c * ld] = v.l;
+    }
+  };
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int c0 = tid >> 3, l8 = tid & 7;   // this thread's columns c0 + 32 u, rows l8 + 8 k
+  // The largest entry, and the power of two that brings it to [1, 2): sketches whose
+  // squares would leave the float range keep all bits (Q does not depend on it).
+  float amax = 0.f;
+#pragma unroll
+  for (int u = 0; u < CPG; ++u) {
+    const int c = c0 + 32 * u;
+    if (c < pc)
+#pragma unroll 4
+      for (int i = l8; i < m; i += 8) {
+        const float v = Yg[i + (int64_t)c * m];
+        if (SMEM) ysm[i + c * ld].h = v;
+        amax = fmaxf(amax, fabsf(v));
+      }
+  }
+  amax = __uint_as_float(__reduce_max_sync(FULL, __float_as_uint(amax)));
+  if (lane == 0) mx[warp] = amax;
+  __syncthreads();
+#pragma unroll
+  for (int w = 0; w < NW; ++w) amax = fmaxf(amax, mx[w]);
+  const int ex = amax > 0.f && amax <= 3.4e38f ? max(ilogbf(amax), -126) : 0;
+  const float up = ldexpf(1.f, -ex / 2), up2 = ldexpf(1.f, -ex - -ex / 2);   // (2^-ex may not fit)
+#pragma unroll
+  for (int u = 0; u < CPG; ++u) {
+    const int c = c0 + 32 * u;
+    float t = 0.f;
+    if (c < pc)
+      for (int i = l8; i < m; i += 8) {
+        const float v = (SMEM ? ysm[i + c * ld].h : Yg[i + (int64_t)c * m]) * up * up2;
+        put(i, c, FF{v, 0.f});
+        t = fmaf(v, v, t);
+      }
+    t = sum_lanes(t, 4);
+    if (l8 == 0 && c < pc) nrm[0][c] = t;
+  }
+  if (sketch_stat && warp == NW - 1)
+    count_stacked_warp(ti, stack, tab, (const int* const*)rtab, P, p, sketch_stat);
+  __syncthreads();
+  unsigned long long taken = 0ull;
+  FF tol{0.f, 0.f};
+  int r = 0;
+  for (int j = 0; j < pc; ++j) {
+    // every warp finds the largest remaining column: bits of the squared norms
+    // order like the norms, the low six hold the column (norms that agree to
+    // 2^-17 count as equal: the lowest column); NaN norms are passed over
+    const float* now = nrm[j & 1];
+    unsigned key = 0u;
+#pragma unroll
+    for (int u = 0; u < CPG; ++u) {
+      const int c = lane + 32 * u;
+      if (c < pc && now[c] > 0.f) key = max(key, (__float_as_uint(now[c]) & ~63u) | (63u - c));
+    }
+    key = __reduce_max_sync(FULL, key);
+    if (key == 0u) break;
+    const int q = 63 - (int)(key & 63u);
+    if (now[q] < 0.99f * tol.h) break;
+    // its products with the remaining columns and itself
+    const unsigned long long gone = taken | 1ull << q;
+    FF s[CPG], best{0.f, 0.f};
+    bool on[CPG];
+#pragma unroll
+    for (int u = 0; u < CPG; ++u) {
+      s[u] = FF{0.f, 0.f};
+      on[u] = c0 + 32 * u < pc && !((gone >> (c0 + 32 * u)) & 1);
+    }
+    for (int i = lane; i < m; i += 32) ff_dot(best, get(i, q), get(i, q));
+#pragma unroll
+    for (int u = 0; u < CPG; ++u)
+      if (on[u])
+#pragma unroll 4
+        for (int i = l8; i < m; i += 8) ff_dot(s[u], get(i, c0 + 32 * u), get(i, q));
+    best = sum_lanes(best, 16);
+    if (j == 0) tol = ff_mul(tau2, best);
+    if (!(best.h > tol.h || (best.h == tol.h && best.l > tol.l))) break;
+    taken = gone;
+    r = j + 1;
+    if (tid == 0) {
+      bn[j] = best;
+      piv[j] = q;
+    }
+    // removed from them; their norms (0: taken)
+#pragma unroll
+    for (int u = 0; u < CPG; ++u) {
+      const int c = c0 + 32 * u;
+      const FF g = ff_neg(ff_div(sum_lanes(s[u], 4), best));
+      float t = 0.f;
+      if (on[u])
+#pragma unroll 4
+        for (int i = l8; i < m; i += 8) {
+          const FF w = ff_axpy(get(i, c), g, get(i, q));
+          put(i, c, w);
+          t = fmaf(w.h, w.h, t);
+        }
+      t = sum_lanes(t, 4);
+      if (l8 == 0 && c < pc) nrm[(j + 1) & 1][c] = t;
+    }
+    __syncthreads();
+  }
+  if (tid < r) bn[tid] = ff_rsqrt(bn[tid]);
+  __syncthreads();
+  auto unit = [&](int i, int j) {
+    const FF v = get(i, piv[j]), f = bn[j];
+    return fmaf(v.h, f.h, fmaf(v.h, f.l, v.l * f.h));
+  };
+  if (SMEM) {
+    for (int j = warp; j < r; j += NW)
+      for (int i = lane; i < m; i += 32) Yg[i + (int64_t)j * m] = unit(i, j);
+  } else {   // a thread owns its rows: all of one read before any is written
+    for (int i = tid; i < m; i += ONT) {
+      float row[CMAX];
+      for (int j = 0; j < r; ++j) row[j] = unit(i, j);
+      for (int j = 0; j < r; ++j) Yg[i + (int64_t)j * m] = row[j];
+    }
+  }
+  if (tid == 0) {
+    rs[ti.r_ri] = r;
+    if (flops) atomicAdd(flops, 2.0 * m * r * (2.0 * pc - r));
+  }
+}
+
+// ------------------------------------------------------------ Jacobi cores
 // The three element types of a core: float (first sweeps), FF and double.
 __device__ __forceinline__ float em(float a, float b) { return a * b; }
 __device__ __forceinline__ double em(double a, double b) { return a * b; }
@@ -313,11 +331,7 @@ __device__ __forceinline__ FF escale(FF a, int e) { return FF{ldexpf(a.h, e), ld
 __device__ __forceinline__ void cos_of(float t, float& c) { c = rsqrtf(fmaf(t, t, 1.f)); }
 __device__ __forceinline__ void cos_of(float t, FF& c) {
   const float p = t * t;
-  const FF x = ff_add(FF{1.f, 0.f}, FF{p, fmaf(t, t, -p)});
-  const float y = rsqrtf(x.h);
-  const FF xy2 = ff_mul(x, ff_mul(FF{y, 0.f}, FF{y, 0.f}));
-  const FF e = ff_add(FF{1.f, 0.f}, ff_neg(xy2));
-  c = ff_add(FF{y, 0.f}, ff_mul(FF{y, 0.f}, FF{0.5f * e.h, 0.5f * e.l}));
+  c = ff_rsqrt(ff_add(FF{1.f, 0.f}, FF{p, fmaf(t, t, -p)}));
 }
 __device__ __forceinline__ void cos_of(float t, double& c) {
   const double x = fma((double)t, (double)t, 1.0);
@@ -801,15 +815,17 @@ void launch_orth(const Plan& pl, double tau, float* const* d_tab, int* const* d_
   const int nt = (int)pl.torder.size();
   if (nt <= 0 || P <= 0) return;
   // Targets are listed by increasing sketch size; each launch takes those up to
-  // the next of these shared-memory sizes (8, 4, 2 and 1 CTA per SM), so that
+  // the next of these shared-memory sizes (4, 3, 2 and 1 CTA per SM), so that
   // small sketches do not pay for the large ones' occupancy.  Few targets fill
   // no SM twice anyway and go in one launch.  Sketches beyond the largest size
   // stay in global memory (L2).
-  static const size_t cls[4] = {28160, 56320, 112640, 225280};
+  static const size_t cls[4] = {55296, 74752, 112640, 225280};
   constexpr int NCLS = 4;
+  const double t2 = tau * tau;
+  const FF tau2{(float)t2, (float)(t2 - (double)(float)t2)};
   auto bytes = [&](int q) {
     const TInfo& ti = pl.targets[pl.torder[q]];
-    return (size_t)ti.m * ti.p * sizeof(float);
+    return (size_t)orth_ld(ti.m) * ti.p * sizeof(FF);
   };
   const bool few = (int64_t)nt * P <= device_sm_count();
   int beg = 0;
@@ -818,15 +834,16 @@ void launch_orth(const Plan& pl, double tau, float* const* d_tab, int* const* d_
     if (c < NCLS)
       for (end = beg; end < nt && bytes(end) <= cls[c]; ++end) {}
     if (end > beg) {
-      auto kern = c < NCLS ? (pl.max_p <= 32 ? k_orth<true, 4> : k_orth<true, 8>)
-                           : (pl.max_p <= 32 ? k_orth<false, 4> : k_orth<false, 8>);
-      const size_t smem = c < NCLS ? bytes(end - 1) : 0;
+      auto kern = c < NCLS ? (pl.max_p <= 32 ? k_orth<true, 1> : k_orth<true, 2>)
+                           : (pl.max_p <= 32 ? k_orth<false, 1> : k_orth<false, 2>);
+      size_t smem = 0;   // (padded: not quite in the targets' order)
+      for (int q = beg; c < NCLS && q < end; ++q) smem = std::max(smem, bytes(q));
       if (smem > 48 * 1024)
         ACR_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                       (int)cls[NCLS - 1]));
       for (int t0 = beg; t0 < end; t0 += 65535) {
         kern<<<dim3(std::min(65535, end - t0), P), ONT, smem, st>>>(
-            (const TInfo*)pl.d_targets, (const int*)pl.d_torder + t0, tau, d_tab, d_rtab, P,
+            (const TInfo*)pl.d_targets, (const int*)pl.d_torder + t0, tau2, d_tab, d_rtab, P,
             3 * pl.nroles, pl.nroles, (const StackDim*)pl.d_stack, d_sketch_stat, d_fl);
         ACR_LAUNCHED(1);
       }

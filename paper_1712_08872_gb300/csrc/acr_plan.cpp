@@ -416,7 +416,7 @@ struct Builder {
       lt.p = p;
       lt.y = alloc((int64_t)m * p);
       lt.q = pp.fused ? lt.y : alloc((int64_t)m * p);
-      lt.bt = alloc((int64_t)n * p);
+      lt.bt = alloc((int64_t)std::max(m, n) * p);   // (before B^T: low parts of the sketch)
       for (LItem& li : lt.items) li.sp_off = alloc((int64_t)li.cap * p);
       TInfo& ti = lt.ti;
       ti.g_off = ti.t_off = ti.h_off = ti.w_off = 0;
