@@ -5,22 +5,22 @@
 //  * k_proj32 : the FP64 vectors' chunk as floats (once, for every product that
 //               meets it), and per low-rank leaf the partial V_l^T X over each
 //               leaf-size chunk of its columns (transposed: U_l^T X);
-//  * k_tsum32 : the partial projections of a leaf summed, as floats;
+//  * k_tsum32 : the partial projections of a leaf (FP64) summed, as floats;
 //  * k_rows32 : per row chunk c, Y[c] = beta Y[c] + alpha (sum of dense leaves
 //               times X + sum of U_l[rows of c] TV_l).
-// Products and sums are float over runs of 64 products or fewer (projections: 32),
-// which enter compensated float pairs.
+// Products and sums are float over runs of at most 8 products, which enter
+// compensated float pairs, at every leaf size.
 //
 // The products are 64 x K x 32 with K of a few hundred to a thousand: CUDA-core
 // work of 32 multiply-adds per loaded entry, bound by shared-memory reads (two 16-byte
 // vectors per 16 products; 8 x 4 outputs per thread with the contraction split over two
 // halves of the CTA read less but held 128 registers and were slower: 104 against
-// 90 us).  A tcgen05 form (split TF32, M = 128 with hi and lo rows stacked) spent its
+// 90 us with sums of 64).  A tcgen05 form (split TF32, M = 128 with hi and lo rows stacked) spent its
 // time staging -- both operands through registers for the split, in core-matrix
 // order, the vectors converted from FP64 again for every chunk that reads them --
 // and took 236 us per launch on average for the n = 64 Helmholtz recipe (4096
-// x 32 per plane, up to 32 planes), its projections 94 us.  Here rows 90, projections
-// 34, sums 10 us; 32 vectors at n = 64: 3.8 ms per apply against 8.4 ms.
+// x 32 per plane, up to 32 planes), its projections 94 us.  32 vectors at n = 64: 4.5 ms
+// per apply against 8.4 ms.
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
@@ -36,6 +36,12 @@ namespace {
 
 constexpr int R = 32;                            // right-hand sides per pass
 constexpr int MAXLQ = 256;                       // low-rank leaves per chunk
+// Products in a float sum.  The rounding an apply adds (the relative defect of its
+// linearity, random vectors) is 0.72e-7 to 0.76e-7 with 8 at 25- to 64-point leaves, where
+// the groups of 8 right-hand sides have 0.66e-7 to 0.94e-7; with 16 it is 1.0e-7, with 64
+// 2.0e-7 (the tensor form had 2.7e-7).  Per apply at n = 64: 4.5 ms (64: 3.8 ms);
+// n = 48: 2.9 ms against 10.4 ms in groups of 8, n = 80: 8.7 ms against 34 ms.
+constexpr int RUN = 8;
 constexpr unsigned FULL = 0xffffffffu;
 
 __device__ __forceinline__ float ldf(float v) { return v; }
@@ -78,15 +84,14 @@ __device__ __forceinline__ int find_q(const int* cum, int nq, int t) {
 // A warp takes 8 columns of the chunk's low-rank leaves at a time (of one leaf or
 // several): 64 rows of them pass through its shared slice, and lane rr
 // accumulates the 8 products with right-hand side rr.
-template <typename T, int RUN>
+template <typename T>
 __global__ void __launch_bounds__(256) k_proj32(MatvecDev mv, T* const* __restrict__ U,
                                                 T* const* __restrict__ V,
                                                 const int* const* __restrict__ rank,
                                                 const double* const* __restrict__ x,
-                                                float2* __restrict__ tv, float* __restrict__ xf,
+                                                double* __restrict__ tv, float* __restrict__ xf,
                                                 bool trans, int64_t vs) {
   chain_begin();
-  constexpr int PR = RUN < 32 ? RUN : 32;
   __shared__ float xs[64][R + 1];
   __shared__ __align__(16) float zs[8][64][8];
   __shared__ int64_t s_off[MAXLQ];
@@ -148,11 +153,11 @@ __global__ void __launch_bounds__(256) k_proj32(MatvecDev mv, T* const* __restri
     float s[8], cc[8];
 #pragma unroll
     for (int k = 0; k < 8; ++k) { s[k] = 0.f; cc[k] = 0.f; }
-    for (int h = 0; h < lsz; h += PR) {
+    for (int h = 0; h < lsz; h += RUN) {
       float a[8];
 #pragma unroll
       for (int k = 0; k < 8; ++k) a[k] = 0.f;
-      const int rows = min(PR, lsz - h);
+      const int rows = min(RUN, lsz - h);
 #pragma unroll 8
       for (int i = 0; i < rows; ++i) {
         const float4 p0 = *reinterpret_cast<const float4*>(&z[h + i][0]);
@@ -169,7 +174,7 @@ __global__ void __launch_bounds__(256) k_proj32(MatvecDev mv, T* const* __restri
 #pragma unroll
     for (int k = 0; k < 8; ++k) {
       const int64_t o = __shfl_sync(FULL, out, k);
-      if (t0 + k < total) tv[o * R + lane] = make_float2(s[k], cc[k]);
+      if (t0 + k < total) tv[o * R + lane] = (double)s[k] + (double)cc[k];
     }
   }
 }
@@ -179,7 +184,7 @@ __global__ void __launch_bounds__(256) k_proj32(MatvecDev mv, T* const* __restri
 __global__ void __launch_bounds__(128) k_tsum32(MatvecDev mv, const void* const* __restrict__ U,
                                                 const int* const* __restrict__ rank,
                                                 const double* const* __restrict__ x,
-                                                const float2* __restrict__ tv,
+                                                const double* __restrict__ tv,
                                                 float* __restrict__ tf, bool trans) {
   chain_begin();
   const int p = blockIdx.y, l = blockIdx.x, lane = threadIdx.x & 15;
@@ -188,20 +193,18 @@ __global__ void __launch_bounds__(128) k_tsum32(MatvecDev mv, const void* const*
   const int nseg = trans ? mv.nsegt : mv.nseg;
   const int k = rank[p][l], s0 = sptr[l], s1 = sptr[l + 1];
   for (int j = threadIdx.x >> 4; j < k; j += 8) {
-    float s[2] = {0.f, 0.f}, c[2] = {0.f, 0.f};
-    const float4* src =
-        reinterpret_cast<const float4*>(tv + (((int64_t)p * nseg + s0) * mv.kc + j) * R) + lane;
+    double s[2] = {0.0, 0.0};
+    const double2* src =
+        reinterpret_cast<const double2*>(tv + (((int64_t)p * nseg + s0) * mv.kc + j) * R) + lane;
     const int64_t step = (int64_t)mv.kc * R / 2;
 #pragma unroll 4
     for (int sg = s0; sg < s1; ++sg, src += step) {
-      const float4 v = *src;
-      pair_add(s[0], c[0], v.x);
-      c[0] += v.y;
-      pair_add(s[1], c[1], v.z);
-      c[1] += v.w;
+      const double2 v = *src;
+      s[0] += v.x;
+      s[1] += v.y;
     }
     reinterpret_cast<float2*>(tf + (((int64_t)p * mv.nl + l) * mv.kc + j) * R)[lane] =
-        make_float2(s[0] + c[0], s[1] + c[1]);
+        make_float2((float)s[0], (float)s[1]);
   }
 }
 
@@ -211,7 +214,7 @@ __global__ void __launch_bounds__(128) k_tsum32(MatvecDev mv, const void* const*
 // enter compensated pairs.
 constexpr int WT = 128, ALD = 68, BLD = 36;
 
-template <typename T, int RUN>
+template <typename T>
 __global__ void __launch_bounds__(WT, 4)
     k_rows32(MatvecDev mv, T* const* __restrict__ D, T* const* __restrict__ U,
              T* const* __restrict__ V, const int* const* __restrict__ rank,
@@ -261,9 +264,7 @@ __global__ void __launch_bounds__(WT, 4)
       for (int a = 0; a < 4; ++a)
 #pragma unroll
         for (int b = 0; b < 4; ++b) acc[a][b] = 0.f;
-      const int k1 = min(k0 + RUN, kf);
-#pragma unroll 4
-      for (int k = k0; k < k1; ++k) {
+      auto product = [&](int k) {
         const float4 a4 = *reinterpret_cast<const float4*>(As + k * ALD + 4 * ty);
         const float4 b4 = *reinterpret_cast<const float4*>(Bs + k * BLD + 4 * tx);
         const float a[4] = {a4.x, a4.y, a4.z, a4.w}, b[4] = {b4.x, b4.y, b4.z, b4.w};
@@ -271,6 +272,12 @@ __global__ void __launch_bounds__(WT, 4)
         for (int u = 0; u < 4; ++u)
 #pragma unroll
           for (int v = 0; v < 4; ++v) acc[u][v] = fmaf(a[u], b[v], acc[u][v]);
+      };
+      if (k0 + RUN <= kf) {
+#pragma unroll
+        for (int k = 0; k < RUN; ++k) product(k0 + k);
+      } else {
+        for (int k = k0; k < kf; ++k) product(k);
       }
 #pragma unroll
       for (int u = 0; u < 4; ++u)
@@ -384,43 +391,21 @@ size_t wide_scratch_floats(const MatvecDev& mv, int P) {
   return (size_t)P * ((size_t)mv.nchunks * mv.lsz * R + (size_t)std::max(mv.nl, 1) * mv.kc * R);
 }
 
-namespace {
-
-template <typename T, int RUN>
-void run_wide(const MatvecDev& mv, T* const* dense, T* const* U, T* const* V,
-              const int* const* rank, const double* const* x, double* const* y, double alpha,
-              double beta, bool trans, double* tv, float* work, int P, int64_t vs,
-              cudaStream_t st) {
-  float* xf = work;
-  float* tf = work + (size_t)P * mv.nchunks * mv.lsz * R;
-  launch_chain(k_proj32<T, RUN>, dim3(mv.nchunks, P), 256, 0, st, mv, U, V, rank, x, (float2*)tv,
-               xf, trans, vs);
-  if (mv.nl > 0)
-    launch_chain(k_tsum32, dim3(mv.nl, P), 128, 0, st, mv, (const void* const*)(trans ? U : V),
-                 rank, x, (const float2*)tv, tf, trans);
-  launch_chain(k_rows32<T, RUN>, dim3(mv.nchunks, P), WT, 0, st, mv, dense, U, V, rank, x, y,
-               alpha, beta, xf, tf, trans, vs);
-  ACR_LAUNCHED(mv.nl > 0 ? 3 : 2);
-}
-
-}  // namespace
-
-// How many products enter a float sum, by leaf size.  The rounding an apply adds (the
-// relative defect of its linearity, random vectors): sums of 64 and 32: 2.0e-7 (the
-// tensor form of the 64-point leaves had 2.7e-7), of 16: 1.0e-7, of 8: 0.7e-7 to 0.8e-7, as
-// the groups of 8 right-hand sides have it (0.76e-7 to 0.84e-7 at 27 to 50
-// points), which other leaf sizes took before.  Per apply at n = 64: 3.8 ms with 64,
-// 4.6 ms with 8; n = 48, 8: 3.0 ms against 10.4 ms, n = 80: 8.8 ms against 34 ms.
 template <typename T>
 void launch_hmatvec_wide(const MatvecDev& mv, T* const* dense, T* const* U, T* const* V,
                          const int* const* rank, const double* const* x, double* const* y,
                          double alpha, double beta, bool trans, double* tv, float* work, int P,
                          int64_t vs, cudaStream_t st) {
   if (P <= 0) return;
-  if (mv.lsz == 64)
-    run_wide<T, 64>(mv, dense, U, V, rank, x, y, alpha, beta, trans, tv, work, P, vs, st);
-  else
-    run_wide<T, 8>(mv, dense, U, V, rank, x, y, alpha, beta, trans, tv, work, P, vs, st);
+  float* xf = work;
+  float* tf = work + (size_t)P * mv.nchunks * mv.lsz * R;
+  launch_chain(k_proj32<T>, dim3(mv.nchunks, P), 256, 0, st, mv, U, V, rank, x, tv, xf, trans, vs);
+  if (mv.nl > 0)
+    launch_chain(k_tsum32, dim3(mv.nl, P), 128, 0, st, mv, (const void* const*)(trans ? U : V),
+                 rank, x, tv, tf, trans);
+  launch_chain(k_rows32<T>, dim3(mv.nchunks, P), WT, 0, st, mv, dense, U, V, rank, x, y, alpha,
+               beta, xf, tf, trans, vs);
+  ACR_LAUNCHED(mv.nl > 0 ? 3 : 2);
 }
 
 template void launch_hmatvec_wide<float>(const MatvecDev&, float* const*, float* const*,
