@@ -27,6 +27,7 @@
 
 #include "acr.h"
 #include "acr_internal.h"
+#include "acr_tables.h"
 
 namespace acr {
 
@@ -397,11 +398,7 @@ class Engine : public EngineBase {
     size_t rank_cnt = 0;
     size_t need = 0, rank_need = 0;    // by the counting pass
     std::vector<void*> old;            // outgrown
-    struct {                           // the pointer tables of the last plan run
-      int64_t epoch = -1;
-      int nr = 0, pc = 0;
-      const void *scr = nullptr, *rscr = nullptr;
-      size_t stride = 0, rstride = 0;  // scratch bytes and rank slots per plane
+    struct : ScratchTables {           // the pointer tables of the last plan run
       std::vector<void*> host;
       void** dev = nullptr;
     } tabs;
@@ -420,6 +417,7 @@ class Engine : public EngineBase {
     if (k.ranks) cudaFree(k.ranks);
     k.scratch = nullptr; k.ranks = nullptr;
     k.bytes = k.rank_cnt = 0;
+    k.tabs.epoch = -1;
   }
   size_t scratch_budget = 0;
   double* d_coefs = nullptr;         // 1, -1 and the sign of products with coefficient 2
@@ -658,6 +656,7 @@ class Engine : public EngineBase {
       if (p) w->old.push_back(p);
       p = (V)q;
       have = need;
+      w->tabs.epoch = -1;
     };
     try {
       grow(w->scratch, 1, w->bytes, bytes);
@@ -822,9 +821,10 @@ class Engine : public EngineBase {
       // its planes' scratch is large enough (one H-inverse runs some 250 plans on the
       // same two H-matrices per plane: a copy before each of them cost as much as
       // a small plan's kernel).  New ones spread the planes over all of the scratch.
-      const bool same = tabs.epoch == ring.epoch && tabs.nr == nr && tabs.pc == pc &&
-                        tabs.scr == scr_base && tabs.rscr == scr_rank_base &&
-                        tabs.stride >= per_plane && tabs.rstride >= ranks && [&] {
+      const size_t have = dry ? w->need : w->bytes;
+      const size_t have_r = dry ? w->rank_need : w->rank_cnt;
+      const bool same = tabs.serve(ring.epoch, nr, pc, scr_base, scr_rank_base, per_plane, ranks,
+                                   have, have_r) && [&] {
                           for (int r = 0; r < nr; ++r)
                             for (int p = 0; p < pc; ++p) {
                               const HM& h = roles[r][c0 + p];
@@ -835,8 +835,6 @@ class Engine : public EngineBase {
                           return true;
                         }();
       if (!same) {
-        const size_t have = dry ? w->need : w->bytes;
-        const size_t have_r = dry ? w->rank_need : w->rank_cnt;
         tabs.nr = nr;
         tabs.pc = pc;
         tabs.scr = scr_base;
