@@ -870,11 +870,15 @@ class Engine : public EngineBase {
           timed(2, [&] { launch_core<T>(pl, eps, kc, c_role, d_tab, d_rtab, pc, d_err, st, fl(2)); });
           continue;
         }
-        if constexpr (std::is_same<T, float>::value)
+        if constexpr (std::is_same<T, float>::value) {
+          if (sg.kind != ST_ORTH) throw AcrError{S_UNSUPPORTED, "a plan stage without a kernel"};
           timed(1, [&] { launch_orth(pl, tau_orth(), d_tab, d_rtab, pc, st, d_sketch_stat, fl(1)); });
-        else
+        } else {
+          if (sg.kind != ST_PCHOL && sg.kind != ST_PCHOL + 16)
+            throw AcrError{S_UNSUPPORTED, "a plan stage without a kernel"};
           timed(1, [&] { launch_pchol<T>(pl, sg.beg, sg.end, sg.kind == ST_PCHOL, tau_orth(), d_tab,
                                          d_rtab, pc, st, d_sketch_stat, fl(1)); });
+        }
       }
     }
   }

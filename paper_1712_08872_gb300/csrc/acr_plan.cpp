@@ -567,6 +567,7 @@ struct Builder {
       if (!lts.empty()) P.stages.push_back(Stage{ST_CORE, 0, (int)lts.size()});
       return;
     }
+    // (unfused cores: the host check of the plans only; the engine has no kernel for ST_EIG)
     // H = (B^T)^T B^T   (r x r), core eigen-decomposition
     g0 = (int)P.groups.size();
     for (size_t i = 0; i < lts.size(); ++i) {
