@@ -63,7 +63,8 @@ __global__ void __launch_bounds__(256) k_stencil_poisson(const double* __restric
 }
 
 // (the FP64 pipe bounds it before memory does: three multiply-adds per axis, the
-// upwind choice by the sign bit instead of FP64 comparisons)
+// upwind choice by the bits instead of FP64 comparisons; a NaN is upstream of neither
+// side, as with fmax and fmin, and shows in the centre)
 __global__ void __launch_bounds__(256) k_stencil_codi(const double* __restrict__ beta,
                                                       double* __restrict__ coef, int n,
                                                       double ih2, double ih) {
@@ -75,10 +76,11 @@ __global__ void __launch_bounds__(256) k_stencil_codi(const double* __restrict__
 #pragma unroll
   for (int a = 0; a < 3; ++a) {
     const double b = beta[a * N + p];
-    const bool neg = __double2hiint(b) < 0;
+    const long long bits = __double_as_longlong(b);
+    const bool neg = bits < 0, nan = (bits & 0x7fffffffffffffffll) > 0x7ff0000000000000ll;
     c += fabs(b) * ih;
-    const double lo = -ih2 - (neg ? 0.0 : b) * ih;   // upstream for b > 0
-    const double hi = -ih2 + (neg ? b : 0.0) * ih;   // upstream for b < 0
+    const double lo = -ih2 - (neg || nan ? 0.0 : b) * ih;    // upstream for b > 0
+    const double hi = -ih2 + (neg && !nan ? b : 0.0) * ih;   // upstream for b < 0
     coef[(2 * a + 1) * N + p] = in[2 * a] ? lo : 0.0;
     coef[(2 * a + 2) * N + p] = in[2 * a + 1] ? hi : 0.0;
   }
