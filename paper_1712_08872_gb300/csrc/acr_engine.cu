@@ -2596,7 +2596,14 @@ acr_status acr_spmv(const acr_grid* grid, const double* coef, const double* x, d
                     int32_t nrhs, cudaStream_t stream) {
   if (!grid_ok(grid) || !coef || !x || !y || nrhs < 1) return ACR_ERR_INVALID_ARG;
   return guarded([&] {
-    acr::launch_spmv(coef, x, y, grid->nx, stream, nrhs);
+    const int64_t N = (int64_t)grid->nx * grid->nx * grid->nx;
+    // vectors that are another one's result (y = x + N: the powers A x, A^2 x, ...) one after
+    // the other, else in groups
+    const auto a = reinterpret_cast<uintptr_t>(x), b = reinterpret_cast<uintptr_t>(y);
+    const uintptr_t bytes = sizeof(double) * (uintptr_t)N * nrhs;
+    const int group = a < b + bytes && b < a + bytes ? 1 : nrhs;
+    for (int k = 0; k < nrhs; k += group)
+      acr::launch_spmv(coef, x + k * N, y + k * N, grid->nx, stream, group);
     return 0;
   });
 }

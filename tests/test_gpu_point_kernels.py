@@ -39,3 +39,22 @@ def test_codi_stencil_of_nan_and_infinite_velocities():
             assert np.array_equal(np.isfinite(got[k]), fin), k
             assert np.array_equal(got[k][~fin], want[~fin]), k
             assert np.abs(got[k][fin] - want[fin]).max() <= 2.3e-16 * np.abs(want[fin]).max(), k
+
+
+@pytest.mark.parametrize("n", [7, 33])
+def test_spmv_of_vectors_that_are_results(n):
+    """y = x + N: each vector is the result of the one before; equal to single products."""
+    acr = _acr()
+    N = n ** 3
+    gen = torch.Generator(device="cuda:0")
+    gen.manual_seed(5)
+    kappa = 1.0 + torch.rand(N, dtype=torch.float64, device="cuda:0", generator=gen)
+    coef = torch.empty(7 * N, dtype=torch.float64, device="cuda:0")
+    acr.acr_stencil_poisson(n, kappa, coef)
+    v = torch.zeros(7, N, dtype=torch.float64, device="cuda:0")
+    v[0] = kappa / n ** 2
+    want = v.clone()
+    for k in range(6):
+        acr.acr_spmv(n, coef, want[k], want[k + 1], 1)
+    acr.acr_spmv(n, coef, v.reshape(-1), v.reshape(-1)[N:], 6)
+    assert torch.equal(v, want)
