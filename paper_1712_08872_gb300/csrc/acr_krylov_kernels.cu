@@ -76,8 +76,8 @@ __global__ void __launch_bounds__(256) k_stencil_codi(const double* __restrict__
 #pragma unroll
   for (int a = 0; a < 3; ++a) {
     const double b = beta[a * N + p];
-    const long long bits = __double_as_longlong(b);
-    const bool neg = bits < 0, nan = (bits & 0x7fffffffffffffffll) > 0x7ff0000000000000ll;
+    const int hw = __double2hiint(b);
+    const bool neg = hw < 0, nan = ((hw & 0x7fffffff) | (__double2loint(b) != 0)) > 0x7ff00000;
     c += fabs(b) * ih;
     const double lo = -ih2 - (neg || nan ? 0.0 : b) * ih;    // upstream for b > 0
     const double hi = -ih2 + (neg && !nan ? b : 0.0) * ih;   // upstream for b < 0
