@@ -520,13 +520,13 @@ __device__ int jacobi(EL*& A, EL*& A2, EL* V, int r, int lda, float conv, int mo
 // the norm; the float rotations' product made orthonormal (Newton-Schulz, V =
 // W + W (I - W^T W) / 2: exact W^T W, the correction small enough for float; twice
 // for FP64); H transformed by it in the core's full arithmetic; then sweeps in
-// that arithmetic -- float-float to an off-diagonal mass of 1e-16, FP64 to 1e-30 --
+// that arithmetic -- float-float to an off-diagonal mass of 1e-16, or of eps^4 / 100 where
+// that is less (the rank rule compares eigenvalues down to eps^2), FP64 to 1e-30 --
 // which find a nearly diagonal matrix and need one (FP64: two) instead of six
 // to eight, at a twelfth of the operations per float sweep (FP64: a 64th).  The
 // result is no less accurate than with full arithmetic throughout: FP64, 56 columns, all
 // kept: U orthonormal to 6.9e-15 and U V^T to 7.3e-15 of the product (FP64
-// sweeps only: 2.7e-14 and 2.5e-14); float at eps 1e-5: the exact rank of 52 (float-float
-// sweeps only: 54, their stopping rule leaves eigenvalues of 1e-10 mixed).
+// sweeps only: 2.7e-14 and 2.5e-14).
 //
 // Bound by the latency of the ~6 (r - 1) dependent rounds of a core.  Four warps, so that a
 // typical core's round (r = 12: 21 blocks and 72 row pairs of V) is one pass over
@@ -753,7 +753,9 @@ __global__ void __launch_bounds__(CNT) k_core(const TInfo* __restrict__ tis, int
       A[j * lda + i] = t;
     }
     __syncthreads();
-    sweeps += jacobi<E>(A, A2, V, r, lda, F64 ? 1e-30f : 1e-16f, 40, red);
+    const float e2 = (float)(eps * eps);   // (pairs reach ~1e-27)
+    const float conv = F64 ? 1e-30f : fminf(1e-16f, fmaxf(1e-24f, 0.01f * e2 * e2));
+    sweeps += jacobi<E>(A, A2, V, r, lda, conv, 40, red);
   } else if (tid == 0) {
     es(V[0], 1.f);
   }

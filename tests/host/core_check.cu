@@ -241,6 +241,7 @@ int main() {
     core<float>(64, 50, r, 1e-2, 0.5);
     core<float>(100, 300, r, 1e-5, 0.8);
   }
+  for (int k = 0; k < 6; ++k) core<float>(100, 300, 56, 1e-5, 0.8);   // eigenvalues down to eps^2
   std::printf(fail ? "FAILED\n" : "all ok\n");
   return fail ? 1 : 0;
 }
