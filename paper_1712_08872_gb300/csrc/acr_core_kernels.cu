@@ -864,7 +864,7 @@ void launch_orth(const Plan& pl, double tau, float* const* d_tab, int* const* d_
                            : (pl.max_p <= 32 ? k_orth<false, 1> : k_orth<false, 2>);
       size_t smem = 0;   // (padded: not quite in the targets' order)
       for (int q = beg; c < NCLS && q < end; ++q) smem = std::max(smem, bytes(q));
-      if (smem > 48 * 1024)
+      if (smem > 40 * 1024)   // (48 KB without it, the kernel's own arrays included)
         ACR_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                       (int)cls[NCLS - 1]));
       for (int t0 = beg; t0 < end; t0 += 65535) {
@@ -884,7 +884,7 @@ void launch_core(const Plan& pl, double eps, int kc, int c_role, T* const* d_tab
   const int nt = (int)pl.targets.size();
   if (nt <= 0 || P <= 0) return;
   const size_t smem = core_smem(pl.max_p);
-  if (smem > 48 * 1024)
+  if (smem > 40 * 1024)
     ACR_CUDA(cudaFuncSetAttribute(k_core<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                   (int)core_smem(CMAX)));
   for (int t0 = 0; t0 < nt; t0 += 65535) {

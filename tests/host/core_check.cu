@@ -233,6 +233,10 @@ int main() {
     orth_ranks(36, 27, 1e-6, scale);
     orth_ranks(64, 32, 1e-5, scale);
     orth_ranks(100, 56, 1e-6, scale);
+    orth_ranks(144, 40, 1e-5, scale);    // 47.5 KB, beside the kernel's own arrays
+    orth_ranks(288, 42, 1e-5, scale);
+    orth_ranks(400, 32, 1e-6, scale);
+    orth_ranks(800, 34, 1e-5, scale);    // a whole SM's
     orth_ranks(1152, 56, 1e-5, scale);   // beyond shared memory
   }
   for (int r : {1, 2, 3, 12, 31, 56}) {
