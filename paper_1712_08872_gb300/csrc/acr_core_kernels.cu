@@ -5,6 +5,7 @@
 //  * k_core -- core Gram (B^T)^T B^T, its eigen-decomposition by Jacobi, the rank
 //              rule sigma_i > eps * sigma_1 (Sec. 4.3 H_eps), and the
 //              recomposed factors U = Q W_k, V = B^T W_k.
+#include <cooperative_groups.h>
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -15,6 +16,8 @@
 #include "acr_internal.h"
 
 namespace acr {
+
+namespace cg = cooperative_groups;
 
 namespace {
 
@@ -138,7 +141,12 @@ __device__ __forceinline__ FF sum_lanes(FF a, int top) {
 // Bound by the latency of the r dependent steps where few targets are left, else by
 // the ~30 operations per remaining entry and step: Y stays in shared memory, 8 lanes
 // own a column (CPG columns; the sums of a column take three exchanges), taken columns
-// stay where they are, and a step has one barrier.  n = 64 setup: 31 ms, n = 80: 94 ms
+// stay where they are, and a step has one barrier.  Sketches of which an SM holds only one
+// or none (m = 512 to 2048 at n = 128) are shared by a cluster of OCL CTAs by rows,
+// which push their parts of the sums into one another's shared memory: n = 128 setup 368
+// ms for the bases (larger ones in global memory: 785; the cluster only beyond one SM's
+// 220 KB: 370, and 94 in place of 89 at n = 80; from 54 KB on: 647 and 100).  Beyond the
+// cluster's memory they stay in global memory.  n = 64 setup: 30 ms, n = 80: 89 ms
 // (a warp per four columns: 41 and 127; plain float columns with a second projection
 // per step: 24 and 75, rank decisions off by 1%, orthogonality up to 3e-7; six
 // launches with FP64 pivoted Cholesky: 95 ms at n = 64).
@@ -147,40 +155,72 @@ constexpr int ONT = 256;
 // row length of the staged columns: two neighbours' 8 rows meet no bank conflict
 __host__ __device__ constexpr int orth_ld(int m) { return (m + 7) / 16 * 16 + 8; }
 
-template <bool SMEM, int CPG>
-__global__ void __launch_bounds__(ONT, CPG == 1 ? 5 : 3)
-    k_orth(const TInfo* __restrict__ tis, const int* __restrict__ order, FF tau2,
-           float* const* __restrict__ tab, int* const* __restrict__ rtab, int P, int scr_buf,
-           int scr_rbuf, const StackDim* __restrict__ stack,
-           unsigned long long* __restrict__ sketch_stat, double* __restrict__ flops) {
+constexpr int OCL = 8;   // CTAs of a cluster: the 8 lanes of a column write to one each
+enum OrthMode { ORTH_SM, ORTH_CLUSTER, ORTH_GLOBAL };
+
+template <int MODE, int CPG>
+__device__ __forceinline__ void orth(const TInfo& ti, int rank, FF tau2,
+                                     float* const* __restrict__ tab, int* const* __restrict__ rtab,
+                                     int P, int scr_buf, int scr_rbuf,
+                                     const StackDim* __restrict__ stack,
+                                     unsigned long long* __restrict__ sketch_stat,
+                                     double* __restrict__ flops) {
   constexpr int NW = ONT / 32;
+  constexpr bool SMEM = MODE != ORTH_GLOBAL, CL = MODE == ORTH_CLUSTER;
   extern __shared__ FF ysm[];
   __shared__ float nrm[2][CMAX];   // squared norms of the remaining columns, by parity of the step
   __shared__ FF bn[CMAX];          // of each basis column: its squared norm, then the reciprocal norm
   __shared__ int piv[CMAX];        // and its place
   __shared__ float mx[NW];
+  // the cluster's parts of the sums, written by its CTAs: products with the columns and of
+  // the column taken (last); norms; largest entries
+  __shared__ FF pdot[CL ? OCL : 1][CL ? CMAX + 1 : 1];
+  __shared__ float pnrm[CL ? OCL : 1][CL ? CMAX : 1], pmax[OCL];
+  cg::cluster_group cl = cg::this_cluster();
   const int p = blockIdx.y;
-  const TInfo ti = tis[order[blockIdx.x]];
   float* scr = tab[scr_buf * P + p];
   int* rs = rtab[scr_rbuf * P + p];
-  if (!scr || !rs) return;
-  const int m = ti.m, pc = ti.p, ld = SMEM ? orth_ld(m) : m;
-  float* Yg = scr + ti.y_off;
+  if (!scr || !rs) return;   // (the whole cluster)
+  if constexpr (CL) cl.sync();   // every CTA has started
+  // this CTA's rows
+  const int mr = CL ? (ti.m + OCL - 1) / OCL : ti.m, r0 = CL ? rank * mr : 0;
+  const int m = CL ? max(0, min(mr, ti.m - r0)) : ti.m, pc = ti.p;
+  const int64_t gld = ti.m;
+  const int ld = SMEM ? orth_ld(mr) : ti.m;
+  float* Yg = scr + ti.y_off + r0;
   float* Yl = scr + ti.bt_off;   // low parts beyond shared memory: B^T comes later
   auto get = [&](int i, int c) {
     if constexpr (SMEM) return ysm[i + c * ld];
-    else return FF{Yg[i + (int64_t)c * ld], Yl[i + (int64_t)c * ld]};
+    else return FF{Yg[i + gld * c], Yl[i + gld * c]};
   };
   auto put = [&](int i, int c, FF v) {
     if constexpr (SMEM) {
       ysm[i + c * ld] = v;
     } else {
-      Yg[i + (int64_t)c * ld] = v.h;
-      Yl[i + (int64_t)c * ld] = v.l;
+      Yg[i + gld * c] = v.h;
+      Yl[i + gld * c] = v.l;
     }
   };
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int c0 = tid >> 3, l8 = tid & 7;   // this thread's columns c0 + 32 u, rows l8 + 8 k
+  // a column's norm (the sum over this CTA's rows, in all 8 lanes) to the next step, in a
+  // cluster through every CTA's parts
+  auto give_norm = [&](float t, int c, float* next) {
+    if (c >= pc) return;
+    if constexpr (CL) *cl.map_shared_rank(&pnrm[rank][c], l8) = t;
+    else if (l8 == 0) next[c] = t;
+  };
+  auto take_norms = [&](float* next) {
+    if constexpr (CL) {
+      cl.sync();
+      if (tid < pc) {
+        float t = 0.f;
+#pragma unroll
+        for (int k = 0; k < OCL; ++k) t += pnrm[k][tid];
+        next[tid] = t;
+      }
+    }
+  };
   // The largest entry, and the power of two that brings it to [1, 2): sketches whose
   // squares would leave the float range keep all bits (Q does not depend on it).
   float amax = 0.f;
@@ -190,7 +230,7 @@ __global__ void __launch_bounds__(ONT, CPG == 1 ? 5 : 3)
     if (c < pc)
 #pragma unroll 4
       for (int i = l8; i < m; i += 8) {
-        const float v = Yg[i + (int64_t)c * m];
+        const float v = Yg[i + gld * c];
         if (SMEM) ysm[i + c * ld].h = v;
         amax = fmaxf(amax, fabsf(v));
       }
@@ -200,6 +240,12 @@ __global__ void __launch_bounds__(ONT, CPG == 1 ? 5 : 3)
   __syncthreads();
 #pragma unroll
   for (int w = 0; w < NW; ++w) amax = fmaxf(amax, mx[w]);
+  if constexpr (CL) {
+    if (tid < OCL) *cl.map_shared_rank(&pmax[rank], tid) = amax;
+    cl.sync();
+#pragma unroll
+    for (int k = 0; k < OCL; ++k) amax = fmaxf(amax, pmax[k]);
+  }
   const int ex = amax > 0.f && amax <= 3.4e38f ? max(ilogbf(amax), -126) : 0;
   const float up = ldexpf(1.f, -ex / 2), up2 = ldexpf(1.f, -ex - -ex / 2);   // (2^-ex may not fit)
 #pragma unroll
@@ -208,14 +254,14 @@ __global__ void __launch_bounds__(ONT, CPG == 1 ? 5 : 3)
     float t = 0.f;
     if (c < pc)
       for (int i = l8; i < m; i += 8) {
-        const float v = (SMEM ? ysm[i + c * ld].h : Yg[i + (int64_t)c * m]) * up * up2;
+        const float v = (SMEM ? ysm[i + c * ld].h : Yg[i + gld * c]) * up * up2;
         put(i, c, FF{v, 0.f});
         t = fmaf(v, v, t);
       }
-    t = sum_lanes(t, 4);
-    if (l8 == 0 && c < pc) nrm[0][c] = t;
+    give_norm(sum_lanes(t, 4), c, nrm[0]);
   }
-  if (sketch_stat && warp == NW - 1)
+  take_norms(nrm[0]);
+  if (sketch_stat && rank == 0 && warp == NW - 1)
     count_stacked_warp(ti, stack, tab, (const int* const*)rtab, P, p, sketch_stat);
   __syncthreads();
   unsigned long long taken = 0ull;
@@ -252,6 +298,25 @@ __global__ void __launch_bounds__(ONT, CPG == 1 ? 5 : 3)
 #pragma unroll 4
         for (int i = l8; i < m; i += 8) ff_dot(s[u], get(i, c0 + 32 * u), get(i, q));
     best = sum_lanes(best, 16);
+#pragma unroll
+    for (int u = 0; u < CPG; ++u) s[u] = sum_lanes(s[u], 4);
+    if constexpr (CL) {   // the sums over the cluster, by every CTA in the same order
+#pragma unroll
+      for (int u = 0; u < CPG; ++u)
+        if (on[u]) *cl.map_shared_rank(&pdot[rank][c0 + 32 * u], l8) = s[u];
+      if (tid < OCL) *cl.map_shared_rank(&pdot[rank][CMAX], tid) = best;
+      cl.sync();
+      best = FF{0.f, 0.f};
+#pragma unroll
+      for (int k = 0; k < OCL; ++k) best = ff_add(best, pdot[k][CMAX]);
+#pragma unroll
+      for (int u = 0; u < CPG; ++u)
+        if (on[u]) {
+          s[u] = FF{0.f, 0.f};
+#pragma unroll
+          for (int k = 0; k < OCL; ++k) s[u] = ff_add(s[u], pdot[k][c0 + 32 * u]);
+        }
+    }
     if (j == 0) tol = ff_mul(tau2, best);
     if (!(best.h > tol.h || (best.h == tol.h && best.l > tol.l))) break;
     taken = gone;
@@ -264,7 +329,7 @@ __global__ void __launch_bounds__(ONT, CPG == 1 ? 5 : 3)
 #pragma unroll
     for (int u = 0; u < CPG; ++u) {
       const int c = c0 + 32 * u;
-      const FF g = ff_neg(ff_div(sum_lanes(s[u], 4), best));
+      const FF g = ff_neg(ff_div(s[u], best));
       float t = 0.f;
       if (on[u])
 #pragma unroll 4
@@ -273,9 +338,9 @@ __global__ void __launch_bounds__(ONT, CPG == 1 ? 5 : 3)
           put(i, c, w);
           t = fmaf(w.h, w.h, t);
         }
-      t = sum_lanes(t, 4);
-      if (l8 == 0 && c < pc) nrm[(j + 1) & 1][c] = t;
+      give_norm(sum_lanes(t, 4), c, nrm[(j + 1) & 1]);
     }
+    take_norms(nrm[(j + 1) & 1]);
     __syncthreads();
   }
   if (tid < r) bn[tid] = ff_rsqrt(bn[tid]);
@@ -286,18 +351,37 @@ __global__ void __launch_bounds__(ONT, CPG == 1 ? 5 : 3)
   };
   if (SMEM) {
     for (int j = warp; j < r; j += NW)
-      for (int i = lane; i < m; i += 32) Yg[i + (int64_t)j * m] = unit(i, j);
+      for (int i = lane; i < m; i += 32) Yg[i + gld * j] = unit(i, j);
   } else {   // a thread owns its rows: all of one read before any is written
     for (int i = tid; i < m; i += ONT) {
       float row[CMAX];
       for (int j = 0; j < r; ++j) row[j] = unit(i, j);
-      for (int j = 0; j < r; ++j) Yg[i + (int64_t)j * m] = row[j];
+      for (int j = 0; j < r; ++j) Yg[i + gld * j] = row[j];
     }
   }
-  if (tid == 0) {
+  if (tid == 0 && rank == 0) {
     rs[ti.r_ri] = r;
-    if (flops) atomicAdd(flops, 2.0 * m * r * (2.0 * pc - r));
+    if (flops) atomicAdd(flops, 2.0 * ti.m * r * (2.0 * pc - r));
   }
+}
+
+template <int MODE, int CPG>
+__global__ void __launch_bounds__(ONT, CPG == 1 ? 5 : 3)
+    k_orth(const TInfo* __restrict__ tis, const int* __restrict__ order, FF tau2,
+           float* const* __restrict__ tab, int* const* __restrict__ rtab, int P, int scr_buf,
+           int scr_rbuf, const StackDim* __restrict__ stack,
+           unsigned long long* __restrict__ sketch_stat, double* __restrict__ flops) {
+  orth<MODE, CPG>(tis[order[blockIdx.x]], 0, tau2, tab, rtab, P, scr_buf, scr_rbuf, stack,
+                  sketch_stat, flops);
+}
+template <int CPG>
+__global__ void __cluster_dims__(OCL, 1, 1) __launch_bounds__(ONT, CPG == 1 ? 5 : 3)
+    k_orth_cluster(const TInfo* __restrict__ tis, const int* __restrict__ order, FF tau2,
+                   float* const* __restrict__ tab, int* const* __restrict__ rtab, int P,
+                   int scr_buf, int scr_rbuf, const StackDim* __restrict__ stack,
+                   unsigned long long* __restrict__ sketch_stat, double* __restrict__ flops) {
+  orth<ORTH_CLUSTER, CPG>(tis[order[blockIdx.x / OCL]], blockIdx.x % OCL, tau2, tab, rtab, P,
+                          scr_buf, scr_rbuf, stack, sketch_stat, flops);
 }
 
 // ------------------------------------------------------------ Jacobi cores
@@ -841,34 +925,37 @@ void launch_orth(const Plan& pl, double tau, float* const* d_tab, int* const* d_
   const int nt = (int)pl.torder.size();
   if (nt <= 0 || P <= 0) return;
   // Targets are listed by increasing sketch size; each launch takes those up to
-  // the next of these shared-memory sizes (4, 3, 2 and 1 CTA per SM), so that
-  // small sketches do not pay for the large ones' occupancy.  Few targets fill
-  // no SM twice anyway and go in one launch.  Sketches beyond the largest size
+  // the next of these shared-memory sizes (4, 3 and 2 CTAs per SM; one CTA of a cluster
+  // of OCL), so that small sketches do not pay for the large ones' occupancy.  Few
+  // targets fill no SM twice anyway and need no classes.  Sketches beyond the largest size
   // stay in global memory (L2).
-  static const size_t cls[4] = {55296, 74752, 112640, 225280};
   constexpr int NCLS = 4;
+  static const size_t cls[NCLS] = {55296, 74752, 112640, 221184};
   const double t2 = tau * tau;
   const FF tau2{(float)t2, (float)(t2 - (double)(float)t2)};
-  auto bytes = [&](int q) {
+  auto bytes = [&](int q, int c) {   // per CTA
     const TInfo& ti = pl.targets[pl.torder[q]];
-    return (size_t)orth_ld(ti.m) * ti.p * sizeof(FF);
+    const int rows = c < NCLS - 1 ? ti.m : (ti.m + OCL - 1) / OCL;
+    return (size_t)orth_ld(rows) * ti.p * sizeof(FF);
   };
-  const bool few = (int64_t)nt * P <= device_sm_count();
+  const bool few = (int64_t)nt * P <= device_sm_count(), narrow = pl.max_p <= 32;
   int beg = 0;
-  for (int c = few ? NCLS - 1 : 0; c <= NCLS && beg < nt; ++c) {
+  for (int c = few ? NCLS - 2 : 0; c <= NCLS && beg < nt; ++c) {
     int end = nt;
     if (c < NCLS)
-      for (end = beg; end < nt && bytes(end) <= cls[c]; ++end) {}
+      for (end = beg; end < nt && bytes(end, c) <= cls[c]; ++end) {}
     if (end > beg) {
-      auto kern = c < NCLS ? (pl.max_p <= 32 ? k_orth<true, 1> : k_orth<true, 2>)
-                           : (pl.max_p <= 32 ? k_orth<false, 1> : k_orth<false, 2>);
+      auto kern = c < NCLS - 1    ? (narrow ? k_orth<ORTH_SM, 1> : k_orth<ORTH_SM, 2>)
+                  : c == NCLS - 1 ? (narrow ? k_orth_cluster<1> : k_orth_cluster<2>)
+                                  : (narrow ? k_orth<ORTH_GLOBAL, 1> : k_orth<ORTH_GLOBAL, 2>);
       size_t smem = 0;   // (padded: not quite in the targets' order)
-      for (int q = beg; c < NCLS && q < end; ++q) smem = std::max(smem, bytes(q));
+      for (int q = beg; c < NCLS && q < end; ++q) smem = std::max(smem, bytes(q, c));
       if (smem > 40 * 1024)   // (48 KB without it, the kernel's own arrays included)
         ACR_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      (int)cls[NCLS - 1]));
-      for (int t0 = beg; t0 < end; t0 += 65535) {
-        kern<<<dim3(std::min(65535, end - t0), P), ONT, smem, st>>>(
+                                      (int)cls[c < NCLS - 1 ? NCLS - 2 : NCLS - 1]));
+      const int wide = c == NCLS - 1 ? OCL : 1;   // CTAs per target
+      for (int t0 = beg; t0 < end; t0 += 65535 / OCL) {
+        kern<<<dim3(std::min(65535 / OCL, end - t0) * wide, P), ONT, smem, st>>>(
             (const TInfo*)pl.d_targets, (const int*)pl.d_torder + t0, tau2, d_tab, d_rtab, P,
             3 * pl.nroles, pl.nroles, (const StackDim*)pl.d_stack, d_sketch_stat, d_fl);
         ACR_LAUNCHED(1);

@@ -236,9 +236,11 @@ int main() {
     orth_ranks(144, 40, 1e-5, scale);    // 47.5 KB, beside the kernel's own arrays
     orth_ranks(288, 42, 1e-5, scale);
     orth_ranks(400, 32, 1e-6, scale);
-    orth_ranks(800, 34, 1e-5, scale);    // a whole SM's
-    orth_ranks(1152, 56, 1e-5, scale);   // beyond shared memory
+    orth_ranks(800, 34, 1e-5, scale);    // a cluster's, with rows to spare
+    orth_ranks(1152, 56, 1e-5, scale);
   }
+  orth_ranks(1001, 30, 1e-5, 1.0);       // a cluster's, whose last CTA has fewer rows
+  orth_ranks(4096, 56, 1e-5, 1.0);       // beyond a cluster's shared memory
   for (int r : {1, 2, 3, 12, 31, 56}) {
     core<double>(64, 50, r, 1e-2, 0.5);
     core<double>(100, 300, r, 1e-7, 0.8);

@@ -10,11 +10,11 @@ import re
 import pytest
 
 ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
-SOURCE = os.path.join(ROOT, "paper_1712_08872_gb300", "csrc", "acr_setup_kernels.cu")
+CSRC = os.path.join(ROOT, "paper_1712_08872_gb300", "csrc")
 
 
-def kernel_body(name):
-    with open(SOURCE) as fh:
+def kernel_body(source, name):
+    with open(os.path.join(CSRC, source)) as fh:
         text = re.sub(r"//[^\n]*", "", fh.read())
     at = text.index("{", text.index(name + "("))
     depth = 0
@@ -26,10 +26,12 @@ def kernel_body(name):
 
 
 # (kernel, what a CTA sets in its own shared memory that others write into)
-@pytest.mark.parametrize("name,setup", [("k_leaf_inv_d", "step[tid] = -1;"),
-                                        ("k_leaf_inv_f", None)])
-def test_cluster_has_started_before_the_first_remote_write(name, setup):
-    body = kernel_body(name)
+@pytest.mark.parametrize("source,name,setup", [
+    ("acr_setup_kernels.cu", "k_leaf_inv_d", "step[tid] = -1;"),
+    ("acr_setup_kernels.cu", "k_leaf_inv_f", None),
+    ("acr_core_kernels.cu", "void orth", None)])
+def test_cluster_has_started_before_the_first_remote_write(source, name, setup):
+    body = kernel_body(source, name)
     remote = body.index("map_shared_rank")
     sync, arrive, wait = (body.find(c) for c in ("cl.sync()", "cl.barrier_arrive()",
                                                  "cl.barrier_wait()"))
