@@ -4,8 +4,8 @@ Workload (default): the nonsymmetric convection-diffusion operator
 -Lap u + beta . grad u at n = 128 (2,097,152 unknowns), beta =
 (50,50,50)(1 + 0.5 sin 2 pi x sin 2 pi y), first-order upwind, f ~ U(-1,1)
 (seed 20); ACR with eps = 1e-2, eta = 2, leaf 64, factors in FP32 (the mixed
-form: FP64 leaf inverses, recompression cores and Krylov); FP64
-GMRES(30), right-preconditioned, rtol 1e-8.
+form: leaf inverses refined to float, bases and cores in float-float);
+FP64 GMRES(30), right-preconditioned, rtol 1e-8.
 
 One step = acr_setup (coefficients already on the device) + acr_krylov_solve
 + acr_destroy.  `value` is seconds per solve for the whole job: with N
@@ -502,7 +502,8 @@ def main():
         traffic = bpf * ds.flops / ds.launches if (bpf is not None and ds.launches) else None
         roof = {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
                 "frac": achieved / peak, "traffic": traffic, "traffic_unit": "bytes per launch",
-                "traffic_source": tsrc, "kernel": "k_ggemm/k_gdot<float> (grouped GEMM family)",
+                "traffic_source": tsrc, "kernel": "k_gcat/k_gbundle/k_tdot/k_gdot_warp<float>, k_gwarp where tuned "
+                          "(grouped GEMM family)",
                 "peak_source": "derived: %d SMs x 128 FP32 lanes x 2 x max SM clock" % sms,
                 "launches": ds.launches, "ms_total": ds.ms}
     else:
@@ -713,7 +714,7 @@ def main():
             "scaling": "weak", "vs_baseline": None, "dtype": "f32", "data": "synthetic",
             "config": {"workload": "codi_n128_acr_gmres30", "n": n, "unknowns": N, "eps": eps,
                        "eta": eta, "leaf": leaf, "rank_cap": args.rank_cap,
-                       "form": "FP32 factors; FP64 leaf inverses, cores and GMRES",
+                       "form": "FP32 factors; leaf inverses refined to float, bases and cores float-float; FP64 GMRES",
                        "parallelism": "replicas" if world > 1 else "single",
                        "l2": "inputs larger than L2 (factors tens of GB)"},
             "iterations": solve_info.iterations, "rel_residual": solve_info.rel_residual,

@@ -132,7 +132,7 @@ typedef struct {
 } acr_kernel_stat;
 
 typedef struct {
-  acr_kernel_stat gemm;      /* grouped small GEMMs (k_ggemm) */
+  acr_kernel_stat gemm;      /* grouped small GEMMs (k_gcat, k_gbundle, k_tdot, k_gdot_warp; tuned shapes) */
   acr_kernel_stat orth;      /* FP64 pivoted-Cholesky cores (k_pchol); float factors: basis kernel (k_orth) */
   acr_kernel_stat eig;       /* core Grams, Jacobi cores and recomposition (k_core) */
   acr_kernel_stat leaf_inv;  /* dense leaf inverses (k_leaf_inv; refined float for float factors) */

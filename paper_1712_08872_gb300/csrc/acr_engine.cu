@@ -883,8 +883,8 @@ class Engine : public EngineBase {
     }
   }
 
-  // One GEMM stage of a plan (grouped small GEMMs on the CUDA cores; float
-  // Grams with compensated accumulation and FP64 results).
+  // One GEMM stage of a plan (grouped small GEMMs on the CUDA cores, in the storage
+  // precision; what decides ranks has stages of its own).
   void gemm_stage(const Plan& pl, const Stage& sg, T* const* d_tab, const int* const* d_rtab,
                   int pc, cudaStream_t st) {
     double* f = sg.tag >= 0 ? fl(5 + sg.tag) : fl(0);
@@ -905,9 +905,9 @@ class Engine : public EngineBase {
 
   double tau_orth() const {
     // range-finder truncation: three orders below eps, never below the
-    // relative noise floor of the sketch in the storage precision (the
-    // Grams are FP64-accurate in every form: 1e-7 for FP64 data, 1e-6 for
-    // float data, whose own rounding is ~6e-8)
+    // relative noise floor of the sketch: 1e-7 for FP64 data (the square root
+    // of a Gram's rounding, with a margin), 1e-6 for float data, whose own rounding is ~6e-8 (its basis
+    // is float-float: k_orth)
     const double floor_ = sizeof(T) == 8 ? 1e-7 : 1e-6;
     return std::max(1e-3 * eps, floor_);
   }

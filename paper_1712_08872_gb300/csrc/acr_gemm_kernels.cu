@@ -1673,7 +1673,7 @@ void launch_ggemm(const Plan& pl, int gbeg, int gend, T* const* d_tab, const int
   // A stage of few groups per plane leaves most of the SMs idle whenever few
   // planes are left: its outputs' columns are then split over 2 or 4 CTAs.  (By the
   // plan alone, not by P: a plane's result must not depend on the batch.)
-  const int zsplit = ng <= 38 ? 4 : ng <= 76 ? 2 : 1;
+  const int zsplit = 4 * ng <= PART_SMS ? 4 : 2 * ng <= PART_SMS ? 2 : 1;
   const int maxg = 65535;
   for (int g0 = 0; g0 < ng; g0 += maxg) {
     dim3 grid(std::min(maxg, ng - g0), P);
@@ -1682,10 +1682,10 @@ void launch_ggemm(const Plan& pl, int gbeg, int gend, T* const* d_tab, const int
     // warp per group for the inner products, and for the small-output
     // sketch / projection stages where the multiply type is float (the FP64
     // instance of the warp kernel holds ~200 registers: one CTA per SM)
-    // variant 1 swaps the warp-per-group and CTA-per-group inner-product
-    // kernels; for float it gives the staged kernel 3 CTAs per SM and 80
-    // registers (no spills) instead of 4 CTAs and 64 registers, for double
-    // half the staging per K-step.  Variant 2 (float, non-dot stages) runs
+    // Variant 0: k_gcat.  Variant 1 swaps the warp-per-group and CTA-per-group
+    // inner-product kernels and takes k_ggemm, item by item, for the others
+    // (float: 3 CTAs per SM and 80 registers; double: half the staging per
+    // K-step).  Variant 2 (float, non-dot stages) runs
     // one warp per group (k_gwarp, 8 columns per pass); variant 3 as 2, with
     // the wide groups on the tensor cores; variant 4 as 2 with 32 columns per
     // pass; variant 5 (float, inner-product stages) 8 x 8 warp tiles.

@@ -621,11 +621,11 @@ bool same_a(const Plan& pl, const GGroup& x, const GGroup& y) {
 }
 
 // Bundles of a factor stage's narrow groups, in the order of their first group.
-// Small stages keep more, smaller bundles (at least ~150, one per SM, where
-// there are that many groups).
+// Small stages keep more, smaller bundles (at least one per SM, where there are
+// that many groups).
 void make_bundles(Plan& plan, Stage& sg) {
   const int beg = sg.beg + sg.nwide, n = sg.end - beg;
-  const int most = std::max(1, std::min(BUNDLE_MAX, n / 152));
+  const int most = std::max(1, std::min(BUNDLE_MAX, n / PART_SMS));
   std::unordered_map<uint64_t, int> open;   // key -> its last bundle
   open.reserve(n);
   std::vector<int> of(n), size, first;      // bundle of each group; size and first group of each

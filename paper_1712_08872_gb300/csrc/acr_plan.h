@@ -129,6 +129,9 @@ inline bool tag_is_dot(int t) {
 // blocks), so that a kernel can stage those operands once per bundle.
 struct Stage { int kind; int beg, end; int tag = -1; int nwide = 0; int bbeg = 0, bend = 0; };
 constexpr int BUNDLE_MAX = 16;   // groups per bundle
+// SMs of the part that stages of few groups are dealt for (a fixed number: how a sum is
+// split must not depend on the device or the batch)
+constexpr int PART_SMS = 152;
 
 // Operand roles: role r owns buffers 3r (dense), 3r+1 (U), 3r+2 (V) and
 // rank buffer r.  The scratch real buffer is 3*nroles, the scratch rank
