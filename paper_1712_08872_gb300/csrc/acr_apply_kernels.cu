@@ -407,10 +407,11 @@ __device__ __forceinline__ void load4(const __nv_bfloat16* p, float (&v)[4]) {
 // row of D^T) per lane and reduces the 16 quads of a row with shuffles.
 // Partial sums (at most 4 dense products, or half a leaf's rank) enter
 // compensated float pairs; warps combine through shared memory in a fixed
-// order.  Bound by HBM where many planes are left: n = 128, FP32, one apply (18 GB)
-// 6.37 ms, transposed 7.81 ms; with the dense loop unrolled twice 6.92 and 8.60 ms
-// (n = 64: 1.147 and 1.413 against 1.175 and 1.468): eight loads in flight per
-// thread are paid for with resident warps.
+// order.  Bound by HBM where many planes are left: n = 128, FP32, one apply (24.4 GB)
+// 6.38 ms, transposed 7.83 ms, with one dense leaf in flight per CTA; two (the loop
+// unrolled twice, eight 16-byte loads per thread) take 6.95 and 8.65 ms.  Bfloat16, whose
+// loads are half as wide: two in flight 5.69 and 7.41 ms, one 5.96 and 7.47 ms.  n = 64: 1.16
+// against 1.19 and 1.01 against 1.07 ms.
 template <typename T>
 __global__ void __launch_bounds__(256) k_hmv_rows_v1(MatvecDev mv, T* const* __restrict__ D,
                                                      T* const* __restrict__ U,
@@ -472,6 +473,8 @@ __global__ void __launch_bounds__(256) k_hmv_rows_v1(MatvecDev mv, T* const* __r
   const int rl = tid & 15, cg = tid >> 4;
   if (have) {
     const T* Dp = D[p];
+    constexpr int LEAVES = sizeof(T) == 2 ? 2 : 1;   // in flight
+#pragma unroll LEAVES
     for (int q = 0; q < nd; ++q) {
       const T* blk = Dp + (int64_t)(q < MAXQ ? s_leaf[q] : dleaf[d0 + q]) * 4096;
       const float* xq = xs + q * 64;

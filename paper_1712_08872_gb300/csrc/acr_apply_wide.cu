@@ -12,10 +12,11 @@
 // compensated float pairs, at every leaf size.
 //
 // The products are 64 x K x 32 with K of a few hundred to a thousand: CUDA-core
-// work of 32 multiply-adds per loaded entry, bound by shared-memory reads (two 16-byte
-// vectors per 16 products; 8 x 4 outputs per thread with the contraction split over two
-// halves of the CTA read less but held 128 registers and were slower: 104 against
-// 90 us with sums of 64).  A tcgen05 form (split TF32, M = 128 with hi and lo rows stacked) spent its
+// work of 32 multiply-adds per loaded entry, bound by issue slots (2.6 of 4 per clock, FMA
+// pipe 48%: the compensated additions take nearly as many as the products) and shared
+// memory at half its rate (two 16-byte vectors per 16 products; 8 x 4 outputs per thread
+// with the contraction split over two halves of the CTA read less but held 128 registers
+// and were slower: 104 against 90 us with sums of 64).  A tcgen05 form (split TF32, M = 128 with hi and lo rows stacked) spent its
 // time staging -- both operands through registers for the split, in core-matrix
 // order, the vectors converted from FP64 again for every chunk that reads them --
 // and took 236 us per launch on average for the n = 64 Helmholtz recipe (4096
