@@ -913,12 +913,27 @@ class Engine : public EngineBase {
   }
 
   // ------------------------------------------------------------ H-inverse
-  void hinv(int t, const std::vector<std::vector<HM>>& roles, void* d_xdense, int P,
+  // The device table of the planes' dense leaves, for the leaf inverses of one H-inverse: kept
+  // until the ring that holds it comes round (small scratch makes an inverse push many tables).
+  struct LeafTable {
+    std::vector<void*> host;
+    int64_t epoch = -1;
+    void* dev = nullptr;
+  };
+  void* leaf_table(LeafTable& t, cudaStream_t st) {
+    if (t.epoch != ring.epoch) {
+      t.dev = ring.push(t.host.data(), sizeof(void*) * t.host.size(), st);
+      t.epoch = ring.epoch;   // (the push itself may have begun a new one)
+    }
+    return t.dev;
+  }
+  void hinv(int t, const std::vector<std::vector<HM>>& roles, LeafTable& leaves, int P,
             cudaStream_t st) {
     const Cluster& c = S.cl[t];
     if (c.child[0] < 0) {
       int nd = S.node(t, t);
-      timed(3, [&] { launch_leaf_inv<T>((T* const*)d_xdense, S.dense_off(S.bn[nd].leaf), S.lsz, P,
+      T* const* xd = (T* const*)leaf_table(leaves, st);
+      timed(3, [&] { launch_leaf_inv<T>(xd, S.dense_off(S.bn[nd].leaf), S.lsz, P,
                                         d_err, st, fl(3), d_sketch_stat + 2); });
       return;
     }
@@ -931,12 +946,12 @@ class Engine : public EngineBase {
       op.prods.push_back(OpDesc::Prod{an, bn, ar, br, coef});
       return op;
     };
-    hinv(t1, roles, d_xdense, P, st);
+    hinv(t1, roles, leaves, P, st);
     run_merged({mk(n12, 1, -1, n11, 0, n12, 0, 0),      // T12 = X11 A12
                 mk(n21, 1, -1, n21, 0, n11, 0, 0)},     // T21 = A21 X11
                roles, P, st);
     run_split(mk(n22, 0, 0, n21, 0, n12, 1, 1), roles, P, st);    // S = A22 - A21 T12
-    hinv(t2, roles, d_xdense, P, st);
+    hinv(t2, roles, leaves, P, st);
     run_merged({mk(n12, 0, -1, n12, 1, n22, 0, 1),      // X12 = -T12 X22
                 mk(n21, 0, -1, n22, 0, n21, 1, 1)},     // X21 = -X22 T21
                roles, P, st);
@@ -958,10 +973,9 @@ class Engine : public EngineBase {
   void hinv_batch(std::vector<std::vector<HM>> roles, cudaStream_t st) {
     const int P = (int)roles[0].size();
     if (P == 0) return;
-    std::vector<void*> xd(P);
-    for (int p = 0; p < P; ++p) xd[p] = roles[0][p].dense;
-    void* d_xdense = ring.push(xd.data(), sizeof(void*) * P, st);
-    hinv(0, roles, d_xdense, P, st);
+    LeafTable leaves;
+    for (int p = 0; p < P; ++p) leaves.host.push_back(roles[0][p].dense);
+    hinv(0, roles, leaves, P, st);
     for (HM& h : roles[1]) free_hm(h);   // reusable by later launches (stream order)
   }
 
